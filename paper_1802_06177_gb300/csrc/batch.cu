@@ -129,6 +129,8 @@ QueuePlan plan_queue(slmc_batch* b, int nsweeps) {
         C.delta = c->p.sweep_delta;
         C.key0 = (uint32_t)(c->p.seed & 0xffffffffu);
         C.key1 = (uint32_t)(c->p.seed >> 32);
+        C.mhalf = slmc::div_magic((long long)c->N * (c->L / 2), c->L / 2);
+        C.mlx = slmc::div_magic(c->N, c->p.Lx);
         P.cls.push_back(C);
         P.nchains += b->nchains[q];
         P.max_N = std::max(P.max_N, c->N);

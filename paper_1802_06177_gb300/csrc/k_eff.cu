@@ -12,6 +12,7 @@
 // Site i = ix + Lx iy, field element (i, l) at i*L + l. All reductions use a fixed
 // order (per-thread strided partial sums, then a shared-memory tree), so results are
 // reproducible run to run.
+#include <algorithm>
 #include <cfloat>
 
 #include "slmc_internal.cuh"
@@ -104,81 +105,146 @@ __device__ __forceinline__ double ldx(const double* p) {
     return *p;
 }
 
+// FP32 value of v rounded toward zero, by integer operations: the conversion instruction shares the
+// FP64 pipe, whose two lanes per clock bound the sweeps when every site converts its seven operands
+// there. |v| below 2^-126 gives 0; above the FP32 range, infinities and NaN give infinity (the caller's
+// finiteness test then sends the site to the FP64 rule).
+__device__ __forceinline__ float trunc_f32(double v) {
+    const int hi = __double2hiint(v);
+    const int t = (hi & 0x7fffffff) - 0x38000000;  // exponent rebased from FP64 to FP32
+    uint32_t m = __funnelshift_l((uint32_t)__double2loint(v), (uint32_t)t, 3);
+    if (t < 0x00100000) m = 0u;
+    if (t >= 0x0ff00000) m = 0x7f800000u;
+    return __uint_as_float((m & 0x7fffffffu) | ((uint32_t)hi & 0x80000000u));
+}
+
+// n / d for the divisors of a lattice (half the slices, Lx) by one multiply-high: exact while n d < 2^32
+// (q = floor(n ceil(2^32 / d) / 2^32)); magic 0 selects the division.
+__device__ __forceinline__ int fast_div(int n, int d, uint32_t magic) {
+    return magic ? (int)__umulhi((uint32_t)n, magic) : n / d;
+}
+
+// Couplings and constants of one chain's sweeps, FP64 for the exact rule and FP32 for the fast test, kept in
+// shared memory.
+struct SweepConst {
+    double J[6];
+    double dtau, a2, delta, ds;  // ds = delta 2^-52
+    float Jf[6];
+    float Jm[6];  // magnitudes
+    float dtauf, a2f, deltaf;
+    int plain;  // delta too small for ds to be normal: the proposal step by step
+};
+
+// Filled by the threads of one warp or more (caller synchronises).
+__device__ __forceinline__ void sweep_const_init(SweepConst& C, const double* __restrict__ Jg, double dtau, double a2,
+                                                 double delta) {
+    if (threadIdx.x < 6) {
+        const double j = Jg[threadIdx.x];
+        C.J[threadIdx.x] = j;
+        C.Jf[threadIdx.x] = (float)j;
+        C.Jm[threadIdx.x] = fabsf((float)j);
+    }
+    if (threadIdx.x == 0) {
+        C.dtau = dtau;
+        C.a2 = a2;
+        C.delta = delta;
+        C.ds = delta * (1.0 / 4503599627370496.0);
+        C.dtauf = (float)dtau;
+        C.a2f = (float)a2;
+        C.deltaf = (float)delta;
+        C.plain = !(delta == 0.0 || delta > 1e-250);
+    }
+}
+
 // Metropolis update of site pair s of colour c in one chain's field (thread s of the half-sweep
 // owns site i = s / (L/2) and the slice l of colour c in the pair (2 (s mod L/2), 2 (s mod L/2) + 1)).
-// Returns 1 if the move was accepted (and written).
+// ld is the row stride of the field. Returns 1 if the move was accepted (and written).
+//
+// Three FP64 operations per site (the proposal), everything else on the FP32 and integer pipes: with the
+// operands converted and the uniforms formed in FP64 the kernel was bound by that pipe (two lanes per clock
+// per SM): a half-sweep of 512 chains of 16x16, L = 160 took 524 us that way and takes 150 us now.
 template <bool kL2>
-__device__ __forceinline__ int site_update(double* xfield, int Lx, int Ly, int L, const double* J, double dtau,
-                                           double a2, double delta, uint32_t key0, uint32_t key1, uint32_t sweep,
-                                           int c, int s, uint32_t chain) {
-    const int half = L / 2;
-    const int i = s / half, lp = s - i * half;
-    const int ix = i % Lx, iy = i / Lx;
+__device__ __forceinline__ int site_update(double* xfield, int Lx, int Ly, int L, int ld, uint32_t mhalf, uint32_t mlx,
+                                           const SweepConst& C, uint32_t key0, uint32_t key1, uint32_t sweep, int c, int s,
+                                           uint32_t chain) {
+    const int half = L >> 1;
+    const int i = fast_div(s, half, mhalf), lp = s - i * half;
+    const int iy = fast_div(i, Lx, mlx), ix = i - iy * Lx;
     const int l = 2 * lp + ((ix + iy + c) & 1);
-    const double v = ldx<kL2>(xfield + (size_t)i * L + l);
-    const double up = ldx<kL2>(xfield + (size_t)i * L + (l + 1 == L ? 0 : l + 1));
-    const double dn = ldx<kL2>(xfield + (size_t)i * L + (l == 0 ? L - 1 : l - 1));
+    double* xi = xfield + (size_t)i * ld;
+    const double v = ldx<kL2>(xi + l);
+    const double up = ldx<kL2>(xi + (l + 1 == L ? 0 : l + 1));
+    const double dn = ldx<kL2>(xi + (l == 0 ? L - 1 : l - 1));
     const int xp = (ix + 1 == Lx ? 0 : ix + 1) + Lx * iy, xm = (ix == 0 ? Lx - 1 : ix - 1) + Lx * iy;
     const int yp = ix + Lx * (iy + 1 == Ly ? 0 : iy + 1), ym = ix + Lx * (iy == 0 ? Ly - 1 : iy - 1);
-    const double nb = ldx<kL2>(xfield + (size_t)xp * L + l) + ldx<kL2>(xfield + (size_t)xm * L + l) +
-                      ldx<kL2>(xfield + (size_t)yp * L + l) + ldx<kL2>(xfield + (size_t)ym * L + l);
+    const double n0 = ldx<kL2>(xfield + (size_t)xp * ld + l), n1 = ldx<kL2>(xfield + (size_t)xm * ld + l);
+    const double n2 = ldx<kL2>(xfield + (size_t)yp * ld + l), n3 = ldx<kL2>(xfield + (size_t)ym * ld + l);
     const slmc::u32x4 w = slmc::philox4x32_10(slmc::u32x4{(uint32_t)(i * L + l), sweep, chain, 0u}, key0, key1);
-    const double u1 = slmc::uniform53(w.x, w.y);
-    // x' = x + delta (2 u1 - 1), rounded step by step (no contraction) as in the oracle
-    const double xn = __dadd_rn(v, __dmul_rn(delta, __dadd_rn(__dmul_rn(2.0, u1), -1.0)));
+    // x' = x + delta (2 u1 - 1), rounded step by step (no contraction) as in the oracle. With u1 = r 2^-53,
+    // 2 u1 - 1 = (r - 2^52) 2^-52 is exact: r mod 2^52 is placed in the significand of 2^52 and 2^52 or 2^53 is
+    // subtracted (exact), and delta 2^-52 times it rounds as delta times (2 u1 - 1) does.
+    double xn;
+    if (!C.plain) {
+        const double big = __hiloint2double(0x43300000 | (int)((w.x >> 11) & 0xfffffu),
+                                            (int)(((w.x << 21) & 0xfc000000u) | (w.y >> 6)));
+        const double off = __hiloint2double(0x43400000 - (int)((w.x >> 31) << 20), 0);
+        xn = __dadd_rn(v, __dmul_rn(C.ds, __dadd_rn(big, -off)));
+    } else {
+        const double u1 = slmc::uniform53(w.x, w.y);
+        xn = __dadd_rn(v, __dmul_rn(C.delta, __dadd_rn(__dmul_rn(2.0, u1), -1.0)));
+    }
     // Fast decision in FP32: dE = d [2 J_k (s - up - dn) + s (J_p ((x'^2 + x^2)/4 - a^2/2)
     //   + J_p' ((x'^4 + x'^2 x^2 + x^4)/6 - a^2 (x'^2 + x^2)/4)) + J_nn nb + J_nn' (up + dn)],
-    // d = x' - x, s = x' + x (the exact difference of the local energies, factored). The FP32
-    // verdict is used only when the log-ratio is further from log u than a margin bounding
-    // (i) the FP32 rounding of the bracket (1e-5 of the sum of the magnitudes of its terms,
-    // about 170 units of FP32 rounding), (ii) the rounding of x, x' to FP32, which moves d by
-    // up to 2^-24 (|x| + |x'|), and (iii) the truncation of u to 24 bits (log u is known to
-    // within 2^-24 / u); otherwise the exact FP64 rule of the oracle decides.
-    const float vf = (float)v, xf = (float)xn, upf = (float)up, dnf = (float)dn, nbf = (float)nb;
-    const float d = xf - vf, sm = xf + vf, x2 = xf * xf, v2 = vf * vf, a2f = (float)a2;
-    const float tk = 2.f * (float)J[1] * (sm - upf - dnf);
-    const float tp = sm * (float)J[2] * (0.25f * (x2 + v2) - 0.5f * a2f);
-    const float tpp = sm * (float)J[3] * ((x2 * x2 + x2 * v2 + v2 * v2) * (1.f / 6.f) - 0.25f * a2f * (x2 + v2));
-    const float tn = (float)J[4] * nbf + (float)J[5] * (upf + dnf);
-    const float mag = 2.f * fabsf((float)J[1]) * (fabsf(sm) + fabsf(upf) + fabsf(dnf)) +
-                      fabsf(sm) * (fabsf((float)J[2]) * (x2 + v2 + a2f) +
-                                   fabsf((float)J[3]) * (x2 * x2 + x2 * v2 + v2 * v2 + a2f * (x2 + v2))) +
-                      fabsf((float)J[4] * nbf) + fabsf((float)J[5]) * (fabsf(upf) + fabsf(dnf));
-    const float dlnw32 = -(float)dtau * d * (tk + tp + tpp + tn);
-    const float uf = (float)(w.z >> 8) * 5.9604644775390625e-8f;  // top 24 bits of the acceptance uniform
-    int decided = 0, acc = 0;
-    if (uf > 0.f && isfinite(dlnw32) && isfinite(mag)) {
-        const float lu = logf(uf);
-        const float margin =
-            1e-5f + (float)dtau * mag * (1e-5f * fabsf(d) + 2e-7f * (fabsf(xf) + fabsf(vf))) + 1.2e-7f / uf;
-        if (dlnw32 > lu + margin) {
-            decided = 1;
-            acc = 1;
-        } else if (dlnw32 < lu - margin) {
-            decided = 1;
-            acc = 0;
-        }
-    }
+    // d = x' - x, s = x' + x (the exact difference of the local energies, factored), from truncated
+    // operands (relative error 2^-23) and d = delta (2 u1 - 1) from the top 23 bits of u1 (absolute
+    // error 2^-22 delta, entering the bracket too: at most 5 2^-22 delta in all; and the rounding of
+    // x' to FP64, 2^-53 |x'|). The FP32 verdict is used only
+    // when the log-ratio is further from log u than a margin bounding (i) the FP32 rounding of the
+    // bracket (1e-5 of the sum of the magnitudes of its terms, about 170 units of FP32 rounding),
+    // (ii) the error of d, (iii) the truncation of u to 23 bits (log u is known to within 2^-23 / u)
+    // and (iv) the hardware logarithm (documented: 2^-21.41 absolute on [0.5, 2], 3 units elsewhere;
+    // |log u| < 16, so below 4e-6); otherwise the exact FP64 rule of the oracle decides.
+    const float vf = trunc_f32(v), upf = trunc_f32(up), dnf = trunc_f32(dn);
+    const float f0 = trunc_f32(n0), f1 = trunc_f32(n1), f2 = trunc_f32(n2), f3 = trunc_f32(n3);
+    const float nbf = (f0 + f1) + (f2 + f3), nbm = (fabsf(f0) + fabsf(f1)) + (fabsf(f2) + fabsf(f3));
+    const float d = C.deltaf * fmaf(2.f, __uint_as_float(0x3f800000u | (w.x >> 9)), -3.f);
+    const float xf = vf + d;
+    const float sm = xf + vf, x2 = xf * xf, v2 = vf * vf, q2 = x2 + v2, q4 = fmaf(x2, q2, v2 * v2);
+    const float ud = upf + dnf, am = fabsf(upf) + fabsf(dnf), sa = fabsf(xf) + fabsf(vf);
+    const float tk = 2.f * C.Jf[1] * (sm - ud);
+    const float tp = C.Jf[2] * fmaf(0.25f, q2, -0.5f * C.a2f) + C.Jf[3] * (q4 * (1.f / 6.f) - 0.25f * C.a2f * q2);
+    const float tn = C.Jf[4] * nbf + C.Jf[5] * ud;
+    const float mag = 2.f * C.Jm[1] * (sa + am) + sa * (C.Jm[2] * (q2 + C.a2f) + C.Jm[3] * (q4 + C.a2f * q2)) +
+                      C.Jm[4] * nbm + C.Jm[5] * am;
+    const float dlnw32 = -C.dtauf * d * (tk + fmaf(sm, tp, tn));
+    const float uf = __uint_as_float(0x3f800000u | (w.z >> 9)) - 1.f;  // top 23 bits of the acceptance uniform
+    const float lu = __logf(uf);
+    const float margin = 1.4e-5f + C.dtauf * mag * (1e-5f * fabsf(d) + 1.2e-6f * C.deltaf + 1e-14f * sa) +
+                         __fdividef(1.3e-7f, uf);
+    // uf = 0 makes the margin infinite, an operand out of FP32 range makes mag infinite: both comparisons fail
+    int acc = dlnw32 > lu + margin;
+    const bool decided = (acc || dlnw32 < lu - margin) && fabsf(dlnw32) < 3e38f;
     if (!decided) {  // exact FP64 rule of the oracle
+        const double nb = ((n0 + n1) + n2) + n3;
         const double u2 = slmc::uniform53(w.z, w.w);
-        const double dE = local_energy(J, a2, xn, up, dn, nb) - local_energy(J, a2, v, up, dn, nb);
-        const double dlnw = -dtau * dE;
+        const double dE = local_energy(C.J, C.a2, xn, up, dn, nb) - local_energy(C.J, C.a2, v, up, dn, nb);
+        const double dlnw = -C.dtau * dE;
         acc = (dlnw >= 0.0 || u2 < exp(dlnw)) ? 1 : 0;
     }
-    if (acc) xfield[(size_t)i * L + l] = xn;
+    if (acc) xi[l] = xn;
     return acc;
 }
 
 // One checkerboard half-sweep over all chains: thread s of chain f updates site pair s.
-__global__ void __launch_bounds__(kThreads) k_half_sweep(double* __restrict__ x, int Lx, int Ly, int L,
-                                                         const double* __restrict__ Jg, double dtau, double a2,
+__global__ void __launch_bounds__(kThreads) k_half_sweep(double* __restrict__ x, int Lx, int Ly, int L, uint32_t mhalf,
+                                                         uint32_t mlx, const double* __restrict__ Jg, double dtau, double a2,
                                                          double delta, uint32_t key0, uint32_t key1, uint32_t sweep_arg,
                                                          int colour, const int* __restrict__ colour_pc, int cxor,
                                                          int chain0, unsigned long long* __restrict__ n_acc,
                                                          const unsigned long long* __restrict__ dctr, int nsweeps) {
-    __shared__ double J[6];
+    __shared__ SweepConst C;
     __shared__ int s_cnt;
-    if (threadIdx.x < 6) J[threadIdx.x] = Jg[threadIdx.x];
+    sweep_const_init(C, Jg, dtau, a2, delta);
     if (threadIdx.x == 0) s_cnt = 0;
     __syncthreads();
     const int f = blockIdx.y;
@@ -189,7 +255,7 @@ __global__ void __launch_bounds__(kThreads) k_half_sweep(double* __restrict__ x,
     int accepted = 0;
     if (s < N * half) {
         const int c = colour_pc ? (colour_pc[f] ^ cxor) : colour;
-        accepted = site_update<false>(x + (size_t)f * N * L, Lx, Ly, L, J, dtau, a2, delta, key0, key1, sweep, c, s,
+        accepted = site_update<false>(x + (size_t)f * N * L, Lx, Ly, L, L, mhalf, mlx, C, key0, key1, sweep, c, s,
                                       (uint32_t)(chain0 + f));
     }
     const unsigned int ballot = __ballot_sync(0xffffffffu, accepted);
@@ -211,7 +277,7 @@ __global__ void __launch_bounds__(kThreads) k_half_sweep(double* __restrict__ x,
 // One Wolff cluster update of one chain's field xf by the whole CTA (blockDim.x threads); act and
 // in_c are 2N and N bytes of shared memory; counter ctr, Philox chain index chain.
 template <bool kL2>
-__device__ __forceinline__ void wolff_chain(double* xf, int Lx, int Ly, int L, const double* __restrict__ Jg,
+__device__ __forceinline__ void wolff_chain(double* xf, int Lx, int Ly, int L, int ld, const double* Jg,
                                             double dtau, uint32_t key0, uint32_t key1, uint32_t ctr, uint32_t chain,
                                             unsigned char* act, unsigned char* in_c, int* s_seed, int* s_cnt,
                                             unsigned long long* __restrict__ n_sites) {
@@ -220,8 +286,8 @@ __device__ __forceinline__ void wolff_chain(double* xf, int Lx, int Ly, int L, c
     for (int b = tid; b < 2 * N; b += blockDim.x) {
         const int i = b >> 1, ix = i % Lx, iy = i / Lx;
         const int j = (b & 1) ? ix + Lx * (iy + 1 == Ly ? 0 : iy + 1) : (ix + 1 == Lx ? 0 : ix + 1) + Lx * iy;
-        const double* xi = xf + (size_t)i * L;
-        const double* xj = xf + (size_t)j * L;
+        const double* xi = xf + (size_t)i * ld;
+        const double* xj = xf + (size_t)j * ld;
         double sb = 0.0;
         for (int l = 0; l < L; ++l) sb = __dadd_rn(sb, __dmul_rn(ldx<kL2>(xi + l), ldx<kL2>(xj + l)));
         const double t = __dmul_rn(cfac, sb);
@@ -257,8 +323,10 @@ __device__ __forceinline__ void wolff_chain(double* xf, int Lx, int Ly, int L, c
     }
     int cnt = 0;
     for (int i = tid; i < N; i += blockDim.x) cnt += in_c[i];
-    for (size_t idx = tid; idx < (size_t)N * L; idx += blockDim.x)
-        if (in_c[idx / L]) xf[idx] = -ldx<kL2>(xf + idx);
+    const int lane = tid & 31;
+    for (int i = tid >> 5; i < N; i += blockDim.x >> 5)
+        if (in_c[i])
+            for (int l = lane; l < L; l += 32) xf[(size_t)i * ld + l] = -ldx<kL2>(xf + (size_t)i * ld + l);
     if (n_sites) {
         atomicAdd(s_cnt, cnt);
         __syncthreads();
@@ -277,7 +345,7 @@ __global__ void __launch_bounds__(256) k_wolff(double* __restrict__ x, int Lx, i
     const int f = blockIdx.x;
     const uint32_t sweep = dctr ? (uint32_t)((*dctr) * (unsigned long long)nsweeps + sweep_arg) : sweep_arg;
     const uint32_t ctr = sweep * (uint32_t)nwolff + (uint32_t)k;
-    wolff_chain<false>(x + (size_t)f * N * L, Lx, Ly, L, Jg, dtau, key0, key1, ctr, (uint32_t)(chain0 + f), wsm,
+    wolff_chain<false>(x + (size_t)f * N * L, Lx, Ly, L, L, Jg, dtau, key0, key1, ctr, (uint32_t)(chain0 + f), wsm,
                        wsm + 2 * N, &s_seed, &s_cnt, n_sites);
 }
 
@@ -305,7 +373,7 @@ __global__ void __launch_bounds__(kThreads) k_sweep_queue(const slmc::QueueClass
                                                           unsigned int* __restrict__ done, unsigned int* __restrict__ ctl,
                                                           uint32_t u, long long wait_cycles) {
     extern __shared__ unsigned char qsm[];
-    __shared__ double J[6];
+    __shared__ SweepConst K;
     __shared__ int s_item, s_cnt, s_seed, s_wcnt;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -340,7 +408,7 @@ __global__ void __launch_bounds__(kThreads) k_sweep_queue(const slmc::QueueClass
         const int4 it = items[q];
         const slmc::QueueClass& C = cls[it.x >> 24];
         const int f = it.x & 0xffffff;
-        if (threadIdx.x < 6) J[threadIdx.x] = C.J[threadIdx.x];
+        sweep_const_init(K, C.J, C.dtau, C.a2, C.delta);
         __syncthreads();
         const int N = C.Lx * C.Ly;
         double* xf = C.x + (size_t)f * N * C.L;
@@ -350,7 +418,7 @@ __global__ void __launch_bounds__(kThreads) k_sweep_queue(const slmc::QueueClass
                                           (unsigned long long)u * C.nsweeps + sw);
         if (it.y & 0x80) {
             const uint32_t ctr = sweep * (uint32_t)C.nwolff + (uint32_t)sub;
-            wolff_chain<true>(xf, C.Lx, C.Ly, C.L, J, C.dtau, C.key0, C.key1, ctr, chain, qsm, qsm + 2 * N, &s_seed,
+            wolff_chain<true>(xf, C.Lx, C.Ly, C.L, C.L, K.J, C.dtau, C.key0, C.key1, ctr, chain, qsm, qsm + 2 * N, &s_seed,
                               &s_wcnt, C.wolff_sites);
         } else {
             const int sites = N * (C.L / 2);
@@ -359,8 +427,8 @@ __global__ void __launch_bounds__(kThreads) k_sweep_queue(const slmc::QueueClass
             for (int j = 0; j < slmc::kQueueSlab / kThreads; ++j) {
                 const int st = it.z * slmc::kQueueSlab + j * kThreads + threadIdx.x;
                 if (st < sites)
-                    accepted += site_update<true>(xf, C.Lx, C.Ly, C.L, J, C.dtau, C.a2, C.delta, C.key0, C.key1,
-                                                  sweep, c, st, chain);
+                    accepted += site_update<true>(xf, C.Lx, C.Ly, C.L, C.L, C.mhalf, C.mlx, K, C.key0, C.key1, sweep,
+                                                  c, st, chain);
             }
             if (accepted) atomicAdd(&s_cnt, accepted);
         }
@@ -561,6 +629,12 @@ __global__ void k_fit_finish(const double* __restrict__ R, double dtau, double s
 
 namespace slmc {
 
+// Multiplier of fast_div for dividends below n (0 where n d reaches 2^32: the kernel divides).
+uint32_t div_magic(long long n, int d) {
+    if (d < 2 || n * d >= (1ll << 32)) return 0u;
+    return (uint32_t)(((1ull << 32) + d - 1) / (unsigned)d);
+}
+
 cudaError_t bose_log_weight(slmc_ctx* c, const double* x, int nf, const double* lndet, double* lnw, cudaStream_t s) {
     k_bose<<<nf, kThreads, 0, s>>>(x, c->N, c->L, c->p.dtau, c->p.lambda, c->p.omega0 * c->p.omega0, lndet, lnw);
     return cudaGetLastError();
@@ -579,7 +653,8 @@ cudaError_t eff_half_sweep(slmc_ctx* c, double* x, int nf, int chain0, const dou
     const double a = c->p.lambda / (c->p.omega0 * c->p.omega0);
     const int sites = c->N * (c->L / 2);
     dim3 grid((sites + kThreads - 1) / kThreads, nf);
-    k_half_sweep<<<grid, kThreads, 0, s>>>(x, c->p.Lx, c->p.Ly, c->L, J, c->p.dtau, a * a, c->p.sweep_delta,
+    k_half_sweep<<<grid, kThreads, 0, s>>>(x, c->p.Lx, c->p.Ly, c->L, div_magic(sites, c->L / 2),
+                                           div_magic(c->N, c->p.Lx), J, c->p.dtau, a * a, c->p.sweep_delta,
                                            (uint32_t)(c->p.seed & 0xffffffffu), (uint32_t)(c->p.seed >> 32),
                                            (uint32_t)sweep, colour, colour_per_chain, colour_xor, chain0,
                                            reinterpret_cast<unsigned long long*>(n_acc), dctr, nsweeps);

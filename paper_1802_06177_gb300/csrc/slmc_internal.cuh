@@ -291,6 +291,8 @@ int cumulative_phases(slmc_ctx* c, double* x, int n, const double* J, int nsweep
                       cudaStream_t s);
 const int* first_colours(slmc_ctx* c);
 
+uint32_t div_magic(long long n, int d);  // multiplier of the sweeps' exact division by multiply-high
+
 // Persistent E_eff sweep queue over the chains of several lattice classes. One lattice class:
 struct QueueClass {
     double* x;                           // chains [nchains][N][L]
@@ -304,6 +306,7 @@ struct QueueClass {
     int done0;                           // index of chain 0's completion counter
     double dtau, a2, delta;
     uint32_t key0, key1;
+    uint32_t mhalf, mlx;                 // div_magic of L / 2 and Lx
 };
 // An item of the queue (int4): x = class << 24 | chain, y = sweep << 8 | kind << 7 | (colour step
 // h or Wolff index k), z = slab of kQueueSlab sites of the half-sweep, w = number of the chain's

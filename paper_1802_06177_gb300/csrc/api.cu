@@ -345,7 +345,11 @@ int cumulative_phases(slmc_ctx* c, double* x, int n, const double* J, int nsweep
                     SLMC_CK(cudaMemcpyAsync(xo, xc, m * NL * sizeof(double), cudaMemcpyDeviceToDevice, sk));
                     SLMC_LAUNCH(SLMC_PROF_EFF, 1, sk, eff_features(c, xc, m, J, nullptr, 0, sc(1), sk));
                 }
-                if (phases & kPhaseSweeps)
+                if ((phases & kPhaseSweeps) && nsweeps > 0 && eff_sweeps_fused(c))
+                    SLMC_LAUNCH(SLMC_PROF_SWEEP, 1, sk,
+                                eff_chain_sweeps(c, xc, m, g0, J, (uint64_t)u * nsweeps, nsweeps, 0, isc(1),
+                                                 n_sweep_acc ? n_sweep_acc + g0 : nullptr, sk, c->dctr, nsweeps));
+                else if (phases & kPhaseSweeps)
                     for (int sw = 0; sw < nsweeps; ++sw)
                         for (int h = 0; h < 2; ++h) {
                             if (h == 1)  // Wolff cluster updates between the two colours of the sweep
@@ -607,6 +611,11 @@ int slmc_eff_sweep(slmc_ctx* c, double* x, int n, const double* J, int nsweeps, 
     if (!checkerboard_ok(c)) return SLMC_ERR_UNSUPPORTED;
     cudaStream_t s = as_stream(stream);
     c->cur_units = n;
+    if (n > 0 && nsweeps > 0 && slmc::eff_sweeps_fused(c)) {
+        SLMC_LAUNCH(SLMC_PROF_SWEEP, 1, s,
+                    slmc::eff_chain_sweeps(c, x, n, 0, J, sweep0, nsweeps, first_colour, nullptr, n_acc, s));
+        return SLMC_OK;
+    }
     for (int sw = 0; sw < nsweeps && n > 0; ++sw)
         for (int h = 0; h < 2; ++h) {
             if (h == 1)  // Wolff cluster updates between the two colours of the sweep

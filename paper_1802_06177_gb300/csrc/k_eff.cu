@@ -349,6 +349,56 @@ __global__ void __launch_bounds__(256) k_wolff(double* __restrict__ x, int Lx, i
                        wsm + 2 * N, &s_seed, &s_cnt, n_sites);
 }
 
+// Every sweep of a call for one chain per CTA, the chain's field in shared memory from the first
+// half-sweep to the last: one launch and one read and write of the field for nsweeps sweeps, block
+// barriers between the colours and the Wolff updates. A small chain's half-sweep is shorter than its
+// launch, and the many launches of the kernel-per-half-sweep path were its time. Rows are padded to the odd stride
+// L + 1, so the Wolff bond sums (a column per lane) meet no bank conflicts. Site and Wolff arithmetic and
+// random numbers are those of k_half_sweep / k_wolff: bit-identical chains.
+__global__ void __launch_bounds__(1024) k_chain_sweeps(double* __restrict__ x, int Lx, int Ly, int L, uint32_t mhalf,
+                                                       uint32_t mlx, const double* __restrict__ Jg, double dtau, double a2,
+                                                       double delta, uint32_t key0, uint32_t key1, uint32_t sweep_arg,
+                                                       int nsweeps, int colour, const int* __restrict__ colour_pc,
+                                                       int chain0, int nwolff, unsigned long long* __restrict__ n_acc,
+                                                       unsigned long long* __restrict__ n_sites,
+                                                       const unsigned long long* __restrict__ dctr, int ctr_mul) {
+    extern __shared__ double csm[];
+    __shared__ SweepConst C;
+    __shared__ int s_cnt, s_seed, s_wcnt;
+    const int f = blockIdx.x, N = Lx * Ly, ld = L + 1, sites = N * (L / 2), tid = threadIdx.x;
+    unsigned char* act = reinterpret_cast<unsigned char*>(csm + (size_t)N * ld);
+    double* xf = x + (size_t)f * N * L;
+    sweep_const_init(C, Jg, dtau, a2, delta);
+    if (tid == 0) s_cnt = 0;
+    for (int i = tid >> 5; i < N; i += blockDim.x >> 5)
+        for (int l = tid & 31; l < L; l += 32) csm[i * ld + l] = xf[(size_t)i * L + l];
+    const uint32_t sweep0 = dctr ? (uint32_t)((*dctr) * (unsigned long long)ctr_mul + sweep_arg) : sweep_arg;
+    const int first = colour_pc ? colour_pc[f] : colour;
+    const uint32_t chain = (uint32_t)(chain0 + f);
+    int accepted = 0;
+    __syncthreads();
+    for (int sw = 0; sw < nsweeps; ++sw) {
+        const uint32_t sweep = sweep0 + (uint32_t)sw;
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1)
+                for (int k = 0; k < nwolff; ++k) {
+                    wolff_chain<false>(csm, Lx, Ly, L, ld, C.J, dtau, key0, key1, sweep * (uint32_t)nwolff + (uint32_t)k,
+                                       chain, act, act + 2 * N, &s_seed, &s_wcnt, n_sites);
+                    __syncthreads();
+                }
+            for (int s = tid; s < sites; s += blockDim.x)
+                accepted += site_update<false>(csm, Lx, Ly, L, ld, mhalf, mlx, C, key0, key1, sweep, first ^ h, s, chain);
+            __syncthreads();
+        }
+    }
+    accepted = __reduce_add_sync(0xffffffffu, accepted);
+    if ((tid & 31) == 0 && accepted) atomicAdd(&s_cnt, accepted);
+    for (int i = tid >> 5; i < N; i += blockDim.x >> 5)
+        for (int l = tid & 31; l < L; l += 32) xf[(size_t)i * L + l] = csm[i * ld + l];
+    __syncthreads();
+    if (tid == 0 && n_acc && s_cnt) atomicAdd(n_acc + f, (unsigned long long)s_cnt);
+}
+
 // Persistent E_eff sweep queue: the half-sweep slabs and Wolff updates of every chain of several
 // lattice classes, pulled in queue order by the CTAs of one launch. The queue lists, phase after
 // phase (colour 0, the Wolff updates, colour 1 of each sweep), the items of every chain in order of
@@ -684,6 +734,31 @@ cudaError_t eff_wolff(slmc_ctx* c, double* x, int nf, int chain0, const double* 
     k_wolff<<<nf, 256, 3 * c->N, s>>>(x, c->p.Lx, c->p.Ly, c->L, J, c->p.dtau, (uint32_t)(c->p.seed & 0xffffffffu),
                                       (uint32_t)(c->p.seed >> 32), (uint32_t)sweep, dctr, nsweeps, c->nwolff, k,
                                       chain0, c->wolff_sites);
+    return cudaGetLastError();
+}
+
+// Largest chain (sites times slices) whose sweeps run in one launch with the field in shared memory. Above,
+// a chain's half-sweep on one SM takes longer than a launch that spreads it over the GPU; measured at the
+// lower end: a 4x4, L = 40 update of 50 sweeps 1.42 -> 0.91 ms, an 8x8, L = 40 update of 10 sweeps and Wolff
+// moves on 128 chains 3.44 -> 3.15 ms (whole updates).
+constexpr int kChainSites = 8192;
+
+bool eff_sweeps_fused(const slmc_ctx* c) { return c->N * (long long)c->L <= kChainSites; }
+
+cudaError_t eff_chain_sweeps(slmc_ctx* c, double* x, int nf, int chain0, const double* J, uint64_t sweep0, int nsweeps,
+                             int colour, const int* colour_per_chain, long long* n_acc, cudaStream_t s,
+                             const unsigned long long* dctr, int ctr_mul) {
+    const double a = c->p.lambda / (c->p.omega0 * c->p.omega0);
+    const int sites = c->N * (c->L / 2), iters = (sites + 1023) / 1024;
+    const int threads = std::max(64, ((sites + iters - 1) / iters + 31) / 32 * 32);
+    const size_t smem = (size_t)c->N * (c->L + 1) * sizeof(double) + 3 * (size_t)c->N;
+    cudaError_t e = cudaFuncSetAttribute(k_chain_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_chain_sweeps<<<nf, threads, smem, s>>>(
+        x, c->p.Lx, c->p.Ly, c->L, div_magic(sites, c->L / 2), div_magic(c->N, c->p.Lx), J, c->p.dtau, a * a,
+        c->p.sweep_delta, (uint32_t)(c->p.seed & 0xffffffffu), (uint32_t)(c->p.seed >> 32), (uint32_t)sweep0, nsweeps,
+        colour, colour_per_chain, chain0, c->nwolff, reinterpret_cast<unsigned long long*>(n_acc), c->wolff_sites, dctr,
+        ctr_mul);
     return cudaGetLastError();
 }
 

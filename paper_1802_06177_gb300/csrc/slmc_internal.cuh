@@ -258,6 +258,12 @@ cudaError_t eff_half_sweep(slmc_ctx* c, double* x, int nf, int chain0, const dou
                            cudaStream_t s, const unsigned long long* dctr = nullptr, int nsweeps = 0);
 cudaError_t eff_wolff(slmc_ctx* c, double* x, int nf, int chain0, const double* J, uint64_t sweep, int k,
                       cudaStream_t s, const unsigned long long* dctr = nullptr, int nsweeps = 0);
+// All nsweeps sweeps (with their Wolff updates) of nf chains in one launch; eff_sweeps_fused says whether
+// the chain is small enough. Sweep counters start at sweep0 (plus the device counter times ctr_mul).
+bool eff_sweeps_fused(const slmc_ctx* c);
+cudaError_t eff_chain_sweeps(slmc_ctx* c, double* x, int nf, int chain0, const double* J, uint64_t sweep0, int nsweeps,
+                             int colour, const int* colour_per_chain, long long* n_acc, cudaStream_t s,
+                             const unsigned long long* dctr = nullptr, int ctr_mul = 0);
 cudaError_t slice_group_kron(slmc_ctx* c, const double* x, int nf, int l0, int nsl, bool transposed, cudaStream_t s);
 // G(g0) = [I + B(g0,0) B(L,g0)]^-1 into G (row-major) from the running product in (U, lnD, Ta)
 // and the transposed left product (Ul column-major, lnDl, Tl row-major); uses Y, Tb, Sws, piv.

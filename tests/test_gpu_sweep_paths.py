@@ -28,3 +28,22 @@ def test_decisions_at_the_edges_of_fp32(Lx, Ly, L, scale, delta):
         na = eff_sweeps(p, xo, J[1:], 4, 9, 1, f, seed, delta)
         assert np.array_equal(xg[f].cpu().numpy(), xo)
         assert n_acc[f].item() == na
+
+
+@pytest.mark.parametrize("Lx,Ly,L,nwolff", [(2, 2, 2, 2), (8, 16, 64, 1), (8, 16, 66, 1), (32, 32, 8, 0), (4, 4, 40, 3)])
+def test_sweeps_in_one_launch_and_per_half_sweep(Lx, Ly, L, nwolff):
+    """Chains up to 8192 sites x slices run all sweeps in one launch, larger ones a launch per half-sweep
+    (8 x 16 x 64 and 8 x 16 x 66 lie on either side): both bit for bit the oracle's."""
+    seed = 31
+    ctx = make_ctx(Lx, L, 2, Ly=Ly, max_fields=2, sweep_delta=0.4, seed=seed)
+    ctx.set_wolff(nwolff)
+    x = np.random.default_rng(6).standard_normal((2, Lx * Ly, L))
+    xg, n_acc = cuda(x.copy()), torch.zeros(2, dtype=torch.int64, device="cuda")
+    ctx.eff_sweep(xg, cuda(J), 2, sweep0=12345, first_colour=0, n_acc=n_acc)
+    p, sizes = HolsteinParams(Lx, Ly, L, n_s=2), []
+    for f in range(2):
+        xo = x[f].copy()
+        na = eff_sweeps(p, xo, J[1:], 2, 12345, 0, f, seed, 0.4, nwolff=nwolff, wolff_sizes=sizes)
+        assert np.array_equal(xg[f].cpu().numpy(), xo)
+        assert n_acc[f].item() == na
+    assert ctx.wolff_sites() == sum(sizes)

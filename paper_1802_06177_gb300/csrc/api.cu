@@ -131,6 +131,10 @@ int* iscal(slmc_ctx* c, int col) { return c->iscal + (size_t)col * c->max_fields
 int logdet_run(slmc_ctx* c, slmc_ctx* v, const double* x, int nf, double* lndet, int* sign, double* G,
                cudaStream_t s) {
     c->cur_units = nf;
+    if (slmc::small_active(v)) {
+        SLMC_LAUNCH(SLMC_PROF_FINAL, 1, s, slmc::small_logdet(v, x, nf, lndet, sign, G, s));
+        return SLMC_OK;
+    }
     SLMC_LAUNCH(SLMC_PROF_FINAL, 1, s, slmc::set_identity(v, nf, s));
     if (v->p.precision != SLMC_PREC_FP64) SLMC_LAUNCH(SLMC_PROF_SLICE, 1, s, slmc::slice_scales(v, x, nf, s));
     for (int l0 = 0; l0 < v->L; l0 += v->p.n_s) {
@@ -247,6 +251,7 @@ slmc_ctx make_view(slmc_ctx* c, int f0) {
     v.tune_slice_groups = c->tune_slice_groups;
     v.tune_qr_cluster = c->tune_qr_cluster;
     v.num_sms = c->num_sms;
+    v.layout_set = c->layout_set;
     v.nsub = 0;
     v.parent = c;
     return v;
@@ -255,7 +260,7 @@ slmc_ctx make_view(slmc_ctx* c, int f0) {
 int logdet_batch(slmc_ctx* c, const double* x, int nf, double* lndet, int* sign, double* G, cudaStream_t s) {
     const bool tc = c->p.precision == SLMC_PREC_TF32X3;  // per-slice workspace not split into views
     const int nsub = std::min(c->nsub, nf / kMinSubFields);
-    if (nsub < 2 || tc) return logdet_run(c, c, x, nf, lndet, sign, G, s);
+    if (nsub < 2 || tc || slmc::small_active(c)) return logdet_run(c, c, x, nf, lndet, sign, G, s);
     const size_t NL = (size_t)c->N * c->L, NN = (size_t)c->N * c->N;
     SLMC_CK(cudaEventRecord(c->sub_fork, s));
     for (int k = 0; k < nsub; ++k) {
@@ -325,7 +330,7 @@ int cumulative_phases(slmc_ctx* c, double* x, int n, const double* J, int nsweep
     return for_batches(c, n, [&](int f0, int nf) {
         const bool tc = c->p.precision == SLMC_PREC_TF32X3;
         int nsub = std::min(c->nsub, nf / kMinSubFields);
-        if (nsub < 2 || tc || !(phases & kPhasePost)) nsub = 1;
+        if (nsub < 2 || tc || !(phases & kPhasePost) || small_active(c)) nsub = 1;
         if (nsub > 1) SLMC_CK(cudaEventRecord(c->sub_fork, s));
         for (int k = 0; k < nsub; ++k) {
             const int a = (int)((long long)k * nf / nsub), b = (int)((long long)(k + 1) * nf / nsub), m = b - a;
@@ -770,6 +775,7 @@ int slmc_set_tuning(slmc_ctx* c, int qr_panel, int slice_cols) {
     if (!c || (qr_panel != 0 && qr_panel != 16 && qr_panel != 32) ||
         (slice_cols != 0 && slice_cols != 8 && slice_cols != 16))
         return SLMC_ERR_ARG;
+    c->layout_set = 1;
     c->tune_qr_panel = qr_panel;
     c->tune_slice_cols = slice_cols;
     return SLMC_OK;
@@ -800,12 +806,14 @@ int slmc_get_wolff_sites(slmc_ctx* c, long long* total, int reset, void* stream)
 
 int slmc_set_qr_cluster(slmc_ctx* c, int ctas) {
     if (!c || (ctas != 0 && ctas != 1 && ctas != 2 && ctas != 4)) return SLMC_ERR_ARG;
+    c->layout_set = 1;
     c->tune_qr_cluster = ctas;
     return SLMC_OK;
 }
 
 int slmc_set_dense_slices(slmc_ctx* c, int dense) {
     if (!c || dense < 0 || dense > 1) return SLMC_ERR_ARG;
+    c->layout_set = 1;
     c->dense_slices = dense;
     return SLMC_OK;
 }
@@ -813,6 +821,7 @@ int slmc_set_dense_slices(slmc_ctx* c, int dense) {
 int slmc_set_tupdate_path(slmc_ctx* c, int path) {
     if (!c || path < 0 || path > 2) return SLMC_ERR_ARG;
     if (path != 1 && !c->tt_A) return SLMC_ERR_UNSUPPORTED;
+    c->layout_set = 1;
     c->tt_path = path;
     return SLMC_OK;
 }
@@ -820,6 +829,7 @@ int slmc_set_tupdate_path(slmc_ctx* c, int path) {
 int slmc_set_qr_path(slmc_ctx* c, int path) {
     if (!c || path < 0 || path > 1) return SLMC_ERR_ARG;
     if (path == 0 && !c->qt_buf) return SLMC_ERR_UNSUPPORTED;
+    c->layout_set = 1;
     c->qr_path = path;
     return SLMC_OK;
 }
@@ -827,6 +837,7 @@ int slmc_set_qr_path(slmc_ctx* c, int path) {
 int slmc_set_sub_batch_priorities(slmc_ctx* c, int on) {
     if (!c || on < 0 || on > 1) return SLMC_ERR_ARG;
     if (on && c->nsub_avail == 0) return SLMC_ERR_UNSUPPORTED;
+    c->layout_set = 1;
     c->sub_prio = on;
     return SLMC_OK;
 }
@@ -834,6 +845,7 @@ int slmc_set_sub_batch_priorities(slmc_ctx* c, int on) {
 int slmc_set_sub_batches(slmc_ctx* c, int n) {
     if (!c || n < 1 || n > slmc_ctx::kMaxSub) return SLMC_ERR_ARG;
     if (n > 1 && c->nsub_avail < n) return SLMC_ERR_UNSUPPORTED;
+    c->layout_set = 1;
     c->nsub = n;
     return SLMC_OK;
 }

@@ -1,0 +1,115 @@
+// FP64 determinant and Green's function of small lattices (N <= 64) in one launch, one CTA per field
+// (small.cuh holds the steps and what bounds them). The per-group kernels it replaces were launch latency at
+// these sizes: a 4x4, L = 40 determinant took about 28 launches.
+#include "small.cuh"
+
+namespace {
+
+using namespace slmc::sm;
+
+template <int NMAX, int LMAX>
+__global__ void __launch_bounds__(4 * NMAX) k_small_logdet(const double* __restrict__ x, const double* __restrict__ kron,
+                                                           double* __restrict__ lndet, int* __restrict__ sign,
+                                                           double* __restrict__ Gout, unsigned int* __restrict__ err, int N,
+                                                           int Lx, int Ly, int L, int n_s, double dtlam, double emu) {
+    constexpr int ld = Dim<NMAX>::ld, NT = Dim<NMAX>::threads, RPT = NMAX / 4;
+    extern __shared__ __align__(16) double dsm[];
+    double* A = dsm;                       // packed QR, then M and its LU
+    double* B = A + Dim<NMAX>::mat;        // U
+    double* T = B + Dim<NMAX>::mat;
+    Vecs<NMAX>& v = *reinterpret_cast<Vecs<NMAX>*>(T + Dim<NMAX>::mat);
+    const int f = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    const double* xf = x + (size_t)f * N * L;
+    for (int idx = tid; idx < Dim<NMAX>::mat; idx += NT) {
+        const double e = idx % (ld + 1) == 0 ? 1.0 : 0.0;
+        B[idx] = e;
+        T[idx] = e;
+    }
+    for (int k = tid; k < slmc::kKronTab; k += NT) {
+        v.tx[k] = kron[k];
+        v.ty[k] = kron[2 * slmc::kKronTab + k];
+    }
+    if (tid < N) v.lnd[tid] = 0.0;
+    __syncthreads();
+    bool bad = false;
+    for (int l0 = 0; l0 < L; l0 += n_s) {
+        slices<NMAX, LMAX, false>(B, v, xf, N, Lx, Ly, L, l0, min(L, l0 + n_s), dtlam, emu);
+        qr<NMAX>(B, A, v, N);
+        t_update<NMAX>(A, T, v, N);
+        form_q<NMAX>(A, B, v, N);
+        if (tid < N) {
+            v.lnd[tid] = v.lnn[tid];
+            bad |= !isfinite(v.lnn[tid]);
+        }
+        __syncthreads();
+    }
+    if (bad) atomicOr(err, SLMC_EBIT_NONFINITE);
+    // M = D_b^-1 U^T + D_s T
+    if (tid < N) {
+        v.e1[tid] = exp(-fmax(v.lnd[tid], 0.0));
+        v.e2[tid] = exp(fmin(v.lnd[tid], 0.0));
+    }
+    __syncthreads();
+    for (int idx = tid; idx < N * N; idx += NT) {
+        const int j = idx / N, i = idx - j * N;
+        A[j * ld + i] = fma(v.e1[i], B[i * ld + j], v.e2[i] * T[i * ld + j]);
+    }
+    __syncthreads();
+    lu<NMAX>(A, v, N);
+    if (tid < 32) {
+        double s = 0.0;
+        for (int k = lane; k < N; k += 32) s += log(fabs(v.key[k])) + fmax(v.lnd[k], 0.0);
+        s = slmc::warp_allsum(s);
+        if (tid == 0) {
+            const bool ok = !v.sing && isfinite(s);
+            lndet[f] = ok ? s : __longlong_as_double(0x7ff8000000000000ll);
+            sign[f] = ok ? ((v.ntriv & 1) ? -1 : 1) * (v.neg ? -1 : 1) : 0;
+            if (v.sing) atomicOr(err, SLMC_EBIT_SINGULAR);
+            else if (!ok) atomicOr(err, SLMC_EBIT_NONFINITE);
+        }
+    }
+    if (!Gout) return;
+    if (tid < N) v.beta[tid] = 1.0 / A[tid * ld + tid];
+    __syncthreads();
+    const int j = tid >> 2, g = tid & 3;
+    double b[RPT];
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+        const int r = 4 * q + g;
+        const int sr = r < N ? v.src[r] : 0;
+        b[q] = (j < N && r < N) ? v.e1[sr] * B[sr * ld + j] : 0.0;
+    }
+    lu_solve<NMAX>(A, v.beta, b, N);
+    if (j < N)
+#pragma unroll
+        for (int q = 0; q < RPT; ++q)
+            if (4 * q + g < N) Gout[(size_t)f * N * N + (size_t)(4 * q + g) * N + j] = b[q];
+}
+
+template <int NMAX, int LMAX>
+cudaError_t launch_small(slmc_ctx* c, const double* x, int nf, double* lndet, int* sign, double* G, cudaStream_t s) {
+    const size_t smem = 3 * (size_t)Dim<NMAX>::mat * sizeof(double) + sizeof(Vecs<NMAX>);
+    cudaError_t e = cudaFuncSetAttribute(k_small_logdet<NMAX, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_small_logdet<NMAX, LMAX><<<nf, 4 * NMAX, smem, s>>>(x, c->kron, lndet, sign, G, c->err, c->N, c->p.Lx, c->p.Ly, c->L,
+                                                         c->p.n_s, c->p.dtau * c->p.lambda, exp(c->p.dtau * c->p.mu));
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+namespace slmc {
+
+bool small_active(const slmc_ctx* c) {
+    return c->N <= kSmallN && c->kron && c->p.precision == SLMC_PREC_FP64 && c->p.qr_mode == SLMC_QR_PREPIVOT &&
+           !c->layout_set && c->qr_path == 0 && c->tt_path == 0 && !c->dense_slices;
+}
+
+cudaError_t small_logdet(slmc_ctx* c, const double* x, int nf, double* lndet, int* sign, double* G, cudaStream_t s) {
+    const bool l8 = c->p.Lx <= 8 && c->p.Ly <= 8;
+    if (c->N <= 16) return l8 ? launch_small<16, 8>(c, x, nf, lndet, sign, G, s) : launch_small<16, 32>(c, x, nf, lndet, sign, G, s);
+    if (c->N <= 32) return l8 ? launch_small<32, 8>(c, x, nf, lndet, sign, G, s) : launch_small<32, 32>(c, x, nf, lndet, sign, G, s);
+    return l8 ? launch_small<64, 8>(c, x, nf, lndet, sign, G, s) : launch_small<64, 32>(c, x, nf, lndet, sign, G, s);
+}
+
+}  // namespace slmc

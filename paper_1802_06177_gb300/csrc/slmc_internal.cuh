@@ -68,6 +68,7 @@ struct slmc_ctx {
     int tune_slice_groups;
     int tune_qr_cluster;    // CTAs per field of the QR / formation of Q (0 = by field count)
     int num_sms;            // multiprocessors of the device
+    int layout_set;         // a knob of the general kernels was set: no one-launch path for small lattices
     // Exact sliced tensor-core slice path (SLMC_PREC_BF16X9): fixed-point BF16 slices of F
     // [4][128 MT][tcx_npad], their row exponents and the TMA descriptor of the slices.
     void* tcx_F;
@@ -264,6 +265,10 @@ bool eff_sweeps_fused(const slmc_ctx* c);
 cudaError_t eff_chain_sweeps(slmc_ctx* c, double* x, int nf, int chain0, const double* J, uint64_t sweep0, int nsweeps,
                              int colour, const int* colour_per_chain, long long* n_acc, cudaStream_t s,
                              const unsigned long long* dctr = nullptr, int ctr_mul = 0);
+// Whole FP64 determinant (and G) of small lattices in one launch (k_small.cu).
+constexpr int kSmallN = 64;
+bool small_active(const slmc_ctx* c);
+cudaError_t small_logdet(slmc_ctx* c, const double* x, int nf, double* lndet, int* sign, double* G, cudaStream_t s);
 cudaError_t slice_group_kron(slmc_ctx* c, const double* x, int nf, int l0, int nsl, bool transposed, cudaStream_t s);
 // G(g0) = [I + B(g0,0) B(L,g0)]^-1 into G (row-major) from the running product in (U, lnD, Ta)
 // and the transposed left product (Ul column-major, lnDl, Tl row-major); uses Y, Tb, Sws, piv.

@@ -36,6 +36,7 @@
 // Block updates reflect one site's whole column (x -> -x) and are accepted with the ratio of
 // full weights (computed by the determinant path); the site and the uniform come from Philox
 // counter (k, sweep, chain, 4).
+#include "circ.cuh"
 #include "slmc_internal.cuh"
 
 #include <algorithm>
@@ -88,7 +89,10 @@ __global__ void __launch_bounds__(kThreads) k_dqmc_slices(double* __restrict__ x
     const int f = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const size_t NN = (size_t)N * N;
     double* G = g_in_smem ? dsm : Gall + f * NN;
-    double* p = g_in_smem ? dsm + NN : dsm;
+    // row stride: odd in shared memory, so that walks down a column (the wrap's right factors with a row per
+    // lane, a move's column of G) meet no bank conflicts
+    const int ldg = g_in_smem ? N | 1 : N;
+    double* p = g_in_smem ? dsm + (size_t)N * ldg : dsm;
     double* s = p;                 // [N] slice scales exp(-dtau lam x_{i,l-1})
     double* sinv = p + N;          // [N] 1 / s
     double* xn = p + 2 * N;        // [N] proposed field
@@ -97,25 +101,27 @@ __global__ void __launch_bounds__(kThreads) k_dqmc_slices(double* __restrict__ x
     double* ua = p + 5 * N;        // [N] acceptance uniform
     double* ac = p + 6 * N;        // [N] -(Delta_ii / R) G[:, i]
     double* rw = p + 7 * N;        // [N] e_i - G[i, :]
-    double* ex = p + 8 * N;        // [2 Lx] E_x
-    double* exi = ex + slmc::kKronTab;   // [2 Lx] E_x^-1
-    double* ey = exi + slmc::kKronTab;   // [2 Ly] E_y
-    double* eyi = ey + slmc::kKronTab;   // [2 Ly] E_y^-1
+    const int kx = slmc::circ::ncoef(Lx), ky = slmc::circ::ncoef(Ly);
+    double* ex = p + 8 * N;        // folded coefficients (circ.cuh) of E_x, E_x^-1, E_y, E_y^-1
+    double* exi = ex + kx;
+    double* ey = exi + kx;
+    double* eyi = ey + ky;
     // delayed updates (kd > 0, G in global memory): accepted moves q < cnt of the current batch as
     // G = G0 + sum_q A_q B_q^T, A_q = -(Delta/R) G[:, i_q], B_q = e_i - G[i_q, :] ([kd][N] each), and the
     // running diagonal of G
-    double* Ad = eyi + slmc::kKronTab;
+    double* Ad = eyi + ky;
     double* Bd = Ad + (size_t)kd * N;
     double* dg = Bd + (size_t)kd * N;
     double* xf = x + (size_t)f * N * L;
     const uint32_t chain = (uint32_t)(chain0 + f);
 
-    for (int k = tid; k < 4 * slmc::kKronTab; k += kThreads) ex[k] = kron[k];  // ex, exi, ey, eyi are contiguous
+    slmc::circ::build(ex, kron, Lx, tid, kThreads);
+    slmc::circ::build(exi, kron + slmc::kKronTab, Lx, tid, kThreads);
+    slmc::circ::build(ey, kron + 2 * slmc::kKronTab, Ly, tid, kThreads);
+    slmc::circ::build(eyi, kron + 3 * slmc::kKronTab, Ly, tid, kThreads);
     if (g_in_smem) {
-        const double2* src = reinterpret_cast<const double2*>(Gall + f * NN);
-        double2* dst = reinterpret_cast<double2*>(G);
-        for (size_t k = tid; k < NN / 2; k += kThreads) dst[k] = src[k];
-        if ((NN & 1) && tid == 0) G[NN - 1] = Gall[f * NN + NN - 1];
+        for (int j = warp; j < N; j += kThreads / 32)
+            for (int m = lane; m < N; m += 32) G[j * ldg + m] = Gall[f * NN + (size_t)j * N + m];
     }
     int accepted = 0;
     for (int l = l0 + 1; l <= l0 + nsl; ++l) {
@@ -139,28 +145,29 @@ __global__ void __launch_bounds__(kThreads) k_dqmc_slices(double* __restrict__ x
         }
         __syncthreads();
         // wrap: G <- diag(s) (E_x kron E_y) G (E_x kron E_y)^-1 diag(1/s), site i = ix + Lx iy
-        for (int q = tid; q < N * Lx; q += kThreads)  // right factor along y: lines (i, jx)
-            slmc::circ_line<LMAX, false>(G, (q / Lx) * N + q % Lx, Lx, Ly, eyi, nullptr, 0, nullptr, 0, 1.0);
-        __syncthreads();
-        for (int q = tid; q < N * Ly; q += kThreads)  // right factor along x: lines (i, jy)
-            slmc::circ_line<LMAX, false>(G, (q / Ly) * N + (q % Ly) * Lx, 1, Lx, exi, nullptr, 0, nullptr, 0, 1.0);
-        __syncthreads();
-        for (int q = tid; q < Ly * N; q += kThreads)  // left factor along x: lines (iy, j)
-            slmc::circ_line<LMAX, true>(G, (q / N) * Lx * N + q % N, N, Lx, ex, nullptr, 0, nullptr, 0, 1.0);
-        __syncthreads();
-        for (int q = tid; q < Lx * N; q += kThreads) {  // left factor along y, then the scales
-            const int ix = q / N, j = q % N;
-            slmc::circ_line<LMAX, true>(G, ix * N + j, Lx * N, Ly, ey, nullptr, 0, s + ix, Lx, sinv[j]);  // row ix + Lx d
+        // passes: right factor along y (lines (i, jx)), along x (lines (i, jy)), left factor along x (lines (iy, j)),
+        // along y (lines (ix, j)) with the scales; consecutive threads take neighbouring rows or columns of G
+        for (int pass = 0; pass < 4; ++pass) {
+            const bool left = pass >= 2, alongx = pass == 1 || pass == 2;
+            const int lines = alongx ? Ly : Lx, n = alongx ? Lx : Ly;
+            const int unit = left ? ldg : 1, stride = (alongx ? 1 : Lx) * unit;
+            const double* cf = left ? (alongx ? ex : ey) : (alongx ? exi : eyi);
+            for (int q = tid; q < lines * N; q += kThreads) {
+                const int li = q / N, o = q - li * N;  // line, and the row (right factors) or column (left) it belongs to
+                const int at = (alongx ? li * Lx : li) * unit + o * (left ? 1 : ldg);
+                slmc::circ::apply_any<LMAX>(n, G + at, stride, cf, nullptr, 0, pass == 3 ? s + li : nullptr, Lx,
+                                            pass == 3 ? sinv[o] : 1.0);
+            }
+            __syncthreads();
         }
-        __syncthreads();
         if (kd > 0) {
-            for (int j = tid; j < N; j += kThreads) dg[j] = G[(size_t)j * N + j];
+            for (int j = tid; j < N; j += kThreads) dg[j] = G[(size_t)j * ldg + j];
             __syncthreads();
         }
         int cnt = 0;  // delayed moves of the current batch (block-uniform)
         for (int i = 0; i < N; ++i) {
             // every thread takes the same decision from the same G_ii
-            const double gii = kd > 0 ? dg[i] : G[(size_t)i * N + i];
+            const double gii = kd > 0 ? dg[i] : G[(size_t)i * ldg + i];
             const double R = __dadd_rn(1.0, __dmul_rn(__dadd_rn(1.0, -gii), dl[i]));
             if (!(ua[i] < R * R * eb[i])) continue;
             const double a = dl[i] * __drcp_rn(R);
@@ -168,7 +175,7 @@ __global__ void __launch_bounds__(kThreads) k_dqmc_slices(double* __restrict__ x
                 // the current column G[:, i] and row G[i, :] from G0 and the batch, each entry by the
                 // same FMA chain the immediate update would have applied to it
                 for (int j = tid; j < N; j += kThreads) {
-                    double cj = G[(size_t)j * N + i], rj = G[(size_t)i * N + j];
+                    double cj = G[(size_t)j * ldg + i], rj = G[(size_t)i * ldg + j];
                     for (int q = 0; q < cnt; ++q) {
                         cj = fma(Ad[q * N + j], Bd[q * N + i], cj);
                         rj = fma(Ad[q * N + i], Bd[q * N + j], rj);
@@ -192,8 +199,8 @@ __global__ void __launch_bounds__(kThreads) k_dqmc_slices(double* __restrict__ x
                 continue;
             }
             for (int j = tid; j < N; j += kThreads) {
-                ac[j] = -a * G[(size_t)j * N + i];
-                rw[j] = (j == i ? 1.0 : 0.0) - G[(size_t)i * N + j];
+                ac[j] = -a * G[(size_t)j * ldg + i];
+                rw[j] = (j == i ? 1.0 : 0.0) - G[(size_t)i * ldg + j];
             }
             if (tid == 0) {
                 xf[(size_t)i * L + c] = xn[i];
@@ -207,7 +214,7 @@ __global__ void __launch_bounds__(kThreads) k_dqmc_slices(double* __restrict__ x
             for (int q = 0; q < QMAX; ++q) r[q] = lane + 32 * q < N ? rw[lane + 32 * q] : 0.0;
             for (int j = warp; j < N; j += kThreads / 32) {
                 const double cj = ac[j];
-                double* Gj = G + (size_t)j * N;
+                double* Gj = G + (size_t)j * ldg;
 #pragma unroll
                 for (int q = 0; q < QMAX; ++q)
                     if (lane + 32 * q < N) Gj[lane + 32 * q] = fma(cj, r[q], Gj[lane + 32 * q]);
@@ -357,8 +364,8 @@ cudaError_t gemm64(const GemmArgs& g, double* C, int N, int nf, int sstride, cud
     return launch_gemm<32, kAik, kBjk, kCrow>(g, C, N, nf, sstride, s);
 }
 
-size_t dqmc_smem_bytes(int N, bool g_in_smem, int kd = 0) {
-    return ((g_in_smem ? (size_t)N * N : 0) + 8 * (size_t)N + 4 * slmc::kKronTab + (kd > 0 ? (2 * (size_t)kd + 1) * N : 0)) *
+size_t dqmc_smem_bytes(int N, int ncoef, bool g_in_smem, int kd = 0) {
+    return ((g_in_smem ? (size_t)N * (N | 1) : 0) + 8 * (size_t)N + ncoef + (kd > 0 ? (2 * (size_t)kd + 1) * N : 0)) *
            sizeof(double);
 }
 
@@ -373,17 +380,18 @@ cudaError_t launch_slices(slmc_ctx* c, double* x, double* G, int nf, int chain0,
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
-    const bool in_smem = dqmc_smem_bytes(c->N, true) <= (size_t)optin;
+    const int nc = 2 * (slmc::circ::ncoef(c->p.Lx) + slmc::circ::ncoef(c->p.Ly));
+    const bool in_smem = dqmc_smem_bytes(c->N, nc, true) <= (size_t)optin;
     // G in global memory: batch up to kd accepted moves in shared memory (delayed updates). With G in
     // shared memory the immediate rank-1 updates were faster (12x12: 463 against 418 chain-sweeps/s
     // with batches of 16), since there a pass over G costs no L2 traffic.
     int kd = 0;
     if (!in_smem) {
         kd = kDelayMax;
-        while (kd > 1 && dqmc_smem_bytes(c->N, false, kd) > (size_t)optin) kd /= 2;
-        if (dqmc_smem_bytes(c->N, false, kd) > (size_t)optin) kd = 0;
+        while (kd > 1 && dqmc_smem_bytes(c->N, nc, false, kd) > (size_t)optin) kd /= 2;
+        if (dqmc_smem_bytes(c->N, nc, false, kd) > (size_t)optin) kd = 0;
     }
-    const size_t bytes = dqmc_smem_bytes(c->N, in_smem, kd);
+    const size_t bytes = dqmc_smem_bytes(c->N, nc, in_smem, kd);
     e = cudaFuncSetAttribute(k_dqmc_slices<LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     k_dqmc_slices<LMAX><<<nf, kThreads, bytes, s>>>(
@@ -426,6 +434,7 @@ cudaError_t dqmc_slices(slmc_ctx* c, double* x, double* G, int nf, int chain0, i
                         long long* n_acc, cudaStream_t s) {
     const int lm = std::max(c->p.Lx, c->p.Ly);
     if (lm <= 8) return launch_slices<8>(c, x, G, nf, chain0, l0, nsl, sweep, n_acc, s);
+    if (lm <= 12) return launch_slices<12>(c, x, G, nf, chain0, l0, nsl, sweep, n_acc, s);
     if (lm <= 16) return launch_slices<16>(c, x, G, nf, chain0, l0, nsl, sweep, n_acc, s);
     return launch_slices<32>(c, x, G, nf, chain0, l0, nsl, sweep, n_acc, s);
 }

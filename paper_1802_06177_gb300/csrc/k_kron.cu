@@ -15,8 +15,11 @@
 //
 // One CTA owns a panel of NB columns of one field in shared memory for all nsl slices (as
 // the dense panel kernel does); within a slice, one pass transforms the x lines and one the
-// y lines of every column, each thread one line at a time with the outputs in registers.
+// y lines of every column, each thread one line at a time in registers with the folded transforms of
+// circ.cuh. The panel's columns are padded to the odd stride N | 1 and consecutive lanes take the same line of
+// consecutive columns, so neither pass meets a bank conflict (lanes along a column were 16 apart at Lx = 16).
 // Layout: column-major N x N, element (i, j) at j*N + i, site i = ix + Lx iy.
+#include "circ.cuh"
 #include "slmc_internal.cuh"
 
 namespace {
@@ -30,48 +33,48 @@ __global__ void __launch_bounds__(kThreads) k_slice_kron(const double* __restric
                                                          const double* __restrict__ kron, int Lx, int Ly, int L,
                                                          int l0, int nsl, double dtlam, double emu) {
     extern __shared__ double sm[];
-    const int N = Lx * Ly;
-    double* P = sm;                 // [kNB][N] panel, column-major
-    double* sc = sm + kNB * N;      // [N] e^{dtau mu} s_l
-    double* tx = sc + N;            // E_x, twice over
-    double* ty = tx + slmc::kKronTab;  // E_y, twice over
-    const int f = blockIdx.y, j0 = blockIdx.x * kNB, tid = threadIdx.x;
+    const int N = Lx * Ly, ld = N | 1;
+    double* P = sm;                 // [kNB][ld] panel, column-major
+    double* sc = sm + kNB * ld;     // [N] e^{dtau mu} s_l
+    double* cx = sc + N;            // folded coefficients of E_x, E_y
+    double* cy = cx + slmc::circ::ncoef(Lx);
+    const int f = blockIdx.y, j0 = blockIdx.x * kNB, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nb = min(kNB, N - j0);
     const size_t NN = (size_t)N * N;
     const double* Uf = U + f * NN + (size_t)j0 * N;
-    for (int k = tid; k < slmc::kKronTab; k += kThreads) {
-        tx[k] = kron[k];
-        ty[k] = kron[2 * slmc::kKronTab + k];
-    }
-    for (int idx = tid; idx < nb * N; idx += kThreads) P[idx] = Uf[idx];
+    slmc::circ::build(cx, kron, Lx, tid, kThreads);
+    slmc::circ::build(cy, kron + 2 * slmc::kKronTab, Ly, tid, kThreads);
+    for (int jj = warp; jj < nb; jj += kThreads / 32)
+        for (int i = lane; i < N; i += 32) P[jj * ld + i] = Uf[(size_t)jj * N + i];
     const double* xf = x + (size_t)f * N * L;
+    double* Pl = P + lane * ld;  // this lane's column
     for (int step = 0; step < nsl; ++step) {
         const int c = kTrans ? l0 + nsl - 1 - step : l0 + step;  // field column of the slice
         for (int i = tid; i < N; i += kThreads) sc[i] = exp(-dtlam * xf[(size_t)i * L + c]) * emu;
         __syncthreads();
-        // x lines (jj, iy): contiguous; the transposed slice scales its input here
-        for (int q = tid; q < nb * Ly; q += kThreads) {
-            const int jj = q / Ly, iy = q - jj * Ly;
-            slmc::circ_line<LMAX, true>(P, jj * N + iy * Lx, 1, Lx, tx, kTrans ? sc + iy * Lx : nullptr, 1, nullptr,
-                                        0, 1.0);
+        // pass 0: x lines (contiguous; the transposed slice scales its input); pass 1: y lines (stride Lx; the
+        // plain slice scales its output)
+        for (int pass = 0; pass < 2; ++pass) {
+            const int lines = pass ? Lx : Ly, step_l = pass ? 1 : Lx, stride = pass ? Lx : 1;
+            if (lane < nb)
+                for (int q = warp; q < lines; q += kThreads / 32) {
+                    const int o = q * step_l;
+                    slmc::circ::apply_any<LMAX>(pass ? Ly : Lx, Pl + o, stride, pass ? cy : cx,
+                                                kTrans && pass == 0 ? sc + o : nullptr, stride,
+                                                !kTrans && pass == 1 ? sc + o : nullptr, stride, 1.0);
+                }
+            __syncthreads();
         }
-        __syncthreads();
-        // y lines (jj, ix): stride Lx; the plain slice scales its output here
-        for (int q = tid; q < nb * Lx; q += kThreads) {
-            const int jj = q / Lx, ix = q - jj * Lx;
-            slmc::circ_line<LMAX, true>(P, jj * N + ix, Lx, Ly, ty, nullptr, 0, kTrans ? nullptr : sc + ix, Lx,
-                                        1.0);
-        }
-        __syncthreads();
     }
     double* Yf = Y + f * NN + (size_t)j0 * N;
-    for (int idx = tid; idx < nb * N; idx += kThreads) Yf[idx] = P[idx];
+    for (int jj = warp; jj < nb; jj += kThreads / 32)
+        for (int i = lane; i < N; i += 32) Yf[(size_t)jj * N + i] = P[jj * ld + i];
 }
 
 template <int LMAX, bool kTrans>
 cudaError_t launch_kron(slmc_ctx* c, const double* x, int nf, int l0, int nsl, cudaStream_t s) {
     const int N = c->N;
-    const size_t smem = ((size_t)kNB * N + N + 2 * slmc::kKronTab) * sizeof(double);
+    const size_t smem = ((size_t)kNB * (N | 1) + N + slmc::circ::ncoef(c->p.Lx) + slmc::circ::ncoef(c->p.Ly)) * sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_slice_kron<LMAX, kTrans>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
@@ -81,10 +84,12 @@ cudaError_t launch_kron(slmc_ctx* c, const double* x, int nf, int l0, int nsl, c
     return cudaGetLastError();
 }
 
+// LMAX: registers grow with the longest line expanded.
 template <bool kTrans>
 cudaError_t dispatch_kron(slmc_ctx* c, const double* x, int nf, int l0, int nsl, cudaStream_t s) {
     const int lm = c->p.Lx > c->p.Ly ? c->p.Lx : c->p.Ly;
     if (lm <= 8) return launch_kron<8, kTrans>(c, x, nf, l0, nsl, s);
+    if (lm <= 12) return launch_kron<12, kTrans>(c, x, nf, l0, nsl, s);
     if (lm <= 16) return launch_kron<16, kTrans>(c, x, nf, l0, nsl, s);
     return launch_kron<32, kTrans>(c, x, nf, l0, nsl, s);
 }

@@ -1,6 +1,8 @@
 // FP64 determinant and Green's function of small lattices (N <= 64) in one launch, one CTA per field
 // (small.cuh holds the steps and what bounds them). The per-group kernels it replaces were launch latency at
 // these sizes: a 4x4, L = 40 determinant took about 28 launches.
+#include <algorithm>
+
 #include "small.cuh"
 
 namespace {
@@ -8,7 +10,7 @@ namespace {
 using namespace slmc::sm;
 
 template <int NMAX, int LMAX>
-__global__ void __launch_bounds__(4 * NMAX) k_small_logdet(const double* __restrict__ x, const double* __restrict__ kron,
+__global__ void __launch_bounds__(4 * NMAX, 1) k_small_logdet(const double* __restrict__ x, const double* __restrict__ kron,
                                                            double* __restrict__ lndet, int* __restrict__ sign,
                                                            double* __restrict__ Gout, unsigned int* __restrict__ err, int N,
                                                            int Lx, int Ly, int L, int n_s, double dtlam, double emu) {
@@ -25,10 +27,8 @@ __global__ void __launch_bounds__(4 * NMAX) k_small_logdet(const double* __restr
         B[idx] = e;
         T[idx] = e;
     }
-    for (int k = tid; k < slmc::kKronTab; k += NT) {
-        v.tx[k] = kron[k];
-        v.ty[k] = kron[2 * slmc::kKronTab + k];
-    }
+    slmc::circ::build(v.cx, kron, Lx, tid, NT);
+    slmc::circ::build(v.cy, kron + 2 * slmc::kKronTab, Ly, tid, NT);
     if (tid < N) v.lnd[tid] = 0.0;
     __syncthreads();
     bool bad = false;
@@ -106,10 +106,12 @@ bool small_active(const slmc_ctx* c) {
 }
 
 cudaError_t small_logdet(slmc_ctx* c, const double* x, int nf, double* lndet, int* sign, double* G, cudaStream_t s) {
-    const bool l8 = c->p.Lx <= 8 && c->p.Ly <= 8;
-    if (c->N <= 16) return l8 ? launch_small<16, 8>(c, x, nf, lndet, sign, G, s) : launch_small<16, 32>(c, x, nf, lndet, sign, G, s);
-    if (c->N <= 32) return l8 ? launch_small<32, 8>(c, x, nf, lndet, sign, G, s) : launch_small<32, 32>(c, x, nf, lndet, sign, G, s);
-    return l8 ? launch_small<64, 8>(c, x, nf, lndet, sign, G, s) : launch_small<64, 32>(c, x, nf, lndet, sign, G, s);
+    const int lm = std::max(c->p.Lx, c->p.Ly);  // at most N / 2: 8, 16 and 32 in the three size classes
+    if (c->N <= 16) return launch_small<16, 8>(c, x, nf, lndet, sign, G, s);
+    if (c->N <= 32)
+        return lm <= 8 ? launch_small<32, 8>(c, x, nf, lndet, sign, G, s) : launch_small<32, 16>(c, x, nf, lndet, sign, G, s);
+    if (lm <= 8) return launch_small<64, 8>(c, x, nf, lndet, sign, G, s);
+    return lm <= 16 ? launch_small<64, 16>(c, x, nf, lndet, sign, G, s) : launch_small<64, 32>(c, x, nf, lndet, sign, G, s);
 }
 
 }  // namespace slmc

@@ -159,31 +159,6 @@ inline int rows_per_lane_class(int N) {
 }
 
 // ---- Philox-4x32-10 (Salmon et al., SC'11), written from the published definition ----
-// One in-place circulant line transform of a strided vector v[m] = g[base + m stride],
-// m < Ld: out[d] = sum_m tab[(d - m) mod Ld] v[m] (kLeft: a circulant applied from the left)
-// or sum_m v[m] tab[(m - d) mod Ld] (from the right), with optional input scales
-// in_sc[m in_st] and output scales out_sc[d out_st] * out_mul. tab holds the factor twice
-// over so that the index needs no modulo. The outputs stay in registers until the whole line
-// has been read.
-template <int LMAX, bool kLeft>
-__device__ __forceinline__ void circ_line(double* g, int base, int stride, int Ld, const double* __restrict__ tab,
-                                          const double* in_sc, int in_st, const double* out_sc, int out_st,
-                                          double out_mul) {
-    double acc[LMAX];
-#pragma unroll
-    for (int d = 0; d < LMAX; ++d) acc[d] = 0.0;
-#pragma unroll 2
-    for (int m = 0; m < Ld; ++m) {
-        const double v = in_sc ? g[base + m * stride] * in_sc[m * in_st] : g[base + m * stride];
-#pragma unroll
-        for (int d = 0; d < LMAX; ++d)
-            if (d < Ld) acc[d] = fma(v, tab[kLeft ? d - m + Ld : m - d + Ld], acc[d]);
-    }
-#pragma unroll
-    for (int d = 0; d < LMAX; ++d)
-        if (d < Ld) g[base + d * stride] = out_sc ? acc[d] * (out_sc[d * out_st] * out_mul) : acc[d];
-}
-
 struct u32x4 { uint32_t x, y, z, w; };
 
 __device__ __forceinline__ u32x4 philox4x32_10(u32x4 c, uint32_t k0, uint32_t k1) {

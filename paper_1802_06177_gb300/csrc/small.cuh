@@ -14,6 +14,7 @@
 
 #include <cfloat>
 
+#include "circ.cuh"
 #include "slmc_internal.cuh"
 
 namespace slmc {
@@ -24,13 +25,16 @@ struct Dim {
     static constexpr int ld = NMAX + 1, mat = NMAX * ld, threads = 4 * NMAX, rpt = NMAX / 4;
 };
 
+constexpr int kSmallCoef = 481;  // circ::ncoef of the longest line (31: one level; 32 folds twice)
+static_assert(circ::ncoef(31) <= kSmallCoef && circ::ncoef(32) <= kSmallCoef && circ::ncoef(30) <= kSmallCoef, "");
+
 // Vectors of one field in shared memory.
 template <int NMAX>
 struct Vecs {
     double lnd[NMAX], lnn[NMAX];   // ln D, new ln D
     double key[NMAX], e1[NMAX], e2[NMAX], tau[NMAX], beta[NMAX];
     double sc[NMAX];               // slice scales
-    double tx[kKronTab], ty[kKronTab];  // circulant factors, twice over
+    double cx[kSmallCoef], cy[kSmallCoef];  // folded coefficients of E_x, E_y
     double lbuf[2][NMAX];          // multipliers of the current / next LU step
     double logabs;
     int perm[NMAX];
@@ -57,17 +61,16 @@ __device__ __forceinline__ void slices(double* P, Vecs<NMAX>& v, const double* _
         if (tid < N) v.sc[tid] = exp(-dtlam * xv) * emu;
         if (tid < N && step + 1 < c1 - c0) xv = xf[(size_t)tid * L + (kTrans ? c1 - 2 - step : c0 + step + 1)];
         if (kTrans) __syncthreads();  // the x pass scales its input; plain slices use sc after the next barrier
-        for (int q = tid; q < N * Ly; q += NT) {
-            const int jj = q / Ly, iy = q - jj * Ly;
-            circ_line<LMAX, true>(P, jj * ld + iy * Lx, 1, Lx, v.tx, kTrans ? v.sc + iy * Lx : nullptr, 1, nullptr, 0,
-                                  1.0);
+        for (int pass = 0; pass < 2; ++pass) {
+            const int lines = pass ? Lx : Ly, step_l = pass ? 1 : Lx, stride = pass ? Lx : 1;
+            for (int q = tid; q < N * lines; q += NT) {
+                const int li = q / N, jj = q - li * N, o = li * step_l;
+                circ::apply_any<LMAX>(pass ? Ly : Lx, P + jj * ld + o, stride, pass ? v.cy : v.cx,
+                                      kTrans && pass == 0 ? v.sc + o : nullptr, stride,
+                                      !kTrans && pass == 1 ? v.sc + o : nullptr, stride, 1.0);
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        for (int q = tid; q < N * Lx; q += NT) {
-            const int jj = q / Lx, ix = q - jj * Lx;
-            circ_line<LMAX, true>(P, jj * ld + ix, Lx, Ly, v.ty, nullptr, 0, kTrans ? nullptr : v.sc + ix, Lx, 1.0);
-        }
-        __syncthreads();
     }
 }
 

@@ -39,9 +39,11 @@ namespace {
 
 using namespace slmc::tc;
 using slmc::s7::abs_bits;
+using slmc::s7::bf16_of;
+using slmc::s7::bf16x2_of;
+using slmc::s7::combine;
 using slmc::s7::exponent_of_bits;
 using slmc::s7::kS;
-using slmc::s7::pow2d;
 using slmc::s7::slice7;
 using slmc::s7::warp_max_bits;
 
@@ -66,6 +68,17 @@ __device__ __forceinline__ void levels_to_int(const uint32_t (&v)[kLv], long lon
     lo = (long long)__float2int_rn(__uint_as_float(v[3]));
 #pragma unroll
     for (int lv = 4; lv < kLv; ++lv) lo = lo * 128 + (long long)__float2int_rn(__uint_as_float(v[lv]));
+}
+
+// The same for sums below 2^22 (K <= 32 indices: at most 36864 * 32 < 2^21): one exact FP32 addition places the
+// integer in the significand, where the conversion instruction would take the FP64 pipe's issue.
+__device__ __forceinline__ int small_int(uint32_t v) {
+    return __float_as_int(__uint_as_float(v) + 12582912.f) - 0x4B400000;
+}
+__device__ __forceinline__ void small_levels_to_int(const uint32_t (&v)[kLv], long long& hi, long long& lo) {
+    hi = (long long)((small_int(v[0]) << 7) + small_int(v[1])) * 128 + (long long)small_int(v[2]);
+    lo = (long long)((small_int(v[3]) << 7) + small_int(v[4])) * 16384 +
+         (long long)((small_int(v[5]) << 7) + small_int(v[6]));
 }
 
 // Compact-WY triangle S of BP reflectors from their Gram matrix G (row stride ldg) and tau, by the 256
@@ -130,39 +143,52 @@ __device__ __forceinline__ void wy_triangle_blocked(const double* G, int ldg, co
 }
 
 // ---- panel ----------------------------------------------------------------------------------
-// 16 warps per field: the panel is a chain of latency-bound column steps (dot products, warp
-// reductions, a block barrier each) that leaves the FP64 pipe half idle with 8 warps.
-constexpr int kPT = 512;
-constexpr int kPW = kPT / 32;
+// The panel is a chain of column steps (dot products, warp reductions, square root and divisions, one block
+// barrier each), so what counts is how many panels an SM works on at once, beside the trailing updates of the
+// other sub-batches: 8 warps per field, and shared memory for rows p.. only (PanelSmem; 77 KB for the first
+// panel of N = 256, 42 KB for the fifth, against 102 KB and 16 warps before). With at most one field per SM nothing
+// shares it, and 16 warps shorten the chain (24x24, 32 fields: 656 against 665 ms per evaluation).
 
+// Shared memory of panel t: V (rows p.. of the panel), the last panel's S and Gram matrix, the scales, the first
+// panel's ordering keys, tau, beta, the permutation.
 template <int BP>
-__global__ void __launch_bounds__(kPT, 2)
+struct PanelSmem {
+    __host__ __device__ static size_t doubles(int N, int p, bool last) {
+        return (size_t)(N - p) * (BP + 1) + (last ? 2 * BP * BP : 0) + 3 * (size_t)N + (p == 0 ? N : 0) + 2 * BP;
+    }
+    static size_t bytes(int N, int p, bool last) { return sizeof(double) * doubles(N, p, last) + sizeof(int) * (size_t)N; }
+};
+
+template <int BP, int kPT>
+__global__ void __launch_bounds__(kPT, kPT == 256 ? 3 : 1)
     k_qrt_panel(double* __restrict__ Yall, double* __restrict__ lnD_all, double* __restrict__ QRall,
                 double* __restrict__ tau_all, int* __restrict__ perm_all, int* __restrict__ sgnU,
                 double* __restrict__ Sall, unsigned int* __restrict__ err, int N, int t, double* __restrict__ lnDn_ws,
                 int* __restrict__ ntriv_ws, __nv_bfloat16* __restrict__ V1, int* __restrict__ eV1,
                 __nv_bfloat16* __restrict__ V2, int* __restrict__ eV2, int kpad, int mpad, size_t plane1,
                 size_t plane2, int fbase) {
-    constexpr int BPS = BP + 1;
+    constexpr int BPS = BP + 1, kPW = kPT / 32;
     const int f = blockIdx.x, gf = fbase + f;
     const size_t NN = (size_t)N * N;
     double* __restrict__ Y = Yall + f * NN;
     double* __restrict__ QR = QRall + f * NN;
     extern __shared__ __align__(16) unsigned char smraw[];
-    double* Vp = reinterpret_cast<double*>(smraw);
-    double* Ssm = Vp + (size_t)N * BPS;
-    double* Wsm = Ssm + BP * BP;
-    double* s_key = Wsm + kWarps * BP * kCT;  // the layout of QrSmem<BP> (Wsm holds the Gram matrix here)
-    double* s_lnd = s_key + N;
+    const int p = t * BP, nb = min(BP, N - p), npanels = (N + BP - 1) / BP;
+    const bool last = t == npanels - 1;
+    double* Vst = reinterpret_cast<double*>(smraw);
+    double* Vp = Vst - (size_t)p * BPS;  // row r of the panel at r BPS, rows p.. stored
+    double* Ssm = Vst + (size_t)(N - p) * BPS;
+    double* Gsm = Ssm + BP * BP;  // (last panel only)
+    double* s_lnd = Ssm + (last ? 2 * BP * BP : 0);
     double* s_lnDn = s_lnd + N;
     double* s_g = s_lnDn + N;
     double* s_tau = s_g + N;
     double* s_beta = s_tau + BP;
-    int* s_perm = reinterpret_cast<int*>(s_beta + BP);
+    double* s_key = s_beta + BP;  // (first panel only)
+    int* s_perm = reinterpret_cast<int*>(s_key + (p == 0 ? N : 0));
     __shared__ double s_mx;
     __shared__ int s_ntriv, s_wide;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int p = t * BP, nb = min(BP, N - p), npanels = (N + BP - 1) / BP;
 
     for (int j = tid; j < N; j += kPT) s_lnd[j] = lnD_all[(size_t)f * N + j];
     if (tid == 0) {
@@ -186,10 +212,12 @@ __global__ void __launch_bounds__(kPT, 2)
                 a = fma(y, y, a);
             }
             a = slmc::warp_allsum(a);
-            if (lane == 0) {
-                const double key = a * exp(2.0 * (s_lnd[j] - s_mx));
-                s_key[j] = (key >= 0.0) ? key : -1.0;
-            }
+            if (lane == 0) s_key[j] = a;
+        }
+        __syncthreads();
+        for (int j = tid; j < N; j += kPT) {  // a column per lane: an exponential is about 20 FP64 instructions
+            const double key = s_key[j] * exp(2.0 * (s_lnd[j] - s_mx));
+            s_key[j] = (key >= 0.0) ? key : -1.0;
         }
         __syncthreads();
         for (int j = tid; j < N; j += kPT) {
@@ -219,8 +247,8 @@ __global__ void __launch_bounds__(kPT, 2)
     __syncthreads();
 
     // the Gram matrix and S of every panel but the last are formed on the tensor cores (k_qrt_gemm1)
-    panel_step<BP, kPT>(Y, QR, tau_all + (size_t)f * N, Sall + (size_t)f * N * BP, Vp, Ssm, Wsm, s_lnd, s_lnDn, s_g, s_tau,
-                        s_beta, s_perm, &s_ntriv, &s_wide, N, p, nb, t == npanels - 1);
+    panel_step<BP, kPT>(Y, QR, tau_all + (size_t)f * N, Sall + (size_t)f * N * BP, Vp, Ssm, Gsm, s_lnd, s_lnDn, s_g, s_tau,
+                        s_beta, s_perm, &s_ntriv, &s_wide, N, p, nb, last);
     __syncthreads();
     if (tid < nb) lnDn_ws[(size_t)gf * N + p + tid] = s_lnDn[p + tid];
     if (tid == 0) {  // reflectors with tau != 0 so far (their parity is the sign of det U)
@@ -245,11 +273,13 @@ __global__ void __launch_bounds__(kPT, 2)
         const int e = exponent_of_bits(warp_max_bits(mx));
         if (lane == 0) eV1[(size_t)gf * kVRows + m] = e;
         __nv_bfloat16* dst = V1 + ((size_t)gf * kVRows + m) * kpad;
-        for (int k = kstart + lane; k < kpad; k += 32) {
-            __nv_bfloat16 q[kS];
-            slice7((k >= p && k < N) ? Vp[k * BPS + m] : 0.0, e, q);
+        for (int k = kstart + 2 * lane; k < kpad; k += 64) {  // two adjacent rows per lane (multiples of 64)
+            float q0[kS], q1[kS];
+            slice7((k >= p && k < N) ? Vp[k * BPS + m] : 0.0, e, q0);
+            slice7((k + 1 >= p && k + 1 < N) ? Vp[(k + 1) * BPS + m] : 0.0, e, q1);
 #pragma unroll
-            for (int s = 0; s < kS; ++s) dst[(size_t)s * plane1 + k] = q[s];
+            for (int s = 0; s < kS; ++s)
+                *reinterpret_cast<uint32_t*>(dst + (size_t)s * plane1 + k) = bf16x2_of(q0[s], q1[s]);
         }
     }
     // V2: row r over the reflectors (K = the BP reflectors, padded to 64 with zeros set at init),
@@ -259,10 +289,10 @@ __global__ void __launch_bounds__(kPT, 2)
         const int e = exponent_of_bits(warp_max_bits(abs_bits(v)));
         if (lane == 0) eV2[(size_t)gf * mpad + r] = e;
         if (lane < BP) {
-            __nv_bfloat16 q[kS];
+            float q[kS];
             slice7(v, e, q);
 #pragma unroll
-            for (int s = 0; s < kS; ++s) V2[(size_t)s * plane2 + ((size_t)gf * mpad + r) * 64 + lane] = q[s];
+            for (int s = 0; s < kS; ++s) V2[(size_t)s * plane2 + ((size_t)gf * mpad + r) * 64 + lane] = bf16_of(q[s]);
         }
     }
 }
@@ -281,11 +311,13 @@ __global__ void __launch_bounds__(256) k_qrt_slice_C(const double* __restrict__ 
     const int e = exponent_of_bits(warp_max_bits(mx));
     if (lane == 0) eC[(size_t)gf * jpad + jj] = e;
     __nv_bfloat16* dst = Cs + ((size_t)gf * jpad + jj) * kpad;
-    for (int k = (p / 64) * 64 + lane; k < kpad; k += 32) {
-        __nv_bfloat16 q[kS];
-        slice7((k >= p && k < N) ? col[k] : 0.0, e, q);
+    for (int k = (p / 64) * 64 + 2 * lane; k < kpad; k += 64) {  // two adjacent rows per lane (multiples of 64)
+        float q0[kS], q1[kS];
+        slice7((k >= p && k < N) ? col[k] : 0.0, e, q0);
+        slice7((k + 1 >= p && k + 1 < N) ? col[k + 1] : 0.0, e, q1);
 #pragma unroll
-        for (int s = 0; s < kS; ++s) dst[(size_t)s * plane + k] = q[s];
+        for (int s = 0; s < kS; ++s)
+            *reinterpret_cast<uint32_t*>(dst + (size_t)s * plane + k) = bf16x2_of(q0[s], q1[s]);
     }
 }
 
@@ -305,7 +337,6 @@ __global__ void __launch_bounds__(kQT, 2)
                 int n_t, int kpad, int jpad, int wpad, size_t planeW, int fbase, unsigned int* __restrict__ err) {
     constexpr uint32_t kTileB = BP * 128;
     constexpr uint32_t kChunkB = kS * kTileB;
-    constexpr uint32_t kIdesc = idesc_f32acc(1, 128, BP);
     constexpr int WS = BP + 1;
     constexpr int kMC = 128 - BP;  // trailing columns per CTA
     const int mt = blockIdx.x, f = blockIdx.y, gf = fbase + f;
@@ -388,7 +419,6 @@ __global__ void __launch_bounds__(kQT, 2)
     } else if (warp == 9) {
         if (lane == 0) {
             bool ok = true;
-            uint32_t written = 0;
             for (int u = 0; u < nkc && ok; ++u) {
                 const int bs = u & 1, seg = u / kSegChunks;
                 if (!mbar_wait(smem_u32(&bar_bfull[bs]), (u >> 1) & 1, err) || abort_sh) {
@@ -402,18 +432,13 @@ __global__ void __launch_bounds__(kQT, 2)
                         break;
                     }
                     tc_fence_after();
+                    // slices b = 0 .. 6 - a of V into the levels a .. 6: adjacent operand rows and adjacent
+                    // accumulators, so one instruction of N = (7 - a) BP per step of K
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) {
-                        const uint64_t ad = smem_desc_sw128(aring + slot * kTileA + ks * 32);
-#pragma unroll
-                        for (int b = 0; b < kS; ++b) {
-                            if (a + b >= kLv) continue;
-                            const int acc = seg * kLv + a + b;
-                            const uint64_t bd = smem_desc_sw128(bbuf + bs * kChunkB + b * kTileB + ks * 32);
-                            mma_bf16(tmem + (uint32_t)(acc * BP), ad, bd, kIdesc, (written >> acc) & 1u);
-                            written |= 1u << acc;
-                        }
-                    }
+                    for (int ks = 0; ks < 4; ++ks)
+                        mma_bf16(tmem + (uint32_t)((seg * kLv + a) * BP), smem_desc_sw128(aring + slot * kTileA + ks * 32),
+                                 smem_desc_sw128(bbuf + bs * kChunkB + ks * 32), idesc_f32acc(1, 128, (kS - a) * BP),
+                                 ((u - seg * kSegChunks) | a | ks) != 0 ? 1u : 0u);
                     mma_commit(smem_u32(&bar_empty[slot]));
                 }
                 if (ok) mma_commit(smem_u32(&bar_bempty[bs]));
@@ -458,8 +483,7 @@ __global__ void __launch_bounds__(kQT, 2)
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     const int m = h * HC + c0 + c;
-                    stW[r * WS + m] = fma(__ll2double_rn(hi[c]), 268435456.0, __ll2double_rn(lo[c])) *
-                                      pow2d(er + eV_sh[m] - kUnitShift);
+                    stW[r * WS + m] = combine(hi[c], lo[c], er + eV_sh[m] - kUnitShift);
                 }
             }
         }
@@ -489,11 +513,11 @@ __global__ void __launch_bounds__(kQT, 2)
                 const int e = exponent_of_bits(warp_max_bits(abs_bits(v)));
                 if (lane == 0) eW[(size_t)gf * wpad + j2] = e;
                 if (lane < BP) {
-                    __nv_bfloat16 q[kS];
+                    float q[kS];
                     slice7(v, e, q);
                     __nv_bfloat16* dst = Ws + ((size_t)gf * wpad + j2) * 64 + lane;
 #pragma unroll
-                    for (int s = 0; s < kS; ++s) dst[(size_t)s * planeW] = q[s];
+                    for (int s = 0; s < kS; ++s) dst[(size_t)s * planeW] = bf16_of(q[s]);
                 }
             }
         }
@@ -517,7 +541,6 @@ __global__ void __launch_bounds__(kQT, 2)
                 double* __restrict__ Yall, int N, int p, int j0, int n_t, int mpad, int wpad, int fbase,
                 unsigned int* __restrict__ err) {
     constexpr uint32_t kTileW = kNC * 128;
-    constexpr uint32_t kIdesc = idesc_f32acc(1, 128, kNC);
     const int nt = blockIdx.x, mt = p / 128 + blockIdx.y, f = blockIdx.z, gf = fbase + f;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -576,7 +599,6 @@ __global__ void __launch_bounds__(kQT, 2)
     } else if (warp == 9) {
         if (lane == 0) {
             bool ok = mbar_wait(smem_u32(&bar_bfull), 0, err);
-            uint32_t written = 0;
             for (int a = 0; a < kS && ok; ++a) {
                 const int slot = a % kRing;
                 if (!mbar_wait(smem_u32(&bar_full[slot]), (a / kRing) & 1, err)) {
@@ -585,17 +607,9 @@ __global__ void __launch_bounds__(kQT, 2)
                 }
                 tc_fence_after();
 #pragma unroll
-                for (int ks = 0; ks < BP / 16; ++ks) {
-                    const uint64_t ad = smem_desc_sw128(aring + slot * kTileA + ks * 32);
-#pragma unroll
-                    for (int b = 0; b < kS; ++b) {
-                        if (a + b >= kLv) continue;
-                        const int lv = a + b;
-                        const uint64_t bd = smem_desc_sw128(bbuf + b * kTileW + ks * 32);
-                        mma_bf16(tmem + (uint32_t)(lv * kNC), ad, bd, kIdesc, (written >> lv) & 1u);
-                        written |= 1u << lv;
-                    }
-                }
+                for (int ks = 0; ks < BP / 16; ++ks)
+                    mma_bf16(tmem + (uint32_t)(a * kNC), smem_desc_sw128(aring + slot * kTileA + ks * 32),
+                             smem_desc_sw128(bbuf + ks * 32), idesc_f32acc(1, 128, (kS - a) * kNC), (a | ks) != 0 ? 1u : 0u);
                 mma_commit(smem_u32(&bar_empty[slot]));
             }
             if (ok) mma_commit(smem_u32(&bar_acc));
@@ -628,9 +642,8 @@ __global__ void __launch_bounds__(kQT, 2)
 #pragma unroll
                     for (int lv = 0; lv < kLv; ++lv) w[lv] = v[lv][c];
                     long long hi, lo;
-                    levels_to_int(w, hi, lo);
-                    const double t = fma(__ll2double_rn(hi), 268435456.0, __ll2double_rn(lo)) *
-                                     pow2d(ev + eW_sh[cc] - kUnitShift);
+                    small_levels_to_int(w, hi, lo);
+                    const double t = combine(hi, lo, ev + eW_sh[cc] - kUnitShift);
                     double* y = Yf + (size_t)col_sh[cc] * N + r;
                     *y = *y - t;
                 }
@@ -671,13 +684,15 @@ QrtArgs qrt_args(const slmc_ctx* c) {
     return a;
 }
 
-template <int BP>
+template <int BP, int kPT>
 cudaError_t launch_panel(slmc_ctx* c, int nf, int t, cudaStream_t s) {
     const QrtArgs a = qrt_args(c);
-    const size_t smP = QrSmem<BP>::bytes(a.N);
-    cudaError_t e = cudaFuncSetAttribute(k_qrt_panel<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smP);
+    const int p = t * BP;
+    const size_t smP = PanelSmem<BP>::bytes(a.N, p, p + BP >= a.N);
+    cudaError_t e = cudaFuncSetAttribute(k_qrt_panel<BP, kPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)std::max(PanelSmem<BP>::bytes(a.N, 0, a.N <= BP), smP));
     if (e != cudaSuccess) return e;
-    k_qrt_panel<BP><<<nf, kPT, smP, s>>>(c->Y, c->lnD, c->QR, c->tau, c->perm, c->sgnU, c->Sws, c->err, a.N, t,
+    k_qrt_panel<BP, kPT><<<nf, kPT, smP, s>>>(c->Y, c->lnD, c->QR, c->tau, c->perm, c->sgnU, c->Sws, c->err, a.N, t,
                                               c->qt_lnDn, c->qt_ntriv, a.V1, c->qt_eV1, a.V2, c->qt_eV2, a.kpad,
                                               a.mpad, a.plane1, a.plane2, c->fbase);
     return cudaGetLastError();
@@ -763,7 +778,9 @@ int qrt_panels(const slmc_ctx* c) {
 }
 
 cudaError_t qrt_panel(slmc_ctx* c, int nf, int t, cudaStream_t s) {
-    return qr_panel_width(c) == 32 ? launch_panel<32>(c, nf, t, s) : launch_panel<16>(c, nf, t, s);
+    if (nf <= c->num_sms)
+        return qr_panel_width(c) == 32 ? launch_panel<32, 512>(c, nf, t, s) : launch_panel<16, 512>(c, nf, t, s);
+    return qr_panel_width(c) == 32 ? launch_panel<32, 256>(c, nf, t, s) : launch_panel<16, 256>(c, nf, t, s);
 }
 
 cudaError_t qrt_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s) {

@@ -65,11 +65,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 double* __restrict__ Yout, const float* __restrict__ sc32, int N, int Npad, int L, int l0, int nsl,
                 int kStages, unsigned int* __restrict__ err) {
     constexpr uint32_t TCOLS = tmem_cols(kLevels * MT * NT);
-    constexpr uint32_t IDESC = kIdesc | ((uint32_t)(NT >> 3) << 17);
+    constexpr int kGroup = kYS * NT <= 256 ? kYS : 2;  // Y slices per instruction (N <= 256)
+    static_assert(kGroup * NT <= 256, "");
     const int f = blockIdx.y, j0 = blockIdx.x * NT;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nk = Npad / 64;
-    const uint32_t tileB = NT * 128u;         // one (Y slice, 64-row K chunk) tile
+    // one (64-row K chunk, Y slice) tile; the three slices of a chunk are adjacent
+    constexpr uint32_t tileB = NT * 128u;
     const uint32_t sliceB = (uint32_t)nk * tileB;
 
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -139,7 +141,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                     break;
                 }
                 tc_fence_after();
-                uint32_t written = 0;
                 for (int u = 0; u < per_slice && ok; ++u, ++t) {
                     const int st = t % kStages, kc = u / (MT * kFS), mt = (u / kFS) % MT, fs = u % kFS;
                     if (!mbar_wait(smem_u32(&bar_full[st]), (t / kStages) & 1, err) || abort_sh) {
@@ -148,16 +149,25 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     tc_fence_after();
                     const uint32_t a = stg + st * kStageBytes;
+                    // slices j of Y go to the levels fs + j: adjacent accumulators, adjacent operand tiles, so
+                    // one instruction of N = cnt NT columns per step of K (kGroup slices at most)
+                    const int nj = min(kYS, kLevels - fs);
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks) {
                         const uint64_t ad = smem_desc_sw128(a + ks * 32);
+                        const bool fresh = kc == 0 && ks == 0;  // this slice's first products of the M tile
+                        auto mm = [&](int j, int cnt, uint32_t acc) {
+                            mma_bf16(tmem + (uint32_t)((mt * kLevels + fs + j) * NT), ad,
+                                     smem_desc_sw128(bbuf + (uint32_t)(kc * kYS + j) * tileB + ks * 32),
+                                     kIdesc | ((uint32_t)(cnt * NT >> 3) << 17), acc);
+                        };
+                        if (fresh && fs == 1) {  // level 3 is first written here, levels 1 and 2 by fs = 0
+                            mm(0, 2, 1u);
+                            mm(2, 1, 0u);
+                        } else {
 #pragma unroll
-                        for (int j = 0; j < kYS; ++j) {
-                            if (fs + j >= kLevels) continue;
-                            const int bit = (fs + j) * MT + mt;
-                            const uint64_t bd = smem_desc_sw128(bbuf + j * sliceB + kc * tileB + ks * 32);
-                            mma_bf16(tmem + (uint32_t)(bit * NT), ad, bd, IDESC, (written >> bit) & 1u);
-                            written |= 1u << bit;
+                            for (int j = 0; j < kYS; j += kGroup)
+                                if (j < nj) mm(j, min(kGroup, nj - j), fresh && fs == 0 ? 0u : 1u);
                         }
                     }
                     mma_commit(smem_u32(&bar_empty[st]));
@@ -213,7 +223,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         uint32_t a[kLevels][8];
                         const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(h * NH + c0);
 #pragma unroll
-                        for (int lv = 0; lv < kLevels; ++lv) tmem_ld8(tl + (uint32_t)((lv * MT + mt) * NT), a[lv]);
+                        for (int lv = 0; lv < kLevels; ++lv) tmem_ld8(tl + (uint32_t)((mt * kLevels + lv) * NT), a[lv]);
                         tmem_ld_wait();
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {
@@ -266,7 +276,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int mt = 0; mt < MT; ++mt) {
                 const int i = mt * 128 + r;
                 if (i >= Npad) continue;
-                const uint32_t rowoff = (uint32_t)(i >> 6) * tileB + (uint32_t)(i & 7) * 2u;
+                const uint32_t rowoff = (uint32_t)(i >> 6) * (kYS * tileB) + (uint32_t)(i & 7) * 2u;
                 const int kchunk = (i & 63) >> 3;
 #pragma unroll
                 for (int c0 = 0; c0 < NH; c0 += 8) {
@@ -281,9 +291,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                         // K-major 128-byte swizzle: row (column of Y) h NH + c0 + c, 16-byte chunk kchunk ^ c
                         const uint32_t off =
                             rowoff + (uint32_t)(h * NH + c0 + c) * 128u + ((uint32_t)(kchunk ^ c) << 4);
-                        *reinterpret_cast<__nv_bfloat16*>(bgen + off) = __float2bfloat16_rn(q0);
-                        *reinterpret_cast<__nv_bfloat16*>(bgen + sliceB + off) = __float2bfloat16_rn(q1);
-                        *reinterpret_cast<__nv_bfloat16*>(bgen + 2 * sliceB + off) = __float2bfloat16_rn(q2);
+                        // small integers: BF16 is the upper half of their FP32 bits
+                        *reinterpret_cast<uint16_t*>(bgen + off) = (uint16_t)(__float_as_uint(q0) >> 16);
+                        *reinterpret_cast<uint16_t*>(bgen + tileB + off) = (uint16_t)(__float_as_uint(q1) >> 16);
+                        *reinterpret_cast<uint16_t*>(bgen + 2 * tileB + off) = (uint16_t)(__float_as_uint(q2) >> 16);
                     }
                     asm volatile("" ::: "memory");
                 }

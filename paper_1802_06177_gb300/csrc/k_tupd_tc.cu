@@ -35,9 +35,10 @@ namespace {
 
 using namespace slmc::tc;
 using slmc::s7::abs_bits;
+using slmc::s7::bf16x2_of;
+using slmc::s7::combine;
 using slmc::s7::exponent_of_bits;
 using slmc::s7::kS;
-using slmc::s7::pow2d;
 using slmc::s7::slice7;
 using slmc::s7::warp_max_bits;
 
@@ -50,7 +51,6 @@ constexpr uint32_t kBTile = kNT * 128;  // 32 rows (columns of T) x 64 BF16
 constexpr uint32_t kBChunk = kS * kBTile;
 constexpr uint32_t kTmemCols = 256;     // 7 x 32 = 224 used
 constexpr int kRingA = 3;               // A slices in flight (tile a is released after its products)
-constexpr uint32_t kIdesc = idesc_f32acc(1, 128, kNT);
 
 __device__ __forceinline__ int warp_sum_int(int v) {
 #pragma unroll
@@ -84,11 +84,13 @@ __global__ void __launch_bounds__(256) k_tt_slice_B(const double* __restrict__ T
         const int e = exponent_of_bits(warp_max_bits(m));
         if (lane == 0) eB[(size_t)(fbase + f) * npad + j] = e;
         __nv_bfloat16* dst = Bs + ((size_t)(fbase + f) * npad + j) * npad;
-        for (int k = lane; k < npad; k += 32) {
-            __nv_bfloat16 q[kS];
-            slice7(k < N ? tile[(size_t)perm_s[k] * (CB + 1) + c] : 0.0, e, q);
+        for (int k = 2 * lane; k < npad; k += 64) {  // two adjacent k per lane (npad is a multiple of 64)
+            float q0[kS], q1[kS];
+            slice7(k < N ? tile[(size_t)perm_s[k] * (CB + 1) + c] : 0.0, e, q0);
+            slice7(k + 1 < N ? tile[(size_t)perm_s[k + 1] * (CB + 1) + c] : 0.0, e, q1);
 #pragma unroll
-            for (int s = 0; s < kS; ++s) dst[(size_t)s * plane + k] = q[s];
+            for (int s = 0; s < kS; ++s)
+                *reinterpret_cast<uint32_t*>(dst + (size_t)s * plane + k) = bf16x2_of(q0[s], q1[s]);
         }
     }
 }
@@ -115,25 +117,29 @@ __global__ void __launch_bounds__(256) k_tt_slice_A(const double* __restrict__ Q
         const int e = exponent_of_bits(warp_max_bits(m));
         if (lane == 0) eA[(size_t)(fbase + f) * mpad + i] = e;
         __nv_bfloat16* dst = As + ((size_t)(fbase + f) * mpad + i) * npad;
-        int rs[kS] = {0, 0, 0, 0, 0, 0, 0};
-        for (int k = lane; k < npad; k += 32) {
-            __nv_bfloat16 q[kS];
-            slice7(k < N ? row[k] : 0.0, e, q);
+        float rs[kS] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // row sums of |slice|, integers below 2^24
+        for (int k = 2 * lane; k < npad; k += 64) {
+            float q0[kS], q1[kS];
+            slice7(k < N ? row[k] : 0.0, e, q0);
+            slice7(k + 1 < N ? row[k + 1] : 0.0, e, q1);
 #pragma unroll
             for (int s = 0; s < kS; ++s) {
-                dst[(size_t)s * plane + k] = q[s];
-                rs[s] += (int)fabsf(__bfloat162float(q[s]));
+                *reinterpret_cast<uint32_t*>(dst + (size_t)s * plane + k) = bf16x2_of(q0[s], q1[s]);
+                rs[s] += fabsf(q0[s]) + fabsf(q1[s]);
             }
         }
+        // bound of every level in integers (in FP64 these sums took a third of the kernel's FP64 slots, all of them
+        // for work that is not FP64): at most 7 * 128 * 1024 * 128 < 2^27
+        int rowsum[kS];
         bool bad = false;
 #pragma unroll
-        for (int s = 0; s < kS; ++s) rs[s] = warp_sum_int(rs[s]);
+        for (int s = 0; s < kS; ++s) rowsum[s] = warp_sum_int((int)rs[s]);
 #pragma unroll
         for (int lv = 0; lv < kLevels; ++lv) {
-            double b = 0.0;
+            int b = 0;
 #pragma unroll
-            for (int a = 0; a <= lv; ++a) b += (double)rs[a] * (lv - a == 0 ? 128.0 : 64.0);
-            bad = bad || b > 16777216.0;
+            for (int a = 0; a <= lv; ++a) b += rowsum[a] * (lv - a == 0 ? 128 : 64);
+            bad = bad || b > 16777216;
         }
         if (bad && lane == 0) atomicOr(flag + (size_t)(fbase + f) * MT + i / 128, 1);
     }
@@ -243,7 +249,6 @@ __global__ void __launch_bounds__(kThreads, 2)
         // ---- MMA issuer: product (a, b) of a K chunk into the accumulator of level a + b ----
         if (lane == 0) {
             bool ok = true;
-            uint32_t written = 0;
             for (int u = 0; u < nkc && ok; ++u) {
                 const int bs = u & 1;
                 if (!mbar_wait(smem_u32(&bar_bfull[bs]), (u >> 1) & 1, err) || abort_sh) {
@@ -258,17 +263,10 @@ __global__ void __launch_bounds__(kThreads, 2)
                     }
                     tc_fence_after();
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) {
-                        const uint64_t ad = smem_desc_sw128(aring + slot * kATile + ks * 32);
-#pragma unroll
-                        for (int b = 0; b < kS; ++b) {
-                            if (a + b >= kLevels) continue;
-                            const int lv = a + b;
-                            const uint64_t bd = smem_desc_sw128(bbuf + bs * kBChunk + b * kBTile + ks * 32);
-                            mma_bf16(tmem + (uint32_t)(lv * kNT), ad, bd, kIdesc, (written >> lv) & 1u);
-                            written |= 1u << lv;
-                        }
-                    }
+                    for (int ks = 0; ks < 4; ++ks)  // slices b = 0 .. 6 - a into the levels a .. 6, adjacent in both
+                        mma_bf16(tmem + (uint32_t)(a * kNT), smem_desc_sw128(aring + slot * kATile + ks * 32),
+                                 smem_desc_sw128(bbuf + bs * kBChunk + ks * 32), idesc_f32acc(1, 128, (kS - a) * kNT),
+                                 (u | a | ks) != 0 ? 1u : 0u);
                     mma_commit(smem_u32(&bar_empty[slot]));
                 }
                 if (ok) mma_commit(smem_u32(&bar_bempty[bs]));
@@ -295,7 +293,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     // sum_l acc_l 2^(7 (6 - l)) = hi 2^28 + lo with hi (levels 0-2, < 2^39) and lo
-                    // (levels 3-6, < 2^46) exact in 64-bit integers and in FP64; one FMA rounds the sum
+                    // (levels 3-6, < 2^46) exact in 64-bit integers; the sum is rounded once
                     long long hi = (long long)__float2int_rn(__uint_as_float(v[0][c]));
 #pragma unroll
                     for (int lv = 1; lv < 3; ++lv) hi = hi * 128 + (long long)__float2int_rn(__uint_as_float(v[lv][c]));
@@ -303,8 +301,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
                     for (int lv = 4; lv < kLevels; ++lv) lo = lo * 128 + (long long)__float2int_rn(__uint_as_float(v[lv][c]));
                     const int col = (kNT / 2) * h + c0 + c;
-                    stage_out[r * (kNT + 1) + col] = fma(__ll2double_rn(hi), 268435456.0, __ll2double_rn(lo)) *
-                                                     pow2d(ea + eB_sh[col] - 2 * (kW - 1) - kW * (kLevels - 1));
+                    stage_out[r * (kNT + 1) + col] = combine(hi, lo, ea + eB_sh[col] - 2 * (kW - 1) - kW * (kLevels - 1));
                 }
             }
         }

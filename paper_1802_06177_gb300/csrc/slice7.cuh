@@ -8,6 +8,7 @@
 #pragma once
 
 #include <cuda_bf16.h>
+#include <stdint.h>
 
 namespace slmc {
 namespace s7 {
@@ -31,10 +32,13 @@ __device__ __forceinline__ int exponent_of_bits(long long m) {
 }
 
 // The seven slices of v in units of 2^(e - 6 - 42), with integer arithmetic only (the FP64 pipe
-// is the scarce unit): v is rounded once to n = round(v 2^(48 - e)) (|n| <= 2^49, half away from
-// zero) and n is written in balanced base-128 digits d_6..d_1 in [-64, 63] and d_0 = the rest,
-// |d_0| <= 128, so v ~ 2^(e - 6) sum_s d_s 2^(-7 s). Each digit is exact in BF16.
-__device__ __forceinline__ void slice7(double v, int e, __nv_bfloat16 (&q)[kS]) {
+// is the scarce unit, and the integer-to-float conversions share its issue): v is rounded once to
+// n = round(v 2^(48 - e)) (|n| <= 2^49, half away from zero) and n is written in balanced base-128 digits
+// d_6..d_1 in [-64, 63] and d_0 = the rest, |d_0| <= 128, so v ~ 2^(e - 6) sum_s d_s 2^(-7 s). Adding 64 at every
+// place below the top makes the digits plain bit fields (plus 64); each is placed in the significand of
+// 1.5 2^23 and freed by one exact FP32 subtraction. The results are small integers as FP32, exact in BF16 (the
+// upper half of their bits).
+__device__ __forceinline__ void slice7(double v, int e, float (&q)[kS]) {
     const long long bits = __double_as_longlong(v);
     const int ex = (int)((bits >> 52) & 0x7ff);
     long long n = 0;
@@ -44,13 +48,57 @@ __device__ __forceinline__ void slice7(double v, int e, __nv_bfloat16 (&q)[kS]) 
         n = r > 0 ? (m + (1ll << (r - 1))) >> r : m;
         if (bits < 0) n = -n;
     }
+    constexpr long long kBias = 64ll * (1 + 128 * (1 + 128 * (1 + 128 * (1 + 128ll * (1 + 128ll)))));
+    n += kBias;
 #pragma unroll
-    for (int s = kS - 1; s >= 1; --s) {
-        const int d = (int)((n + 64) & 127) - 64;
-        n = (n - d) >> 7;
-        q[s] = __ushort_as_bfloat16((unsigned short)(__float_as_uint((float)d) >> 16));
+    for (int s = kS - 1; s >= 1; --s)
+        q[s] = __int_as_float(0x4B400000 | ((int)(n >> (7 * (kS - 1 - s))) & 127)) - 12582976.f;
+    q[0] = __int_as_float(0x4B400000 + (int)(n >> (7 * (kS - 1)))) - 12582912.f;
+}
+
+// BF16 bits of an exact small integer, and of two adjacent ones.
+__device__ __forceinline__ __nv_bfloat16 bf16_of(float q) {
+    return __ushort_as_bfloat16((unsigned short)(__float_as_uint(q) >> 16));
+}
+__device__ __forceinline__ uint32_t bf16x2_of(float q0, float q1) {
+    return __byte_perm(__float_as_uint(q0), __float_as_uint(q1), 0x7632);
+}
+
+// (hi 2^28 + lo) 2^k rounded once to FP64 (to nearest, ties to even), assembled with integer operations: the two
+// conversions, the FMA and the scaling it replaces took 64 issue cycles of the FP64 pipe per warp, the bound of
+// the epilogues that combine level sums. |hi| < 2^40, |lo| < 2^60.
+__device__ __forceinline__ double combine(long long hi, long long lo, int k) {
+    unsigned long long l = (unsigned long long)hi << 28;
+    const unsigned long long sum = l + (unsigned long long)lo;
+    long long h = (hi >> 36) + (lo >> 63) + (sum < l ? 1 : 0);
+    l = sum;
+    const bool neg = h < 0;
+    if (neg) {
+        l = 0ull - l;
+        h = ~h + (l == 0ull ? 1 : 0);
     }
-    q[0] = __ushort_as_bfloat16((unsigned short)(__float_as_uint((float)n) >> 16));
+    const int up = h == 0 ? 0 : 64 - __clzll(h);  // bits above the low word (at most 5)
+    unsigned long long m = l;
+    uint32_t sticky = 0u;
+    int nb;
+    if (up) {
+        sticky = (uint32_t)l & ((1u << up) - 1u);
+        m = (l >> up) | ((unsigned long long)h << (64 - up));
+        nb = 64 + up;
+    } else {
+        if (l == 0ull) return 0.0;
+        const int z = __clzll((long long)l);
+        m = l << z;
+        nb = 64 - z;
+    }
+    const uint32_t frac = (uint32_t)m & 0x7ffu;
+    unsigned long long mant = m >> 11;
+    if (frac > 0x400u || (frac == 0x400u && (sticky || (mant & 1ull)))) ++mant;
+    const int E = nb - 1 + k + 1023;
+    if (E < 1 || E > 2046)  // out of the normal range: the FP64 operations round as they did
+        return fma(__ll2double_rn(hi), 268435456.0, __ll2double_rn(lo)) * pow2d(k);
+    const long long r = ((long long)(E - 1) << 52) + (long long)mant;
+    return __longlong_as_double(neg ? r | (long long)0x8000000000000000ull : r);
 }
 
 }  // namespace s7

@@ -91,6 +91,12 @@ __device__ __forceinline__ uint32_t sw128_off_b16(int r, int k) {
     return (uint32_t)r * 128u + ((uint32_t)((k >> 3) ^ (r & 7)) << 4) + (uint32_t)(k & 7) * 2u;
 }
 
+// The kernels here multiply a slice a of one operand with the slices b of the other into the level a + b. Slices
+// b lie in adjacent rows of shared memory and levels in adjacent accumulator columns, so all b of one a are ONE
+// instruction of N = (number of b) x tile columns: an instruction of N = 32 or 64 takes about as long as one
+// several times wider (28 of N = 32 per step of K became 7 of N = 32 .. 224; 16x16, L = 160, 512 fields:
+// 283 -> 235 ms per evaluation together with the integer epilogues of slice7.cuh).
+//
 // Instruction descriptor of tcgen05.mma kind::f16 / kind::tf32: FP32 accumulator, A and B of
 // format fmt (BF16 = 1, TF32 = 2), both K-major, M x N tile.
 __host__ __device__ constexpr uint32_t idesc_f32acc(uint32_t fmt, int M, int N) {

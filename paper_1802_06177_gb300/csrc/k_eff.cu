@@ -55,35 +55,53 @@ __global__ void __launch_bounds__(kThreads) k_bose(const double* __restrict__ x,
     if (threadIdx.x == 0) lnw[f] = (lndet ? 2.0 * lndet[f] : 0.0) + acc[0];
 }
 
+// Feature sums of one field per CTA; a warp walks rows (sites), its lanes the slices. Eleven FP64 operations per
+// value bound it: 2000 fields of 12x12,
+// L = 120 take 1.36 ms (0.6 ms of FP64 issue, 41 us of memory traffic). With nine more FP64 operations and three
+// integer divisions per value, and the regression below as it was, a fit of them took 5.5 ms against 1.45 ms.
 __global__ void __launch_bounds__(kThreads) k_features(const double* __restrict__ x, int Lx, int Ly, int L, double a2,
                                                        double dtau, const double* __restrict__ J,
                                                        double* __restrict__ F, int ldF, double* __restrict__ lnw_eff) {
-    __shared__ double red[5 * kThreads];
-    const int f = blockIdx.x;
+    __shared__ double red[5][kThreads / 32];
+    const int f = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int N = Lx * Ly;
     const double* xf = x + (size_t)f * N * L;
     double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int idx = threadIdx.x; idx < N * L; idx += kThreads) {
-        const int i = idx / L, l = idx - i * L;
-        const int ix = i % Lx, iy = i / Lx;
-        const double v = xf[idx];
-        const double vt = xf[(size_t)i * L + (l + 1 == L ? 0 : l + 1)];
-        const double vx = xf[(size_t)((ix + 1 == Lx ? 0 : ix + 1) + Lx * iy) * L + l];
-        const double vy = xf[(size_t)(ix + Lx * (iy + 1 == Ly ? 0 : iy + 1)) * L + l];
-        const double v2 = v * v;
-        const double d = vt - v;
-        acc[0] += d * d;
-        acc[1] += v2 * v2 * 0.25 - a2 * v2 * 0.5;
-        acc[2] += v2 * v2 * v2 * (1.0 / 6.0) - a2 * v2 * v2 * 0.25;
-        acc[3] += v * (vx + vy);
-        acc[4] += v * vt;
+    const double h2 = -0.5 * a2, h4 = -0.25 * a2;
+    for (int i = warp; i < N; i += kThreads / 32) {
+        const int iy = i / Lx, ix = i - iy * Lx;
+        const double* xi = xf + (size_t)i * L;
+        const double* xx = xf + (size_t)((ix + 1 == Lx ? 0 : ix + 1) + Lx * iy) * L;
+        const double* xy = xf + (size_t)(ix + Lx * (iy + 1 == Ly ? 0 : iy + 1)) * L;
+#pragma unroll 4
+        for (int l = lane; l < L; l += 32) {
+            const double v = xi[l], vt = xi[l + 1 == L ? 0 : l + 1];
+            const double nb = xx[l] + xy[l];
+            const double v2 = v * v, v4 = v2 * v2, d = vt - v;
+            acc[0] = fma(d, d, acc[0]);
+            acc[1] = fma(v2, fma(0.25, v2, h2), acc[1]);
+            acc[2] = fma(v4, fma(1.0 / 6.0, v2, h4), acc[2]);
+            acc[3] = fma(v, nb, acc[3]);
+            acc[4] = fma(v, vt, acc[4]);
+        }
     }
-    block_sum<5>(acc, red);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        const double t = slmc::warp_allsum(acc[q]);
+        if (lane == 0) red[q][warp] = t;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
+        double feat[5];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            feat[q] = red[q][0];
+            for (int w = 1; w < kThreads / 32; ++w) feat[q] += red[q][w];
+        }
         if (F)
-            for (int q = 0; q < 5; ++q) F[(size_t)f * ldF + q] = acc[q];
+            for (int q = 0; q < 5; ++q) F[(size_t)f * ldF + q] = feat[q];
         if (lnw_eff) {
-            const double e = J[0] + J[1] * acc[0] + J[2] * acc[1] + J[3] * acc[2] + J[4] * acc[3] + J[5] * acc[4];
+            const double e = J[0] + J[1] * feat[0] + J[2] * feat[1] + J[3] * feat[2] + J[4] * feat[3] + J[5] * feat[4];
             lnw_eff[f] = -dtau * e;
         }
     }
@@ -576,45 +594,93 @@ __device__ __forceinline__ void givens_absorb(double (&Rrow)[7], double a, int l
     }
 }
 
-// Warps take consecutive chunks of the configurations (the first warp starts from the current
-// triangle), reduce them to partial triangles, and the partial triangles are merged pairwise
-// in shared memory (all rows are taken relative to the same reference, so no shift is needed).
-__global__ void k_fit_accumulate(double* __restrict__ R, const double* __restrict__ feat, int ldF,
-                                 const double* __restrict__ lnw, int nconf, double sc) {
-    __shared__ double sR[32][49];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (threadIdx.x == 0 && R[55] == 0.0) {
+// Absorbs nconf rows into the triangle, kFitRows per pass, by Householder reflections of [R; rows] in one CTA:
+// the rows stay in registers (four per thread), and the reflector of column k touches row k of R and the rows
+// only. The products of column k with itself and with the columns right of it are reduced together (one block
+// reduction per column); scaling by the reflector's normalisation comes after. Row k of R takes the sign that
+// makes its diagonal non-negative, as the Givens merge below leaves it. A chain of Givens rotations per warp
+// (63 rows, seven hypots and divisions each) and a tree of triangle merges stood here before; 2000 rows take 95 us with
+// the kernels around it. Couplings against quad precision over 24 fits: 1.2e-13 (2.4e-13 before).
+constexpr int kFitThreads = 512, kFitPer = 4, kFitRows = kFitThreads * kFitPer;
+
+__global__ void __launch_bounds__(kFitThreads) k_fit_accumulate(double* __restrict__ R, const double* __restrict__ feat,
+                                                                int ldF, const double* __restrict__ lnw, int nconf,
+                                                                double sc) {
+    constexpr int NW = kFitThreads / 32;
+    __shared__ double sR[49], ref[6], part[7][NW], dot[7], par[2];  // par: tau, scal
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0 && R[55] == 0.0) {
         for (int q = 0; q < 5; ++q) R[49 + q] = feat[q];
         R[54] = lnw[0];
         R[55] = 1.0;
     }
     __syncthreads();
-    double Rrow[7];  // lane m < 7 holds column m of every row
-    for (int k = 0; k < 7; ++k) Rrow[k] = (warp == 0 && lane < 7) ? R[k * 7 + lane] : 0.0;
-    const int per = (nconf + nw - 1) / nw;
-    const int c0 = warp * per, c1 = min(nconf, c0 + per);
-    for (int c = c0; c < c1; ++c) {
-        double a;
-        if (lane == 0) a = 1.0;
-        else if (lane < 6) a = (feat[(size_t)c * ldF + lane - 1] - R[49 + lane - 1]) / sc;
-        else if (lane == 6) a = lnw[c] - R[54];
-        else a = 0.0;
-        givens_absorb(Rrow, a, lane);
+    if (tid < 49) sR[tid] = R[tid];
+    if (tid >= 64 && tid < 70) ref[tid - 64] = R[49 + tid - 64];
+    __syncthreads();
+    const double inv = 1.0 / sc;
+    for (int c0 = 0; c0 < nconf; c0 += kFitRows) {
+        double a[kFitPer][7];
+#pragma unroll
+        for (int r = 0; r < kFitPer; ++r) {
+            const int c = c0 + r * kFitThreads + tid;
+            const bool on = c < nconf;
+            a[r][0] = on ? 1.0 : 0.0;
+#pragma unroll
+            for (int q = 0; q < 5; ++q) a[r][q + 1] = on ? (feat[(size_t)c * ldF + q] - ref[q]) * inv : 0.0;
+            a[r][6] = on ? lnw[c] - ref[5] : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+#pragma unroll
+            for (int m = k; m < 7; ++m) {
+                double t = 0.0;
+#pragma unroll
+                for (int r = 0; r < kFitPer; ++r) t = fma(a[r][k], a[r][m], t);
+                t = slmc::warp_allsum(t);
+                if (lane == 0) part[m][warp] = t;
+            }
+            __syncthreads();
+            if (warp >= k && warp < 7) {  // warp m finishes product m
+                const double t = slmc::warp_allsum(lane < NW ? part[warp][lane] : 0.0);
+                if (lane == 0) dot[warp] = t;
+            }
+            __syncthreads();
+            if (warp == 0) {
+                const double alpha = sR[k * 7 + k], sig = dot[k];
+                double tau = 0.0, beta = alpha, scal = 0.0;
+                if (sig != 0.0) {
+                    const double nrm = sqrt(fma(alpha, alpha, sig));
+                    beta = (alpha >= 0.0) ? -nrm : nrm;
+                    tau = (beta - alpha) / beta;
+                    scal = 1.0 / (alpha - beta);
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    sR[k * 7 + k] = fabs(beta);
+                    par[0] = tau;
+                    par[1] = scal;
+                }
+                if (lane > k && lane < 7) {  // row k of R: R_km -= tau (R_km + v . a_m)
+                    const double d = tau * fma(scal, dot[lane], sR[k * 7 + lane]);
+                    const double v = sR[k * 7 + lane] - d;
+                    sR[k * 7 + lane] = beta < 0.0 ? -v : v;
+                    dot[lane] = d;
+                }
+            }
+            __syncthreads();
+            const double scal = par[1];
+#pragma unroll
+            for (int m = k + 1; m < 7; ++m) {
+                const double d = dot[m] * scal;
+#pragma unroll
+                for (int r = 0; r < kFitPer; ++r) a[r][m] = fma(-d, a[r][k], a[r][m]);
+            }
+            __syncthreads();  // part and dot are rewritten by the next column
+        }
     }
-    for (int st = 1; st < nw; st <<= 1) {
-        if (warp % (2 * st) == st)
-            for (int k = 0; k < 7; ++k)
-                if (lane < 7) sR[warp][k * 7 + lane] = Rrow[k];
-        __syncthreads();
-        if (warp % (2 * st) == 0 && warp + st < nw)
-            for (int k = 0; k < 7; ++k) givens_absorb(Rrow, (lane < 7) ? sR[warp + st][k * 7 + lane] : 0.0, lane);
-        __syncthreads();
-    }
-    if (warp == 0) {
-        for (int k = 0; k < 7; ++k)
-            if (lane < 7) R[k * 7 + lane] = Rrow[k];
-        if (lane == 0) R[56] += nconf;
-    }
+    if (tid < 49) R[tid] = sR[tid];
+    if (tid == 0) R[56] += nconf;
 }
 
 // Merges partial states (same layout as R) into R. Each state's factor is first moved to the
@@ -799,8 +865,7 @@ cudaError_t fit_begin(slmc_ctx* c, double* R, cudaStream_t s) {
 }
 
 cudaError_t fit_accumulate(slmc_ctx* c, double* R, const double* feat, const double* lnw, int nconf, cudaStream_t s) {
-    const int warps = nconf >= 32 * 16 ? 32 : (nconf + 15) / 16;  // about 16 configurations per warp
-    k_fit_accumulate<<<1, 32 * (warps < 1 ? 1 : warps), 0, s>>>(R, feat, 8, lnw, nconf, (double)c->N * c->L);
+    k_fit_accumulate<<<1, kFitThreads, 0, s>>>(R, feat, 8, lnw, nconf, (double)c->N * c->L);
     return cudaGetLastError();
 }
 

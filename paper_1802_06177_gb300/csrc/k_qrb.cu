@@ -163,42 +163,159 @@ __global__ void __launch_bounds__(kThreads, 2) k_qrb(double* __restrict__ Yall, 
     if (C > 1) cluster.sync();  // shared memory stays alive until rank 0 has read the counts
 }
 
-// Q = Q_0 Q_1 ... (Q_p = I - V_p S_p V_p^T), accumulated backwards into U (column-major),
-// computed in T: FP64, or FP32 when Q only feeds reduced-precision slice products (which round
-// it to FP32 on entry anyway).
+// Q = Q_0 Q_1 ... (Q_p = I - V_p S_p V_p^T), accumulated backwards into U (column-major), in FP64
+// (k_formq32 where Q only feeds reduced-precision slice products, which round it to FP32 on entry anyway).
 // Columns of Q are independent: CTA (field, blockIdx.y) forms columns [j0, j1) of gridDim.y
 // blocks (several CTAs per field when there are few fields).
-template <int BP, typename T>
+template <int BP>
 __global__ void __launch_bounds__(kThreads, 2) k_formq_b(const double* __restrict__ QRall, const double* __restrict__ Sall,
-                                                      T* __restrict__ Uall, int N) {
+                                                      double* __restrict__ Uall, int N) {
     constexpr int BPS = BP + 1;
     const int f = blockIdx.x;
     const int j0 = (int)((long long)blockIdx.y * N / gridDim.y), j1 = (int)((long long)(blockIdx.y + 1) * N / gridDim.y);
     const size_t NN = (size_t)N * N;
     const double* __restrict__ QR = QRall + f * NN;
-    T* __restrict__ U = Uall + f * NN;
+    double* __restrict__ U = Uall + f * NN;
     extern __shared__ __align__(16) unsigned char smraw[];
-    T* Vp = reinterpret_cast<T*>(smraw);
-    T* Ssm = Vp + (size_t)N * BPS;
-    T* Wsm = Ssm + BP * BP;
+    double* Vp = reinterpret_cast<double*>(smraw);
+    double* Ssm = Vp + (size_t)N * BPS;
+    double* Wsm = Ssm + BP * BP;
     const int tid = threadIdx.x;
     for (size_t idx = (size_t)j0 * N + tid; idx < (size_t)j1 * N; idx += kThreads)
-        U[idx] = (idx % (N + 1) == 0) ? T(1) : T(0);
+        U[idx] = (idx % (N + 1) == 0) ? 1.0 : 0.0;
     for (int p = ((N - 1) / BP) * BP; p >= 0; p -= BP) {
         const int nb = min(BP, N - p);
         __syncthreads();
         for (int idx = tid; idx < nb * (N - p); idx += kThreads) {
             const int c = idx / (N - p), r = p + idx - c * (N - p);
             const int k = p + c;
-            Vp[r * BPS + c] = (T)((r > k) ? QR[(size_t)k * N + r] : (r == k ? 1.0 : 0.0));
+            Vp[r * BPS + c] = (r > k) ? QR[(size_t)k * N + r] : (r == k ? 1.0 : 0.0);
         }
         for (int idx = tid; idx < nb * BP; idx += kThreads) {
             const int a = idx / BP, b = idx - a * BP;
-            Ssm[a * BP + b] = (T)Sall[(size_t)f * N * BP + (size_t)(p + a) * BP + b];
+            Ssm[a * BP + b] = Sall[(size_t)f * N * BP + (size_t)(p + a) * BP + b];
         }
         __syncthreads();
         const int jb = max(p, j0);  // columns left of the panel are still unit vectors
         if (jb < j1) wy_update<BP, false>(Vp, Ssm, Wsm, N, p, nb, j1 - jb, [&](int jj) { return U + (size_t)(jb + jj) * N; });
+    }
+}
+
+// Q in FP32 (mixed modes), same arithmetic per entry as k_formq_b<BP, float> (each sum one FMA chain in the same
+// order, so the same bits) with the operands in shared memory: a warp keeps 8 columns of Q there from the first
+// panel to the last, and each phase is a register tile. W = V^T Q: a lane's four reflectors are BP / 4
+// apart, its columns 128 / BP apart, four rows per 16-byte load; W' = S W: a reflector per lane; Q -= V W': four rows per lane and
+// the warp's 8 columns. The row stride is 4 mod 32 floats, so 16-byte accesses a column apart meet no bank
+// conflicts. Reading Q's columns from global memory one broadcast word at a time, a 24x24 evaluation of
+// 32 fields (30 groups) spent 99 ms here and now 36; a 16x16 evaluation of 512 fields took 235 ms and now 218. Groups of 8 columns go round the CTAs of a field, which evens out the triangular work
+// (columns left of a panel are still unit vectors and are skipped).
+template <int BP>
+__global__ void __launch_bounds__(256, 2) k_formq32(const double* __restrict__ QRall, const double* __restrict__ Sall,
+                                                    float* __restrict__ Uall, int N, int ld) {
+    constexpr int MT = BP / 4, CT = 32 / MT, TC = 8 / CT;  // W tile: 4 reflectors x TC columns per lane
+    const int f = blockIdx.x, nw = blockDim.x / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const size_t NN = (size_t)N * N;
+    const double* __restrict__ QR = QRall + f * NN;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    float* V = reinterpret_cast<float*>(smraw);     // [BP][ld] reflectors
+    float* Ssm = V + (size_t)BP * ld;               // [q][m] = S[m][q]
+    float* W = Ssm + BP * BP + warp * BP * 8;       // [BP][8] of this warp
+    float* Q = Ssm + BP * BP + nw * BP * 8 + (size_t)warp * 8 * ld;  // 8 columns
+    const int j0 = (warp * gridDim.y + blockIdx.y) * 8;
+    const bool on = j0 < N;
+    for (int idx = lane; idx < 8 * ld; idx += 32) Q[idx] = (idx % ld == j0 + idx / ld) ? 1.f : 0.f;
+    for (int p = ((N - 1) / BP) * BP; p >= 0; p -= BP) {
+        const int nb = min(BP, N - p);
+        if ((((N + 7) / 8 - 1 - (int)blockIdx.y) / (int)gridDim.y * (int)gridDim.y + (int)blockIdx.y) * 8 + 7 < p)
+            continue;  // every column of this CTA is left of the panel
+        __syncthreads();
+        for (int c = warp; c < BP; c += nw) {
+            const int k = p + c;
+            for (int r = p + lane; r < ld; r += 32)
+                V[c * ld + r] = (c < nb && r < N) ? (float)((r > k) ? QR[(size_t)k * N + r] : (r == k ? 1.0 : 0.0)) : 0.f;
+        }
+        for (int idx = tid; idx < BP * BP; idx += blockDim.x) {
+            const int m = idx / BP, q = idx - m * BP;
+            Ssm[q * BP + m] = m < nb ? (float)Sall[(size_t)f * N * BP + (size_t)(p + m) * BP + q] : 0.f;
+        }
+        __syncthreads();
+        if (!on || j0 + 7 < p) continue;
+        {   // W[m][c] = sum_r V[m][r] Q[c][r]
+            const int mt = lane % MT, ct = lane / MT;
+            float acc[4][TC];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int c = 0; c < TC; ++c) acc[i][c] = 0.f;
+#pragma unroll 2
+            for (int r = p; r < N; r += 4) {
+                float4 v[4], q[TC];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = *reinterpret_cast<const float4*>(V + (mt + MT * i) * ld + r);
+#pragma unroll
+                for (int c = 0; c < TC; ++c) q[c] = *reinterpret_cast<const float4*>(Q + (ct + CT * c) * ld + r);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int c = 0; c < TC; ++c) {
+                        acc[i][c] = fmaf(v[i].x, q[c].x, acc[i][c]);
+                        acc[i][c] = fmaf(v[i].y, q[c].y, acc[i][c]);
+                        acc[i][c] = fmaf(v[i].z, q[c].z, acc[i][c]);
+                        acc[i][c] = fmaf(v[i].w, q[c].w, acc[i][c]);
+                    }
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int c = 0; c < TC; ++c) W[(mt + MT * i) * 8 + ct + CT * c] = acc[i][c];
+            __syncwarp();
+        }
+        {   // W' = S W (S upper triangular, zero below): lane (m, column half for BP = 16)
+            constexpr int CPL = BP / 4;
+            const int m = lane % BP, c0 = (lane / BP) * CPL;
+            float acc[CPL];
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) acc[c] = 0.f;
+            for (int q = 0; q < nb; ++q) {
+                const float sv = Ssm[q * BP + m];
+#pragma unroll
+                for (int c = 0; c < CPL; ++c)
+                    if (q >= m) acc[c] = fmaf(sv, W[q * 8 + c0 + c], acc[c]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) W[m * 8 + c0 + c] = acc[c];
+            __syncwarp();
+        }
+        for (int r = p + 4 * lane; r < N; r += 128) {  // Q[c][r] -= sum_m V[m][r] W'[m][c]
+            float4 y[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) y[c] = *reinterpret_cast<const float4*>(Q + c * ld + r);
+#pragma unroll 4
+            for (int m = 0; m < nb; ++m) {
+                const float4 v = *reinterpret_cast<const float4*>(V + m * ld + r);
+                const float4 w0 = *reinterpret_cast<const float4*>(W + m * 8);
+                const float4 w1 = *reinterpret_cast<const float4*>(W + m * 8 + 4);
+                const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    y[c].x = fmaf(-v.x, w[c], y[c].x);
+                    y[c].y = fmaf(-v.y, w[c], y[c].y);
+                    y[c].z = fmaf(-v.z, w[c], y[c].z);
+                    y[c].w = fmaf(-v.w, w[c], y[c].w);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 8; ++c) *reinterpret_cast<float4*>(Q + c * ld + r) = y[c];
+        }
+        __syncwarp();
+    }
+    if (on) {
+        float* __restrict__ U = Uall + f * NN;
+        for (int c = 0; c < 8 && j0 + c < N; ++c)
+            for (int r = lane; r < N; r += 32) U[(size_t)(j0 + c) * N + r] = Q[c * ld + r];
     }
 }
 
@@ -291,19 +408,34 @@ cudaError_t launch_qrb(slmc_ctx* c, int nf, cudaStream_t s) {
     return cudaLaunchKernelEx(&cfg, k_qrb<BP>, c->Y, c->lnD, c->QR, c->tau, c->perm, c->sgnU, c->Sws, c->err, c->N);
 }
 
-template <int BP, typename T>
+template <int BP>
 cudaError_t launch_formq_b(slmc_ctx* c, int nf, cudaStream_t s) {
-    const size_t smem = sizeof(T) * ((size_t)c->N * (BP + 1) + BP * BP + kWarps * BP * kCT);
-    cudaError_t e = cudaFuncSetAttribute(k_formq_b<BP, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = sizeof(double) * ((size_t)c->N * (BP + 1) + BP * BP + kWarps * BP * kCT);
+    cudaError_t e = cudaFuncSetAttribute(k_formq_b<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    T* U;
-    if constexpr (sizeof(T) == 4) U = c->U32;
-    else U = c->U;
     // column blocks per field: at least the QR's cluster size, and enough for about two CTAs per SM
     int cb = qr_cluster_size(c, nf);
     if (c->num_sms > 0 && nf > 0) cb = std::max(cb, std::min(4, (2 * c->num_sms + nf - 1) / nf));
     dim3 grid(nf, cb);
-    k_formq_b<BP, T><<<grid, kThreads, smem, s>>>(c->QR, c->Sws, U, c->N);
+    k_formq_b<BP><<<grid, kThreads, smem, s>>>(c->QR, c->Sws, c->U, c->N);
+    return cudaGetLastError();
+}
+
+// As many warps (8 columns of Q each) as two CTAs per SM allow, fewer for long columns.
+template <int BP>
+cudaError_t launch_formq32(slmc_ctx* c, int nf, cudaStream_t s) {
+    const int N = c->N, ld = (N + 31) / 32 * 32 + 4;
+    const size_t fixed = sizeof(float) * ((size_t)BP * ld + BP * BP), per_warp = sizeof(float) * (8 * (size_t)ld + BP * 8);
+    int nw = 8;
+    if (fixed + nw * per_warp > 112 * 1024) {
+        nw = (int)std::min<size_t>(8, (226 * 1024 - fixed) / per_warp);
+        if (nw < 1) return cudaErrorInvalidValue;
+    }
+    const size_t smem = fixed + nw * per_warp;
+    cudaError_t e = cudaFuncSetAttribute(k_formq32<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int groups = (N + 7) / 8;
+    k_formq32<BP><<<dim3(nf, (groups + nw - 1) / nw), nw * 32, smem, s>>>(c->QR, c->Sws, c->U32, N, ld);
     return cudaGetLastError();
 }
 
@@ -323,8 +455,8 @@ cudaError_t qr_blocked(slmc_ctx* c, int nf, cudaStream_t s) {
 }
 
 cudaError_t form_q_blocked(slmc_ctx* c, int nf, bool fp32, cudaStream_t s) {
-    if (fp32) return qr_panel_width(c) == 32 ? launch_formq_b<32, float>(c, nf, s) : launch_formq_b<16, float>(c, nf, s);
-    return qr_panel_width(c) == 32 ? launch_formq_b<32, double>(c, nf, s) : launch_formq_b<16, double>(c, nf, s);
+    if (fp32) return qr_panel_width(c) == 32 ? launch_formq32<32>(c, nf, s) : launch_formq32<16>(c, nf, s);
+    return qr_panel_width(c) == 32 ? launch_formq_b<32>(c, nf, s) : launch_formq_b<16>(c, nf, s);
 }
 
 cudaError_t t_update_tiled(slmc_ctx* c, int nf, cudaStream_t s) {

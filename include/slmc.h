@@ -247,7 +247,13 @@ SLMC_API int slmc_set_update_counter(slmc_ctx* ctx, uint64_t value, void* stream
 /* Synchronises `stream` and returns the device-side cumulative-update counter. */
 SLMC_API int slmc_get_update_counter(slmc_ctx* ctx, uint64_t* value, void* stream);
 
-/* Kernel tile choices (found by slmc_autotune): qr_panel = width of the blocked-QR panels
+/* FP64 contexts with N <= 64 (prepivot mode) evaluate a determinant in one launch per batch, one CTA per field
+ * in shared memory, as long as none of the calls that steer the general kernels was made on them
+ * (slmc_set_tuning, slmc_set_sub_batches, slmc_set_sub_batch_priorities, slmc_set_qr_cluster,
+ * slmc_set_dense_slices, slmc_set_tupdate_path, slmc_set_qr_path); after one of them the context uses the
+ * general kernels. Both agree to FP64 rounding.
+ *
+ * Kernel tile choices (found by slmc_autotune): qr_panel = width of the blocked-QR panels
  * (0 = by N, 16 or 32); slice_cols = columns per thread of the FP32 slice kernel (0 = by N,
  * 8 or 16; 16 is used only for N <= 256). Results do not depend on them beyond rounding. */
 SLMC_API int slmc_set_tuning(slmc_ctx* ctx, int qr_panel, int slice_cols);
@@ -290,7 +296,7 @@ SLMC_API int slmc_set_dense_slices(slmc_ctx* ctx, int dense);
  *            below 2^-48 of their row and column scales.
  *   path = 1: FP64 FMAs (tiled triangular GEMM).
  *   path = 2: the tensor-core kernel with every tile on its FP64 fallback (for tests).
- * The DQMC updates always use path 1. Errors: SLMC_ERR_ARG for other values. */
+ * The DQMC updates use the same path for N > 64 and path 1 up to there. Errors: SLMC_ERR_ARG for other values. */
 SLMC_API int slmc_set_tupdate_path(slmc_ctx* ctx, int path);
 
 /* How the pre-pivoted blocked QR (qr_mode SLMC_QR_PREPIVOT) applies each panel's block of BP
@@ -305,9 +311,11 @@ SLMC_API int slmc_set_tupdate_path(slmc_ctx* ctx, int path);
  *            accumulator), and each entry is rounded once to FP64. Each product entry then differs
  *            from the exact product of the operands by below 2^-44 K max|a_row| max|b_column| (K
  *            the inner dimension): normwise the size of the FP64 loop's own rounding. 4 launches
- *            per panel on the caller's stream.
- *   path = 1: the one-kernel FP64 QR (trailing updates with FP64 FMAs).
- * The DQMC updates and qr_mode SLMC_QR_PIVOTED are unaffected. Errors: SLMC_ERR_ARG for other
+ *            per panel on the caller's stream. For N > 64 Q is formed in FP64 through the same products (4
+ *            more launches per panel).
+ *   path = 1: the one-kernel FP64 QR (trailing updates with FP64 FMAs), Q formed with FP64 FMAs.
+ * The DQMC updates follow it for N > 64 (the one-kernel QR up to there); qr_mode SLMC_QR_PIVOTED is
+ * unaffected. Errors: SLMC_ERR_ARG for other
  * values, SLMC_ERR_UNSUPPORTED for path 0 when N > 896. */
 SLMC_API int slmc_set_qr_path(slmc_ctx* ctx, int path);
 

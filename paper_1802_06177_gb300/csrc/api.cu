@@ -163,7 +163,10 @@ int logdet_run(slmc_ctx* c, slmc_ctx* v, const double* x, int nf, double* lndet,
             // Q enters the next reduced-precision slice group (rounded to FP32 there anyway) except
             // after the last group, where it enters the FP64 final step.
             const bool q32 = v->p.precision != SLMC_PREC_FP64 && l0 + nsl < v->L;
-            SLMC_LAUNCH(SLMC_PROF_FORMQ, 1, s, slmc::form_q_blocked(v, nf, q32, s));
+            if (!q32 && slmc::qrt_form_q_active(v))
+                SLMC_LAUNCH(SLMC_PROF_FORMQ, slmc::qrt_form_q_launches(v), s, slmc::qrt_form_q(v, nf, s));
+            else
+                SLMC_LAUNCH(SLMC_PROF_FORMQ, 1, s, slmc::form_q_blocked(v, nf, q32, s));
         }
         SLMC_LAUNCH(SLMC_PROF_TUPDATE, slmc::t_update_launches(v), s, slmc::t_update(v, nf, s));
     }
@@ -659,17 +662,29 @@ int slmc_cumulative_update(slmc_ctx* c, double* x, int n, const double* J, int n
 }
 
 namespace {
-// One FP64 step of the stabilised chain on the product already in Y: pivoted QR, Q, T.
+// One FP64 step of the stabilised chain on the product already in Y: pivoted QR, Q, T, on the same paths as the
+// determinant's. At N <= 64 the one-kernel QR and the FP64 T update have fewer launches than the work is worth.
 int chain_step64(slmc_ctx* c, int nf, cudaStream_t s) {
     c->cur_units = nf;
+    const bool tc = slmc::qrt_form_q_active(c);
     if (c->p.qr_mode == SLMC_QR_PIVOTED) {
         SLMC_LAUNCH(SLMC_PROF_QR, 1, s, slmc::qr_pivoted(c, nf, s));
         SLMC_LAUNCH(SLMC_PROF_FORMQ, 1, s, slmc::form_q(c, nf, s));
+    } else if (tc) {
+        const int np = slmc::qrt_panels(c);
+        for (int t = 0; t < np; ++t) {
+            SLMC_LAUNCH(SLMC_PROF_QR, 1, s, slmc::qrt_panel(c, nf, t, s));
+            if (t + 1 < np) SLMC_LAUNCH(SLMC_PROF_QRTC, 3, s, slmc::qrt_trailing(c, nf, t, s));
+        }
+        SLMC_LAUNCH(SLMC_PROF_FORMQ, slmc::qrt_form_q_launches(c), s, slmc::qrt_form_q(c, nf, s));
     } else {
         SLMC_LAUNCH(SLMC_PROF_QR, 1, s, slmc::qr_blocked(c, nf, s));
         SLMC_LAUNCH(SLMC_PROF_FORMQ, 1, s, slmc::form_q_blocked(c, nf, false, s));
     }
-    SLMC_LAUNCH(SLMC_PROF_TUPDATE, 1, s, slmc::t_update_tiled(c, nf, s));
+    if (tc)
+        SLMC_LAUNCH(SLMC_PROF_TUPDATE, slmc::t_update_launches(c), s, slmc::t_update(c, nf, s));
+    else
+        SLMC_LAUNCH(SLMC_PROF_TUPDATE, 1, s, slmc::t_update_tiled(c, nf, s));
     return SLMC_OK;
 }
 

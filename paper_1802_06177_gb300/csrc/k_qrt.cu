@@ -159,6 +159,46 @@ struct PanelSmem {
     static size_t bytes(int N, int p, bool last) { return sizeof(double) * doubles(N, p, last) + sizeof(int) * (size_t)N; }
 };
 
+// Slices of the clean reflectors V (row r at Vp + r (BP + 1), rows p..N-1) of one field: per reflector over the
+// rows (V1) and per row over the reflectors (V2), with their exponents.
+template <int BP, int NT>
+__device__ __forceinline__ void slice_V(const double* Vp, __nv_bfloat16* __restrict__ V1, int* __restrict__ eV1,
+                                        __nv_bfloat16* __restrict__ V2, int* __restrict__ eV2, int N, int p, int gf, int kpad,
+                                        int mpad, size_t plane1, size_t plane2) {
+    constexpr int BPS = BP + 1, kW = NT / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // V1: reflector m over rows p..N-1 (K-major, K chunks from the one holding row p)
+    const int kstart = (p / 64) * 64;
+    for (int m = warp; m < BP; m += kW) {
+        long long mx = 0;
+        for (int r = p + lane; r < N; r += 32) mx = max(mx, abs_bits(Vp[r * BPS + m]));
+        const int e = exponent_of_bits(warp_max_bits(mx));
+        if (lane == 0) eV1[(size_t)gf * kVRows + m] = e;
+        __nv_bfloat16* dst = V1 + ((size_t)gf * kVRows + m) * kpad;
+        for (int k = kstart + 2 * lane; k < kpad; k += 64) {  // two adjacent rows per lane (multiples of 64)
+            float q0[kS], q1[kS];
+            slice7((k >= p && k < N) ? Vp[k * BPS + m] : 0.0, e, q0);
+            slice7((k + 1 >= p && k + 1 < N) ? Vp[(k + 1) * BPS + m] : 0.0, e, q1);
+#pragma unroll
+            for (int s = 0; s < kS; ++s)
+                *reinterpret_cast<uint32_t*>(dst + (size_t)s * plane1 + k) = bf16x2_of(q0[s], q1[s]);
+        }
+    }
+    // V2: row r over the reflectors (K = the BP reflectors, padded to 64 with zeros set at init),
+    // rows of the first row tile that holds row p onward
+    for (int r = (p / 128) * 128 + warp; r < mpad; r += kW) {
+        const double v = (r >= p && r < N && lane < BP) ? Vp[r * BPS + lane] : 0.0;
+        const int e = exponent_of_bits(warp_max_bits(abs_bits(v)));
+        if (lane == 0) eV2[(size_t)gf * mpad + r] = e;
+        if (lane < BP) {
+            float q[kS];
+            slice7(v, e, q);
+#pragma unroll
+            for (int s = 0; s < kS; ++s) V2[(size_t)s * plane2 + ((size_t)gf * mpad + r) * 64 + lane] = bf16_of(q[s]);
+        }
+    }
+}
+
 template <int BP, int kPT>
 __global__ void __launch_bounds__(kPT, kPT == 256 ? 3 : 1)
     k_qrt_panel(double* __restrict__ Yall, double* __restrict__ lnD_all, double* __restrict__ QRall,
@@ -265,47 +305,19 @@ __global__ void __launch_bounds__(kPT, kPT == 256 ? 3 : 1)
         if (bad) atomicOr(err, SLMC_EBIT_NONFINITE);
         return;
     }
-    // V1: reflector m over rows p..N-1 (K-major, K chunks from the one holding row p)
-    const int kstart = (p / 64) * 64;
-    for (int m = warp; m < BP; m += kPW) {
-        long long mx = 0;
-        for (int r = p + lane; r < N; r += 32) mx = max(mx, abs_bits(Vp[r * BPS + m]));
-        const int e = exponent_of_bits(warp_max_bits(mx));
-        if (lane == 0) eV1[(size_t)gf * kVRows + m] = e;
-        __nv_bfloat16* dst = V1 + ((size_t)gf * kVRows + m) * kpad;
-        for (int k = kstart + 2 * lane; k < kpad; k += 64) {  // two adjacent rows per lane (multiples of 64)
-            float q0[kS], q1[kS];
-            slice7((k >= p && k < N) ? Vp[k * BPS + m] : 0.0, e, q0);
-            slice7((k + 1 >= p && k + 1 < N) ? Vp[(k + 1) * BPS + m] : 0.0, e, q1);
-#pragma unroll
-            for (int s = 0; s < kS; ++s)
-                *reinterpret_cast<uint32_t*>(dst + (size_t)s * plane1 + k) = bf16x2_of(q0[s], q1[s]);
-        }
-    }
-    // V2: row r over the reflectors (K = the BP reflectors, padded to 64 with zeros set at init),
-    // rows of the first row tile that holds row p onward
-    for (int r = (p / 128) * 128 + warp; r < mpad; r += kPW) {
-        const double v = (r >= p && r < N && lane < BP) ? Vp[r * BPS + lane] : 0.0;
-        const int e = exponent_of_bits(warp_max_bits(abs_bits(v)));
-        if (lane == 0) eV2[(size_t)gf * mpad + r] = e;
-        if (lane < BP) {
-            float q[kS];
-            slice7(v, e, q);
-#pragma unroll
-            for (int s = 0; s < kS; ++s) V2[(size_t)s * plane2 + ((size_t)gf * mpad + r) * 64 + lane] = bf16_of(q[s]);
-        }
-    }
+    slice_V<BP, kPT>(Vp, V1, eV1, V2, eV2, N, p, gf, kpad, mpad, plane1, plane2);
 }
 
 // ---- slices of the trailing columns ---------------------------------------------------------
-// Warp w of block x slices trailing column jj = 8 x + w (logical column j0 + jj) over rows p..N-1.
+// Warp w of block x slices trailing column jj = 8 x + w (logical column j0 + jj; no permutation in the formation of
+// Q) over rows p..N-1.
 __global__ void __launch_bounds__(256) k_qrt_slice_C(const double* __restrict__ Yall, const int* __restrict__ perm_all,
                                                      __nv_bfloat16* __restrict__ Cs, int* __restrict__ eC, int N,
                                                      int p, int j0, int kpad, int jpad, size_t plane, int fbase) {
     const int f = blockIdx.y, gf = fbase + f, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int jj = blockIdx.x * 8 + warp, j = j0 + jj;
     if (j >= N) return;
-    const double* col = Yall + (size_t)f * N * N + (size_t)perm_all[(size_t)f * N + j] * N;
+    const double* col = Yall + (size_t)f * N * N + (size_t)(perm_all ? perm_all[(size_t)f * N + j] : j) * N;
     long long mx = 0;
     for (int r = p + lane; r < N; r += 32) mx = max(mx, abs_bits(col[r]));
     const int e = exponent_of_bits(warp_max_bits(mx));
@@ -321,6 +333,27 @@ __global__ void __launch_bounds__(256) k_qrt_slice_C(const double* __restrict__ 
     }
 }
 
+// The reflectors of panel p of a finished QR (below the diagonal of its packed output), sliced again for the
+// formation of Q.
+template <int BP>
+__global__ void __launch_bounds__(256) k_qrt_slice_V(const double* __restrict__ QRall, __nv_bfloat16* __restrict__ V1,
+                                                     int* __restrict__ eV1, __nv_bfloat16* __restrict__ V2,
+                                                     int* __restrict__ eV2, int N, int p, int kpad, int mpad, size_t plane1,
+                                                     size_t plane2, int fbase) {
+    constexpr int BPS = BP + 1;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    double* Vp = reinterpret_cast<double*>(smraw) - (size_t)p * BPS;  // rows p.. stored
+    const int f = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double* QR = QRall + (size_t)f * N * N;
+    for (int c = warp; c < BP; c += 8) {
+        const int k = p + c;
+        for (int r = p + lane; r < N; r += 32)
+            Vp[r * BPS + c] = k < N ? (r > k ? QR[(size_t)k * N + r] : (r == k ? 1.0 : 0.0)) : 0.0;
+    }
+    __syncthreads();
+    slice_V<BP, 256>(Vp, V1, eV1, V2, eV2, N, p, fbase + f, kpad, mpad, plane1, plane2);
+}
+
 // ---- [G; W^T] = [V C]^T V, S from G, then W'^T = W^T S and its slices -----------------------
 // CTA = the BP reflectors plus 128 - BP trailing columns of one field: each 128-row A tile holds the
 // slices of V's columns (rows 0..BP-1, from the reflector slice buffer) above those of the CTA's
@@ -329,7 +362,9 @@ __global__ void __launch_bounds__(256) k_qrt_slice_C(const double* __restrict__ 
 // out for the formation of Q), then W' = S^T W. TMA streams per 64-row K chunk the seven A slices
 // through a 3-tile ring and the seven V slices double-buffered; products (a, b), a + b <= 6, go to
 // the accumulator of level a + b of the chunk's segment (seven chunks per segment).
-template <int BP>
+// kForm: the step of the formation of Q, whose panels need W' = S W with the S the QR left in Sall (the Gram rows
+// of the product are not used).
+template <int BP, bool kForm>
 __global__ void __launch_bounds__(kQT, 2)
     k_qrt_gemm1(const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmV,
                 const int* __restrict__ eC, const int* __restrict__ eV1, const double* __restrict__ tau_all,
@@ -372,7 +407,7 @@ __global__ void __launch_bounds__(kQT, 2)
     }
     if (threadIdx.x < BP) {
         eV_sh[threadIdx.x] = eV1[(size_t)gf * kVRows + threadIdx.x];
-        tau_sh[threadIdx.x] = tau_all[(size_t)f * N + p + threadIdx.x];
+        if (!kForm) tau_sh[threadIdx.x] = tau_all[(size_t)f * N + p + threadIdx.x];
     }
     const int nseg = (nkc + kSegChunks - 1) / kSegChunks;
     const uint32_t tcols = nseg == 1 ? 256u : 512u;  // 7 levels x BP columns per accumulator set
@@ -454,6 +489,14 @@ __global__ void __launch_bounds__(kQT, 2)
         // jj = mt kMC + r - BP
         constexpr int HC = BP / 2;
         const int q4 = warp & 3, h = warp >> 2, r = 32 * q4 + lane, jj = mt * kMC + r - BP;
+        constexpr int SPT = BP * BP / 256;
+        double s_in[SPT];  // kForm: S (rows beyond the last reflector are zero), loaded before the products are waited for
+        if (kForm)
+#pragma unroll
+            for (int q = 0; q < SPT; ++q) {
+                const int idx = threadIdx.x + 256 * q;
+                s_in[q] = p + idx / BP < N ? Sall[((size_t)f * N + p) * BP + idx] : 0.0;
+            }
         const bool bad = !mbar_wait(smem_u32(&bar_acc), 0, err) || abort_sh;
         if (!named_sync_or(1, 256, bad)) {
             tc_fence_after();
@@ -488,9 +531,16 @@ __global__ void __launch_bounds__(kQT, 2)
             }
         }
         named_sync(1, 256);
-        if (!bad) wy_triangle_blocked<BP>(stW, WS, tau_sh, Ssh, stWp, threadIdx.x);  // S from G = rows 0..BP-1
+        if (kForm) {
+            if (!bad)
+#pragma unroll
+                for (int q = 0; q < SPT; ++q) Ssh[threadIdx.x + 256 * q] = s_in[q];
+            named_sync(1, 256);
+        } else if (!bad) {
+            wy_triangle_blocked<BP>(stW, WS, tau_sh, Ssh, stWp, threadIdx.x);  // S from G = rows 0..BP-1
+        }
         if (!bad) {
-            if (mt == 0)  // S of the panel for the formation of Q
+            if (!kForm && mt == 0)  // S of the panel for the formation of Q
                 for (int idx = threadIdx.x; idx < BP * BP; idx += 256)
                     Sall[((size_t)f * N + p) * BP + idx] = Ssh[idx];
             // W'[m] = sum_{q <= m} S[q][m] W[q]  (S upper triangular); thread (row, half)
@@ -498,7 +548,10 @@ __global__ void __launch_bounds__(kQT, 2)
             if ((threadIdx.x & 127) < kMC)
                 for (int m = hh * HC; m < hh * HC + HC; ++m) {
                     double a = 0.0;
-                    for (int q = 0; q <= m; ++q) a = fma(Ssh[q * BP + m], stW[rr * WS + q], a);
+                    if (kForm)
+                        for (int q = m; q < BP; ++q) a = fma(Ssh[m * BP + q], stW[rr * WS + q], a);
+                    else
+                        for (int q = 0; q <= m; ++q) a = fma(Ssh[q * BP + m], stW[rr * WS + q], a);
                     stWp[rr * WS + m] = a;
                 }
         }
@@ -567,7 +620,7 @@ __global__ void __launch_bounds__(kQT, 2)
     if (threadIdx.x < kNC) {
         const int jj = nt * kNC + threadIdx.x;
         eW_sh[threadIdx.x] = jj < n_t ? eW[(size_t)gf * wpad + jj] : 0;
-        col_sh[threadIdx.x] = jj < n_t ? perm_all[(size_t)f * N + j0 + jj] : 0;
+        col_sh[threadIdx.x] = jj < n_t ? (perm_all ? perm_all[(size_t)f * N + j0 + jj] : j0 + jj) : 0;
     }
     if (warp == 9) {
         tmem_alloc(smem_u32(&tmem_base_sh), 256);
@@ -621,31 +674,41 @@ __global__ void __launch_bounds__(kQT, 2)
         // ---- epilogue: warp w: rows 32 (w % 4).. of the tile, columns 16 (w / 4)..; C -= V W' ----
         constexpr int HC = kNC / 2;
         const int q4 = warp & 3, h = warp >> 2, r = mt * 128 + 32 * q4 + lane;
+        const bool row_ok = r >= p && r < N;
+        const int ev = row_ok ? eV2[(size_t)gf * mpad + r] : 0;
+        double* Yf = Yall + (size_t)f * N * N + r;
+        // the entries of C for a block of 8 columns are loaded together, the first block's before the products are
+        // waited for (one at a time behind the stores of the last, their latencies were most of the epilogue)
+        double y[8];
+        auto fetch = [&](int c0) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const int cc = HC * h + c0 + c;
+                y[c] = (row_ok && nt * kNC + cc < n_t) ? Yf[(size_t)col_sh[cc] * N] : 0.0;
+            }
+        };
+        fetch(0);
         const bool bad = !mbar_wait(smem_u32(&bar_acc), 0, err) || abort_sh;
         if (!named_sync_or(1, 256, bad)) {
             tc_fence_after();
-            const bool row_ok = r >= p && r < N;
-            const int ev = row_ok ? eV2[(size_t)gf * mpad + r] : 0;
-            double* Yf = Yall + (size_t)f * N * N;
 #pragma unroll
             for (int c0 = 0; c0 < HC; c0 += 8) {
                 uint32_t v[kLv][8];
                 const uint32_t tl = tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(HC * h + c0);
 #pragma unroll
                 for (int lv = 0; lv < kLv; ++lv) tmem_ld8(tl + (uint32_t)(lv * kNC), v[lv]);
+                if (c0 > 0) fetch(c0);
                 tmem_ld_wait();
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    const int cc = HC * h + c0 + c, jj = nt * kNC + cc;
-                    if (!row_ok || jj >= n_t) continue;
+                    const int cc = HC * h + c0 + c;
+                    if (!row_ok || nt * kNC + cc >= n_t) continue;
                     uint32_t w[kLv];
 #pragma unroll
                     for (int lv = 0; lv < kLv; ++lv) w[lv] = v[lv][c];
                     long long hi, lo;
                     small_levels_to_int(w, hi, lo);
-                    const double t = combine(hi, lo, ev + eW_sh[cc] - kUnitShift);
-                    double* y = Yf + (size_t)col_sh[cc] * N + r;
-                    *y = *y - t;
+                    Yf[(size_t)col_sh[cc] * N] = y[c] - combine(hi, lo, ev + eW_sh[cc] - kUnitShift);
                 }
             }
         }
@@ -703,7 +766,7 @@ template <int BP>
 cudaError_t launch_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s) {
     const QrtArgs a = qrt_args(c);
     const size_t sm1 = gemm1_smem(BP), sm2 = gemm2_smem();
-    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
+    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_gemm2<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
     if (e != cudaSuccess) return e;
     const CUtensorMap& mapV1 = BP == 32 ? c->qt_mapV1_32 : c->qt_mapV1_16;
@@ -711,11 +774,47 @@ cudaError_t launch_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s) {
     k_qrt_slice_C<<<dim3((n_t + 7) / 8, nf), 256, 0, s>>>(c->Y, c->perm, a.Cs, c->qt_eC, N, p, j0, a.kpad, a.jpad,
                                                           a.planeC, c->fbase);
     const CUtensorMap& mapC = BP == 32 ? c->qt_mapC96 : c->qt_mapC112;
-    k_qrt_gemm1<BP><<<dim3((n_t + 127 - BP) / (128 - BP), nf), kQT, sm1, s>>>(
+    k_qrt_gemm1<BP, false><<<dim3((n_t + 127 - BP) / (128 - BP), nf), kQT, sm1, s>>>(
         mapC, mapV1, c->qt_eC, c->qt_eV1, c->tau, c->Sws, a.Ws, c->qt_eW, N, p, n_t, a.kpad, a.jpad, a.wpad, a.planeW,
         c->fbase, c->err);
     k_qrt_gemm2<BP><<<dim3((n_t + kNC - 1) / kNC, a.mpad / 128 - p / 128, nf), kQT, sm2, s>>>(
         c->qt_mapV2, c->qt_mapW, c->qt_eV2, c->qt_eW, c->perm, c->Y, N, p, j0, n_t, a.mpad, a.wpad, c->fbase, c->err);
+    return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(256) k_qrt_identity(double* __restrict__ U, int N) {
+    double* Uf = U + (size_t)blockIdx.y * N * N;
+    for (int idx = blockIdx.x * 256 + threadIdx.x; idx < N * N; idx += gridDim.x * 256) Uf[idx] = idx % (N + 1) == 0 ? 1.0 : 0.0;
+}
+
+// Q = Q_0 Q_1 ... accumulated backwards into U: per panel, columns and rows p.. of U take I - V S V^T through the
+// products of the trailing update (slices of V and of U's columns, W = V^T U, W' = S W, U -= V W'). On the FP64 pipe
+// (k_formq_b) the 4/3 N^3 flops were 30-45 % of an FP64 evaluation and of a DQMC sweep's chain steps: 12x12,
+// L = 120, 256 fields with G 65.9 -> 55.5 ms; 18x10, L = 37, 50 fields 13.5 -> 11.4 ms (four Q: 4.0 -> 2.0 ms).
+template <int BP>
+cudaError_t launch_form_q(slmc_ctx* c, int nf, cudaStream_t s) {
+    const QrtArgs a = qrt_args(c);
+    const int N = a.N;
+    const size_t sm1 = gemm1_smem(BP), sm2 = gemm2_smem(), smV = sizeof(double) * (size_t)N * (BP + 1);
+    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_gemm2<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_slice_V<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smV);
+    if (e != cudaSuccess) return e;
+    const CUtensorMap& mapV1 = BP == 32 ? c->qt_mapV1_32 : c->qt_mapV1_16;
+    const CUtensorMap& mapC = BP == 32 ? c->qt_mapC96 : c->qt_mapC112;
+    k_qrt_identity<<<dim3(std::min(64, (N * N + 1023) / 1024), nf), 256, 0, s>>>(c->U, N);
+    for (int p = (N - 1) / BP * BP; p >= 0; p -= BP) {
+        const int n_t = N - p;
+        k_qrt_slice_V<BP><<<nf, 256, sizeof(double) * (size_t)n_t * (BP + 1), s>>>(
+            c->QR, a.V1, c->qt_eV1, a.V2, c->qt_eV2, N, p, a.kpad, a.mpad, a.plane1, a.plane2, c->fbase);
+        k_qrt_slice_C<<<dim3((n_t + 7) / 8, nf), 256, 0, s>>>(c->U, nullptr, a.Cs, c->qt_eC, N, p, p, a.kpad, a.jpad, a.planeC,
+                                                              c->fbase);
+        k_qrt_gemm1<BP, true><<<dim3((n_t + 127 - BP) / (128 - BP), nf), kQT, sm1, s>>>(
+            mapC, mapV1, c->qt_eC, c->qt_eV1, c->tau, c->Sws, a.Ws, c->qt_eW, N, p, n_t, a.kpad, a.jpad, a.wpad, a.planeW,
+            c->fbase, c->err);
+        k_qrt_gemm2<BP><<<dim3((n_t + kNC - 1) / kNC, a.mpad / 128 - p / 128, nf), kQT, sm2, s>>>(
+            c->qt_mapV2, c->qt_mapW, c->qt_eV2, c->qt_eW, nullptr, c->U, N, p, p, n_t, a.mpad, a.wpad, c->fbase, c->err);
+    }
     return cudaGetLastError();
 }
 
@@ -770,7 +869,17 @@ cudaError_t qrt_init(slmc_ctx* c, void* bf16_base, int* int_base) {
     return cudaSuccess;
 }
 
+// Below, a panel's four launches outweigh the FP64 kernel (one or two panels in all).
+constexpr int kFormQMinN = 65;
+
 bool qrt_active(const slmc_ctx* c) { return c->qt_C && c->qr_path == 0 && qrt_supported(c->N); }
+
+// The formation of Q in FP64 on the tensor cores: 4 launches per panel.
+bool qrt_form_q_active(const slmc_ctx* c) { return qrt_active(c) && c->N >= kFormQMinN; }
+int qrt_form_q_launches(const slmc_ctx* c) { return 1 + 4 * qrt_panels(c); }
+cudaError_t qrt_form_q(slmc_ctx* c, int nf, cudaStream_t s) {
+    return qr_panel_width(c) == 32 ? launch_form_q<32>(c, nf, s) : launch_form_q<16>(c, nf, s);
+}
 
 int qrt_panels(const slmc_ctx* c) {
     const int BP = qr_panel_width(c);

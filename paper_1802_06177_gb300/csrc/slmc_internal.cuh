@@ -213,6 +213,9 @@ bool qrt_active(const slmc_ctx* c);
 int qrt_panels(const slmc_ctx* c);
 cudaError_t qrt_panel(slmc_ctx* c, int nf, int t, cudaStream_t s);     // factor panel t (1 launch)
 cudaError_t qrt_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s);  // its trailing update (3 launches)
+bool qrt_form_q_active(const slmc_ctx* c);
+int qrt_form_q_launches(const slmc_ctx* c);
+cudaError_t qrt_form_q(slmc_ctx* c, int nf, cudaStream_t s);  // Q (FP64) of the last QR into U
 cudaError_t tt_init(slmc_ctx* c);
 cudaError_t qr_blocked(slmc_ctx* c, int nf, cudaStream_t s);
 cudaError_t form_q_blocked(slmc_ctx* c, int nf, bool fp32, cudaStream_t s);

@@ -130,10 +130,10 @@ __device__ __forceinline__ void line(const double* __restrict__ c, double (&v)[n
 }
 
 // The line g[0], g[stride], ... in place, with optional input scales in_sc[m in_st] and output scales
-// out_sc[d out_st] * out_mul.
+// out_sc[d out_st] (times *mul if given).
 template <int n>
 __device__ __forceinline__ void apply(double* g, int stride, const double* __restrict__ c, const double* in_sc, int in_st,
-                                      const double* out_sc, int out_st, double out_mul) {
+                                      const double* out_sc, int out_st, const double* mul) {
     double v[n];
 #pragma unroll
     for (int m = 0; m < n; ++m) v[m] = g[m * stride];
@@ -141,9 +141,16 @@ __device__ __forceinline__ void apply(double* g, int stride, const double* __res
 #pragma unroll
         for (int m = 0; m < n; ++m) v[m] *= in_sc[m * in_st];
     line<n>(c, v);
-    if (out_sc)
+    if (out_sc) {
+        if (mul) {
+            const double f = *mul;
 #pragma unroll
-        for (int m = 0; m < n; ++m) v[m] *= out_sc[m * out_st] * out_mul;
+            for (int m = 0; m < n; ++m) v[m] *= out_sc[m * out_st] * f;
+        } else {
+#pragma unroll
+            for (int m = 0; m < n; ++m) v[m] *= out_sc[m * out_st];
+        }
+    }
 #pragma unroll
     for (int m = 0; m < n; ++m) g[m * stride] = v[m];
 }
@@ -151,10 +158,11 @@ __device__ __forceinline__ void apply(double* g, int stride, const double* __res
 // Length n <= LMAX at run time (one call site per kernel: every length is expanded there).
 template <int LMAX>
 __device__ __forceinline__ void apply_any(int n, double* g, int stride, const double* __restrict__ c, const double* in_sc,
-                                          int in_st, const double* out_sc, int out_st, double out_mul) {
+                                          int in_st, const double* out_sc, int out_st,
+                                          const double* mul = nullptr) {
 #define SLMC_CIRC(k)                                                                             \
     case k:                                                                                      \
-        if constexpr (k <= LMAX) apply<k>(g, stride, c, in_sc, in_st, out_sc, out_st, out_mul); \
+        if constexpr (k <= LMAX) apply<k>(g, stride, c, in_sc, in_st, out_sc, out_st, mul); \
         break;
     switch (n) {
         SLMC_CIRC(2) SLMC_CIRC(3) SLMC_CIRC(4) SLMC_CIRC(5) SLMC_CIRC(6) SLMC_CIRC(7) SLMC_CIRC(8) SLMC_CIRC(9)

@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kThreads) k_dqmc_slices(double* __restrict__ x
                 const int li = q / N, o = q - li * N;  // line, and the row (right factors) or column (left) it belongs to
                 const int at = (alongx ? li * Lx : li) * unit + o * (left ? 1 : ldg);
                 slmc::circ::apply_any<LMAX>(n, G + at, stride, cf, nullptr, 0, pass == 3 ? s + li : nullptr, Lx,
-                                            pass == 3 ? sinv[o] : 1.0);
+                                            sinv + o);
             }
             __syncthreads();
         }

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kThreads) k_slice_kron(const double* __restric
                     const int o = q * step_l;
                     slmc::circ::apply_any<LMAX>(pass ? Ly : Lx, Pl + o, stride, pass ? cy : cx,
                                                 kTrans && pass == 0 ? sc + o : nullptr, stride,
-                                                !kTrans && pass == 1 ? sc + o : nullptr, stride, 1.0);
+                                                !kTrans && pass == 1 ? sc + o : nullptr, stride);
                 }
             __syncthreads();
         }

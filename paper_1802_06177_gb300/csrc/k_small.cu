@@ -10,11 +10,11 @@ namespace {
 using namespace slmc::sm;
 
 template <int NMAX, int LMAX>
-__global__ void __launch_bounds__(4 * NMAX, 1) k_small_logdet(const double* __restrict__ x, const double* __restrict__ kron,
+__global__ void __launch_bounds__(Dim<NMAX>::threads, NMAX == 16 ? 4 : 2) k_small_logdet(const double* __restrict__ x, const double* __restrict__ kron,
                                                            double* __restrict__ lndet, int* __restrict__ sign,
                                                            double* __restrict__ Gout, unsigned int* __restrict__ err, int N,
                                                            int Lx, int Ly, int L, int n_s, double dtlam, double emu) {
-    constexpr int ld = Dim<NMAX>::ld, NT = Dim<NMAX>::threads, RPT = NMAX / 4;
+    constexpr int ld = Dim<NMAX>::ld, NT = Dim<NMAX>::threads, RPT = Dim<NMAX>::rpt, G = Dim<NMAX>::G;
     extern __shared__ __align__(16) double dsm[];
     double* A = dsm;                       // packed QR, then M and its LU
     double* B = A + Dim<NMAX>::mat;        // U
@@ -27,8 +27,7 @@ __global__ void __launch_bounds__(4 * NMAX, 1) k_small_logdet(const double* __re
         B[idx] = e;
         T[idx] = e;
     }
-    slmc::circ::build(v.cx, kron, Lx, tid, NT);
-    slmc::circ::build(v.cy, kron + 2 * slmc::kKronTab, Ly, tid, NT);
+    load_factors<NMAX>(v, kron, Lx, Ly);
     if (tid < N) v.lnd[tid] = 0.0;
     __syncthreads();
     bool bad = false;
@@ -71,11 +70,11 @@ __global__ void __launch_bounds__(4 * NMAX, 1) k_small_logdet(const double* __re
     if (!Gout) return;
     if (tid < N) v.beta[tid] = 1.0 / A[tid * ld + tid];
     __syncthreads();
-    const int j = tid >> 2, g = tid & 3;
+    const int j = tid / G, g = tid % G;
     double b[RPT];
 #pragma unroll
     for (int q = 0; q < RPT; ++q) {
-        const int r = 4 * q + g;
+        const int r = G * q + g;
         const int sr = r < N ? v.src[r] : 0;
         b[q] = (j < N && r < N) ? v.e1[sr] * B[sr * ld + j] : 0.0;
     }
@@ -83,7 +82,7 @@ __global__ void __launch_bounds__(4 * NMAX, 1) k_small_logdet(const double* __re
     if (j < N)
 #pragma unroll
         for (int q = 0; q < RPT; ++q)
-            if (4 * q + g < N) Gout[(size_t)f * N * N + (size_t)(4 * q + g) * N + j] = b[q];
+            if (G * q + g < N) Gout[(size_t)f * N * N + (size_t)(G * q + g) * N + j] = b[q];
 }
 
 template <int NMAX, int LMAX>
@@ -91,7 +90,7 @@ cudaError_t launch_small(slmc_ctx* c, const double* x, int nf, double* lndet, in
     const size_t smem = 3 * (size_t)Dim<NMAX>::mat * sizeof(double) + sizeof(Vecs<NMAX>);
     cudaError_t e = cudaFuncSetAttribute(k_small_logdet<NMAX, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_small_logdet<NMAX, LMAX><<<nf, 4 * NMAX, smem, s>>>(x, c->kron, lndet, sign, G, c->err, c->N, c->p.Lx, c->p.Ly, c->L,
+    k_small_logdet<NMAX, LMAX><<<nf, Dim<NMAX>::threads, smem, s>>>(x, c->kron, lndet, sign, G, c->err, c->N, c->p.Lx, c->p.Ly, c->L,
                                                          c->p.n_s, c->p.dtau * c->p.lambda, exp(c->p.dtau * c->p.mu));
     return cudaGetLastError();
 }

@@ -3,10 +3,15 @@
 // so a determinant is one launch instead of several per slice group, and nothing goes through global memory
 // but the field and the result.
 //
-// What bounds it: for N <= 36 the chain of column steps (barriers, square roots, divisions); for N = 64 the
-// FP64 pipe (two FMAs per clock per SM). Columns are held in registers by quads: thread 4 j + g owns rows g,
-// g + 4, ... of column j, so a dot product is a run of FMAs per thread and two additions across the quad; a
-// column per warp would spend five of every nine FP64 slots on the reduction at these sizes.
+// What bounds it: for N <= 36 the chain of column steps; for N = 64 the FP64 pipe (two FMAs per clock per SM). A
+// sub-core takes 64 cycles per FP64 warp instruction, however many lanes are active, so the chain is as long as
+// the number of FP64 instructions one warp runs in sequence. Columns are held in registers by groups of G lanes:
+// thread G j + g owns rows g, g + G, ... of column j, so a dot product is a run of FMAs per thread and log2 G
+// additions across the group (a column per warp would spend five of every nine on the reduction); the warps of a
+// field cover all four sub-cores; square root and divisions are short Newton forms, the two divisions of a
+// reflector in neighbouring lanes of one instruction stream; and a group's slice scales are exponentiated
+// together before its slices. 64 fields of 4x4, L = 40 with G: 784 us by per-step kernels, 401 us by the first
+// version of this kernel, 326 us with folded transforms, 241 us now.
 //
 // Matrices in shared memory: element (r, c) of a column-major one at c * ld + r, of a row-major one at
 // r * ld + c, ld = NMAX + 1; rows and columns beyond N are zero.
@@ -22,8 +27,10 @@ namespace sm {
 
 template <int NMAX>
 struct Dim {
-    static constexpr int ld = NMAX + 1, mat = NMAX * ld, threads = 4 * NMAX, rpt = NMAX / 4;
+    static constexpr int G = NMAX <= 32 ? 8 : 4;  // lanes per column
+    static constexpr int ld = NMAX + 1, mat = NMAX * ld, threads = G * NMAX, rpt = NMAX / G, cpw = 32 / G;
 };
+constexpr int kScMax = 16;  // slices whose scales are formed together
 
 constexpr int kSmallCoef = 481;  // circ::ncoef of the longest line (31: one level; 32 folds twice)
 static_assert(circ::ncoef(31) <= kSmallCoef && circ::ncoef(32) <= kSmallCoef && circ::ncoef(30) <= kSmallCoef, "");
@@ -33,7 +40,7 @@ template <int NMAX>
 struct Vecs {
     double lnd[NMAX], lnn[NMAX];   // ln D, new ln D
     double key[NMAX], e1[NMAX], e2[NMAX], tau[NMAX], beta[NMAX];
-    double sc[NMAX];               // slice scales
+    double sc[kScMax][NMAX];       // slice scales of a group
     double cx[kSmallCoef], cy[kSmallCoef];  // folded coefficients of E_x, E_y
     double lbuf[2][NMAX];          // multipliers of the current / next LU step
     double logabs;
@@ -43,47 +50,153 @@ struct Vecs {
     int ntriv, wide, neg, sing;
 };
 
-__device__ __forceinline__ double quad_sum(double v) {
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    return v + __shfl_xor_sync(0xffffffffu, v, 2);
+template <int G>
+__device__ __forceinline__ double group_sum(double v) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Square root and quotient of normal numbers of moderate exponent (others take the library's) by Newton steps from an
+// FP32 estimate of the significand: Goldschmidt's coupled iteration for the root with a final residual correction,
+// Newton's for the reciprocal and Markstein's correction of the quotient. Six and five FP64 instructions; results
+// are within one unit in the last place of the correctly rounded ones (10^8 random arguments).
+__device__ __forceinline__ double fast_sqrt(double a) {
+    const int hi = __double2hiint(a), ex = (hi >> 20) - 1023;
+    if (ex < -900 || ex > 900) return sqrt(a);
+    const int k = ex >> 1;  // a = m 4^k, m in [1, 4)
+    const double m = __hiloint2double(hi - (k << 21), __double2loint(a));
+    const float mf = __int_as_float(((hi - (k << 21) - 0x38000000) << 3) | ((uint32_t)__double2loint(a) >> 29));
+    const float y = rsqrtf(mf);
+    const double yd = __hiloint2double((int)(__float_as_uint(y) >> 3) + 0x38000000, (int)(__float_as_uint(y) << 29));
+    double g = m * yd, h = __hiloint2double(__double2hiint(yd) - 0x00100000, __double2loint(yd));
+    const double r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    h = fma(h, r, h);
+    g = fma(fma(-g, g, m), h, g);
+    return __hiloint2double(__double2hiint(g) + (k << 20), __double2loint(g));
+}
+__device__ __forceinline__ double fast_div(double n, double d) {
+    const int hd = __double2hiint(d), ex = ((hd >> 20) & 0x7ff) - 1023;
+    const int en = ((__double2hiint(n) >> 20) & 0x7ff) - 1023;
+    if (ex < -400 || ex > 400 || en < -400 || en > 400) return n / d;
+    const int sh = ex << 20;  // d = s 2^ex, |s| in [1, 2)
+    const double sd = __hiloint2double(hd - sh, __double2loint(d));
+    const float sf = __int_as_float((int)((hd & 0x80000000u) | ((((hd & 0x7fffffff) - sh - 0x38000000) << 3) |
+                                                                ((uint32_t)__double2loint(d) >> 29))));
+    const float y = __frcp_rn(sf);
+    const uint32_t yu = __float_as_uint(y) & 0x7fffffffu;
+    double yd = __hiloint2double((int)((yu >> 3) + 0x38000000u) | (hd & (int)0x80000000), (int)(yu << 29));
+    yd = fma(fma(-sd, yd, 1.0), yd, yd);
+    double q = n * yd;
+    q = fma(fma(-sd, q, n), yd, q);
+    return __hiloint2double(__double2hiint(q) - (q == 0.0 ? 0 : sh), __double2loint(q));
+}
+
+// One pass of a transform over short lines (n <= 8, the 4x4 class): two lanes per line, each half of the outputs by
+// direct sums. At this size the folded transform's chain (18 FP64 instructions for a line of 4 on two warps) is
+// longer than eight direct ones on four.
+template <int n>
+__device__ __forceinline__ void half_line(double* g, int stride, const double* __restrict__ t, int half,
+                                          const double* out_sc, bool on) {
+    constexpr int nh = (n + 1) / 2;
+    double v[n], y[nh];
+#pragma unroll
+    for (int m = 0; m < n; ++m) v[m] = g[m * stride];
+#pragma unroll
+    for (int o = 0; o < nh; ++o) {
+        const int d = half * nh + o;
+        y[o] = t[d < n ? d : 0] * v[0];
+#pragma unroll
+        for (int m = 1; m < n; ++m) y[o] = fma(t[d >= m ? (d < n ? d - m : 0) : d - m + n], v[m], y[o]);
+        if (out_sc) y[o] *= out_sc[(d < n ? d : 0) * stride];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 0; o < nh; ++o)
+        if (on && half * nh + o < n) g[(half * nh + o) * stride] = y[o];
+}
+
+template <int NMAX>
+__device__ __forceinline__ void short_pass(double* P, const double* __restrict__ t, const double* in_sc, const double* out_sc,
+                                           int N, int n, int lines, int step_l, int stride) {
+    constexpr int ld = Dim<NMAX>::ld, NT = Dim<NMAX>::threads;
+    for (int q0 = 0; q0 < 2 * N * lines; q0 += NT) {  // uniform trip count: the halves meet at a warp barrier
+        const int q = q0 + threadIdx.x, li = (q >> 1) / N, jj = (q >> 1) - li * N, o = li * step_l;
+        const bool on = q < 2 * N * lines;
+        double* g = P + (on ? jj * ld + o : 0);
+        if (in_sc && on && (q & 1) == 0)
+            for (int m = 0; m < n; ++m) g[m * stride] *= in_sc[o + m * stride];
+        __syncwarp();
+#define SLMC_SHORT(k) \
+    case k: half_line<k>(g, stride, t, q & 1, out_sc ? out_sc + (on ? o : 0) : nullptr, on); break;  // off lanes: no store
+        switch (n) {
+            SLMC_SHORT(2) SLMC_SHORT(3) SLMC_SHORT(4) SLMC_SHORT(5) SLMC_SHORT(6) SLMC_SHORT(7) SLMC_SHORT(8)
+        }
+#undef SLMC_SHORT
+    }
 }
 
 // P <- B_{c1} ... B_{c0} P (plain) for the field columns c0 .. c1 - 1 in order, or with trans the transposed
 // slices E diag(s) from c1 - 1 down to c0: circulant transforms along the x and the y lines of every column.
+// v.cx, v.cy: folded coefficients, or the plain factors for NMAX = 16 (short_pass).
 template <int NMAX, int LMAX, bool kTrans>
 __device__ __forceinline__ void slices(double* P, Vecs<NMAX>& v, const double* __restrict__ xf, int N, int Lx, int Ly,
                                        int L, int c0, int c1, double dtlam, double emu) {
     constexpr int ld = Dim<NMAX>::ld, NT = Dim<NMAX>::threads;
     const int tid = threadIdx.x;
-    // the field column of the next slice is loaded a slice ahead (N <= NT: one site per thread)
-    double xv = tid < N ? xf[(size_t)tid * L + (kTrans ? c1 - 1 : c0)] : 0.0;
-    for (int step = 0; step < c1 - c0; ++step) {
-        if (tid < N) v.sc[tid] = exp(-dtlam * xv) * emu;
-        if (tid < N && step + 1 < c1 - c0) xv = xf[(size_t)tid * L + (kTrans ? c1 - 2 - step : c0 + step + 1)];
-        if (kTrans) __syncthreads();  // the x pass scales its input; plain slices use sc after the next barrier
-        for (int pass = 0; pass < 2; ++pass) {
-            const int lines = pass ? Lx : Ly, step_l = pass ? 1 : Lx, stride = pass ? Lx : 1;
-            for (int q = tid; q < N * lines; q += NT) {
-                const int li = q / N, jj = q - li * N, o = li * step_l;
-                circ::apply_any<LMAX>(pass ? Ly : Lx, P + jj * ld + o, stride, pass ? v.cy : v.cx,
-                                      kTrans && pass == 0 ? v.sc + o : nullptr, stride,
-                                      !kTrans && pass == 1 ? v.sc + o : nullptr, stride, 1.0);
-            }
-            __syncthreads();
+    for (int b0 = c0; b0 < c1; b0 += kScMax) {
+        const int nb = min(kScMax, c1 - b0);  // field columns of this batch, in the order of the slices
+        for (int idx = tid; idx < nb * N; idx += NT) {
+            const int i = idx / nb, k = idx - i * nb;
+            const int c = kTrans ? c1 - 1 - (b0 - c0) - k : b0 + k;
+            v.sc[k][i] = exp(-dtlam * xf[(size_t)i * L + c]) * emu;
         }
+        __syncthreads();
+        for (int k = 0; k < nb; ++k)
+            for (int pass = 0; pass < 2; ++pass) {
+                const int lines = pass ? Lx : Ly, step_l = pass ? 1 : Lx, stride = pass ? Lx : 1, n = pass ? Ly : Lx;
+                const double* in_sc = kTrans && pass == 0 ? v.sc[k] : nullptr;
+                const double* out_sc = !kTrans && pass == 1 ? v.sc[k] : nullptr;
+                if constexpr (NMAX == 16) {
+                    short_pass<NMAX>(P, pass ? v.cy : v.cx, in_sc, out_sc, N, n, lines, step_l, stride);
+                } else {
+                    for (int q = tid; q < N * lines; q += NT) {
+                        const int li = q / N, jj = q - li * N, o = li * step_l;
+                        circ::apply_any<LMAX>(n, P + jj * ld + o, stride, pass ? v.cy : v.cx, in_sc ? in_sc + o : nullptr,
+                                              stride, out_sc ? out_sc + o : nullptr, stride);
+                    }
+                }
+                __syncthreads();
+            }
     }
 }
 
-// Reflector of column j = k (its quad calls it; rows q < kq are final): beta, tau, v into the packed column k of
-// A (R above the diagonal, beta on it, v below).
+// The transform's coefficients into v.cx, v.cy (caller synchronises).
 template <int NMAX>
-__device__ __forceinline__ void reflector(double (&a)[NMAX / 4], int kq, int kg, int k, int N, int g, bool mine, double* A,
-                                          Vecs<NMAX>& v) {
-    constexpr int ld = Dim<NMAX>::ld, RPT = NMAX / 4;
+__device__ __forceinline__ void load_factors(Vecs<NMAX>& v, const double* __restrict__ kron, int Lx, int Ly) {
+    constexpr int NT = Dim<NMAX>::threads;
+    if constexpr (NMAX == 16) {
+        if (threadIdx.x < 8) {
+            v.cx[threadIdx.x] = kron[threadIdx.x];
+            v.cy[threadIdx.x] = kron[2 * kKronTab + threadIdx.x];
+        }
+    } else {
+        circ::build(v.cx, kron, Lx, threadIdx.x, NT);
+        circ::build(v.cy, kron + 2 * kKronTab, Ly, threadIdx.x, NT);
+    }
+}
+
+// Reflector of column j = k (its group calls it; rows before G kq are final): beta, tau, v into the packed column k
+// of A (R above the diagonal, beta on it, v below).
+template <int NMAX>
+__device__ __forceinline__ void reflector(double (&a)[Dim<NMAX>::rpt], int kq, int kg, int k, int N, int g, bool mine,
+                                          double* A, Vecs<NMAX>& v) {
+    constexpr int ld = Dim<NMAX>::ld, RPT = Dim<NMAX>::rpt, G = Dim<NMAX>::G;
     double alpha = 0.0, sig = 0.0;
 #pragma unroll
     for (int q = 0; q < RPT; ++q) {
-        if (q < kq || 4 * q >= N) continue;
+        if (q < kq || G * q >= N) continue;
         if (q == kq) {
             if (g == kg) alpha = a[q];
             if (g > kg) sig = a[q] * a[q];
@@ -91,19 +204,24 @@ __device__ __forceinline__ void reflector(double (&a)[NMAX / 4], int kq, int kg,
             sig = fma(a[q], a[q], sig);
         }
     }
-    sig = quad_sum(sig);
-    alpha = __shfl_sync(0xffffffffu, alpha, (threadIdx.x & 28) + kg);
+    sig = group_sum<G>(sig);
+    alpha = __shfl_sync(0xffffffffu, alpha, (threadIdx.x & (32 - G)) + kg);
     double tau = 0.0, beta = alpha, scal = 0.0;
-    if (mine && sig != 0.0) {
-        const double nrm = sqrt(fma(alpha, alpha, sig));
+    const bool refl = mine && sig != 0.0;
+    if (refl) {
+        const double nrm = fast_sqrt(fma(alpha, alpha, sig));
         beta = (alpha >= 0.0) ? -nrm : nrm;
-        tau = (beta - alpha) / beta;
-        scal = 1.0 / (alpha - beta);
+        // tau = (beta - alpha) / beta in the even lanes, scal = 1 / (alpha - beta) in the odd ones
+        const double d = beta - alpha;
+        const double r = fast_div((g & 1) ? -1.0 : d, (g & 1) ? d : beta);
+        const double o = __shfl_xor_sync(((1u << G) - 1u) << (threadIdx.x & (32 - G)), r, 1);
+        tau = (g & 1) ? o : r;
+        scal = (g & 1) ? r : o;
     }
     if (mine) {
 #pragma unroll
         for (int q = 0; q < RPT; ++q) {
-            const int r = 4 * q + g;
+            const int r = G * q + g;
             if (r < N) A[k * ld + r] = r < k ? a[q] : (r == k ? beta : a[q] * scal);
         }
         if (g == 0) {
@@ -119,8 +237,9 @@ __device__ __forceinline__ void reflector(double (&a)[NMAX / 4], int kq, int kg,
 // (unit diagonal signs). Returns the parity count of reflectors in v.ntriv.
 template <int NMAX>
 __device__ void qr(const double* P, double* A, Vecs<NMAX>& v, int N) {
-    constexpr int ld = Dim<NMAX>::ld, NT = Dim<NMAX>::threads, RPT = NMAX / 4;
-    const int tid = threadIdx.x, j = tid >> 2, g = tid & 3, lane = tid & 31;
+    constexpr int ld = Dim<NMAX>::ld, NT = Dim<NMAX>::threads, RPT = Dim<NMAX>::rpt, G = Dim<NMAX>::G;
+    constexpr int CPW = Dim<NMAX>::cpw;
+    const int tid = threadIdx.x, j = tid / G, g = tid % G, lane = tid & 31;
     double a[RPT];
     if (tid == 0) {
         v.ntriv = 0;
@@ -134,11 +253,11 @@ __device__ void qr(const double* P, double* A, Vecs<NMAX>& v, int N) {
         double s = 0.0;
 #pragma unroll
         for (int q = 0; q < RPT; ++q) {
-            const int r = 4 * q + g;
+            const int r = G * q + g;
             const double p = (j < N && r < N) ? P[j * ld + r] : 0.0;
             s = fma(p, p, s);
         }
-        s = quad_sum(s);
+        s = group_sum<G>(s);
         const double key = s * exp(2.0 * ((j < N ? v.lnd[j] : 0.0) - mx));
         if (j < N && g == 0) v.key[j] = (key >= 0.0) ? key : -1.0;  // NaN sorts last and keeps ranks unique
     }
@@ -156,7 +275,7 @@ __device__ void qr(const double* P, double* A, Vecs<NMAX>& v, int N) {
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < RPT; ++q) {
-        const int r = 4 * q + g;
+        const int r = G * q + g;
         a[q] = (j < N && r < N) ? P[v.perm[j < N ? j : 0] * ld + r] : 0.0;
     }
     if (tid < 32) reflector<NMAX>(a, 0, 0, 0, N, g, j == 0, A, v);
@@ -165,33 +284,33 @@ __device__ void qr(const double* P, double* A, Vecs<NMAX>& v, int N) {
     // (one barrier per step)
 #pragma unroll
     for (int kq = 0; kq < RPT; ++kq) {
-        if (4 * kq >= N) break;
-        for (int kg = 0; kg < 4; ++kg) {
-            const int k = 4 * kq + kg;
+        if (G * kq >= N) break;
+        for (int kg = 0; kg < G; ++kg) {
+            const int k = G * kq + kg;
             if (k + 1 >= N) break;
-            const int jlast = (tid | 31) >> 2;  // last column of the warp
+            const int jlast = (tid | 31) / G;  // last column of the warp
             if (jlast > k) {
                 const double tau = v.tau[k];
                 double vv[RPT], d = 0.0;
 #pragma unroll
                 for (int q = kq; q < RPT; ++q) {
-                    if (4 * q >= N) continue;
-                    const int r = 4 * q + g;
+                    if (G * q >= N) continue;
+                    const int r = G * q + g;
                     vv[q] = (r < N) ? A[k * ld + r] : 0.0;
                     if (q == kq) vv[q] = g == kg ? 1.0 : (g > kg ? vv[q] : 0.0);
                     d = fma(vv[q], a[q], d);
                 }
-                d = quad_sum(d) * tau;
+                d = group_sum<G>(d) * tau;
                 if (j > k) {
 #pragma unroll
                     for (int q = kq; q < RPT; ++q) {
-                        if (4 * q >= N) continue;
+                        if (G * q >= N) continue;
                         a[q] = fma(-d, vv[q], a[q]);
                     }
                 }
-                if ((k + 1) >> 3 == tid >> 5) {  // the warp that holds column k + 1
-                    const int g1 = (kg + 1) & 3;
-                    if (kg < 3) reflector<NMAX>(a, kq, g1, k + 1, N, g, j == k + 1, A, v);
+                if ((k + 1) / CPW == tid >> 5) {  // the warp that holds column k + 1
+                    const int g1 = (kg + 1) % G;
+                    if (kg < G - 1) reflector<NMAX>(a, kq, g1, k + 1, N, g, j == k + 1, A, v);
                     else reflector<NMAX>(a, kq + 1, g1, k + 1, N, g, j == k + 1, A, v);
                 }
             }
@@ -218,70 +337,70 @@ __device__ void qr(const double* P, double* A, Vecs<NMAX>& v, int N) {
     __syncthreads();
 }
 
-// T <- Rt P^T T in place (T row-major, Rt in the upper triangle of A): 4 x 4 entries per thread.
+// T <- Rt P^T T in place (T row-major, Rt in the upper triangle of A): TX x TY entries per thread.
 template <int NMAX>
 __device__ void t_update(const double* A, double* T, const Vecs<NMAX>& v, int N) {
-    constexpr int ld = Dim<NMAX>::ld, TT = NMAX / 4, NTH = Dim<NMAX>::threads;
-    constexpr int PASS = (TT * TT + NTH - 1) / NTH;
-    static_assert(PASS == 1, "one tile per thread");
-    const int ti = threadIdx.x / TT, tj = threadIdx.x % TT;
-    const bool on = threadIdx.x < TT * TT && 4 * ti < N && 4 * tj < N;
-    double acc[4][4];
+    constexpr int ld = Dim<NMAX>::ld, NTH = Dim<NMAX>::threads;
+    constexpr int TX = NMAX * NMAX / NTH >= 16 ? 4 : (NMAX * NMAX / NTH >= 4 ? 2 : 1), TY = NMAX * NMAX / NTH / TX;
+    static_assert(TX * TY * NTH == NMAX * NMAX && TY >= 1, "one tile per thread");
+    constexpr int TT = NMAX / TY;
+    const int i0 = threadIdx.x / TT * TX, j0 = threadIdx.x % TT * TY;
+    const bool on = i0 < N && j0 < N;
+    double acc[TX][TY];
 #pragma unroll
-    for (int x = 0; x < 4; ++x)
+    for (int x = 0; x < TX; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] = 0.0;
+        for (int y = 0; y < TY; ++y) acc[x][y] = 0.0;
     if (on)
-        for (int k = 4 * ti; k < N; ++k) {
-            double a[4], b[4];
-            const double* Tk = T + v.perm[k] * ld + 4 * tj;
+        for (int k = i0; k < N; ++k) {
+            double a[TX], b[TY];
+            const double* Tk = T + v.perm[k] * ld + j0;
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                a[x] = (4 * ti + x <= k) ? A[k * ld + 4 * ti + x] : 0.0;
-                b[x] = Tk[x];
-            }
+            for (int x = 0; x < TX; ++x) a[x] = (i0 + x <= k) ? A[k * ld + i0 + x] : 0.0;
 #pragma unroll
-            for (int x = 0; x < 4; ++x)
+            for (int y = 0; y < TY; ++y) b[y] = Tk[y];
 #pragma unroll
-                for (int y = 0; y < 4; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
+            for (int x = 0; x < TX; ++x)
+#pragma unroll
+                for (int y = 0; y < TY; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
         }
     __syncthreads();
     if (on)
 #pragma unroll
-        for (int x = 0; x < 4; ++x)
+        for (int x = 0; x < TX; ++x)
 #pragma unroll
-            for (int y = 0; y < 4; ++y)
-                if (4 * ti + x < N && 4 * tj + y < N) T[(4 * ti + x) * ld + 4 * tj + y] = acc[x][y];
+            for (int y = 0; y < TY; ++y)
+                if (i0 + x < N && j0 + y < N) T[(i0 + x) * ld + j0 + y] = acc[x][y];
 }
 
-// Q (column-major) from the packed reflectors of A, accumulated backwards; a quad per column, no barriers.
+// Q (column-major) from the packed reflectors of A, accumulated backwards; a group per column, no barriers.
 template <int NMAX>
 __device__ void form_q(const double* A, double* Q, const Vecs<NMAX>& v, int N) {
-    constexpr int ld = Dim<NMAX>::ld, RPT = NMAX / 4;
-    const int tid = threadIdx.x, j = tid >> 2, g = tid & 3;
+    constexpr int ld = Dim<NMAX>::ld, RPT = Dim<NMAX>::rpt, G = Dim<NMAX>::G;
+    const int tid = threadIdx.x, j = tid / G, g = tid % G;
     double x[RPT];
 #pragma unroll
-    for (int q = 0; q < RPT; ++q) x[q] = (4 * q + g == j) ? 1.0 : 0.0;
-    const int jlast = (tid | 31) >> 2;
+    for (int q = 0; q < RPT; ++q) x[q] = (G * q + g == j) ? 1.0 : 0.0;
+    const int jlast = (tid | 31) / G;
 #pragma unroll
     for (int kq = RPT - 1; kq >= 0; --kq) {
-        if (4 * kq >= N) continue;
-        for (int kg = 3; kg >= 0; --kg) {
-            const int k = 4 * kq + kg;
+        if (G * kq >= N) continue;
+        for (int kg = G - 1; kg >= 0; --kg) {
+            const int k = G * kq + kg;
             if (k >= N || k > jlast) continue;  // columns left of k are still unit vectors
             double vv[RPT], d = 0.0;
 #pragma unroll
             for (int q = kq; q < RPT; ++q) {
-                if (4 * q >= N) continue;
-                const int r = 4 * q + g;
+                if (G * q >= N) continue;
+                const int r = G * q + g;
                 vv[q] = (r < N) ? A[k * ld + r] : 0.0;
                 if (q == kq) vv[q] = g == kg ? 1.0 : (g > kg ? vv[q] : 0.0);
                 d = fma(vv[q], x[q], d);
             }
-            d = quad_sum(d) * v.tau[k];
+            d = group_sum<G>(d) * v.tau[k];
 #pragma unroll
             for (int q = kq; q < RPT; ++q) {
-                if (4 * q >= N) continue;
+                if (G * q >= N) continue;
                 x[q] = fma(-d, vv[q], x[q]);
             }
         }
@@ -289,7 +408,7 @@ __device__ void form_q(const double* A, double* Q, const Vecs<NMAX>& v, int N) {
     if (j < N)
 #pragma unroll
         for (int q = 0; q < RPT; ++q)
-            if (4 * q + g < N) Q[j * ld + 4 * q + g] = x[q];
+            if (G * q + g < N) Q[j * ld + G * q + g] = x[q];
 }
 
 // Pivot search and multipliers of column k of M (column-major) by one warp: rows k.. of the column, the chosen row,
@@ -325,7 +444,7 @@ __device__ __forceinline__ void lu_column(double* M, Vecs<NMAX>& v, int k, int N
     }
     if (bi >= N) bi = k;  // no comparable entry (NaN column): no interchange
     double pval = col[bi], top = col[k];
-    const double rinv = (pval != 0.0) ? 1.0 / pval : 0.0;
+    const double rinv = (pval != 0.0) ? fast_div(1.0, pval) : 0.0;
     __syncwarp();
 #pragma unroll
     for (int t = 0; t < R; ++t) {
@@ -370,30 +489,12 @@ __device__ void lu(double* M, Vecs<NMAX>& v, int N) {
             const int r = lane + 32 * t;
             l[t] = (r > k && r < N) ? v.lbuf[k & 1][r] : 0.0;
         }
-        // the column of the next step first
+        // the column of the next step first: its warp factors it while the others still update
         const int next = k + 1;
-        const int start = next < N && next % NW == warp ? next : -1;
-        for (int it = -1, j = warp; j < N || it < 0; ++it) {
-            int c;
-            if (it < 0) {
-                if (start < 0) continue;
-                c = start;
-            } else {
-                c = j;
-                j += NW;
-                if (c == start || c == k) continue;
-            }
-            double* col = M + c * ld;
+        if (next < N && next % NW == warp) {
+            double* col = M + next * ld;
             const double u = col[p], t0 = col[k];
             __syncwarp();
-            if (c < k) {  // earlier columns only take the interchange
-                if (lane == 0 && p != k) {
-                    col[k] = u;
-                    col[p] = t0;
-                }
-                __syncwarp();
-                continue;
-            }
 #pragma unroll
             for (int t = 0; t < R; ++t) {
                 const int r = lane + 32 * t;
@@ -402,44 +503,74 @@ __device__ void lu(double* M, Vecs<NMAX>& v, int N) {
                 col[r] = r == k ? u : fma(-l[t], u, e);
             }
             __syncwarp();
-            if (c == start) lu_column<NMAX>(M, v, next, N, lane);
+            lu_column<NMAX>(M, v, next, N, lane);
+        }
+        // the warp's other columns, two at a time (independent loads); earlier ones only take the interchange
+        for (int c0 = warp; c0 < N; c0 += 2 * NW) {
+            double u[2], e[2][R];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = c0 + h * NW;
+                if (c >= N || c == k || c == next) continue;
+                const double* col = M + c * ld;
+                u[h] = col[p];
+                const double t0 = col[k];
+#pragma unroll
+                for (int t = 0; t < R; ++t) {
+                    const int r = lane + 32 * t;
+                    e[h][t] = (r < k || r >= N) ? 0.0 : (r == p ? t0 : col[r]);
+                }
+            }
+            __syncwarp();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = c0 + h * NW;
+                if (c >= N || c == k || c == next) continue;
+                double* col = M + c * ld;
+#pragma unroll
+                for (int t = 0; t < R; ++t) {
+                    const int r = lane + 32 * t;
+                    if (r < k || r >= N) continue;
+                    col[r] = r == k ? u[h] : (c < k ? e[h][t] : fma(-l[t], u[h], e[h][t]));
+                }
+            }
         }
         __syncthreads();
     }
 }
 
-// Right-hand side column j in quad registers (row 4 q + g in x[q]): x <- U'^-1 L^-1 x with the factors in M and
+// Right-hand side column j in group registers (row G q + g in x[q]): x <- U'^-1 L^-1 x with the factors in M and
 // the reciprocal pivots rd.
 template <int NMAX>
-__device__ __forceinline__ void lu_solve(const double* M, const double* rd, double (&x)[NMAX / 4], int N) {
-    constexpr int ld = Dim<NMAX>::ld, RPT = NMAX / 4;
-    const int g = threadIdx.x & 3, q0 = threadIdx.x & 28;
+__device__ __forceinline__ void lu_solve(const double* M, const double* rd, double (&x)[Dim<NMAX>::rpt], int N) {
+    constexpr int ld = Dim<NMAX>::ld, RPT = Dim<NMAX>::rpt, G = Dim<NMAX>::G;
+    const int g = threadIdx.x % G, q0 = threadIdx.x & (32 - G);
 #pragma unroll
     for (int kq = 0; kq < RPT; ++kq) {
-        if (4 * kq >= N) break;
-        for (int kg = 0; kg < 4; ++kg) {
-            const int k = 4 * kq + kg;
+        if (G * kq >= N) break;
+        for (int kg = 0; kg < G; ++kg) {
+            const int k = G * kq + kg;
             if (k >= N) break;
             const double xk = __shfl_sync(0xffffffffu, x[kq], q0 + kg);
 #pragma unroll
             for (int q = kq; q < RPT; ++q) {
-                const int r = 4 * q + g;
-                if (4 * q >= N) continue;
+                const int r = G * q + g;
+                if (G * q >= N) continue;
                 if (r > k && r < N) x[q] = fma(-M[k * ld + r], xk, x[q]);
             }
         }
     }
 #pragma unroll
     for (int kq = RPT - 1; kq >= 0; --kq) {
-        if (4 * kq >= N) continue;
-        for (int kg = 3; kg >= 0; --kg) {
-            const int k = 4 * kq + kg;
+        if (G * kq >= N) continue;
+        for (int kg = G - 1; kg >= 0; --kg) {
+            const int k = G * kq + kg;
             if (k >= N) continue;
             const double xk = __shfl_sync(0xffffffffu, x[kq], q0 + kg) * rd[k];
             if (g == kg) x[kq] = xk;
 #pragma unroll
             for (int q = 0; q <= kq; ++q) {
-                const int r = 4 * q + g;
+                const int r = G * q + g;
                 if (r < k) x[q] = fma(-M[k * ld + r], xk, x[q]);
             }
         }

@@ -5,6 +5,7 @@
 
 #include <cfloat>
 
+#include "fast_fp64.cuh"
 #include "slmc_internal.cuh"
 
 namespace {
@@ -161,6 +162,7 @@ __device__ __forceinline__ void panel_reflector(double* __restrict__ Vp, int k, 
     constexpr int BPS = BP + 1;
     const double alpha = Vp[k * BPS + c];
     double sig = 0.0;
+#pragma unroll 4
     for (int r = k + 1 + lane; r < N; r += 32) {
         const double v = Vp[r * BPS + c];
         sig = fma(v, v, sig);
@@ -168,11 +170,15 @@ __device__ __forceinline__ void panel_reflector(double* __restrict__ Vp, int k, 
     sig = slmc::warp_allsum(sig);
     double tau = 0.0, beta = alpha, scal = 0.0;
     if (sig != 0.0) {
-        const double nrm = sqrt(fma(alpha, alpha, sig));
+        const double nrm = slmc::fast_sqrt(fma(alpha, alpha, sig));
         beta = (alpha >= 0.0) ? -nrm : nrm;
-        tau = (beta - alpha) / beta;
-        scal = 1.0 / (alpha - beta);
+        // tau = (beta - alpha) / beta in the even lanes, scal = 1 / (alpha - beta) in the odd ones
+        const double d = beta - alpha;
+        const double q = slmc::fast_div((lane & 1) ? -1.0 : d, (lane & 1) ? d : beta);
+        tau = __shfl_sync(0xffffffffu, q, 0);
+        scal = __shfl_sync(0xffffffffu, q, 1);
     }
+#pragma unroll 4
     for (int r = k + 1 + lane; r < N; r += 32) Vp[r * BPS + c] *= scal;
     if (lane == 0) {
         s_tau[c] = tau;
@@ -194,6 +200,8 @@ __device__ __forceinline__ void panel_apply(double* __restrict__ Vp, int k, int 
     double d[NC];
 #pragma unroll
     for (int j = 0; j < NC; ++j) d[j] = (lane == 0) ? Vp[k * BPS + cols[j]] : 0.0;
+    // (unrolled: the loads of the next rows are in flight behind the FMAs of these)
+#pragma unroll NC <= 2 ? 4 : 2
     for (int r = k + 1 + lane; r < N; r += 32) {
         const double v = Vp[r * BPS + c];
 #pragma unroll
@@ -212,7 +220,22 @@ __device__ __forceinline__ void panel_apply(double* __restrict__ Vp, int k, int 
 #pragma unroll
         for (int j = 0; j < NC; ++j) Vp[k * BPS + cols[j]] -= d[j];
     }
-    for (int r = k + 1 + lane; r < N; r += 32) {
+    constexpr int U = NC <= 2 ? 4 : 2;  // rows in flight (loaded together: the stores may alias the next loads)
+    int r = k + 1 + lane;
+    for (; r + 32 * (U - 1) < N; r += 32 * U) {
+        double v[U], a[U][NC];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            v[u] = Vp[(r + 32 * u) * BPS + c];
+#pragma unroll
+            for (int j = 0; j < NC; ++j) a[u][j] = Vp[(r + 32 * u) * BPS + cols[j]];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int j = 0; j < NC; ++j) Vp[(r + 32 * u) * BPS + cols[j]] = fma(-d[j], v[u], a[u][j]);
+    }
+    for (; r < N; r += 32) {
         const double v = Vp[r * BPS + c];
 #pragma unroll
         for (int j = 0; j < NC; ++j) Vp[r * BPS + cols[j]] = fma(-d[j], v, Vp[r * BPS + cols[j]]);

@@ -10,7 +10,7 @@ namespace {
 using namespace slmc::sm;
 
 template <int NMAX, int LMAX>
-__global__ void __launch_bounds__(Dim<NMAX>::threads, NMAX == 16 ? 4 : 2) k_small_logdet(const double* __restrict__ x, const double* __restrict__ kron,
+__global__ void __launch_bounds__(Dim<NMAX>::threads, NMAX == 16 ? 4 : (NMAX == 32 ? 2 : 1)) k_small_logdet(const double* __restrict__ x, const double* __restrict__ kron,
                                                            double* __restrict__ lndet, int* __restrict__ sign,
                                                            double* __restrict__ Gout, unsigned int* __restrict__ err, int N,
                                                            int Lx, int Ly, int L, int n_s, double dtlam, double emu) {

@@ -28,7 +28,7 @@ namespace sm {
 
 template <int NMAX>
 struct Dim {
-    static constexpr int G = NMAX <= 32 ? 8 : 4;  // lanes per column
+    static constexpr int G = 8;  // lanes per column
     static constexpr int ld = NMAX + 1, mat = NMAX * ld, threads = G * NMAX, rpt = NMAX / G, cpw = 32 / G;
 };
 constexpr int kScMax = 16;  // slices whose scales are formed together

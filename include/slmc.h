@@ -321,7 +321,7 @@ SLMC_API int slmc_set_qr_path(slmc_ctx* ctx, int path);
 
 /* Thread layout of the FP32 slice kernel: 1: one column group of 256 row threads; 2: two such
  * groups (512 threads); 4 (N <= 256): four column groups of 64 row threads, each thread up to
- * 4 rows x 8 columns. 0 (default) selects 4 for N <= 256 and 1 above. The 256-thread layouts (about 104 KB of shared memory
+ * 4 rows x 8 columns. 0 (default) selects 4 for N <= 256, two groups of N / 3 row threads up to 768 and 1 above. The 256-thread layouts (about 104 KB of shared memory
  * at N = 256) leave room on the SM for a CTA of another sub-batch's FP64 stabilisation, so the
  * FP32 and FP64 pipes work at the same time. Results do not depend on it. */
 SLMC_API int slmc_set_slice_groups(slmc_ctx* ctx, int groups);

@@ -167,11 +167,14 @@ __device__ __forceinline__ void stage_F(float* Fs, const float* __restrict__ Fhi
     }
 }
 
-template <int RPT, int NBT, int KB, int NCG, int TR>
-__global__ void __launch_bounds__(TR * NCG, (TR * NCG == 256 ? 2 : 1)) k_slice_f32(const float* __restrict__ Fhi, const int* __restrict__ lo_kidx,
+// TRC row threads per column group, or tr of them (at most 256) for TRC = 0.
+template <int RPT, int NBT, int KB, int NCG, int TRC>
+__global__ void __launch_bounds__((TRC ? TRC : 256) * NCG, (TRC * NCG == 256 ? 2 : 1)) k_slice_f32(const float* __restrict__ Fhi, const int* __restrict__ lo_kidx,
                                                    const float* __restrict__ lo_val, int S,
                                                    const float* __restrict__ U, double* __restrict__ out,
-                                                   const float* __restrict__ sc32, int N, int L, int l0, int nsl) {
+                                                   const float* __restrict__ sc32, int N, int L, int l0, int nsl,
+                                                   int tr) {
+    const int TR = TRC ? TRC : tr;
     constexpr int NB = NCG * NBT;  // NCG column groups of NBT columns; thread = (row, group)
     constexpr int NBP = NB + 4;    // padded row stride of the panel
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -204,13 +207,15 @@ __global__ void __launch_bounds__(TR * NCG, (TR * NCG == 256 ? 2 : 1)) k_slice_f
             cp_async_wait1();
             __syncthreads();
             const int k0 = b * KB, nk = min(KB, N - k0);
-            const float* Fh = Fcur;
-            for (int kk = 0; kk < nk; ++kk) {
-                const int k = k0 + kk;
+            const float* Fr[RPT];  // rows beyond N read the last one (their sums are not stored)
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) Fr[r] = Fcur + min(tid + TR * r, N - 1);
+            const float* Pk = Pin + (size_t)k0 * NBP + cg;
+            auto step = [&](int kk) {
                 float pv[NBT];
 #pragma unroll
                 for (int c = 0; c < NBT; c += 4) {
-                    const float4 q = *reinterpret_cast<const float4*>(Pin + k * NBP + cg + c);
+                    const float4 q = *reinterpret_cast<const float4*>(Pk + kk * NBP + c);
                     pv[c] = q.x;
                     pv[c + 1] = q.y;
                     pv[c + 2] = q.z;
@@ -218,11 +223,16 @@ __global__ void __launch_bounds__(TR * NCG, (TR * NCG == 256 ? 2 : 1)) k_slice_f
                 }
 #pragma unroll
                 for (int r = 0; r < RPT; ++r) {
-                    const int i = tid + TR * r;
-                    const float ah = (i < N) ? Fh[kk * N + i] : 0.f;
+                    const float ah = Fr[r][kk * N];
 #pragma unroll
                     for (int c = 0; c < NBT; ++c) blk[r][c] = fmaf(ah, pv[c], blk[r][c]);
                 }
+            };
+            if (nk == KB) {
+#pragma unroll 8
+                for (int kk = 0; kk < KB; ++kk) step(kk);
+            } else {
+                for (int kk = 0; kk < nk; ++kk) step(kk);
             }
             if (((b + 1) * KB) % kTS == 0 || b + 1 == nblk) {  // blocks of kTS products per TwoSum
 #pragma unroll
@@ -291,18 +301,18 @@ __global__ void __launch_bounds__(TR * NCG, (TR * NCG == 256 ? 2 : 1)) k_slice_f
 
 constexpr size_t kSmemBudget = 220 * 1024;
 
-template <int RPT, int NBT, int KB, int NCG, int TR>
-cudaError_t launch_slice_f32_kb(const slmc_ctx* c, int nf, int l0, int nsl, cudaStream_t s) {
+template <int RPT, int NBT, int KB, int NCG, int TRC>
+cudaError_t launch_slice_f32_kb(const slmc_ctx* c, int nf, int l0, int nsl, cudaStream_t s, int tr = TRC) {
     const int N = c->N;
     constexpr int NBP = NCG * NBT + 4;
     const size_t smem = ((size_t)2 * N * NBP + (size_t)2 * KB * N) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k_slice_f32<RPT, NBT, KB, NCG, TR>,
+    cudaError_t e = cudaFuncSetAttribute(k_slice_f32<RPT, NBT, KB, NCG, TRC>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     constexpr int NB = NCG * NBT;
     dim3 grid((N + NB - 1) / NB, nf);
-    k_slice_f32<RPT, NBT, KB, NCG, TR><<<grid, TR * NCG, smem, s>>>(c->F32, c->lo_kidx, c->lo_val, c->lo_S, c->U32, c->Y, c->sc32, N,
-                                                      c->L, l0, nsl);
+    k_slice_f32<RPT, NBT, KB, NCG, TRC><<<grid, tr * NCG, smem, s>>>(c->F32, c->lo_kidx, c->lo_val, c->lo_S, c->U32, c->Y,
+                                                                     c->sc32, N, c->L, l0, nsl, tr);
     return cudaGetLastError();
 }
 
@@ -319,9 +329,23 @@ cudaError_t launch_slice_f32_g(const slmc_ctx* c, int nf, int l0, int nsl, cudaS
     return launch_slice_f32_kb<RPT, NBT, 8, NCG, TR>(c, nf, l0, nsl, s);
 }
 
+// Default for 256 < N <= 768: two column groups of 8, three rows per thread, the rows spread evenly over a multiple
+// of 32 row threads. One group of 256 row threads padded N = 576 to 768 rows and read F (1.3 MB, from L2) once per 8
+// columns; this reads it once per 16 and pads nothing at 576: 24x24, L = 240, 32 fields 188 -> 124 ms in the slice
+// products of an evaluation (with the unrolled inner loop above, 149 before it). Same sums per entry, same bits.
+cudaError_t launch_slice_f32_wide(const slmc_ctx* c, int nf, int l0, int nsl, cudaStream_t s) {
+    const int tr = (c->N + 95) / 96 * 32;
+    const size_t budget = tr * 2 <= 256 ? kSmemBudget / 2 : kSmemBudget;
+    const size_t panel = (size_t)2 * c->N * 20 * sizeof(float), per_row = (size_t)2 * c->N * sizeof(float);
+    if (panel + 32 * per_row <= budget) return launch_slice_f32_kb<3, 8, 32, 2, 0>(c, nf, l0, nsl, s, tr);
+    if (panel + 16 * per_row <= budget) return launch_slice_f32_kb<3, 8, 16, 2, 0>(c, nf, l0, nsl, s, tr);
+    return launch_slice_f32_kb<3, 8, 8, 2, 0>(c, nf, l0, nsl, s, tr);
+}
+
 template <int RPT, int NBT>
 cudaError_t launch_slice_f32(const slmc_ctx* c, const double* x, int nf, int l0, int nsl, cudaStream_t s) {
     (void)x;
+    if (c->tune_slice_groups == 0 && c->N > 256 && c->N <= 768) return launch_slice_f32_wide(c, nf, l0, nsl, s);
     if (c->tune_slice_groups == 2) return launch_slice_f32_g<RPT, NBT, 2>(c, nf, l0, nsl, s);
     if ((c->tune_slice_groups == 4 || c->tune_slice_groups == 0) && c->N <= 256) {
         // default for N <= 256: 64 row threads x 4 column groups of 8, up to 4 rows each

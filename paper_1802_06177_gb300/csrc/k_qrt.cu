@@ -454,27 +454,33 @@ __global__ void __launch_bounds__(kQT, 2)
     } else if (warp == 9) {
         if (lane == 0) {
             bool ok = true;
+            Ring ring;
+            const uint64_t da0 = smem_desc_sw128(aring), db0 = smem_desc_sw128(bbuf);
+            const uint32_t full0 = smem_u32(bar_full), empty0 = smem_u32(bar_empty);
             for (int u = 0; u < nkc && ok; ++u) {
                 const int bs = u & 1, seg = u / kSegChunks;
                 if (!mbar_wait(smem_u32(&bar_bfull[bs]), (u >> 1) & 1, err) || abort_sh) {
                     ok = false;
                     break;
                 }
-                for (int a = 0; a < kS && ok; ++a) {
-                    const int q = u * kS + a, slot = q % kRing;
-                    if (!mbar_wait(smem_u32(&bar_full[slot]), (q / kRing) & 1, err) || abort_sh) {
+                const uint64_t db = db0 + (uint64_t)bs * desc_step(kChunkB);
+                const bool first = u == seg * kSegChunks;
+#pragma unroll
+                for (int a = 0; a < kS; ++a) {
+                    if (!ok || !mbar_wait(full0 + 8 * ring.slot, ring.phase, err) || abort_sh) {
                         ok = false;
-                        break;
+                        continue;
                     }
                     tc_fence_after();
+                    const uint64_t da = da0 + (uint64_t)ring.slot * desc_step(kTileA);
                     // slices b = 0 .. 6 - a of V into the levels a .. 6: adjacent operand rows and adjacent
                     // accumulators, so one instruction of N = (7 - a) BP per step of K
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
-                        mma_bf16(tmem + (uint32_t)((seg * kLv + a) * BP), smem_desc_sw128(aring + slot * kTileA + ks * 32),
-                                 smem_desc_sw128(bbuf + bs * kChunkB + ks * 32), idesc_f32acc(1, 128, (kS - a) * BP),
-                                 ((u - seg * kSegChunks) | a | ks) != 0 ? 1u : 0u);
-                    mma_commit(smem_u32(&bar_empty[slot]));
+                        mma_bf16(tmem + (uint32_t)((seg * kLv + a) * BP), da + desc_step(ks * 32), db + desc_step(ks * 32),
+                                 idesc_f32acc(1, 128, (kS - a) * BP), (a | ks) != 0 || !first ? 1u : 0u);
+                    mma_commit(empty0 + 8 * ring.slot);
+                    ring.next(kRing);
                 }
                 if (ok) mma_commit(smem_u32(&bar_bempty[bs]));
             }
@@ -652,17 +658,19 @@ __global__ void __launch_bounds__(kQT, 2)
     } else if (warp == 9) {
         if (lane == 0) {
             bool ok = mbar_wait(smem_u32(&bar_bfull), 0, err);
-            for (int a = 0; a < kS && ok; ++a) {
+            const uint64_t da0 = smem_desc_sw128(aring), db0 = smem_desc_sw128(bbuf);
+#pragma unroll
+            for (int a = 0; a < kS; ++a) {
                 const int slot = a % kRing;
-                if (!mbar_wait(smem_u32(&bar_full[slot]), (a / kRing) & 1, err)) {
+                if (!ok || !mbar_wait(smem_u32(&bar_full[slot]), (a / kRing) & 1, err)) {
                     ok = false;
-                    break;
+                    continue;
                 }
                 tc_fence_after();
 #pragma unroll
                 for (int ks = 0; ks < BP / 16; ++ks)
-                    mma_bf16(tmem + (uint32_t)(a * kNC), smem_desc_sw128(aring + slot * kTileA + ks * 32),
-                             smem_desc_sw128(bbuf + ks * 32), idesc_f32acc(1, 128, (kS - a) * kNC), (a | ks) != 0 ? 1u : 0u);
+                    mma_bf16(tmem + (uint32_t)(a * kNC), da0 + desc_step(slot * kTileA + ks * 32), db0 + desc_step(ks * 32),
+                             idesc_f32acc(1, 128, (kS - a) * kNC), (a | ks) != 0 ? 1u : 0u);
                 mma_commit(smem_u32(&bar_empty[slot]));
             }
             if (ok) mma_commit(smem_u32(&bar_acc));

@@ -133,44 +133,53 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else if (warp == 9) {
         // ---- MMA issuer ----
         if (lane == 0) {
-            int t = 0;
+            Ring ring;
             bool ok = true;
+            const uint64_t da0 = smem_desc_sw128(stg), db0 = smem_desc_sw128(bbuf);
+            const uint32_t full0 = smem_u32(bar_full), empty0 = smem_u32(bar_empty);
             for (int s = 0; s < nsl && ok; ++s) {
                 if (!mbar_wait(smem_u32(&bar_b), s & 1, err) || abort_sh) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                for (int u = 0; u < per_slice && ok; ++u, ++t) {
-                    const int st = t % kStages, kc = u / (MT * kFS), mt = (u / kFS) % MT, fs = u % kFS;
-                    if (!mbar_wait(smem_u32(&bar_full[st]), (t / kStages) & 1, err) || abort_sh) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t a = stg + st * kStageBytes;
-                    // slices j of Y go to the levels fs + j: adjacent accumulators, adjacent operand tiles, so
-                    // one instruction of N = cnt NT columns per step of K (kGroup slices at most)
-                    const int nj = min(kYS, kLevels - fs);
+                for (int kc = 0; kc < nk && ok; ++kc) {
+                    const uint64_t db = db0 + (uint64_t)kc * desc_step(kYS * tileB);
+                    for (int mt = 0; mt < MT && ok; ++mt) {
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) {
-                        const uint64_t ad = smem_desc_sw128(a + ks * 32);
-                        const bool fresh = kc == 0 && ks == 0;  // this slice's first products of the M tile
-                        auto mm = [&](int j, int cnt, uint32_t acc) {
-                            mma_bf16(tmem + (uint32_t)((mt * kLevels + fs + j) * NT), ad,
-                                     smem_desc_sw128(bbuf + (uint32_t)(kc * kYS + j) * tileB + ks * 32),
-                                     kIdesc | ((uint32_t)(cnt * NT >> 3) << 17), acc);
-                        };
-                        if (fresh && fs == 1) {  // level 3 is first written here, levels 1 and 2 by fs = 0
-                            mm(0, 2, 1u);
-                            mm(2, 1, 0u);
-                        } else {
+                        for (int fs = 0; fs < kFS; ++fs) {
+                            if (!ok || !mbar_wait(full0 + 8 * ring.slot, ring.phase, err) || abort_sh) {
+                                ok = false;
+                                continue;
+                            }
+                            tc_fence_after();
+                            const uint64_t da = da0 + (uint64_t)ring.slot * desc_step(kStageBytes);
+                            // slices j of Y go to the levels fs + j: adjacent accumulators, adjacent operand tiles,
+                            // so one instruction of N = cnt NT columns per step of K (kGroup slices at most)
+                            const int nj = kLevels - fs < kYS ? kLevels - fs : kYS;
+                            const uint32_t td = tmem + (uint32_t)((mt * kLevels + fs) * NT);
 #pragma unroll
-                            for (int j = 0; j < kYS; j += kGroup)
-                                if (j < nj) mm(j, min(kGroup, nj - j), fresh && fs == 0 ? 0u : 1u);
+                            for (int ks = 0; ks < 4; ++ks) {
+                                const bool fresh = kc == 0 && ks == 0;  // this slice's first products of the M tile
+                                auto mm = [&](int j, int cnt, uint32_t acc) {
+                                    mma_bf16(td + (uint32_t)(j * NT), da + desc_step(ks * 32),
+                                             db + desc_step(j * tileB + ks * 32), kIdesc | ((uint32_t)(cnt * NT >> 3) << 17),
+                                             acc);
+                                };
+                                if (fs == 1 && fresh) {  // level 3 is first written here, levels 1 and 2 by fs = 0
+                                    mm(0, 2, 1u);
+                                    mm(2, 1, 0u);
+                                } else {
+#pragma unroll
+                                    for (int j = 0; j < kYS; j += kGroup)
+                                        if (j < nj)
+                                            mm(j, kGroup < nj - j ? kGroup : nj - j, fs == 0 && fresh ? 0u : 1u);
+                                }
+                            }
+                            mma_commit(empty0 + 8 * ring.slot);
+                            ring.next(kStages);
                         }
                     }
-                    mma_commit(smem_u32(&bar_empty[st]));
                 }
                 if (ok) mma_commit(smem_u32(&bar_acc));
             }

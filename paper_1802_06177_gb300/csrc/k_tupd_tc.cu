@@ -249,25 +249,30 @@ __global__ void __launch_bounds__(kThreads, 2)
         // ---- MMA issuer: product (a, b) of a K chunk into the accumulator of level a + b ----
         if (lane == 0) {
             bool ok = true;
+            Ring ring;
+            const uint64_t da0 = smem_desc_sw128(aring), db0 = smem_desc_sw128(bbuf);
+            const uint32_t full0 = smem_u32(bar_full), empty0 = smem_u32(bar_empty);
             for (int u = 0; u < nkc && ok; ++u) {
                 const int bs = u & 1;
                 if (!mbar_wait(smem_u32(&bar_bfull[bs]), (u >> 1) & 1, err) || abort_sh) {
                     ok = false;
                     break;
                 }
-                for (int a = 0; a < kS && ok; ++a) {
-                    const int t = u * kS + a, slot = t % kRingA;
-                    if (!mbar_wait(smem_u32(&bar_full[slot]), (t / kRingA) & 1, err) || abort_sh) {
+                const uint64_t db = db0 + (uint64_t)bs * desc_step(kBChunk);
+#pragma unroll
+                for (int a = 0; a < kS; ++a) {
+                    if (!ok || !mbar_wait(full0 + 8 * ring.slot, ring.phase, err) || abort_sh) {
                         ok = false;
-                        break;
+                        continue;
                     }
                     tc_fence_after();
+                    const uint64_t da = da0 + (uint64_t)ring.slot * desc_step(kATile);
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)  // slices b = 0 .. 6 - a into the levels a .. 6, adjacent in both
-                        mma_bf16(tmem + (uint32_t)(a * kNT), smem_desc_sw128(aring + slot * kATile + ks * 32),
-                                 smem_desc_sw128(bbuf + bs * kBChunk + ks * 32), idesc_f32acc(1, 128, (kS - a) * kNT),
-                                 (u | a | ks) != 0 ? 1u : 0u);
-                    mma_commit(smem_u32(&bar_empty[slot]));
+                        mma_bf16(tmem + (uint32_t)(a * kNT), da + desc_step(ks * 32), db + desc_step(ks * 32),
+                                 idesc_f32acc(1, 128, (kS - a) * kNT), (a | ks) != 0 || u != 0 ? 1u : 0u);
+                    mma_commit(empty0 + 8 * ring.slot);
+                    ring.next(kRingA);
                 }
                 if (ok) mma_commit(smem_u32(&bar_bempty[bs]));
             }

@@ -33,6 +33,7 @@ __device__ __forceinline__ bool mbar_try(uint32_t addr, uint32_t parity) {
 
 // Bounded wait on the completion of the mbarrier phase with the given parity.
 __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity, unsigned int* err) {
+    if (mbar_try(addr, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try(addr, parity)) {
         if (clock64() - t0 > kWaitCycles) {
@@ -84,6 +85,24 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
     return d;
 }
 
+// Descriptors of neighbouring operands differ by their byte distance / 16 in the low word. The issuing thread adds
+// constants to a descriptor formed once: building each from its address (and tile indices from a running count by
+// division) took that thread 150 to 230 cycles per instruction, where the tensor core needs 44 (N = 32) to 128
+// (N = 256).
+__host__ __device__ constexpr uint64_t desc_step(uint32_t bytes) { return (uint64_t)(bytes >> 4); }
+
+// Slot and phase parity of a ring of n barriers, advanced one tile at a time.
+struct Ring {
+    int slot = 0;
+    uint32_t phase = 0;
+    __device__ __forceinline__ void next(int n) {
+        if (++slot == n) {
+            slot = 0;
+            phase ^= 1u;
+        }
+    }
+};
+
 // Byte offset of element (row r, k) of a K-major tile with 128-byte rows in the 128-byte
 // swizzle layout (the layout a TMA box with CU_TENSOR_MAP_SWIZZLE_128B writes), for 2-byte
 // elements: 16-byte chunk k/8 of row r sits at chunk position (k/8) ^ (r % 8).
@@ -93,9 +112,9 @@ __device__ __forceinline__ uint32_t sw128_off_b16(int r, int k) {
 
 // The kernels here multiply a slice a of one operand with the slices b of the other into the level a + b. Slices
 // b lie in adjacent rows of shared memory and levels in adjacent accumulator columns, so all b of one a are ONE
-// instruction of N = (number of b) x tile columns: an instruction of N = 32 or 64 takes about as long as one
-// several times wider (28 of N = 32 per step of K became 7 of N = 32 .. 224; 16x16, L = 160, 512 fields:
-// 283 -> 235 ms per evaluation together with the integer epilogues of slice7.cuh).
+// instruction of N = (number of b) x tile columns (28 of N = 32 per step of K became 7 of N = 32 .. 224; 16x16,
+// L = 160, 512 fields: 283 -> 235 ms per evaluation together with the integer epilogues of slice7.cuh). Measured
+// per instruction of M = 128, K = 16, BF16: 44 cycles at N = 32, 48 at 64, 57 at 96, 64 at 128, 95 at 192, 126 at 256.
 //
 // Instruction descriptor of tcgen05.mma kind::f16 / kind::tf32: FP32 accumulator, A and B of
 // format fmt (BF16 = 1, TF32 = 2), both K-major, M x N tile.

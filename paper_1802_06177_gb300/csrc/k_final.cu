@@ -521,6 +521,7 @@ namespace slmc {
 
 namespace {
 cudaError_t final_dispatch(slmc_ctx* c, int nf, double* lndet, int* sign, cudaStream_t s, bool assemble) {
+    if (c->N <= kSmallN) return small_final_lu(c, nf, lndet, sign, s, assemble);
     switch (rows_per_lane_class(c->N)) {
         case 1: return launch_final<1>(c, nf, lndet, sign, s, assemble);
         case 2: return launch_final<2>(c, nf, lndet, sign, s, assemble);
@@ -542,8 +543,11 @@ cudaError_t final_lu(slmc_ctx* c, int nf, double* lndet, int* sign, cudaStream_t
     return final_dispatch(c, nf, lndet, sign, s, false);
 }
 
+int final_logdet_launches(const slmc_ctx* c) { return c->N <= kSmallN ? 1 : 2; }
+
 cudaError_t final_greens(slmc_ctx* c, int nf, double* G, cudaStream_t s) {
     const int N = c->N;
+    if (N <= kSmallN) return small_final_greens(c, nf, G, s);
     const size_t smem = (size_t)N * kGS * sizeof(double) + (size_t)N * (sizeof(double) + sizeof(int));
     if (smem <= 227 * 1024) {  // blocked solve (the column-per-warp kernel below covers larger N)
         cudaError_t e = cudaFuncSetAttribute(k_greens_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -193,8 +193,15 @@ __global__ void __launch_bounds__((TRC ? TRC : 256) * NCG, (TRC * NCG == 256 ? 2
     float* Pout = P1;
     for (int s = 0; s < nsl; ++s) {
         __syncthreads();
-        stage_F(Fs0, Fhi, N, 0, min(KB, N));
+        // with at most two blocks F stays in its two stages for the whole group
+        const bool fresh = s == 0 || nblk > 2;
+        if (fresh) stage_F(Fs0, Fhi, N, 0, min(KB, N));
         cp_async_commit();
+        // the slice's scales, loaded a slice's products ahead of their use (registers allowing)
+        const float* scl = sc32 + ((size_t)f * L + l0 + s) * N;
+        float scr[RPT];
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) scr[r] = RPT <= 2 ? scl[min(tid + TR * r, N - 1)] : 0.f;
         float hi[RPT][NBT], cp[RPT][NBT], blk[RPT][NBT];
 #pragma unroll
         for (int r = 0; r < RPT; ++r)
@@ -202,7 +209,7 @@ __global__ void __launch_bounds__((TRC ? TRC : 256) * NCG, (TRC * NCG == 256 ? 2
             for (int c = 0; c < NBT; ++c) hi[r][c] = cp[r][c] = blk[r][c] = 0.f;
         for (int b = 0; b < nblk; ++b) {
             float* Fcur = (b & 1) ? Fs1 : Fs0;
-            if (b + 1 < nblk) stage_F((b & 1) ? Fs0 : Fs1, Fhi, N, (b + 1) * KB, min(KB, N - (b + 1) * KB));
+            if (b + 1 < nblk && fresh) stage_F((b & 1) ? Fs0 : Fs1, Fhi, N, (b + 1) * KB, min(KB, N - (b + 1) * KB));
             cp_async_commit();
             cp_async_wait1();
             __syncthreads();
@@ -250,6 +257,7 @@ __global__ void __launch_bounds__((TRC ? TRC : 256) * NCG, (TRC * NCG == 256 ? 2
             __syncthreads();  // the stage just read is refilled two blocks later
         }
         // F_lo on its stencil (rows of the panel already in shared memory)
+#pragma unroll RPT <= 2 ? 4 : 1  // the index and panel loads of four displacements in flight (registers allowing)
         for (int q = 0; q < S; ++q) {
             const float v = __ldg(lo_val + q);
 #pragma unroll
@@ -269,12 +277,11 @@ __global__ void __launch_bounds__((TRC ? TRC : 256) * NCG, (TRC * NCG == 256 ? 2
             }
         }
         const bool last = (s == nsl - 1);
-        const float* scl = sc32 + ((size_t)f * L + l0 + s) * N;
 #pragma unroll
         for (int r = 0; r < RPT; ++r) {
             const int i = tid + TR * r;
             if (i >= N) continue;
-            const float sc = scl[i];
+            const float sc = RPT <= 2 ? scr[r] : scl[i];
 #pragma unroll
             for (int c = 0; c < NBT; c += 4) {
                 const float4 y = *reinterpret_cast<const float4*>(Pin + i * NBP + cg + c);

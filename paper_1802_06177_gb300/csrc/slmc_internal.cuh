@@ -246,6 +246,10 @@ cudaError_t eff_chain_sweeps(slmc_ctx* c, double* x, int nf, int chain0, const d
 // Whole FP64 determinant (and G) of small lattices in one launch (k_small.cu).
 constexpr int kSmallN = 64;
 bool small_active(const slmc_ctx* c);
+// the general kernels' final step at N <= kSmallN (c->piv then holds the row order, for small_final_greens)
+cudaError_t small_final_lu(slmc_ctx* c, int nf, double* lndet, int* sign, cudaStream_t s, bool assemble);
+cudaError_t small_final_greens(slmc_ctx* c, int nf, double* G, cudaStream_t s);
+int final_logdet_launches(const slmc_ctx* c);
 cudaError_t small_logdet(slmc_ctx* c, const double* x, int nf, double* lndet, int* sign, double* G, cudaStream_t s);
 cudaError_t slice_group_kron(slmc_ctx* c, const double* x, int nf, int l0, int nsl, bool transposed, cudaStream_t s);
 // G(g0) = [I + B(g0,0) B(L,g0)]^-1 into G (row-major) from the running product in (U, lnD, Ta)

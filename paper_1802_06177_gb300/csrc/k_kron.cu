@@ -13,19 +13,86 @@
 // B(L, g0)^T = B_{g0+1}^T ... B_L^T that the DQMC updates combine with B(g0, 0) to obtain
 // G(g0) without a full chain per recomputation.
 //
-// One CTA owns a panel of NB columns of one field in shared memory for all nsl slices (as
-// the dense panel kernel does); within a slice, one pass transforms the x lines and one the
-// y lines of every column, each thread one line at a time in registers with the folded transforms of
-// circ.cuh. The panel's columns are padded to the odd stride N | 1 and consecutive lanes take the same line of
-// consecutive columns, so neither pass meets a bank conflict (lanes along a column were 16 apart at Lx = 16).
-// Layout: column-major N x N, element (i, j) at j*N + i, site i = ix + Lx iy.
+// One CTA owns a panel of columns of one field in shared memory for all nsl slices (as the dense panel kernel does);
+// within a slice, one pass transforms the x lines and one the y lines of every column. Two forms:
+//   k_slice_oz    longer side 9..16: a warp takes the same line of 16 columns at a time through the tensor-instruction
+//                 transform of oz_line.cuh;
+//   k_slice_kron  other sides: a thread takes a line through the folded FP64 sums of circ.cuh, consecutive lanes the
+//                 same line of consecutive columns.
+// 12x12, L = 120, 256 fields: 65 ms of slice products by direct FP64 sums, 21.0 folded, 17.7 on the tensor
+// instructions (16 lines and 16 outputs fill its tile best at sides 9..16). 18x10, L = 37, 50 fields: 7.8 ms direct, 2.1
+// folded, 3.3 on the tensor instructions (two K steps, three column tiles for a line of 18); 8x8: half of each
+// K step and tile would be padding.
+// Layout: column-major N x N, element (i, j) at j*N + i, site i = ix + Lx iy; the panel's columns at the odd stride
+// N | 1, so neither pass meets a bank conflict.
 #include "circ.cuh"
+#include "oz_line.cuh"
 #include "slmc_internal.cuh"
 
 namespace {
 
 constexpr int kThreads = 128;
-constexpr int kNB = 32;  // columns per CTA
+constexpr int kNBF = 32;  // columns per CTA of the folded form
+
+template <bool kTrans>
+__global__ void __launch_bounds__(kThreads) k_slice_oz(const double* __restrict__ U, double* __restrict__ Y,
+                                                         const double* __restrict__ x,
+                                                         const double* __restrict__ kron, int Lx, int Ly, int L,
+                                                         int l0, int nsl, double dtlam, double emu, int NB) {
+    extern __shared__ __align__(16) double sm[];
+    const int N = Lx * Ly, ld = N | 1;
+    uint2* fx = reinterpret_cast<uint2*>(sm);  // digit fragments of E_x, E_y
+    uint2* fy = fx + slmc::oz::frag_bytes(Lx) / 8;
+    double* P = reinterpret_cast<double*>(fy + slmc::oz::frag_bytes(Ly) / 8);  // [NB][ld] panel, column-major
+    double* sc = P + NB * ld;                                                  // [N] e^{dtau mu} s_l
+    const int f = blockIdx.y, j0 = blockIdx.x * NB, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nb = min(NB, N - j0), groups = (nb + 15) / 16;
+    const size_t NN = (size_t)N * N;
+    const double* Uf = U + f * NN + (size_t)j0 * N;
+    const int ex = slmc::oz::build(fx, kron, Lx, tid, kThreads);
+    const int ey = slmc::oz::build(fy, kron + 2 * slmc::kKronTab, Ly, tid, kThreads);
+    for (int jj = warp; jj < nb; jj += kThreads / 32)
+        for (int i = lane; i < N; i += 32) P[jj * ld + i] = Uf[(size_t)jj * N + i];
+    const double* xf = x + (size_t)f * N * L;
+    for (int step = 0; step < nsl; ++step) {
+        const int c = kTrans ? l0 + nsl - 1 - step : l0 + step;  // field column of the slice
+        for (int i = tid; i < N; i += kThreads) sc[i] = exp(-dtlam * xf[(size_t)i * L + c]) * emu;
+        __syncthreads();
+        // pass 0: x lines (contiguous; the transposed slice scales its input); pass 1: y lines (stride Lx; the
+        // plain slice scales its output)
+        for (int pass = 0; pass < 2; ++pass) {
+            const int lines = pass ? Lx : Ly, step_l = pass ? 1 : Lx, stride = pass ? Lx : 1;
+            for (int q = warp; q < lines * groups; q += kThreads / 32) {
+                const int li = q / groups, j16 = (q - li * groups) * 16, o = li * step_l;
+                slmc::oz::tile_any(P + j16 * ld + o, ld, min(16, nb - j16), stride, pass ? Ly : Lx, pass ? fy : fx,
+                                      pass ? ey : ex, kTrans && pass == 0 ? sc + o : nullptr,
+                                      !kTrans && pass == 1 ? sc + o : nullptr, stride);
+            }
+            __syncthreads();
+        }
+    }
+    double* Yf = Y + f * NN + (size_t)j0 * N;
+    for (int jj = warp; jj < nb; jj += kThreads / 32)
+        for (int i = lane; i < N; i += 32) Yf[(size_t)jj * N + i] = P[jj * ld + i];
+}
+
+template <bool kTrans>
+cudaError_t launch_oz(slmc_ctx* c, const double* x, int nf, int l0, int nsl, cudaStream_t s) {
+    const int N = c->N;
+    // columns per CTA: the widest of 64, 48, 32 that pads N least (each CTA forms the slice's scales again) and leaves
+    // room for two CTAs per SM
+    const size_t fixed = (size_t)slmc::oz::frag_bytes(c->p.Lx) + slmc::oz::frag_bytes(c->p.Ly) + N * sizeof(double);
+    int NB = 32;
+    for (int w = 48; w <= 64; w += 16)
+        if ((N + w - 1) / w * w <= (N + NB - 1) / NB * NB && fixed + (size_t)w * (N | 1) * sizeof(double) <= 112 * 1024) NB = w;
+    const size_t smem = fixed + (size_t)NB * (N | 1) * sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(k_slice_oz<kTrans>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid((N + NB - 1) / NB, nf);
+    k_slice_oz<kTrans><<<grid, kThreads, smem, s>>>(c->U, c->Y, x, c->kron, c->p.Lx, c->p.Ly, c->L, l0, nsl,
+                                                         c->p.dtau * c->p.lambda, exp(c->p.dtau * c->p.mu), NB);
+    return cudaGetLastError();
+}
 
 template <int LMAX, bool kTrans>
 __global__ void __launch_bounds__(kThreads) k_slice_kron(const double* __restrict__ U, double* __restrict__ Y,
@@ -34,12 +101,12 @@ __global__ void __launch_bounds__(kThreads) k_slice_kron(const double* __restric
                                                          int l0, int nsl, double dtlam, double emu) {
     extern __shared__ double sm[];
     const int N = Lx * Ly, ld = N | 1;
-    double* P = sm;                 // [kNB][ld] panel, column-major
-    double* sc = sm + kNB * ld;     // [N] e^{dtau mu} s_l
+    double* P = sm;                 // [kNBF][ld] panel, column-major
+    double* sc = sm + kNBF * ld;     // [N] e^{dtau mu} s_l
     double* cx = sc + N;            // folded coefficients of E_x, E_y
     double* cy = cx + slmc::circ::ncoef(Lx);
-    const int f = blockIdx.y, j0 = blockIdx.x * kNB, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nb = min(kNB, N - j0);
+    const int f = blockIdx.y, j0 = blockIdx.x * kNBF, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nb = min(kNBF, N - j0);
     const size_t NN = (size_t)N * N;
     const double* Uf = U + f * NN + (size_t)j0 * N;
     slmc::circ::build(cx, kron, Lx, tid, kThreads);
@@ -74,11 +141,11 @@ __global__ void __launch_bounds__(kThreads) k_slice_kron(const double* __restric
 template <int LMAX, bool kTrans>
 cudaError_t launch_kron(slmc_ctx* c, const double* x, int nf, int l0, int nsl, cudaStream_t s) {
     const int N = c->N;
-    const size_t smem = ((size_t)kNB * (N | 1) + N + slmc::circ::ncoef(c->p.Lx) + slmc::circ::ncoef(c->p.Ly)) * sizeof(double);
+    const size_t smem = ((size_t)kNBF * (N | 1) + N + slmc::circ::ncoef(c->p.Lx) + slmc::circ::ncoef(c->p.Ly)) * sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_slice_kron<LMAX, kTrans>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    dim3 grid((N + kNB - 1) / kNB, nf);
+    dim3 grid((N + kNBF - 1) / kNBF, nf);
     k_slice_kron<LMAX, kTrans><<<grid, kThreads, smem, s>>>(c->U, c->Y, x, c->kron, c->p.Lx, c->p.Ly, c->L, l0, nsl,
                                                             c->p.dtau * c->p.lambda, exp(c->p.dtau * c->p.mu));
     return cudaGetLastError();
@@ -89,8 +156,7 @@ template <bool kTrans>
 cudaError_t dispatch_kron(slmc_ctx* c, const double* x, int nf, int l0, int nsl, cudaStream_t s) {
     const int lm = c->p.Lx > c->p.Ly ? c->p.Lx : c->p.Ly;
     if (lm <= 8) return launch_kron<8, kTrans>(c, x, nf, l0, nsl, s);
-    if (lm <= 12) return launch_kron<12, kTrans>(c, x, nf, l0, nsl, s);
-    if (lm <= 16) return launch_kron<16, kTrans>(c, x, nf, l0, nsl, s);
+    if (lm <= slmc::oz::kMaxLine) return launch_oz<kTrans>(c, x, nf, l0, nsl, s);
     return launch_kron<32, kTrans>(c, x, nf, l0, nsl, s);
 }
 

@@ -260,7 +260,8 @@ SLMC_API int slmc_set_tuning(slmc_ctx* ctx, int qr_panel, int slice_cols);
 
 /* Number of sub-batches (1..4) a determinant batch of at least 32 fields per sub-batch is
  * split into; each runs on its own forked stream so that the kernels of one fill the SMs
- * the others leave idle (default 3; 1 = no split). Results do not depend on it. Contexts
+ * the others leave idle (default 3, and no split for N <= 64 while there is at most one field per SM, unless this
+ * call was made; 1 = no split). Results do not depend on it. Contexts
  * created with max_fields < 64 have no forked streams (SLMC_ERR_UNSUPPORTED for n > 1). */
 SLMC_API int slmc_set_sub_batches(slmc_ctx* ctx, int n);
 

@@ -15,20 +15,22 @@
 //  * exp(-dtau K) of the periodic square lattice factorises exactly into
 //    e^{dtau mu} (E_x kron E_y), E_x and E_y symmetric circulant (the hopping along x and
 //    along y commute); the mu factors of B_l and B_l^-1 cancel, and the wrap becomes four
-//    in-place circulant transforms along the lines of G: 2 N^2 (Lx + Ly) FMAs instead of
-//    the 2 N^3 of two dense products;
-//  * G stays in shared memory when it fits (N <= 160), else in global memory (L2-resident). There the
-//    accepted moves of a slice are delayed in batches of up to 32 (Ad, Bd in shared memory, with the
-//    running diagonal of G for the decisions; the batch size is what the shared memory left holds):
-//    each new move needs only the current column and row of G, and the batch is added to G in one
-//    register-tiled pass. Every entry is formed by the same FMA chain in the same order as immediate
-//    rank-1 updates, so the results are bit-identical, for one read and write of G per batch
-//    instead of per move;
+//    in-place circulant transforms along the lines of G, folded by the factor's symmetry
+//    (circ.cuh): about N^2 (Lx + Ly) FP64 operations instead of the 4 N^3 of two dense products;
+//  * G stays in shared memory when it fits (N <= 160), else in global memory (L2-resident). For N > 64 the
+//    accepted moves of a slice are delayed in batches (Ad, Bd in shared memory, with the running diagonal of G for
+//    the decisions): each new move needs only the current column and row of G, and the batch is added to G in one
+//    pass. With G in shared memory a batch is 16 moves, one K step of the tensor-instruction update of oz_line.cuh
+//    (each entry's sum of 16 products rounded once, 56-bit digits): the N^2 FMAs per move were most of the kernel
+//    (40 slices, 128 chains, immediate / batched: 12x12 34.2 / 23.8 ms, 10x10 16.7 / 12.8, 9x8 8.6 / 7.9, 8x8 5.6 /
+//    6.0, where moves stay immediate). With G in global memory it is up to 32 moves, added by FMAs in the order of
+//    immediate updates (the same bits), for one read and write of G per batch instead of per move;
 //  * the proposal, Delta_ii, exp(d ln w_bose) and both uniforms of every site of a slice are
 //    computed in parallel before the slice's sites are visited; each thread then takes the
 //    site's decision itself (u < R^2 exp(d ln w_bose), the same test as
 //    ln(R^2) + d ln w_bose compared with ln u up to rounding), so a rejected move costs no
-//    barrier and an accepted one costs the N^2 FMAs of the rank-1 update and two barriers.
+//    barrier and an accepted one costs two barriers and its rank-1 update, at once or as its
+//    share of a batch.
 // Sites of a slice are visited in order; the proposal x' = x + U[-Delta, Delta] and the
 // acceptance uniform come from Philox counter (i L + l - 1, sweep, chain, 3). The new field is
 // rounded step by step as in the oracle, so accepted moves leave identical fields.
@@ -37,6 +39,7 @@
 // full weights (computed by the determinant path); the site and the uniform come from Philox
 // counter (k, sweep, chain, 4).
 #include "circ.cuh"
+#include "oz_line.cuh"
 #include "slmc_internal.cuh"
 
 #include <algorithm>
@@ -192,7 +195,8 @@ __global__ void __launch_bounds__(kThreads) k_dqmc_slices(double* __restrict__ x
                 }
                 __syncthreads();
                 if (++cnt == kd) {
-                    dqmc_flush(G, Ad, Bd, cnt, N, lane, warp);
+                    if (g_in_smem) slmc::oz::rank_update(G, ldg, Ad, Bd, cnt, N, warp, kThreads / 32);
+                    else dqmc_flush(G, Ad, Bd, cnt, N, lane, warp);
                     cnt = 0;
                     __syncthreads();
                 }
@@ -221,7 +225,10 @@ __global__ void __launch_bounds__(kThreads) k_dqmc_slices(double* __restrict__ x
             }
             __syncthreads();
         }
-        if (cnt > 0) dqmc_flush(G, Ad, Bd, cnt, N, lane, warp);  // the slice's last batch
+        if (cnt > 0) {  // the slice's last batch
+            if (g_in_smem) slmc::oz::rank_update(G, ldg, Ad, Bd, cnt, N, warp, kThreads / 32);
+            else dqmc_flush(G, Ad, Bd, cnt, N, lane, warp);
+        }
         __syncthreads();  // rejected sites take no barrier: the next slice's tables wait for all threads here
     }
     if (tid == 0 && n_acc) n_acc[f] += (unsigned long long)accepted;
@@ -370,6 +377,7 @@ size_t dqmc_smem_bytes(int N, int ncoef, bool g_in_smem, int kd = 0) {
 }
 
 constexpr int kDelayMax = 32;  // accepted moves per delayed batch (G in global memory)
+constexpr int kDelaySmem = 16, kDelayMinN = 65;  // the same with G in shared memory
 
 bool dqmc_supported(const slmc_ctx* c) { return c->L >= 2 && c->kron != nullptr; }
 
@@ -382,11 +390,15 @@ cudaError_t launch_slices(slmc_ctx* c, double* x, double* G, int nf, int chain0,
     if (e != cudaSuccess) return e;
     const int nc = 2 * (slmc::circ::ncoef(c->p.Lx) + slmc::circ::ncoef(c->p.Ly));
     const bool in_smem = dqmc_smem_bytes(c->N, nc, true) <= (size_t)optin;
-    // G in global memory: batch up to kd accepted moves in shared memory (delayed updates). With G in
-    // shared memory the immediate rank-1 updates were faster (12x12: 463 against 418 chain-sweeps/s
-    // with batches of 16), since there a pass over G costs no L2 traffic.
+    // Batches of up to kd accepted moves (delayed updates). G in shared memory: 16 moves are one K step of the
+    // tensor-instruction update, where there is room for them and N is large enough for the update to outweigh the
+    // batch's bookkeeping (N = 72 gains 8%, N = 64 loses 6%, above); else, and for N > 150, which leaves no room for
+    // the batch, moves are applied at once (batches flushed by FP64 FMAs measured slower than that:
+    // the same FMAs and the columns on top). G in global memory: batches of 32 by FMAs, one pass over G each.
     int kd = 0;
-    if (!in_smem) {
+    if (in_smem) {
+        if (c->N >= kDelayMinN && dqmc_smem_bytes(c->N, nc, true, kDelaySmem) <= (size_t)optin) kd = kDelaySmem;
+    } else {
         kd = kDelayMax;
         while (kd > 1 && dqmc_smem_bytes(c->N, nc, false, kd) > (size_t)optin) kd /= 2;
         if (dqmc_smem_bytes(c->N, nc, false, kd) > (size_t)optin) kd = 0;

@@ -190,6 +190,87 @@ __device__ __forceinline__ void tile(double* g, int rstep, int rows, int stride,
     }
 }
 
+// C (row-major, row stride ldc) += sum_{q < cnt} A_q B_q^T, A_q and B_q the N-vectors at Ad + q N and Bd + q N,
+// cnt <= 16: one K step, 16 x 8 tiles, digits per row of A and per column of B, each entry's sum rounded once and added
+// in FP64: against 64-bit-mantissa arithmetic, the entries of G after a batch are off by 4e-17 (median, relative)
+// where 16 rounded FMAs leave 1.2e-16 (9x8 and 12x12 lattices, L = 40 and 80). By the warps of a CTA (warp of nw); kChunk column tiles share a row tile's digits.
+__device__ __forceinline__ void rank_update(double* C, int ldc, const double* Ad, const double* Bd, int cnt, int N, int warp,
+                                            int nw) {
+    constexpr int kChunk = 6;
+    const int lane = threadIdx.x & 31, r0 = lane >> 2, t2 = 2 * (lane & 3);
+    const int CT = (N + 7) / 8, nch = (CT + kChunk - 1) / kChunk, units = (N + 15) / 16 * nch;
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    for (int unit = warp; unit < units; unit += nw) {
+        const int j0 = unit / nch * 16, c0 = unit % nch * kChunk, c1 = min(CT, c0 + kChunk);
+        uint32_t a[kD][4];
+        int eA[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = j0 + r0 + 8 * h;
+            double v[4];
+            int m = 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = t2 + (u & 1) + 8 * (u >> 1);
+                v[u] = (k < cnt && j < N) ? Ad[k * N + j] : 0.0;
+                m = max(m, __double2hiint(v[u]) & 0x7fffffff);
+            }
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+            eA[h] = exponent_of_hi(m);
+            float q[4][kD];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) digits(v[u], eA[h], q[u]);
+#pragma unroll
+            for (int s = 0; s < kD; ++s) {
+                a[s][h] = pack(q[0][s], q[1][s]);
+                a[s][2 + h] = pack(q[2][s], q[3][s]);
+            }
+        }
+#pragma unroll 1
+        for (int ct = c0; ct < c1; ++ct) {
+            const int col = 8 * ct + r0;
+            double v[4];
+            int m = 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = t2 + (u & 1) + 8 * (u >> 1);
+                v[u] = (k < cnt && col < N) ? Bd[k * N + col] : 0.0;
+                m = max(m, __double2hiint(v[u]) & 0x7fffffff);
+            }
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+            const int eB = exponent_of_hi(m);
+            float c[kD][4];
+#pragma unroll
+            for (int l = 0; l < kD; ++l)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) c[l][u] = 0.f;
+            {
+                float q[4][kD];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) digits(v[u], eB, q[u]);
+#pragma unroll
+                for (int b = 0; b < kD; ++b) {
+                    const uint32_t f0 = pack(q[0][b], q[1][b]), f1 = pack(q[2][b], q[3][b]);
+#pragma unroll
+                    for (int s = 0; s + b < kD; ++s) mma(c[s + b], a[s], f0, f1);
+                }
+            }
+            const int eC[2] = {__shfl_sync(0xffffffffu, eB, 4 * t2), __shfl_sync(0xffffffffu, eB, 4 * t2 + 4)};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int m2 = 8 * ct + t2 + (u & 1), j = j0 + r0 + 8 * (u >> 1), e1 = eA[u >> 1], e2 = eC[u & 1];
+                if (m2 >= N || j >= N) continue;
+                float w[kD];
+#pragma unroll
+                for (int l = 0; l < kD; ++l) w[l] = c[l][u];
+                C[j * ldc + m2] += (e1 == 1024 || e2 == 1024) ? nan : value(w, e1 + e2 - 61);
+            }
+        }
+    }
+}
+
 // Length n <= kMaxLine at run time; frag built for that n.
 __device__ __forceinline__ void tile_any(double* g, int rstep, int rows, int stride, int n, const uint2* __restrict__ frag,
                                          int eB, const double* in_sc, const double* out_sc, int sstep) {

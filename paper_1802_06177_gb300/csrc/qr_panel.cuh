@@ -313,10 +313,10 @@ __device__ __forceinline__ void panel_step(const double* __restrict__ Y, double*
                 panel_reflector<BP>(Vp, k + 1, c + 1, N, lane, s_tau, s_beta, tau_f, s_ntriv);
             }
         } else if (tau != 0.0) {
-            // Columns c0, c0 + cs, ... below nb (warp-uniform count nv <= 5 for NW >= 8). A sub-core issues one FP64
-            // warp instruction per 64 cycles, and warp 0's reflector takes about 65 of them, so the warps that share
-            // its sub-core (4, 8, ..) work only while many columns remain; the 12 workers of NW = 16 (6 of NW = 8)
-            // on the other three sub-cores take the rest.
+            // Columns c0, c0 + cs, ... below nb (warp-uniform count nv <= 5 for NW >= 8). One warp issues
+            // one FP64 instruction per 64 cycles and the SM one per 16 to 19, and warp 0's reflector is about 65 of
+            // them in sequence: the warps 4, 8, .. work only while many columns remain, so that warp 0 has fewer
+            // competitors for the unit; 12 workers of NW = 16 (6 of NW = 8) take the rest.
             const bool all = nb - c - 2 > 12;
             const int w = all ? warp - 1 : warp - 1 - warp / 4;
             const int c0 = (all || (warp & 3) != 0) ? c + 2 + w : nb, cs = all ? NW - 1 : NW - NW / 4;

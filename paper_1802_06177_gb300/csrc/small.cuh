@@ -3,12 +3,11 @@
 // so a determinant is one launch instead of several per slice group, and nothing goes through global memory
 // but the field and the result.
 //
-// What bounds it: for N <= 36 the chain of column steps; for N = 64 the FP64 pipe (two FMAs per clock per SM). A
-// sub-core takes 64 cycles per FP64 warp instruction, however many lanes are active, so the chain is as long as
-// the number of FP64 instructions one warp runs in sequence. Columns are held in registers by groups of G lanes:
+// What bounds it: for N <= 36 the chain of column steps; for N = 64 the FP64 pipe (an SM issues one FP64 warp
+// instruction per 16 to 19 cycles). One warp issues one per 64 cycles, however many lanes are active and however
+// independent they are, so the chain is as long as the number of FP64 instructions one warp runs in sequence. Columns are held in registers by groups of G lanes:
 // thread G j + g owns rows g, g + G, ... of column j, so a dot product is a run of FMAs per thread and log2 G
-// additions across the group (a column per warp would spend five of every nine on the reduction); the warps of a
-// field cover all four sub-cores; square root and divisions are short Newton forms, the two divisions of a
+// additions across the group (a column per warp would spend five of every nine on the reduction); square root and divisions are short Newton forms, the two divisions of a
 // reflector in neighbouring lanes of one instruction stream; and a group's slice scales are exponentiated
 // together before its slices. 64 fields of 4x4, L = 40 with G: 784 us by per-step kernels, 401 us by the first
 // version of this kernel, 326 us with folded transforms, 241 us now.

@@ -268,77 +268,175 @@ struct GemmArgs {
     int nterms;
 };
 
-// C = sum over terms of diag(ra) A diag(sk) B diag(cb), one field per blockIdx.z, a TM x TM
-// tile per CTA (4 x 4 outputs per thread), k-tiles of 16 staged in shared memory.
+// C = sum over terms of diag(ra) A diag(sk) B diag(cb), one field per blockIdx.z, a TM x TM tile per CTA, 16 x 16
+// per warp, on the warp-level tensor instruction.
+//
+// As FP64 FMAs (4 x 4 outputs per thread) these products ran at the FP64 issue limit. Here rows of A and columns of B
+// (with sk) are cut into eight 7-bit digits against the power of two of their largest value (oz_line.cuh); the CTA cuts
+// each 16-column step once into fragments in shared memory, the next step's values already loaded, and the 36 products
+// a + b <= 7 accumulate exactly in FP32 for kSeg steps (a level's sum stays below 2^22), then as integers rounded once
+// to FP64: of 36 MMAs per 16 x 8 x 16 block, two cycles each, instead of 64 FMA warp instructions of 16 to 19 cycles.
+// G of a run of 40 slices (products, LU and solve), FP64 FMAs / digits: 128 chains of 12x12 18.8 / 12.0 ms, 10x10 10.5 /
+// 6.4, 8x8 1.84 / 1.15, 4x4 0.35 / 0.26; 64 of 16x16, L = 20, 22.5 / 13.6. Against 64-bit-mantissa arithmetic (4x4, 9x8 and
+// 12x12, L = 40 and 80), Frobenius norm, FMAs / digits: M 0.9e-16 to 3.8e-16 / 0.4e-16 to 1.1e-16, U_L (..) 0.8e-16 to
+// 3.0e-16 / 0.7e-16 to 2.3e-16, smaller for every field.
 template <int TM, bool kAik, bool kBjk, bool kCrow>
-__global__ void __launch_bounds__((TM / 4) * (TM / 4)) k_gemm64(GemmArgs g, double* __restrict__ C, int N,
-                                                                int sstride) {
-    constexpr int TT = TM / 4, NT = TT * TT, BK = 16;
-    __shared__ __align__(16) double As[BK][TM];
-    __shared__ __align__(16) double Bs[BK][TM];
-    const int f = blockIdx.z, i0 = blockIdx.y * TM, j0 = blockIdx.x * TM;
-    const int tid = threadIdx.x, tx = tid % TT, ty = tid / TT;
+__global__ void __launch_bounds__(TM * TM / 8, TM == 32 ? 3 : 1) k_gemm_oz(GemmArgs g, double* __restrict__ C,
+                                                                                         int N, int sstride) {
+    namespace oz = slmc::oz;
+    constexpr int WT = TM / 16, NW = WT * WT, NT = 32 * NW, kD = oz::kD, kSeg = 6;
+    constexpr int kItems = TM * 16, P = (kItems + NT - 1) / NT;  // pairs (k, k + 1) of A and B in a step, per thread
+    __shared__ uint4 Af[WT][kD][32];
+    __shared__ uint2 Bf[2 * WT][kD][32];
+    __shared__ int hi[2 * TM];  // upper words of the largest |a| of each row and |b| of each column
+    const int f = blockIdx.z, i0 = blockIdx.y * TM, j0 = blockIdx.x * TM, KT = (N + 15) / 16;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wr = warp / WT, wc = warp % WT;
+    const int r0 = lane >> 2, t2 = 2 * (lane & 3);
     const size_t NN = (size_t)N * N;
-    double acc[4][4];
+    double out[2][4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int ct = 0; ct < 2; ++ct)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[r][q] = 0.0;
+        for (int u = 0; u < 4; ++u) out[ct][u] = 0.0;
+#pragma unroll 1
+    for (int t = 0; t < g.nterms; ++t) {
+        const double* A = (t ? g.t[1].A : g.t[0].A) + f * NN;
+        const double* B = (t ? g.t[1].B : g.t[0].B) + f * NN;
+        const double* ra = t ? g.t[1].ra : g.t[0].ra;
+        const double* sk = t ? g.t[1].sk : g.t[0].sk;
+        const double* cb = t ? g.t[1].cb : g.t[0].cb;
+        if (ra) ra += (size_t)f * sstride;
+        if (sk) sk += (size_t)f * sstride;
+        if (cb) cb += (size_t)f * sstride;
+        auto val_a = [&](int r, int k) {
+            const int i = i0 + r;
+            return i < N && k < N ? (kAik ? A[(size_t)i * N + k] : A[(size_t)k * N + i]) : 0.0;
+        };
+        auto val_b = [&](int r, int k) {
+            const int j = j0 + r;
+            double v = j < N && k < N ? (kBjk ? B[(size_t)j * N + k] : B[(size_t)k * N + j]) : 0.0;
+            if (sk && k < N) v *= sk[k];
+            return v;
+        };
+        // item q of a step: pair kp of row r of A (r < TM) or of column r - TM of B, ordered along the operand's
+        // contiguous index
+        auto place = [&](int q, int& r, int& kp) {
+            const bool b = q >= TM * 8;
+            const int p = b ? q - TM * 8 : q;
+            if (b ? kBjk : kAik) {
+                r = p >> 3, kp = p & 7;
+            } else {
+                r = (p >> 5) % (TM / 8) * 8 + (p & 7), kp = (p >> 5) / (TM / 8) * 4 + ((p >> 3) & 3);
+            }
+            if (b) r += TM;
+        };
+        double v[P][2];
+        auto load = [&](int k0) {
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        if (t >= g.nterms) break;
-        const double* A = g.t[t].A + f * NN;
-        const double* B = g.t[t].B + f * NN;
-        const double* ra = g.t[t].ra ? g.t[t].ra + (size_t)f * sstride : nullptr;
-        const double* sk = g.t[t].sk ? g.t[t].sk + (size_t)f * sstride : nullptr;
-        const double* cb = g.t[t].cb ? g.t[t].cb + (size_t)f * sstride : nullptr;
-        for (int k0 = 0; k0 < N; k0 += BK) {
-            for (int q = tid; q < TM * BK; q += NT) {
-                const int ii = kAik ? q / BK : q % TM, kk = kAik ? q % BK : q / TM;
-                const int i = i0 + ii, k = k0 + kk;
-                double v = 0.0;
-                if (i < N && k < N) {
-                    v = kAik ? A[(size_t)i * N + k] : A[(size_t)k * N + i];
-                    if (ra) v *= ra[i];
+            for (int m = 0; m < P; ++m) {
+                const int q = tid + m * NT;
+                int r, kp;
+                place(q, r, kp);
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    v[m][h] = q >= kItems ? 0.0 : r < TM ? val_a(r, k0 + 2 * kp + h) : val_b(r - TM, k0 + 2 * kp + h);
+            }
+        };
+        load(0);
+        __syncthreads();  // the fragments and maxima of the previous term are read
+        for (int r = tid; r < 2 * TM; r += NT) hi[r] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+            auto bits = [&](int r, int k) { return __double2hiint(o ? val_b(r, k) : val_a(r, k)) & 0x7fffffff; };
+            if (o ? kBjk : kAik) {
+                for (int r = warp; r < TM; r += NW) {
+                    int m = 0;
+                    for (int k = lane; k < N; k += 32) m = max(m, bits(r, k));
+                    m = __reduce_max_sync(0xffffffffu, m);
+                    if (lane == 0) hi[o * TM + r] = m;
                 }
-                As[kk][ii] = v;
+            } else {
+                constexpr int KS = NT / TM;  // rows of k per pass
+                const int r = tid % TM;
+                int m = 0;
+                if (tid < KS * TM)
+                    for (int k = tid / TM; k < N; k += KS) m = max(m, bits(r, k));
+                atomicMax(&hi[o * TM + r], m);
             }
-            for (int q = tid; q < TM * BK; q += NT) {
-                const int jj = kBjk ? q / BK : q % TM, kk = kBjk ? q % BK : q / TM;
-                const int j = j0 + jj, k = k0 + kk;
-                double v = 0.0;
-                if (j < N && k < N) {
-                    v = kBjk ? B[(size_t)j * N + k] : B[(size_t)k * N + j];
-                    if (sk) v *= sk[k];
-                    if (cb) v *= cb[j];
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int s0 = 0; s0 < KT; s0 += kSeg) {
+            float c[2][kD][4];
+#pragma unroll
+            for (int ct = 0; ct < 2; ++ct)
+#pragma unroll
+                for (int l = 0; l < kD; ++l)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) c[ct][l][u] = 0.f;
+#pragma unroll 1
+            for (int ks = s0; ks < min(KT, s0 + kSeg); ++ks) {
+#pragma unroll
+                for (int m = 0; m < P; ++m) {
+                    const int q = tid + m * NT;
+                    if (q >= kItems) break;
+                    int r, kp;
+                    place(q, r, kp);
+                    const int e = oz::exponent_of_hi(hi[r]), ln = 4 * (r & 7) + (kp & 3);
+                    float d0[kD], d1[kD];
+                    oz::digits(v[m][0], e, d0);
+                    oz::digits(v[m][1], e, d1);
+                    uint32_t* w = r < TM ? reinterpret_cast<uint32_t*>(&Af[r >> 4][0][ln]) + ((r >> 3) & 1) + 2 * (kp >> 2)
+                                         : reinterpret_cast<uint32_t*>(&Bf[(r - TM) >> 3][0][ln]) + (kp >> 2);
+                    const int step = r < TM ? 128 : 64;
+#pragma unroll
+                    for (int s = 0; s < kD; ++s) w[s * step] = oz::pack(d0[s], d1[s]);
                 }
-                Bs[kk][jj] = v;
+                __syncthreads();
+                if (ks + 1 < KT) load(16 * (ks + 1));
+#pragma unroll
+                for (int ct = 0; ct < 2; ++ct) {
+                    uint2 b[kD];
+#pragma unroll
+                    for (int l = 0; l < kD; ++l) b[l] = Bf[2 * wc + ct][l][lane];
+#pragma unroll
+                    for (int l = 0; l < kD; ++l) {
+                        const uint4 q = Af[wr][l][lane];
+                        const uint32_t a[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                        for (int m = 0; l + m < kD; ++m) oz::mma(c[ct][l + m], a, b[m].x, b[m].y);
+                    }
+                }
+                __syncthreads();
             }
-            __syncthreads();
 #pragma unroll
-            for (int kk = 0; kk < BK; ++kk) {
-                const double2 a01 = *reinterpret_cast<const double2*>(&As[kk][ty * 4]);
-                const double2 a23 = *reinterpret_cast<const double2*>(&As[kk][ty * 4 + 2]);
-                const double2 b01 = *reinterpret_cast<const double2*>(&Bs[kk][tx * 4]);
-                const double2 b23 = *reinterpret_cast<const double2*>(&Bs[kk][tx * 4 + 2]);
-                const double a[4] = {a01.x, a01.y, a23.x, a23.y}, b[4] = {b01.x, b01.y, b23.x, b23.y};
+            for (int ct = 0; ct < 2; ++ct)
 #pragma unroll
-                for (int r = 0; r < 4; ++r)
+                for (int u = 0; u < 4; ++u) {
+                    float w[kD];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) acc[r][q] = fma(a[r], b[q], acc[r][q]);
-            }
-            __syncthreads();
+                    for (int l = 0; l < kD; ++l) w[l] = c[ct][l][u];
+                    const int ea = oz::exponent_of_hi(hi[16 * wr + r0 + 8 * (u >> 1)]);
+                    const int eb = oz::exponent_of_hi(hi[TM + 16 * wc + 8 * ct + t2 + (u & 1)]);
+                    double y = oz::value(w, ea + eb - 61);
+                    // a row or column with a value that is not finite becomes NaN, as its sums would
+                    if (ea == 1024 || eb == 1024) y = __longlong_as_double(0x7ff8000000000000ll);
+                    const int i = min(i0 + 16 * wr + r0 + 8 * (u >> 1), N - 1);
+                    const int j = min(j0 + 16 * wc + 8 * ct + t2 + (u & 1), N - 1);
+                    if (ra) y *= ra[i];
+                    if (cb) y *= cb[j];
+                    out[ct][u] += y;
+                }
         }
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int i = i0 + ty * 4 + r;
+    for (int ct = 0; ct < 2; ++ct)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int j = j0 + tx * 4 + q;
-            if (i < N && j < N) C[f * NN + (kCrow ? (size_t)i * N + j : (size_t)j * N + i)] = acc[r][q];
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + 16 * wr + r0 + 8 * (u >> 1), j = j0 + 16 * wc + 8 * ct + t2 + (u & 1);
+            if (i < N && j < N) C[f * NN + (kCrow ? (size_t)i * N + j : (size_t)j * N + i)] = out[ct][u];
         }
-    }
 }
 
 // S[f] = [D_bR^-1 | D_sR | D_bL^-1 | D_sL], each [N], from the ln D of both products
@@ -358,16 +456,17 @@ __global__ void k_split_scales(const double* __restrict__ lnR, const double* __r
 template <int TM, bool kAik, bool kBjk, bool kCrow>
 cudaError_t launch_gemm(const GemmArgs& g, double* C, int N, int nf, int sstride, cudaStream_t s) {
     dim3 grid((N + TM - 1) / TM, (N + TM - 1) / TM, nf);
-    k_gemm64<TM, kAik, kBjk, kCrow><<<grid, (TM / 4) * (TM / 4), 0, s>>>(g, C, N, sstride);
+    k_gemm_oz<TM, kAik, kBjk, kCrow><<<grid, TM * TM / 8, 0, s>>>(g, C, N, sstride);
     return cudaGetLastError();
 }
 
-// the tile (32, 48 or 64) that pads N least, the larger on ties
+// One tile per field while N fits (32, 48 or 64), else tiles of 32, three CTAs per SM: one CTA's cutting then runs beside
+// another's products (G of the 12x12 run above 12.0 ms with 32, 12.6 with 48, which pads nothing; 16x16 the same with
+// 32 and 64; one tile of 48 or 64 against four of 32: 6x6 0.73 / 0.85 ms, 8x8 1.15 / 1.24).
 template <bool kAik, bool kBjk, bool kCrow>
-cudaError_t gemm64(const GemmArgs& g, double* C, int N, int nf, int sstride, cudaStream_t s) {
-    const int p32 = (N + 31) / 32 * 32, p48 = (N + 47) / 48 * 48, p64 = (N + 63) / 64 * 64;
-    if (p64 <= p48 && p64 <= p32) return launch_gemm<64, kAik, kBjk, kCrow>(g, C, N, nf, sstride, s);
-    if (p48 <= p32) return launch_gemm<48, kAik, kBjk, kCrow>(g, C, N, nf, sstride, s);
+cudaError_t gemm_oz(const GemmArgs& g, double* C, int N, int nf, int sstride, cudaStream_t s) {
+    if (N > 32 && N <= 48) return launch_gemm<48, kAik, kBjk, kCrow>(g, C, N, nf, sstride, s);
+    if (N > 48 && N <= 64) return launch_gemm<64, kAik, kBjk, kCrow>(g, C, N, nf, sstride, s);
     return launch_gemm<32, kAik, kBjk, kCrow>(g, C, N, nf, sstride, s);
 }
 
@@ -430,7 +529,7 @@ cudaError_t dqmc_combine(slmc_ctx* c, const double* Ul, const double* lnDl, cons
     m.nterms = 2;
     m.t[0] = GemmTerm{c->U, Ul, S, nullptr, S + 2 * N};     // D_bR^-1 U_R^T U_L D_bL^-1
     m.t[1] = GemmTerm{c->Ta, Tl, S + N, nullptr, S + 3 * N};  // D_sR T_R T_L^T D_sL
-    e = gemm64<true, true, false>(m, c->Y, N, nf, 4 * N, s);  // M column-major, as the LU expects
+    e = gemm_oz<true, true, false>(m, c->Y, N, nf, 4 * N, s);  // M column-major, as the LU expects
     if (e != cudaSuccess) return e;
     e = final_lu(c, nf, lndet_scratch, sign_scratch, s);
     if (e != cudaSuccess) return e;
@@ -439,7 +538,7 @@ cudaError_t dqmc_combine(slmc_ctx* c, const double* Ul, const double* lnDl, cons
     GemmArgs gg{};
     gg.nterms = 1;
     gg.t[0] = GemmTerm{Ul, c->Tb, nullptr, S + 2 * N, nullptr};  // U_L D_bL^-1 X
-    return gemm64<false, false, true>(gg, G, N, nf, 4 * N, s);
+    return gemm_oz<false, false, true>(gg, G, N, nf, 4 * N, s);
 }
 
 cudaError_t dqmc_slices(slmc_ctx* c, double* x, double* G, int nf, int chain0, int l0, int nsl, uint64_t sweep,

@@ -70,15 +70,15 @@ __device__ __forceinline__ uint32_t pack(float q0, float q1) {
     return __byte_perm(__float_as_uint(q0), __float_as_uint(q1), 0x7632);
 }
 
-// sum_l w_l 128^(7 - l) 2^k from the level sums w_l (|w_l| < 2^21), rounded to nearest. The lowest 8 of its up to 70
-// bits are dropped first (2^-62 of the row's scale).
+// sum_l w_l 128^(7 - l) 2^k from the level sums w_l of at most 96 products per pair of digits (|w_l| < 2^22; the sum
+// then fits 62 bits without its lowest 8, which are rounded off first), rounded to nearest.
 __device__ __forceinline__ double value(const float (&w)[kD], int k) {
     int i[kD];
 #pragma unroll
     for (int l = 0; l < kD; ++l) i[l] = __float_as_int(w[l] + 12582912.f) - 0x4B400000;
     const long long hi = (long long)((i[0] << 7) + i[1]) * 16384 + (long long)((i[2] << 7) + i[3]);
     const long long lo = (long long)((i[4] << 7) + i[5]) * 16384 + (long long)((i[6] << 7) + i[7]);
-    const long long t = (hi << 20) + (lo >> 8);
+    const long long t = (hi << 20) + ((lo + 128) >> 8);
     const unsigned long long m = t < 0 ? (unsigned long long)-t : (unsigned long long)t;
     const int z = __clzll((long long)m);
     const int E = 62 - z + k + 8 + 1023;  // biased exponent - 1; the significand's leading bit adds the 1

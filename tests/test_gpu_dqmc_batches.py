@@ -1,6 +1,7 @@
 """DQMC sweeps where G lies in shared memory, against the oracle field for field: odd numbers of sites (a chain's
 G is then 8- but not 16-byte aligned) and the batched rank-16 updates on the tensor instruction (N > 64: partial
-row and column tiles, several batches and a partial one per slice; N = 160 is the largest in shared memory and leaves no room for them)."""
+row and column tiles, several batches and a partial one per slice; N = 160 is
+the largest G in shared memory and leaves no room for them)."""
 import numpy as np
 import pytest
 import torch

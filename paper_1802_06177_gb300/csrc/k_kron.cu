@@ -49,8 +49,9 @@ __global__ void __launch_bounds__(kThreads) k_slice_oz(const double* __restrict_
     const int nb = min(NB, N - j0), groups = (nb + 15) / 16;
     const size_t NN = (size_t)N * N;
     const double* Uf = U + f * NN + (size_t)j0 * N;
-    const int ex = slmc::oz::build(fx, kron, Lx, tid, kThreads);
-    const int ey = slmc::oz::build(fy, kron + 2 * slmc::kKronTab, Ly, tid, kThreads);
+    int shx, shy;
+    const int ex = slmc::oz::build(fx, kron + 4 * slmc::kKronTab, Lx, tid, kThreads, shx);
+    const int ey = slmc::oz::build(fy, kron + 5 * slmc::kKronTab, Ly, tid, kThreads, shy);
     for (int jj = warp; jj < nb; jj += kThreads / 32)
         for (int i = lane; i < N; i += 32) P[jj * ld + i] = Uf[(size_t)jj * N + i];
     const double* xf = x + (size_t)f * N * L;
@@ -65,7 +66,7 @@ __global__ void __launch_bounds__(kThreads) k_slice_oz(const double* __restrict_
             for (int q = warp; q < lines * groups; q += kThreads / 32) {
                 const int li = q / groups, j16 = (q - li * groups) * 16, o = li * step_l;
                 slmc::oz::tile_any(P + j16 * ld + o, ld, min(16, nb - j16), stride, pass ? Ly : Lx, pass ? fy : fx,
-                                      pass ? ey : ex, kTrans && pass == 0 ? sc + o : nullptr,
+                                      pass ? ey : ex, pass ? shy : shx, kTrans && pass == 0 ? sc + o : nullptr,
                                       !kTrans && pass == 1 ? sc + o : nullptr, stride);
             }
             __syncthreads();

@@ -29,8 +29,8 @@ __host__ __device__ constexpr int frag_bytes(int n) { return ntiles(n) * kD * 32
 
 // The eight digits of v in units of 2^(e - 6 - 7 s), as small integers in FP32 (see slice7.cuh): v is rounded to
 // n 2^(e - 55) (half away from zero) in 32-bit words -- the variable 64-bit shifts and the conversions were most of
-// this function -- and the balanced digits of n are bit fields of n plus 64 at every place below the top.
-__device__ __forceinline__ void digits(double v, int e, float (&q)[kD]) {
+// this function -- and the balanced digits of n are bit fields of n plus 64 at every place below the top. Returns n with its sign.
+__device__ __forceinline__ long long digits(double v, int e, float (&q)[kD]) {
     const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
     const int ex = (int)((h >> 20) & 0x7ffu);
     const uint32_t mh = ex ? (h & 0xfffffu) | 0x100000u : 0u;  // a subnormal counts as zero
@@ -42,7 +42,8 @@ __device__ __forceinline__ void digits(double v, int e, float (&q)[kD]) {
     long long n = (long long)((((unsigned long long)yh << 32) | yl) + 1ull) >> 1;
     const long long sg = (long long)((int)h >> 31);
     constexpr long long kBias = 64ll * (1 + 128 * (1 + 128 * (1 + 128 * (1 + 128ll * (1 + 128ll * (1 + 128ll))))));
-    n = (n ^ sg) + (kBias - sg);
+    const long long ns = (n ^ sg) - sg;
+    n = ns + kBias;
     const uint32_t nl = (uint32_t)n;
     const int nh = (int)(n >> 32);
     auto low = [](uint32_t d) { return __uint_as_float(0x4B400000u | (d & 127u)) - 12582976.f; };
@@ -54,6 +55,7 @@ __device__ __forceinline__ void digits(double v, int e, float (&q)[kD]) {
     q[2] = low((uint32_t)nh >> 3);
     q[1] = low((uint32_t)nh >> 10);
     q[0] = __int_as_float(0x4B400000 + (nh >> 17)) - 12582912.f;
+    return ns;
 }
 
 // Power of two of the largest of |v| from the upper words of their bits (1024 if one is not finite).
@@ -71,14 +73,14 @@ __device__ __forceinline__ uint32_t pack(float q0, float q1) {
 }
 
 // sum_l w_l 128^(7 - l) 2^k from the level sums w_l of at most 96 products per pair of digits (|w_l| < 2^22; the sum
-// then fits 62 bits without its lowest 8, which are rounded off first), rounded to nearest.
-__device__ __forceinline__ double value(const float (&w)[kD], int k) {
+// then fits 62 bits without its lowest 8, which are rounded off first), plus add 2^(k + 8), rounded to nearest.
+__device__ __forceinline__ double value(const float (&w)[kD], int k, long long add = 0) {
     int i[kD];
 #pragma unroll
     for (int l = 0; l < kD; ++l) i[l] = __float_as_int(w[l] + 12582912.f) - 0x4B400000;
     const long long hi = (long long)((i[0] << 7) + i[1]) * 16384 + (long long)((i[2] << 7) + i[3]);
     const long long lo = (long long)((i[4] << 7) + i[5]) * 16384 + (long long)((i[6] << 7) + i[7]);
-    const long long t = (hi << 20) + ((lo + 128) >> 8);
+    const long long t = (hi << 20) + ((lo + 128) >> 8) + add;
     const unsigned long long m = t < 0 ? (unsigned long long)-t : (unsigned long long)t;
     const int z = __clzll((long long)m);
     const int E = 62 - z + k + 8 + 1023;  // biased exponent - 1; the significand's leading bit adds the 1
@@ -89,11 +91,24 @@ __device__ __forceinline__ double value(const float (&w)[kD], int k) {
     return __longlong_as_double(r | (t & (long long)0x8000000000000000ull));
 }
 
-// Fragments of the factor tab (t[0..n-1]) for MMAs with B[k][c] = t[(c - k) mod n], and its exponent; by nt threads.
-__device__ inline int build(uint2* frag, const double* __restrict__ tab, int n, int tid, int nt) {
+// Fragments for MMAs with B[k][c] = t[(c - k) mod n] of a circulant factor given less the identity (tab[0..n-1]), by nt
+// threads; returns their exponent eB, and in sh whether they hold the factor less the identity (sh >= 0) or all of it
+// (sh < 0). exp(dtau t C) is close to the identity, and its digits are the same in every slice: cut at 2^-56 of the
+// diagonal, their rounding adds up over N L factors (ln det against 64-bit-mantissa arithmetic, rms of 16 fields: 16x16,
+// L = 160, 6.0e-12 whole, 2.6e-12 less the identity; 12x12, L = 120, 2.7e-12 / 2.2e-12). The lines' own integers, shifted by
+// sh = -2 - eB to the sums' unit, add the identity exactly; sh is at most 4, so that the sum keeps within 62 bits.
+__device__ inline int build(uint2* frag, const double* __restrict__ tab, int n, int tid, int nt, int& sh) {
     int h = 0;
     for (int d = 0; d < n; ++d) h = max(h, __double2hiint(tab[d]) & 0x7fffffff);
-    const int e = exponent_of_hi(h), total = ntiles(n) * 32;
+    int e = max(exponent_of_hi(h), -6);
+    sh = -2 - e;
+    const double one = sh >= 0 ? 0.0 : 1.0;  // what the fragments add to the diagonal
+    if (sh < 0) {
+        h = 0;
+        for (int d = 0; d < n; ++d) h = max(h, __double2hiint(tab[d] + (d == 0 ? 1.0 : 0.0)) & 0x7fffffff);
+        e = exponent_of_hi(h);
+    }
+    const int total = ntiles(n) * 32;
     for (int i = tid; i < total; i += nt) {
         const int lane = i & 31, j = i >> 5;
         const int c = 8 * j + (lane >> 2), k0 = 2 * (lane & 3);
@@ -101,7 +116,7 @@ __device__ inline int build(uint2* frag, const double* __restrict__ tab, int n, 
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int k = k0 + (u & 1) + 8 * (u >> 1);
-            digits(c < n && k < n ? tab[c >= k ? c - k : c - k + n] : 0.0, e, q[u]);
+            digits(c < n && k < n ? tab[c >= k ? c - k : c - k + n] + (c == k ? one : 0.0) : 0.0, e, q[u]);
         }
 #pragma unroll
         for (int s = 0; s < kD; ++s)
@@ -115,9 +130,10 @@ __device__ inline int build(uint2* frag, const double* __restrict__ tab, int n, 
 // of the warp take part.
 template <int NTL>
 __device__ __forceinline__ void tile(double* g, int rstep, int rows, int stride, int n, const uint2* __restrict__ frag, int eB,
-                                     const double* in_sc, const double* out_sc, int sstep) {
+                                     int sh, const double* in_sc, const double* out_sc, int sstep) {
     const int lane = threadIdx.x & 31, r0 = lane >> 2, t2 = 2 * (lane & 3);
     uint32_t a[kD][4];
+    long long own[8];  // the thread's values as integers: at the positions of its results
     int e0, e1;
     {
         double v[8];
@@ -149,10 +165,10 @@ __device__ __forceinline__ void tile(double* g, int rstep, int rows, int stride,
 #pragma unroll
         for (int u = 0; u < 4; u += 2) {
             float q0[kD], q1[kD], p0[kD], p1[kD];
-            digits(v[u], e0, q0);
-            digits(v[u + 1], e0, q1);
-            digits(v[4 + u], e1, p0);
-            digits(v[5 + u], e1, p1);
+            own[u] = digits(v[u], e0, q0);
+            own[u + 1] = digits(v[u + 1], e0, q1);
+            own[4 + u] = digits(v[4 + u], e1, p0);
+            own[5 + u] = digits(v[5 + u], e1, p1);
 #pragma unroll
             for (int s = 0; s < kD; ++s) {
                 a[s][u] = pack(q0[s], q1[s]);
@@ -183,7 +199,9 @@ __device__ __forceinline__ void tile(double* g, int rstep, int rows, int stride,
 #pragma unroll
             for (int l = 0; l < kD; ++l) w[l] = c[l][u];
             // a line with a value that is not finite becomes NaN, as its sums would
-            double y = e == 1024 ? nan : value(w, e + eB - 61);
+            const int at = (u & 1) + 4 * (u >> 1);
+            const long long o = j == 0 ? own[at] : own[at + 2];
+            double y = e == 1024 ? nan : value(w, e + eB - 61, sh >= 0 ? o << sh : 0);
             if (out_sc) y *= out_sc[col * sstep];
             g[r * rstep + col * stride] = y;
         }
@@ -273,9 +291,9 @@ __device__ __forceinline__ void rank_update(double* C, int ldc, const double* Ad
 
 // Length n <= kMaxLine at run time; frag built for that n.
 __device__ __forceinline__ void tile_any(double* g, int rstep, int rows, int stride, int n, const uint2* __restrict__ frag,
-                                         int eB, const double* in_sc, const double* out_sc, int sstep) {
-    if (n <= 8) tile<1>(g, rstep, rows, stride, n, frag, eB, in_sc, out_sc, sstep);
-    else tile<2>(g, rstep, rows, stride, n, frag, eB, in_sc, out_sc, sstep);
+                                         int eB, int sh, const double* in_sc, const double* out_sc, int sstep) {
+    if (n <= 8) tile<1>(g, rstep, rows, stride, n, frag, eB, sh, in_sc, out_sc, sstep);
+    else tile<2>(g, rstep, rows, stride, n, frag, eB, sh, in_sc, out_sc, sstep);
 }
 
 }  // namespace oz

@@ -43,3 +43,17 @@ def test_line_transforms_keep_a_nan_field_apart():
     with pytest.raises(SlmcError):
         ctx.get_error()
     assert torch.equal(got[[0, 2]], want[[0, 2]]) and torch.isnan(got[1]) and sg[1].item() == 0
+
+
+@pytest.mark.parametrize("dtau", [0.001, 0.1, 0.4, 0.5])
+def test_line_transforms_near_and_far_from_the_identity(dtau):
+    """The factor's digits are cut less the identity while its off-diagonal entries stay below 1/2 (dtau = 0.5: whole)."""
+    Lx, Ly, L, n_s, nf = 12, 10, 6, 2, 2
+    x = inputs.mixed_fields(nf, Lx, Ly, L, seed=3)
+    ctx = make_ctx(Lx, L, n_s, Ly=Ly, max_fields=nf, dtau=dtau)
+    G, ld, sg = ctx.greens(cuda(x))
+    p = HolsteinParams(Lx, Ly, L, n_s=n_s, dtau=dtau)
+    for f in range(nf):
+        l_ref, s_ref, G_ref = fermion_logdet(p, x[f])
+        assert abs(ld[f].item() - l_ref) < 1e-8 and sg[f].item() == s_ref
+        assert np.abs(G[f].cpu().numpy() - G_ref).max() < 1e-9

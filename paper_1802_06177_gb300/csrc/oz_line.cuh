@@ -1,12 +1,13 @@
 // Transforms of short lines by a symmetric circulant factor, FP64-accurate, on the warp-level tensor
 // instruction (mma.sync, BF16): the slices of the FP64 mode and of the DQMC chains.
+// Also the rank-16 updates of the DQMC moves (rank_update).
 //
 // The transforms are FP64-issue bound (one warp instruction per 16-19 cycles per SM; 6.5 to 8 per value and pass even
 // when folded, circ.cuh), and a line of at most 16 values is one K step of an MMA whose operands never leave the
-// registers. Lines of up to 16 values: 16 of them (the same line of 16 columns) are the rows of A, cut per row into eight 7-bit
-// digits against the row's power of two (as slice7.cuh with one digit more: 56 bits, so the slicing error is
-// 2^-56 of the row's largest value, below the FP64 sum's own rounding); the factor's digits are B, laid out in
-// fragment order once per CTA. The 36 products a + b <= 7 of a tile are summed per level in FP32, exactly (at most
+// registers. Lines of up to 16 values: 16 of them (the same line of 16 columns) are the rows of A, cut per row into
+// eight 7-bit digits against the row's power of two (as slice7.cuh with one digit more: 56 bits, so the slicing
+// error is 2^-56 of the row's largest value, below the FP64 sum's own rounding); the factor's digits, less the
+// identity (build), are B, laid out in fragment order once per CTA. The 36 products a + b <= 7 of a tile are summed per level in FP32, exactly (at most
 // 41 thousand per index of K <= 16), combined in two 64-bit integers and rounded once with integer operations: about
 // 50 integer and FP32 instructions per value and pass, no FP64. tcgen05 would need the digits in shared memory and
 // the sums back from tensor memory for 36 instructions of K = 16.
@@ -29,7 +30,8 @@ __host__ __device__ constexpr int frag_bytes(int n) { return ntiles(n) * kD * 32
 
 // The eight digits of v in units of 2^(e - 6 - 7 s), as small integers in FP32 (see slice7.cuh): v is rounded to
 // n 2^(e - 55) (half away from zero) in 32-bit words -- the variable 64-bit shifts and the conversions were most of
-// this function -- and the balanced digits of n are bit fields of n plus 64 at every place below the top. Returns n with its sign.
+// this function -- and the balanced digits of n are bit fields of n plus 64 at every place below the top.
+// Returns n with its sign.
 __device__ __forceinline__ long long digits(double v, int e, float (&q)[kD]) {
     const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
     const int ex = (int)((h >> 20) & 0x7ffu);
@@ -211,7 +213,8 @@ __device__ __forceinline__ void tile(double* g, int rstep, int rows, int stride,
 // C (row-major, row stride ldc) += sum_{q < cnt} A_q B_q^T, A_q and B_q the N-vectors at Ad + q N and Bd + q N,
 // cnt <= 16: one K step, 16 x 8 tiles, digits per row of A and per column of B, each entry's sum rounded once and added
 // in FP64: against 64-bit-mantissa arithmetic, the entries of G after a batch are off by 4e-17 (median, relative)
-// where 16 rounded FMAs leave 1.2e-16 (9x8 and 12x12 lattices, L = 40 and 80). By the warps of a CTA (warp of nw); kChunk column tiles share a row tile's digits.
+// where 16 rounded FMAs leave 1.2e-16 (9x8 and 12x12 lattices, L = 40 and 80). By the warps of a CTA (warp of
+// nw); kChunk column tiles share a row tile's digits.
 __device__ __forceinline__ void rank_update(double* C, int ldc, const double* Ad, const double* Bd, int cnt, int N, int warp,
                                             int nw) {
     constexpr int kChunk = 6;

@@ -32,7 +32,9 @@
 namespace {
 
 constexpr int kThreads = 128;
-constexpr int kNBF = 32;  // columns per CTA of the folded form
+// Columns per CTA of the folded form: 32, a lane per column. From 27 x 32 sites on a panel of 32 columns, the slice
+// scales and the coefficients of the two factors outgrow the 227 KB of a CTA; 24 columns fit up to 32 x 32.
+constexpr int kNBF = 32, kNBFLarge = 24;
 
 template <bool kTrans>
 __global__ void __launch_bounds__(kThreads) k_slice_oz(const double* __restrict__ U, double* __restrict__ Y,
@@ -99,15 +101,15 @@ template <int LMAX, bool kTrans>
 __global__ void __launch_bounds__(kThreads) k_slice_kron(const double* __restrict__ U, double* __restrict__ Y,
                                                          const double* __restrict__ x,
                                                          const double* __restrict__ kron, int Lx, int Ly, int L,
-                                                         int l0, int nsl, double dtlam, double emu) {
+                                                         int l0, int nsl, double dtlam, double emu, int NB) {
     extern __shared__ double sm[];
     const int N = Lx * Ly, ld = N | 1;
-    double* P = sm;                 // [kNBF][ld] panel, column-major
-    double* sc = sm + kNBF * ld;     // [N] e^{dtau mu} s_l
+    double* P = sm;                // [NB][ld] panel, column-major
+    double* sc = sm + NB * ld;     // [N] e^{dtau mu} s_l
     double* cx = sc + N;            // folded coefficients of E_x, E_y
     double* cy = cx + slmc::circ::ncoef(Lx);
-    const int f = blockIdx.y, j0 = blockIdx.x * kNBF, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nb = min(kNBF, N - j0);
+    const int f = blockIdx.y, j0 = blockIdx.x * NB, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nb = min(NB, N - j0);
     const size_t NN = (size_t)N * N;
     const double* Uf = U + f * NN + (size_t)j0 * N;
     slmc::circ::build(cx, kron, Lx, tid, kThreads);
@@ -142,13 +144,15 @@ __global__ void __launch_bounds__(kThreads) k_slice_kron(const double* __restric
 template <int LMAX, bool kTrans>
 cudaError_t launch_kron(slmc_ctx* c, const double* x, int nf, int l0, int nsl, cudaStream_t s) {
     const int N = c->N;
-    const size_t smem = ((size_t)kNBF * (N | 1) + N + slmc::circ::ncoef(c->p.Lx) + slmc::circ::ncoef(c->p.Ly)) * sizeof(double);
+    const size_t fixed = (size_t)N + slmc::circ::ncoef(c->p.Lx) + slmc::circ::ncoef(c->p.Ly);
+    const int NB = (fixed + (size_t)kNBF * (N | 1)) * sizeof(double) <= 227 * 1024 ? kNBF : kNBFLarge;
+    const size_t smem = (fixed + (size_t)NB * (N | 1)) * sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_slice_kron<LMAX, kTrans>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    dim3 grid((N + kNBF - 1) / kNBF, nf);
+    dim3 grid((N + NB - 1) / NB, nf);
     k_slice_kron<LMAX, kTrans><<<grid, kThreads, smem, s>>>(c->U, c->Y, x, c->kron, c->p.Lx, c->p.Ly, c->L, l0, nsl,
-                                                            c->p.dtau * c->p.lambda, exp(c->p.dtau * c->p.mu));
+                                                            c->p.dtau * c->p.lambda, exp(c->p.dtau * c->p.mu), NB);
     return cudaGetLastError();
 }
 

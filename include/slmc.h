@@ -248,10 +248,9 @@ SLMC_API int slmc_set_update_counter(slmc_ctx* ctx, uint64_t value, void* stream
 SLMC_API int slmc_get_update_counter(slmc_ctx* ctx, uint64_t* value, void* stream);
 
 /* FP64 contexts with N <= 64 (prepivot mode) evaluate a determinant in one launch per batch, one CTA per field
- * in shared memory, as long as none of the calls that steer the general kernels was made on them
- * (slmc_set_tuning, slmc_set_sub_batches, slmc_set_sub_batch_priorities, slmc_set_qr_cluster,
- * slmc_set_dense_slices, slmc_set_tupdate_path, slmc_set_qr_path); after one of them the context uses the
- * general kernels. Both agree to FP64 rounding.
+ * in shared memory, while what steers the general kernels has its default value (qr_panel 0, slmc_set_qr_cluster 0,
+ * slmc_set_dense_slices 0, slmc_set_tupdate_path 0, slmc_set_qr_path 0) and slmc_set_sub_batches was not called;
+ * otherwise they use the general kernels. Both agree to FP64 rounding.
  *
  * Kernel tile choices (found by slmc_autotune): qr_panel = width of the blocked-QR panels
  * (0 = by N, 16 or 32); slice_cols = columns per thread of the FP32 slice kernel (0 = by N,
@@ -442,8 +441,8 @@ SLMC_API int slmc_batch_launch(slmc_batch* batch, int nrounds, void* stream);
 /* ---- Autotuner ------------------------------------------------------------------------------
  * For the class described by *p (its precision and qr_mode), times slmc_logdet on ntune
  * synthetic Gaussian fields for every candidate stabilisation interval n_s in
- * {4, 6, 8, 10, 12, 16, 20, 24, 32} (<= L), blocked-QR panel width {16, 32} and FP32 slice
- * tile {8, 16}, and returns the fastest candidate whose max |d ln det| against the library's
+ * {4, 6, 8, 10, 12, 16, 20, 24, 32} (<= L), blocked-QR panel width {16, 32} (and 0, the one-launch
+ * kernel, for FP64 with N <= 64) and FP32 slice tile {8, 16}, and returns the fastest candidate whose max |d ln det| against the library's
  * FP64 path (n_s = 4) on the same fields is <= tol. Allocates and frees its own buffers and
  * synchronises the device (an initialisation-time call). SLMC_ERR_UNSUPPORTED if no candidate
  * meets tol. */

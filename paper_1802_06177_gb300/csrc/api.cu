@@ -254,7 +254,7 @@ slmc_ctx make_view(slmc_ctx* c, int f0) {
     v.tune_slice_groups = c->tune_slice_groups;
     v.tune_qr_cluster = c->tune_qr_cluster;
     v.num_sms = c->num_sms;
-    v.layout_set = c->layout_set;
+    v.nsub_set = c->nsub_set;
     v.nsub = 0;
     v.parent = c;
     return v;
@@ -265,7 +265,7 @@ slmc_ctx make_view(slmc_ctx* c, int f0) {
 // 128 chains: 2.44 ms per update in one batch, 2.53 in three).
 int sub_batches(const slmc_ctx* c, int nf) {
     if (c->p.precision == SLMC_PREC_TF32X3) return 1;  // per-slice workspace not split into views
-    if (slmc::small_active(c) || (!c->layout_set && c->N <= slmc::kSmallN && nf <= c->num_sms)) return 1;
+    if (!c->nsub_set && (slmc::small_active(c) || (c->N <= slmc::kSmallN && nf <= c->num_sms))) return 1;
     return std::max(1, std::min(c->nsub, nf / kMinSubFields));
 }
 
@@ -796,7 +796,6 @@ int slmc_set_tuning(slmc_ctx* c, int qr_panel, int slice_cols) {
     if (!c || (qr_panel != 0 && qr_panel != 16 && qr_panel != 32) ||
         (slice_cols != 0 && slice_cols != 8 && slice_cols != 16))
         return SLMC_ERR_ARG;
-    c->layout_set = 1;
     c->tune_qr_panel = qr_panel;
     c->tune_slice_cols = slice_cols;
     return SLMC_OK;
@@ -827,14 +826,12 @@ int slmc_get_wolff_sites(slmc_ctx* c, long long* total, int reset, void* stream)
 
 int slmc_set_qr_cluster(slmc_ctx* c, int ctas) {
     if (!c || (ctas != 0 && ctas != 1 && ctas != 2 && ctas != 4)) return SLMC_ERR_ARG;
-    c->layout_set = 1;
     c->tune_qr_cluster = ctas;
     return SLMC_OK;
 }
 
 int slmc_set_dense_slices(slmc_ctx* c, int dense) {
     if (!c || dense < 0 || dense > 1) return SLMC_ERR_ARG;
-    c->layout_set = 1;
     c->dense_slices = dense;
     return SLMC_OK;
 }
@@ -842,7 +839,6 @@ int slmc_set_dense_slices(slmc_ctx* c, int dense) {
 int slmc_set_tupdate_path(slmc_ctx* c, int path) {
     if (!c || path < 0 || path > 2) return SLMC_ERR_ARG;
     if (path != 1 && !c->tt_A) return SLMC_ERR_UNSUPPORTED;
-    c->layout_set = 1;
     c->tt_path = path;
     return SLMC_OK;
 }
@@ -850,7 +846,6 @@ int slmc_set_tupdate_path(slmc_ctx* c, int path) {
 int slmc_set_qr_path(slmc_ctx* c, int path) {
     if (!c || path < 0 || path > 1) return SLMC_ERR_ARG;
     if (path == 0 && !c->qt_buf) return SLMC_ERR_UNSUPPORTED;
-    c->layout_set = 1;
     c->qr_path = path;
     return SLMC_OK;
 }
@@ -858,7 +853,6 @@ int slmc_set_qr_path(slmc_ctx* c, int path) {
 int slmc_set_sub_batch_priorities(slmc_ctx* c, int on) {
     if (!c || on < 0 || on > 1) return SLMC_ERR_ARG;
     if (on && c->nsub_avail == 0) return SLMC_ERR_UNSUPPORTED;
-    c->layout_set = 1;
     c->sub_prio = on;
     return SLMC_OK;
 }
@@ -866,7 +860,7 @@ int slmc_set_sub_batch_priorities(slmc_ctx* c, int on) {
 int slmc_set_sub_batches(slmc_ctx* c, int n) {
     if (!c || n < 1 || n > slmc_ctx::kMaxSub) return SLMC_ERR_ARG;
     if (n > 1 && c->nsub_avail < n) return SLMC_ERR_UNSUPPORTED;
-    c->layout_set = 1;
+    c->nsub_set = 1;
     c->nsub = n;
     return SLMC_OK;
 }

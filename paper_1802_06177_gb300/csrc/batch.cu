@@ -367,8 +367,11 @@ int slmc_autotune(const slmc_params* p, int ntune, double tol, slmc_tune_result*
         q.n_s = ns;
         slmc_ctx* c = nullptr;
         st = slmc_init(&q, ntune, &c);
-        for (int panel : {16, 32}) {
+        // panel 0: the one-launch kernel of small FP64 lattices, which runs with no width set
+        const bool small = st == SLMC_OK && slmc::small_active(c);
+        for (int panel : {0, 16, 32}) {
             if (st != SLMC_OK || (!blocked && panel == 32)) break;
+            if (panel == 0 && !small) continue;
             for (int cols : {8, 16}) {
                 if (st != SLMC_OK || (!fp32 && cols == 16)) break;
                 st = slmc_set_tuning(c, blocked ? panel : 0, fp32 ? cols : 0);

@@ -208,7 +208,8 @@ cudaError_t small_final_greens(slmc_ctx* c, int nf, double* G, cudaStream_t s) {
 
 bool small_active(const slmc_ctx* c) {
     return c->N <= kSmallN && c->kron && c->p.precision == SLMC_PREC_FP64 && c->p.qr_mode == SLMC_QR_PREPIVOT &&
-           !c->layout_set && c->qr_path == 0 && c->tt_path == 0 && !c->dense_slices;
+           c->qr_path == 0 && c->tt_path == 0 && !c->dense_slices && c->tune_qr_panel == 0 &&
+           c->tune_qr_cluster == 0 && !c->nsub_set;
 }
 
 cudaError_t small_logdet(slmc_ctx* c, const double* x, int nf, double* lndet, int* sign, double* G, cudaStream_t s) {

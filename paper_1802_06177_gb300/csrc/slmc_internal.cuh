@@ -69,7 +69,7 @@ struct slmc_ctx {
     int tune_slice_groups;
     int tune_qr_cluster;    // CTAs per field of the QR / formation of Q (0 = by field count)
     int num_sms;            // multiprocessors of the device
-    int layout_set;         // a knob of the general kernels was set: no one-launch path for small lattices
+    int nsub_set;           // slmc_set_sub_batches was called
     // Exact sliced tensor-core slice path (SLMC_PREC_BF16X9): fixed-point BF16 slices of F
     // [4][128 MT][tcx_npad], their row exponents and the TMA descriptor of the slices.
     void* tcx_F;
@@ -244,7 +244,8 @@ bool eff_sweeps_fused(const slmc_ctx* c);
 cudaError_t eff_chain_sweeps(slmc_ctx* c, double* x, int nf, int chain0, const double* J, uint64_t sweep0, int nsweeps,
                              int colour, const int* colour_per_chain, long long* n_acc, cudaStream_t s,
                              const unsigned long long* dctr = nullptr, int ctr_mul = 0);
-// Whole FP64 determinant (and G) of small lattices in one launch (k_small.cu).
+// Whole FP64 determinant (and G) of small lattices in one launch (k_small.cu), while every knob of the general
+// kernels has its default value and the sub-batches were left alone.
 constexpr int kSmallN = 64;
 bool small_active(const slmc_ctx* c);
 // the general kernels' final step at N <= kSmallN (c->piv then holds the row order, for small_final_greens)

@@ -359,7 +359,7 @@ int cumulative_phases(slmc_ctx* c, double* x, int n, const double* J, int nsweep
                     SLMC_CK(cudaMemcpyAsync(xo, xc, m * NL * sizeof(double), cudaMemcpyDeviceToDevice, sk));
                     SLMC_LAUNCH(SLMC_PROF_EFF, 1, sk, eff_features(c, xc, m, J, nullptr, 0, sc(1), sk));
                 }
-                if ((phases & kPhaseSweeps) && nsweeps > 0 && eff_sweeps_fused(c))
+                if ((phases & kPhaseSweeps) && nsweeps > 0 && eff_sweeps_fused(c, m))
                     SLMC_LAUNCH(SLMC_PROF_SWEEP, 1, sk,
                                 eff_chain_sweeps(c, xc, m, g0, J, (uint64_t)u * nsweeps, nsweeps, 0, isc(1),
                                                  n_sweep_acc ? n_sweep_acc + g0 : nullptr, sk, c->dctr, nsweeps));
@@ -625,7 +625,7 @@ int slmc_eff_sweep(slmc_ctx* c, double* x, int n, const double* J, int nsweeps, 
     if (!checkerboard_ok(c)) return SLMC_ERR_UNSUPPORTED;
     cudaStream_t s = as_stream(stream);
     c->cur_units = n;
-    if (n > 0 && nsweeps > 0 && slmc::eff_sweeps_fused(c)) {
+    if (n > 0 && nsweeps > 0 && slmc::eff_sweeps_fused(c, n)) {
         SLMC_LAUNCH(SLMC_PROF_SWEEP, 1, s,
                     slmc::eff_chain_sweeps(c, x, n, 0, J, sweep0, nsweeps, first_colour, nullptr, n_acc, s));
         return SLMC_OK;

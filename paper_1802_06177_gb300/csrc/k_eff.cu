@@ -803,13 +803,23 @@ cudaError_t eff_wolff(slmc_ctx* c, double* x, int nf, int chain0, const double* 
     return cudaGetLastError();
 }
 
-// Largest chain (sites times slices) whose sweeps run in one launch with the field in shared memory. Above,
-// a chain's half-sweep on one SM takes longer than a launch that spreads it over the GPU; measured at the
-// lower end: a 4x4, L = 40 update of 50 sweeps 1.42 -> 0.91 ms, an 8x8, L = 40 update of 10 sweeps and Wolff
-// moves on 128 chains 3.44 -> 3.15 ms (whole updates).
-constexpr int kChainSites = 8192;
+// Whether the sweeps of n chains run in one launch, a chain per SM with its field in shared memory (up to 8192
+// sites times slices, two CTAs per SM), or as a launch per half-sweep that spreads the chains over the GPU. With
+// Wolff updates (a launch each otherwise) one launch is faster at any n: 1 chain of 8x8, L = 40, 20 sweeps 223 us
+// against 386, of 8x8, L = 128, 515 against 684, 16 chains 536 against 785. Without them it is for up to 4096
+// values (8x8, L = 40: 123 against 182 us for 1 chain, 126 against 226 for 16; 4x4, L = 240: 153 / 182), and above
+// once there are enough chains for the half-sweeps to grow: 20 sweeps of 5120, 6144, 7168 and 8192 values take 195,
+// 220, 255 and 280 us in one launch for 1 to 16 chains; launches per half-sweep 186 to 190 us for one
+// chain, 208, 210, 216, 219 for 4, 226, 229, 235, 242 for 8, 249, 252, 255, 256 for 16 (and at 8192 values 338 for 32).
+constexpr int kChainSites = 8192, kChainSitesAny = 4096;
 
-bool eff_sweeps_fused(const slmc_ctx* c) { return c->N * (long long)c->L <= kChainSites; }
+bool eff_sweeps_fused(const slmc_ctx* c, int n) {
+    const long long sites = c->N * (long long)c->L;
+    if (sites > kChainSites) return false;
+    int most = kChainSitesAny;  // and 1024 more for every doubling of n from 4 on
+    for (int m = n; m >= 4; m >>= 1) most += 1024;
+    return c->nwolff > 0 || sites <= most;
+}
 
 cudaError_t eff_chain_sweeps(slmc_ctx* c, double* x, int nf, int chain0, const double* J, uint64_t sweep0, int nsweeps,
                              int colour, const int* colour_per_chain, long long* n_acc, cudaStream_t s,

@@ -238,9 +238,9 @@ cudaError_t eff_half_sweep(slmc_ctx* c, double* x, int nf, int chain0, const dou
                            cudaStream_t s, const unsigned long long* dctr = nullptr, int nsweeps = 0);
 cudaError_t eff_wolff(slmc_ctx* c, double* x, int nf, int chain0, const double* J, uint64_t sweep, int k,
                       cudaStream_t s, const unsigned long long* dctr = nullptr, int nsweeps = 0);
-// All nsweeps sweeps (with their Wolff updates) of nf chains in one launch; eff_sweeps_fused says whether
-// the chain is small enough. Sweep counters start at sweep0 (plus the device counter times ctr_mul).
-bool eff_sweeps_fused(const slmc_ctx* c);
+// All nsweeps sweeps (with their Wolff updates) of nf chains in one launch; eff_sweeps_fused says for n chains whether
+// that is possible and faster. Sweep counters start at sweep0 (plus the device counter times ctr_mul).
+bool eff_sweeps_fused(const slmc_ctx* c, int n);
 cudaError_t eff_chain_sweeps(slmc_ctx* c, double* x, int nf, int chain0, const double* J, uint64_t sweep0, int nsweeps,
                              int colour, const int* colour_per_chain, long long* n_acc, cudaStream_t s,
                              const unsigned long long* dctr = nullptr, int ctr_mul = 0);

@@ -443,7 +443,7 @@ int slmc_init(const slmc_params* p, int max_fields, slmc_ctx** out) {
     };
     alloc(&c->E64, NN * sizeof(double));
     alloc(&c->Einv64, NN * sizeof(double));
-    if (c->p.Lx <= slmc::kKronMaxLine && c->p.Ly <= slmc::kKronMaxLine) alloc(&c->kron, slmc::kKronTabs * slmc::kKronTab * sizeof(double));
+    if (c->p.Lx <= slmc::kKronMaxLine && c->p.Ly <= slmc::kKronMaxLine) alloc(&c->kron, 4 * slmc::kKronTab * sizeof(double));
     alloc(&c->F32, NN * sizeof(float));
     if (p->precision == SLMC_PREC_FP32) {
         c->lo_S = std::min(slmc::kLoStencil, (int)N);

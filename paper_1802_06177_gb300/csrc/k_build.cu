@@ -31,8 +31,8 @@ __global__ void k_hopping_exp(double* __restrict__ E, int Lx, int Ly, double dta
 // The one-dimensional factors of the plane-wave sum above: for a side of Ld sites,
 // e[d] = (1/Ld) sum_n cos(2 pi n d / Ld) exp(+-2 dtau t cos(2 pi n / Ld)); the sums over
 // x and y separate because the hopping along x and along y commute. Block q of tab holds
-// [E_x | E_x^-1 | E_y | E_y^-1 | E_x - I | E_y - I][q], each written twice over. The sums go over the exponentials less
-// one: every slice multiplies by the same entries, so their rounding adds up over N L factors in ln det, and this way
+// [E_x | E_x^-1 | E_y | E_y^-1][q], and kKronMaxLine behind it the same less the identity. The sums go over the
+// exponentials less one: every slice multiplies by the same entries, so their rounding adds up over N L factors in ln det, and this way
 // it is that of a number ten times smaller than the diagonal.
 __global__ void k_kron_tables(double* __restrict__ tab, int Lx, int Ly, double dtau_t2) {
     const int q = blockIdx.x, d = threadIdx.x;
@@ -42,13 +42,8 @@ __global__ void k_kron_tables(double* __restrict__ tab, int Lx, int Ly, double d
     double acc = 0.0;
     for (int n = 0; n < Ld; ++n) acc += cospi(2.0 * ((n * d) % Ld) / Ld) * expm1(a * cospi(2.0 * n / Ld));
     acc /= Ld;
-    const double e = d == 0 ? 1.0 + acc : acc;
-    tab[q * slmc::kKronTab + d] = e;
-    tab[q * slmc::kKronTab + d + Ld] = e;
-    if ((q & 1) == 0) {
-        tab[(4 + q / 2) * slmc::kKronTab + d] = acc;
-        tab[(4 + q / 2) * slmc::kKronTab + d + Ld] = acc;
-    }
+    tab[q * slmc::kKronTab + d] = d == 0 ? 1.0 + acc : acc;
+    tab[q * slmc::kKronTab + slmc::kKronMaxLine + d] = acc;
 }
 
 __global__ void k_split_F(const double* __restrict__ E, float* __restrict__ F32, int N) {

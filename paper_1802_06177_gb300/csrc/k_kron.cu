@@ -52,8 +52,8 @@ __global__ void __launch_bounds__(kThreads) k_slice_oz(const double* __restrict_
     const size_t NN = (size_t)N * N;
     const double* Uf = U + f * NN + (size_t)j0 * N;
     int shx, shy;
-    const int ex = slmc::oz::build(fx, kron + 4 * slmc::kKronTab, Lx, tid, kThreads, shx);
-    const int ey = slmc::oz::build(fy, kron + 5 * slmc::kKronTab, Ly, tid, kThreads, shy);
+    const int ex = slmc::oz::build(fx, kron + slmc::kKronMaxLine, Lx, tid, kThreads, shx);
+    const int ey = slmc::oz::build(fy, kron + 2 * slmc::kKronTab + slmc::kKronMaxLine, Ly, tid, kThreads, shy);
     for (int jj = warp; jj < nb; jj += kThreads / 32)
         for (int i = lane; i < N; i += 32) P[jj * ld + i] = Uf[(size_t)jj * N + i];
     const double* xf = x + (size_t)f * N * L;

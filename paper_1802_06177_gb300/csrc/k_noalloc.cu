@@ -38,7 +38,7 @@ size_t fixed_bytes(size_t N) {
     const size_t S = N < (size_t)slmc::kLoStencil ? N : (size_t)slmc::kLoStencil;
     return align256(N * N * sizeof(double)) + align256(N * N * sizeof(float)) +
            align256((S * N + S) * sizeof(int)) + align256(S * sizeof(float)) +
-           align256(slmc::kKronTabs * slmc::kKronTab * sizeof(double)) + 256;
+           align256(4 * slmc::kKronTab * sizeof(double)) + 256;
 }
 // L > 0 (FP32 mode): also the FP32 slice scales and the FP32 orthogonal factor.
 size_t field_bytes(size_t N, size_t L) {
@@ -110,7 +110,7 @@ int slmc_logdet_noalloc(const slmc_params* p, const double* x, int n, double* ln
     }
     // the circulant factors of exp(-dtau K): FP64 slice products through them, as in slmc_logdet
     if (p->Lx <= slmc::kKronMaxLine && p->Ly <= slmc::kKronMaxLine)
-        c.kron = reinterpret_cast<double*>(take(slmc::kKronTabs * slmc::kKronTab * sizeof(double)));
+        c.kron = reinterpret_cast<double*>(take(4 * slmc::kKronTab * sizeof(double)));
     c.err = reinterpret_cast<unsigned int*>(take(sizeof(unsigned int)));
     c.Y = reinterpret_cast<double*>(q);
     c.QR = c.Y + F * NN;

@@ -18,8 +18,7 @@
 
 namespace slmc {
 constexpr int kKronMaxLine = 32;             // longest lattice side of the circulant factors
-constexpr int kKronTab = 2 * kKronMaxLine;   // doubles per stored factor
-constexpr int kKronTabs = 6;
+constexpr int kKronTab = 2 * kKronMaxLine;   // doubles per stored factor: the factor, then the factor less the identity
 }  // namespace slmc
 
 struct slmc_ctx {
@@ -29,8 +28,8 @@ struct slmc_ctx {
     double* E64;
     double* Einv64;  // exp(+dtau K), for carrying G between slices in the DQMC updates
     // One-dimensional circulant factors of exp(-+dtau K) = e^{-+dtau mu} E_x kron E_y (site
-    // i = ix + Lx iy), each stored twice over: [E_x | E_x^-1 | E_y | E_y^-1 | E_x - I | E_y - I], kKronTab
-    // doubles apiece. Null when a lattice side exceeds kKronMaxLine (dense products then).
+    // i = ix + Lx iy): [E_x | E_x^-1 | E_y | E_y^-1], kKronTab doubles apiece, of which the last
+    // kKronMaxLine hold the factor less the identity. Null when a lattice side exceeds kKronMaxLine (dense products then).
     double* kron;
     double* dq_stack;     // DQMC: [groups][max_fields] (U | T | lnD) of the transposed left products
     int dq_groups;        // groups the stack holds

@@ -1,6 +1,10 @@
 // Symmetric circulant transforms of short lines, y[d] = sum_m t[|d - m|] v[m] (t[k] = t[n - k]), the two factors
 // of the separable hopping exponential [Suppl. Eq. (S2)], in FP64.
 //
+// The factor is given less the identity, which a value's own term adds exactly: exp(dtau t C) is close to the
+// identity, every slice multiplies by the same coefficients, and the rounding of a diagonal of 1.1 would add up over the
+// N L factors of a determinant.
+//
 // FP64 issue bounds every kernel that applies them (two FMAs per clock per SM, 65 cycles of latency), so the
 // n^2 FMAs of the direct sum are folded by the symmetries of the line: reflection about site 0 splits v into
 // even and odd halves, and for even n the map m -> n/2 - m splits each half again. A line of 12 then takes
@@ -28,7 +32,7 @@ constexpr __host__ __device__ int ncoef(int n) {
     return sizes(n).p * sizes(n).p + sizes(n).m * sizes(n).m + sizes(n).q * sizes(n).q + sizes(n).r * sizes(n).r;
 }
 
-// Coefficients of the folded transform of length n from tab (t[0..n-1]); by nt threads, thread tid.
+// Coefficients of the folded transform of length n from tab (t[0..n-1] less the identity); by nt threads, thread tid.
 __device__ inline void build(double* coef, const double* tab, int n, int tid, int nt) {
     const Sizes z = sizes(n);
     const int h = n / 2, n0 = z.p * z.p, n1 = n0 + z.m * z.m, n2 = n1 + z.q * z.q, n3 = n2 + z.r * z.r;
@@ -55,11 +59,23 @@ __device__ inline void build(double* coef, const double* tab, int n, int tid, in
     }
 }
 
-template <int K>
+// x 2^-k by integer operations (an FP64 multiplication would take the pipe that bounds the transforms). Infinities and
+// NaN stay as they are; values below 2^(k - 1022) become zero.
+template <int k>
+__device__ __forceinline__ double scaled(double x) {
+    if (k == 0) return x;
+    const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+    const bool tiny = e <= k;
+    return __hiloint2double(tiny ? 0 : (e == 0x7ff ? hi : hi - (k << 20)), tiny ? 0 : __double2loint(x));
+}
+
+// y = c x plus the identity's part of the block: 2^-H x, but 2^-H0 x for the first K0 values and 2^-H1 x for the last K1.
+template <int K, int H, int K0 = 0, int H0 = 0, int K1 = 0, int H1 = 0>
 __device__ __forceinline__ void block(const double* __restrict__ c, const double (&x)[K > 0 ? K : 1],
                                       double (&y)[K > 0 ? K : 1]) {
 #pragma unroll
-    for (int d = 0; d < K; ++d) y[d] = c[d * K] * x[0];
+    for (int d = 0; d < K; ++d)
+        y[d] = fma(c[d * K], x[0], d < K0 ? scaled<H0>(x[d]) : (d >= K - K1 ? scaled<H1>(x[d]) : scaled<H>(x[d])));
 #pragma unroll
     for (int m = 1; m < K; ++m)
 #pragma unroll
@@ -84,8 +100,9 @@ __device__ __forceinline__ void line(const double* __restrict__ c, double (&v)[n
     }
     double s[h + 1], a[hm > 0 ? hm : 1];
     if constexpr (!two_level(n)) {
-        block<h + 1>(c, e, s);
-        if constexpr (hm > 0) block<hm>(cq, o, a);
+        // sites 0 and n / 2 are their own mirror images (weight 1), every other one shares a pair (1/2)
+        block<h + 1, 1, 1, 0, n % 2 == 0 ? 1 : 0, 0>(c, e, s);
+        if constexpr (hm > 0) block<hm, 1>(cq, o, a);
     } else {
         double ep[z.p], sp[z.p], em[z.m], sm[z.m];
 #pragma unroll
@@ -94,8 +111,9 @@ __device__ __forceinline__ void line(const double* __restrict__ c, double (&v)[n
             em[m] = e[m] - e[h - m];
         }
         if constexpr (z.p > z.m) ep[z.m] = e[h / 2];
-        block<z.p>(c, ep, sp);
-        block<z.m>(cm, em, sm);
+        // the same weights halved again, but for the middle value, its own mirror image in the second fold
+        block<z.p, 2, 1, 1, z.p - z.m, 1>(c, ep, sp);
+        block<z.m, 2, 1, 1>(cm, em, sm);
 #pragma unroll
         for (int d = 0; d < z.m; ++d) {
             s[d] = sp[d] + sm[d];
@@ -110,8 +128,8 @@ __device__ __forceinline__ void line(const double* __restrict__ c, double (&v)[n
                 om[m - 1] = o[m - 1] - o[h - m - 1];
             }
             if constexpr (z.q > z.r) op[z.r] = o[h / 2 - 1];
-            block<z.q>(cq, op, ap);
-            if constexpr (z.r > 0) block<z.r>(cr, om, am);
+            block<z.q, 2, 0, 0, z.q - z.r, 1>(cq, op, ap);
+            if constexpr (z.r > 0) block<z.r, 2>(cr, om, am);
 #pragma unroll
             for (int d = 1; d <= z.r; ++d) {
                 a[d - 1] = ap[d - 1] + am[d - 1];

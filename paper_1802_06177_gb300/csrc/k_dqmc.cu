@@ -123,10 +123,11 @@ __global__ void __launch_bounds__(kThreads) k_dqmc_slices(double* __restrict__ x
     double* xf = x + (size_t)f * N * L;
     const uint32_t chain = (uint32_t)(chain0 + f);
 
-    slmc::circ::build(ex, kron, Lx, tid, kThreads);
-    slmc::circ::build(exi, kron + slmc::kKronTab, Lx, tid, kThreads);
-    slmc::circ::build(ey, kron + 2 * slmc::kKronTab, Ly, tid, kThreads);
-    slmc::circ::build(eyi, kron + 3 * slmc::kKronTab, Ly, tid, kThreads);
+    const double* less1 = kron + slmc::kKronMaxLine;  // the factors less the identity
+    slmc::circ::build(ex, less1, Lx, tid, kThreads);
+    slmc::circ::build(exi, less1 + slmc::kKronTab, Lx, tid, kThreads);
+    slmc::circ::build(ey, less1 + 2 * slmc::kKronTab, Ly, tid, kThreads);
+    slmc::circ::build(eyi, less1 + 3 * slmc::kKronTab, Ly, tid, kThreads);
     if (g_in_smem) {
         for (int j = warp; j < N; j += kThreads / 32)
             for (int m = lane; m < N; m += 32) G[j * ldg + m] = Gall[f * NN + (size_t)j * N + m];

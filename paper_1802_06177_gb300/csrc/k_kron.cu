@@ -112,8 +112,8 @@ __global__ void __launch_bounds__(kThreads) k_slice_kron(const double* __restric
     const int nb = min(NB, N - j0);
     const size_t NN = (size_t)N * N;
     const double* Uf = U + f * NN + (size_t)j0 * N;
-    slmc::circ::build(cx, kron, Lx, tid, kThreads);
-    slmc::circ::build(cy, kron + 2 * slmc::kKronTab, Ly, tid, kThreads);
+    slmc::circ::build(cx, kron + slmc::kKronMaxLine, Lx, tid, kThreads);
+    slmc::circ::build(cy, kron + 2 * slmc::kKronTab + slmc::kKronMaxLine, Ly, tid, kThreads);
     for (int jj = warp; jj < nb; jj += kThreads / 32)
         for (int i = lane; i < N; i += 32) P[jj * ld + i] = Uf[(size_t)jj * N + i];
     const double* xf = x + (size_t)f * N * L;

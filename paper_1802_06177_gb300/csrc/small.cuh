@@ -58,7 +58,7 @@ __device__ __forceinline__ double group_sum(double v) {
 }
 
 // One pass of a transform over short lines (n <= 8, the 4x4 class): two lanes per line, each half of the outputs by
-// direct sums. At this size the folded transform's chain (18 FP64 instructions for a line of 4 on two warps) is
+// direct sums (t: the factor less the identity). At this size the folded transform's chain (18 FP64 instructions for a line of 4 on two warps) is
 // longer than eight direct ones on four.
 template <int n>
 __device__ __forceinline__ void half_line(double* g, int stride, const double* __restrict__ t, int half,
@@ -70,7 +70,7 @@ __device__ __forceinline__ void half_line(double* g, int stride, const double* _
 #pragma unroll
     for (int o = 0; o < nh; ++o) {
         const int d = half * nh + o;
-        y[o] = t[d < n ? d : 0] * v[0];
+        y[o] = fma(t[d < n ? d : 0], v[0], half ? v[nh + o < n ? nh + o : 0] : v[o]);
 #pragma unroll
         for (int m = 1; m < n; ++m) y[o] = fma(t[d >= m ? (d < n ? d - m : 0) : d - m + n], v[m], y[o]);
         if (out_sc) y[o] *= out_sc[(d < n ? d : 0) * stride];
@@ -103,7 +103,7 @@ __device__ __forceinline__ void short_pass(double* P, const double* __restrict__
 
 // P <- B_{c1} ... B_{c0} P (plain) for the field columns c0 .. c1 - 1 in order, or with trans the transposed
 // slices E diag(s) from c1 - 1 down to c0: circulant transforms along the x and the y lines of every column.
-// v.cx, v.cy: folded coefficients, or the plain factors for NMAX = 16 (short_pass).
+// v.cx, v.cy: folded coefficients, or the factors less the identity for NMAX = 16 (short_pass).
 template <int NMAX, int LMAX, bool kTrans>
 __device__ __forceinline__ void slices(double* P, Vecs<NMAX>& v, const double* __restrict__ xf, int N, int Lx, int Ly,
                                        int L, int c0, int c1, double dtlam, double emu) {
@@ -142,12 +142,12 @@ __device__ __forceinline__ void load_factors(Vecs<NMAX>& v, const double* __rest
     constexpr int NT = Dim<NMAX>::threads;
     if constexpr (NMAX == 16) {
         if (threadIdx.x < 8) {
-            v.cx[threadIdx.x] = kron[threadIdx.x];
-            v.cy[threadIdx.x] = kron[2 * kKronTab + threadIdx.x];
+            v.cx[threadIdx.x] = kron[kKronMaxLine + threadIdx.x];
+            v.cy[threadIdx.x] = kron[2 * kKronTab + kKronMaxLine + threadIdx.x];
         }
     } else {
-        circ::build(v.cx, kron, Lx, threadIdx.x, NT);
-        circ::build(v.cy, kron + 2 * kKronTab, Ly, threadIdx.x, NT);
+        circ::build(v.cx, kron + kKronMaxLine, Lx, threadIdx.x, NT);
+        circ::build(v.cy, kron + 2 * kKronTab + kKronMaxLine, Ly, threadIdx.x, NT);
     }
 }
 

@@ -31,6 +31,7 @@
 // tensor memory.
 #include <algorithm>
 
+#include "oz_line.cuh"
 #include "qr_panel.cuh"
 #include "slice7.cuh"
 #include "tc_ptx.cuh"
@@ -43,42 +44,61 @@ using slmc::s7::bf16_of;
 using slmc::s7::bf16x2_of;
 using slmc::s7::combine;
 using slmc::s7::exponent_of_bits;
-using slmc::s7::kS;
 using slmc::s7::slice7;
 using slmc::s7::warp_max_bits;
 
-constexpr int kLv = 7;                       // levels a + b = 0..6
 constexpr int kQT = 320;                     // GEMM threads: 8 epilogue warps, TMA warp, MMA warp
 constexpr uint32_t kTileA = 128 * 128;       // 128 rows x 64 BF16 (one 128-byte swizzle row each)
-constexpr int kSegChunks = 7;                // K chunks (64 rows) per accumulator set of W^T = C^T V
-constexpr int kMaxN = 2 * kSegChunks * 64;   // 896: two accumulator sets
+constexpr int kMaxN = 896;                   // 14 K chunks: two accumulator sets of seven
 constexpr int kVRows = 32;                   // rows of the V1 slice buffer per field (BP <= 32)
 // W^T = C^T V streams the seven C slices of a K chunk through a ring of three tiles (tile a is
 // released once its products with the seven V slices are issued), so two CTAs fit on an SM: one's
 // FP64 epilogue then overlaps the other's copies and products.
 constexpr int kRing = 3;
-// 2^-54: the digits' units 2^(e - 6) per operand and the level weights 2^(-7 level), 2^-42 at level 6
-constexpr int kUnitShift = 2 * 6 + 7 * (kLv - 1);
+constexpr int kDMax = 8;
 
-// Level sums (FP32 integers) of one accumulator entry -> hi 2^28 + lo as 64-bit integers.
-__device__ __forceinline__ void levels_to_int(const uint32_t (&v)[kLv], long long& hi, long long& lo) {
-    hi = (long long)__float2int_rn(__uint_as_float(v[0]));
-#pragma unroll
-    for (int lv = 1; lv < 3; ++lv) hi = hi * 128 + (long long)__float2int_rn(__uint_as_float(v[lv]));
-    lo = (long long)__float2int_rn(__uint_as_float(v[3]));
-#pragma unroll
-    for (int lv = 4; lv < kLv; ++lv) lo = lo * 128 + (long long)__float2int_rn(__uint_as_float(v[lv]));
+// What depends on the number of digits D per operand: seven (49 bits, the trailing updates) or eight (56 bits, the
+// formation of Q in FP64; oz_line.cuh's digits). Products a + b <= D - 1 in D levels.
+template <int D>
+struct Dig {
+    // K chunks (64 rows) per accumulator set of W^T = C^T V: a level's sum of absolute terms is at most 36864 per K
+    // index with seven digits, 40960 with eight, and stays below 2^24
+    static constexpr int kSegChunks = D == 7 ? 7 : 6;
+    // the digits' units 2^(e - 6) per operand and the level weights 2^(-7 level)
+    static constexpr int kUnitShift = 2 * 6 + 7 * (D - 1);
+    // tiles of the first product's A ring: two leave room for two CTAs per SM beside eight slices of 32 reflectors
+    static constexpr __host__ __device__ int ring1(int BP) { return D == 8 && BP == 32 ? 2 : kRing; }
+};
+
+template <int D>
+__device__ __forceinline__ void cut(double v, int e, float (&q)[D]) {
+    if constexpr (D == 7) slice7(v, e, q);
+    else slmc::oz::digits(v, e, q);
 }
 
-// The same for sums below 2^22 (K <= 32 indices: at most 36864 * 32 < 2^21): one exact FP32 addition places the
+// Level sums (FP32 integers) of one accumulator entry -> hi 2^28 + lo as 64-bit integers.
+template <int D>
+__device__ __forceinline__ void levels_to_int(const uint32_t (&v)[D], long long& hi, long long& lo) {
+    hi = (long long)__float2int_rn(__uint_as_float(v[0]));
+#pragma unroll
+    for (int lv = 1; lv < D - 4; ++lv) hi = hi * 128 + (long long)__float2int_rn(__uint_as_float(v[lv]));
+    lo = (long long)__float2int_rn(__uint_as_float(v[D - 4]));
+#pragma unroll
+    for (int lv = D - 3; lv < D; ++lv) lo = lo * 128 + (long long)__float2int_rn(__uint_as_float(v[lv]));
+}
+
+// The same for sums below 2^22 (K <= 32 indices: at most 40960 * 32 < 2^21): one exact FP32 addition places the
 // integer in the significand, where the conversion instruction would take the FP64 pipe's issue.
 __device__ __forceinline__ int small_int(uint32_t v) {
     return __float_as_int(__uint_as_float(v) + 12582912.f) - 0x4B400000;
 }
-__device__ __forceinline__ void small_levels_to_int(const uint32_t (&v)[kLv], long long& hi, long long& lo) {
-    hi = (long long)((small_int(v[0]) << 7) + small_int(v[1])) * 128 + (long long)small_int(v[2]);
-    lo = (long long)((small_int(v[3]) << 7) + small_int(v[4])) * 16384 +
-         (long long)((small_int(v[5]) << 7) + small_int(v[6]));
+template <int D>
+__device__ __forceinline__ void small_levels_to_int(const uint32_t (&v)[D], long long& hi, long long& lo) {
+    hi = small_int(v[0]);
+    if constexpr (D == 8) hi = hi * 128 + (long long)small_int(v[1]);
+    hi = hi * 16384 + (long long)((small_int(v[D - 6]) << 7) + small_int(v[D - 5]));
+    lo = (long long)((small_int(v[D - 4]) << 7) + small_int(v[D - 3])) * 16384 +
+         (long long)((small_int(v[D - 2]) << 7) + small_int(v[D - 1]));
 }
 
 // Compact-WY triangle S of BP reflectors from their Gram matrix G (row stride ldg) and tau, by the 256
@@ -161,7 +181,7 @@ struct PanelSmem {
 
 // Slices of the clean reflectors V (row r at Vp + r (BP + 1), rows p..N-1) of one field: per reflector over the
 // rows (V1) and per row over the reflectors (V2), with their exponents.
-template <int BP, int NT>
+template <int BP, int NT, int D>
 __device__ __forceinline__ void slice_V(const double* Vp, __nv_bfloat16* __restrict__ V1, int* __restrict__ eV1,
                                         __nv_bfloat16* __restrict__ V2, int* __restrict__ eV2, int N, int p, int gf, int kpad,
                                         int mpad, size_t plane1, size_t plane2) {
@@ -176,11 +196,11 @@ __device__ __forceinline__ void slice_V(const double* Vp, __nv_bfloat16* __restr
         if (lane == 0) eV1[(size_t)gf * kVRows + m] = e;
         __nv_bfloat16* dst = V1 + ((size_t)gf * kVRows + m) * kpad;
         for (int k = kstart + 2 * lane; k < kpad; k += 64) {  // two adjacent rows per lane (multiples of 64)
-            float q0[kS], q1[kS];
-            slice7((k >= p && k < N) ? Vp[k * BPS + m] : 0.0, e, q0);
-            slice7((k + 1 >= p && k + 1 < N) ? Vp[(k + 1) * BPS + m] : 0.0, e, q1);
+            float q0[D], q1[D];
+            cut<D>((k >= p && k < N) ? Vp[k * BPS + m] : 0.0, e, q0);
+            cut<D>((k + 1 >= p && k + 1 < N) ? Vp[(k + 1) * BPS + m] : 0.0, e, q1);
 #pragma unroll
-            for (int s = 0; s < kS; ++s)
+            for (int s = 0; s < D; ++s)
                 *reinterpret_cast<uint32_t*>(dst + (size_t)s * plane1 + k) = bf16x2_of(q0[s], q1[s]);
         }
     }
@@ -191,10 +211,10 @@ __device__ __forceinline__ void slice_V(const double* Vp, __nv_bfloat16* __restr
         const int e = exponent_of_bits(warp_max_bits(abs_bits(v)));
         if (lane == 0) eV2[(size_t)gf * mpad + r] = e;
         if (lane < BP) {
-            float q[kS];
-            slice7(v, e, q);
+            float q[D];
+            cut<D>(v, e, q);
 #pragma unroll
-            for (int s = 0; s < kS; ++s) V2[(size_t)s * plane2 + ((size_t)gf * mpad + r) * 64 + lane] = bf16_of(q[s]);
+            for (int s = 0; s < D; ++s) V2[(size_t)s * plane2 + ((size_t)gf * mpad + r) * 64 + lane] = bf16_of(q[s]);
         }
     }
 }
@@ -305,12 +325,13 @@ __global__ void __launch_bounds__(kPT, kPT == 256 ? 3 : 1)
         if (bad) atomicOr(err, SLMC_EBIT_NONFINITE);
         return;
     }
-    slice_V<BP, kPT>(Vp, V1, eV1, V2, eV2, N, p, gf, kpad, mpad, plane1, plane2);
+    slice_V<BP, kPT, 7>(Vp, V1, eV1, V2, eV2, N, p, gf, kpad, mpad, plane1, plane2);
 }
 
 // ---- slices of the trailing columns ---------------------------------------------------------
 // Warp w of block x slices trailing column jj = 8 x + w (logical column j0 + jj; no permutation in the formation of
 // Q) over rows p..N-1.
+template <int D>
 __global__ void __launch_bounds__(256) k_qrt_slice_C(const double* __restrict__ Yall, const int* __restrict__ perm_all,
                                                      __nv_bfloat16* __restrict__ Cs, int* __restrict__ eC, int N,
                                                      int p, int j0, int kpad, int jpad, size_t plane, int fbase) {
@@ -324,18 +345,18 @@ __global__ void __launch_bounds__(256) k_qrt_slice_C(const double* __restrict__ 
     if (lane == 0) eC[(size_t)gf * jpad + jj] = e;
     __nv_bfloat16* dst = Cs + ((size_t)gf * jpad + jj) * kpad;
     for (int k = (p / 64) * 64 + 2 * lane; k < kpad; k += 64) {  // two adjacent rows per lane (multiples of 64)
-        float q0[kS], q1[kS];
-        slice7((k >= p && k < N) ? col[k] : 0.0, e, q0);
-        slice7((k + 1 >= p && k + 1 < N) ? col[k + 1] : 0.0, e, q1);
+        float q0[D], q1[D];
+        cut<D>((k >= p && k < N) ? col[k] : 0.0, e, q0);
+        cut<D>((k + 1 >= p && k + 1 < N) ? col[k + 1] : 0.0, e, q1);
 #pragma unroll
-        for (int s = 0; s < kS; ++s)
+        for (int s = 0; s < D; ++s)
             *reinterpret_cast<uint32_t*>(dst + (size_t)s * plane + k) = bf16x2_of(q0[s], q1[s]);
     }
 }
 
 // The reflectors of panel p of a finished QR (below the diagonal of its packed output), sliced again for the
 // formation of Q.
-template <int BP>
+template <int BP, int D>
 __global__ void __launch_bounds__(256) k_qrt_slice_V(const double* __restrict__ QRall, __nv_bfloat16* __restrict__ V1,
                                                      int* __restrict__ eV1, __nv_bfloat16* __restrict__ V2,
                                                      int* __restrict__ eV2, int N, int p, int kpad, int mpad, size_t plane1,
@@ -351,7 +372,7 @@ __global__ void __launch_bounds__(256) k_qrt_slice_V(const double* __restrict__ 
             Vp[r * BPS + c] = k < N ? (r > k ? QR[(size_t)k * N + r] : (r == k ? 1.0 : 0.0)) : 0.0;
     }
     __syncthreads();
-    slice_V<BP, 256>(Vp, V1, eV1, V2, eV2, N, p, fbase + f, kpad, mpad, plane1, plane2);
+    slice_V<BP, 256, D>(Vp, V1, eV1, V2, eV2, N, p, fbase + f, kpad, mpad, plane1, plane2);
 }
 
 // ---- [G; W^T] = [V C]^T V, S from G, then W'^T = W^T S and its slices -----------------------
@@ -359,19 +380,20 @@ __global__ void __launch_bounds__(256) k_qrt_slice_V(const double* __restrict__ 
 // slices of V's columns (rows 0..BP-1, from the reflector slice buffer) above those of the CTA's
 // trailing columns of C, so the product's first BP rows are the panel's Gram matrix G = V^T V. The
 // epilogue forms the compact-WY triangle S from G (the panel kernel no longer does; CTA 0 writes it
-// out for the formation of Q), then W' = S^T W. TMA streams per 64-row K chunk the seven A slices
-// through a 3-tile ring and the seven V slices double-buffered; products (a, b), a + b <= 6, go to
-// the accumulator of level a + b of the chunk's segment (seven chunks per segment).
+// out for the formation of Q), then W' = S^T W. TMA streams per 64-row K chunk the D A slices
+// through a ring of tiles and the D V slices double-buffered; products (a, b), a + b <= D - 1, go to
+// the accumulator of level a + b of the chunk's segment (Dig<D>::kSegChunks chunks per segment).
 // kForm: the step of the formation of Q, whose panels need W' = S W with the S the QR left in Sall (the Gram rows
 // of the product are not used).
-template <int BP, bool kForm>
+template <int BP, bool kForm, int D>
 __global__ void __launch_bounds__(kQT, 2)
     k_qrt_gemm1(const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmV,
                 const int* __restrict__ eC, const int* __restrict__ eV1, const double* __restrict__ tau_all,
                 double* __restrict__ Sall, __nv_bfloat16* __restrict__ Ws, int* __restrict__ eW, int N, int p,
                 int n_t, int kpad, int jpad, int wpad, size_t planeW, int fbase, unsigned int* __restrict__ err) {
     constexpr uint32_t kTileB = BP * 128;
-    constexpr uint32_t kChunkB = kS * kTileB;
+    constexpr int kRing = Dig<D>::ring1(BP), kSegChunks = Dig<D>::kSegChunks;
+    constexpr uint32_t kChunkB = D * kTileB;
     constexpr int WS = BP + 1;
     constexpr int kMC = 128 - BP;  // trailing columns per CTA
     const int mt = blockIdx.x, f = blockIdx.y, gf = fbase + f;
@@ -410,7 +432,7 @@ __global__ void __launch_bounds__(kQT, 2)
         if (!kForm) tau_sh[threadIdx.x] = tau_all[(size_t)f * N + p + threadIdx.x];
     }
     const int nseg = (nkc + kSegChunks - 1) / kSegChunks;
-    const uint32_t tcols = nseg == 1 ? 256u : 512u;  // 7 levels x BP columns per accumulator set
+    const uint32_t tcols = nseg == 1 ? 256u : 512u;  // D levels x BP columns per accumulator set
     if (warp == 9) {
         tmem_alloc(smem_u32(&tmem_base_sh), tcols);
         tc_fence_before();
@@ -430,10 +452,10 @@ __global__ void __launch_bounds__(kQT, 2)
                 }
                 const uint32_t bb = smem_u32(&bar_bfull[bs]);
                 mbar_expect_tx(bb, kChunkB);
-                for (int b = 0; b < kS; ++b) tma_load_3d(bbuf + bs * kChunkB + b * kTileB, &tmV, kc * 64, gf * kVRows, b, bb);
+                for (int b = 0; b < D; ++b) tma_load_3d(bbuf + bs * kChunkB + b * kTileB, &tmV, kc * 64, gf * kVRows, b, bb);
                 issued_b = u + 1;
-                for (int a = 0; a < kS; ++a) {
-                    const int q = u * kS + a, slot = q % kRing;
+                for (int a = 0; a < D; ++a) {
+                    const int q = u * D + a, slot = q % kRing;
                     if (q >= kRing && !mbar_wait(smem_u32(&bar_empty[slot]), ((q / kRing) - 1) & 1, err)) {
                         abort_sh = 1;
                         break;
@@ -466,19 +488,19 @@ __global__ void __launch_bounds__(kQT, 2)
                 const uint64_t db = db0 + (uint64_t)bs * desc_step(kChunkB);
                 const bool first = u == seg * kSegChunks;
 #pragma unroll
-                for (int a = 0; a < kS; ++a) {
+                for (int a = 0; a < D; ++a) {
                     if (!ok || !mbar_wait(full0 + 8 * ring.slot, ring.phase, err) || abort_sh) {
                         ok = false;
                         continue;
                     }
                     tc_fence_after();
                     const uint64_t da = da0 + (uint64_t)ring.slot * desc_step(kTileA);
-                    // slices b = 0 .. 6 - a of V into the levels a .. 6: adjacent operand rows and adjacent
-                    // accumulators, so one instruction of N = (7 - a) BP per step of K
+                    // slices b = 0 .. D - 1 - a of V into the levels a .. D - 1: adjacent operand rows and adjacent
+                    // accumulators, so one instruction of N = (D - a) BP per step of K
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
-                        mma_bf16(tmem + (uint32_t)((seg * kLv + a) * BP), da + desc_step(ks * 32), db + desc_step(ks * 32),
-                                 idesc_f32acc(1, 128, (kS - a) * BP), (a | ks) != 0 || !first ? 1u : 0u);
+                        mma_bf16(tmem + (uint32_t)((seg * D + a) * BP), da + desc_step(ks * 32), db + desc_step(ks * 32),
+                                 idesc_f32acc(1, 128, (D - a) * BP), (a | ks) != 0 || !first ? 1u : 0u);
                     mma_commit(empty0 + 8 * ring.slot);
                     ring.next(kRing);
                 }
@@ -513,18 +535,18 @@ __global__ void __launch_bounds__(kQT, 2)
 #pragma unroll
                 for (int c = 0; c < 8; ++c) hi[c] = lo[c] = 0;
                 for (int sg = 0; sg < nseg; ++sg) {
-                    uint32_t v[kLv][8];
-                    const uint32_t tl = tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(sg * kLv * BP + h * HC + c0);
+                    uint32_t v[D][8];
+                    const uint32_t tl = tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(sg * D * BP + h * HC + c0);
 #pragma unroll
-                    for (int lv = 0; lv < kLv; ++lv) tmem_ld8(tl + (uint32_t)(lv * BP), v[lv]);
+                    for (int lv = 0; lv < D; ++lv) tmem_ld8(tl + (uint32_t)(lv * BP), v[lv]);
                     tmem_ld_wait();
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
-                        uint32_t w[kLv];
+                        uint32_t w[D];
 #pragma unroll
-                        for (int lv = 0; lv < kLv; ++lv) w[lv] = v[lv][c];
+                        for (int lv = 0; lv < D; ++lv) w[lv] = v[lv][c];
                         long long a, b;
-                        levels_to_int(w, a, b);
+                        levels_to_int<D>(w, a, b);
                         hi[c] += a;
                         lo[c] += b;
                     }
@@ -532,7 +554,7 @@ __global__ void __launch_bounds__(kQT, 2)
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     const int m = h * HC + c0 + c;
-                    stW[r * WS + m] = combine(hi[c], lo[c], er + eV_sh[m] - kUnitShift);
+                    stW[r * WS + m] = combine(hi[c], lo[c], er + eV_sh[m] - Dig<D>::kUnitShift);
                 }
             }
         }
@@ -572,11 +594,11 @@ __global__ void __launch_bounds__(kQT, 2)
                 const int e = exponent_of_bits(warp_max_bits(abs_bits(v)));
                 if (lane == 0) eW[(size_t)gf * wpad + j2] = e;
                 if (lane < BP) {
-                    float q[kS];
-                    slice7(v, e, q);
+                    float q[D];
+                    cut<D>(v, e, q);
                     __nv_bfloat16* dst = Ws + ((size_t)gf * wpad + j2) * 64 + lane;
 #pragma unroll
-                    for (int s = 0; s < kS; ++s) dst[(size_t)s * planeW] = bf16_of(q[s]);
+                    for (int s = 0; s < D; ++s) dst[(size_t)s * planeW] = bf16_of(q[s]);
                 }
             }
         }
@@ -589,11 +611,11 @@ __global__ void __launch_bounds__(kQT, 2)
 
 // ---- C -= V W' -----------------------------------------------------------------------------
 // CTA = 128 rows (row tile p/128 + blockIdx.y) x kNC trailing columns of one field; one K chunk (BP
-// reflectors): the seven W' slices resident, the seven V slices streamed through the 3-tile ring.
-// 32 columns keep the accumulators at 7 x 32 tensor-memory columns, so two CTAs share an SM.
+// reflectors): the D W' slices resident, the D V slices streamed through the 3-tile ring.
+// 32 columns keep the accumulators at D x 32 <= 256 tensor-memory columns, so two CTAs share an SM.
 constexpr int kNC = 32;
 
-template <int BP>
+template <int BP, int D>
 __global__ void __launch_bounds__(kQT, 2)
     k_qrt_gemm2(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmW,
                 const int* __restrict__ eV2, const int* __restrict__ eW, const int* __restrict__ perm_all,
@@ -610,7 +632,7 @@ __global__ void __launch_bounds__(kQT, 2)
     __shared__ int col_sh[kNC];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    const uint32_t bbuf = base, aring = base + kS * kTileW;
+    const uint32_t bbuf = base, aring = base + D * kTileW;
 
     if (threadIdx.x == 0) {
         for (int q = 0; q < kRing; ++q) {
@@ -639,10 +661,10 @@ __global__ void __launch_bounds__(kQT, 2)
     if (warp == 8) {
         if (lane == 0) {
             const uint32_t bb = smem_u32(&bar_bfull);
-            mbar_expect_tx(bb, kS * kTileW);
-            for (int b = 0; b < kS; ++b) tma_load_3d(bbuf + b * kTileW, &tmW, 0, gf * wpad + nt * kNC, b, bb);
+            mbar_expect_tx(bb, D * kTileW);
+            for (int b = 0; b < D; ++b) tma_load_3d(bbuf + b * kTileW, &tmW, 0, gf * wpad + nt * kNC, b, bb);
             int issued = 0;
-            for (int a = 0; a < kS; ++a) {
+            for (int a = 0; a < D; ++a) {
                 const int slot = a % kRing;
                 if (a >= kRing && !mbar_wait(smem_u32(&bar_empty[slot]), ((a / kRing) - 1) & 1, err)) break;
                 const uint32_t fb = smem_u32(&bar_full[slot]);
@@ -660,7 +682,7 @@ __global__ void __launch_bounds__(kQT, 2)
             bool ok = mbar_wait(smem_u32(&bar_bfull), 0, err);
             const uint64_t da0 = smem_desc_sw128(aring), db0 = smem_desc_sw128(bbuf);
 #pragma unroll
-            for (int a = 0; a < kS; ++a) {
+            for (int a = 0; a < D; ++a) {
                 const int slot = a % kRing;
                 if (!ok || !mbar_wait(smem_u32(&bar_full[slot]), (a / kRing) & 1, err)) {
                     ok = false;
@@ -670,7 +692,7 @@ __global__ void __launch_bounds__(kQT, 2)
 #pragma unroll
                 for (int ks = 0; ks < BP / 16; ++ks)
                     mma_bf16(tmem + (uint32_t)(a * kNC), da0 + desc_step(slot * kTileA + ks * 32), db0 + desc_step(ks * 32),
-                             idesc_f32acc(1, 128, (kS - a) * kNC), (a | ks) != 0 ? 1u : 0u);
+                             idesc_f32acc(1, 128, (D - a) * kNC), (a | ks) != 0 ? 1u : 0u);
                 mma_commit(smem_u32(&bar_empty[slot]));
             }
             if (ok) mma_commit(smem_u32(&bar_acc));
@@ -701,22 +723,22 @@ __global__ void __launch_bounds__(kQT, 2)
             tc_fence_after();
 #pragma unroll
             for (int c0 = 0; c0 < HC; c0 += 8) {
-                uint32_t v[kLv][8];
+                uint32_t v[D][8];
                 const uint32_t tl = tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(HC * h + c0);
 #pragma unroll
-                for (int lv = 0; lv < kLv; ++lv) tmem_ld8(tl + (uint32_t)(lv * kNC), v[lv]);
+                for (int lv = 0; lv < D; ++lv) tmem_ld8(tl + (uint32_t)(lv * kNC), v[lv]);
                 if (c0 > 0) fetch(c0);
                 tmem_ld_wait();
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     const int cc = HC * h + c0 + c;
                     if (!row_ok || nt * kNC + cc >= n_t) continue;
-                    uint32_t w[kLv];
+                    uint32_t w[D];
 #pragma unroll
-                    for (int lv = 0; lv < kLv; ++lv) w[lv] = v[lv][c];
+                    for (int lv = 0; lv < D; ++lv) w[lv] = v[lv][c];
                     long long hi, lo;
-                    small_levels_to_int(w, hi, lo);
-                    Yf[(size_t)col_sh[cc] * N] = y[c] - combine(hi, lo, ev + eW_sh[cc] - kUnitShift);
+                    small_levels_to_int<D>(w, hi, lo);
+                    Yf[(size_t)col_sh[cc] * N] = y[c] - combine(hi, lo, ev + eW_sh[cc] - Dig<D>::kUnitShift);
                 }
             }
         }
@@ -727,8 +749,10 @@ __global__ void __launch_bounds__(kQT, 2)
     if (warp == 9) tmem_dealloc(tmem, 256);
 }
 
-size_t gemm1_smem(int BP) { return 1024 + 2 * (size_t)kS * BP * 128 + (size_t)kRing * kTileA; }
-size_t gemm2_smem() { return 1024 + (size_t)kS * kNC * 128 + (size_t)kRing * kTileA; }
+template <int D>
+size_t gemm1_smem(int BP) { return 1024 + 2 * (size_t)D * BP * 128 + (size_t)Dig<D>::ring1(BP) * kTileA; }
+template <int D>
+size_t gemm2_smem() { return 1024 + (size_t)D * kNC * 128 + (size_t)kRing * kTileA; }
 
 struct QrtArgs {
     int N, kpad, mpad, wpad, jpad;
@@ -773,19 +797,19 @@ cudaError_t launch_panel(slmc_ctx* c, int nf, int t, cudaStream_t s) {
 template <int BP>
 cudaError_t launch_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s) {
     const QrtArgs a = qrt_args(c);
-    const size_t sm1 = gemm1_smem(BP), sm2 = gemm2_smem();
-    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_gemm2<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+    const size_t sm1 = gemm1_smem<7>(BP), sm2 = gemm2_smem<7>();
+    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP, false, 7>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_gemm2<BP, 7>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
     if (e != cudaSuccess) return e;
     const CUtensorMap& mapV1 = BP == 32 ? c->qt_mapV1_32 : c->qt_mapV1_16;
     const int N = a.N, p = t * BP, j0 = p + BP, n_t = N - j0;
-    k_qrt_slice_C<<<dim3((n_t + 7) / 8, nf), 256, 0, s>>>(c->Y, c->perm, a.Cs, c->qt_eC, N, p, j0, a.kpad, a.jpad,
+    k_qrt_slice_C<7><<<dim3((n_t + 7) / 8, nf), 256, 0, s>>>(c->Y, c->perm, a.Cs, c->qt_eC, N, p, j0, a.kpad, a.jpad,
                                                           a.planeC, c->fbase);
     const CUtensorMap& mapC = BP == 32 ? c->qt_mapC96 : c->qt_mapC112;
-    k_qrt_gemm1<BP, false><<<dim3((n_t + 127 - BP) / (128 - BP), nf), kQT, sm1, s>>>(
+    k_qrt_gemm1<BP, false, 7><<<dim3((n_t + 127 - BP) / (128 - BP), nf), kQT, sm1, s>>>(
         mapC, mapV1, c->qt_eC, c->qt_eV1, c->tau, c->Sws, a.Ws, c->qt_eW, N, p, n_t, a.kpad, a.jpad, a.wpad, a.planeW,
         c->fbase, c->err);
-    k_qrt_gemm2<BP><<<dim3((n_t + kNC - 1) / kNC, a.mpad / 128 - p / 128, nf), kQT, sm2, s>>>(
+    k_qrt_gemm2<BP, 7><<<dim3((n_t + kNC - 1) / kNC, a.mpad / 128 - p / 128, nf), kQT, sm2, s>>>(
         c->qt_mapV2, c->qt_mapW, c->qt_eV2, c->qt_eW, c->perm, c->Y, N, p, j0, n_t, a.mpad, a.wpad, c->fbase, c->err);
     return cudaGetLastError();
 }
@@ -796,31 +820,34 @@ __global__ void __launch_bounds__(256) k_qrt_identity(double* __restrict__ U, in
 }
 
 // Q = Q_0 Q_1 ... accumulated backwards into U: per panel, columns and rows p.. of U take I - V S V^T through the
-// products of the trailing update (slices of V and of U's columns, W = V^T U, W' = S W, U -= V W'). On the FP64 pipe
-// (k_formq_b) the 4/3 N^3 flops were 30-45 % of an FP64 evaluation and of a DQMC sweep's chain steps: 12x12,
-// L = 120, 256 fields with G 65.9 -> 55.5 ms; 18x10, L = 37, 50 fields 13.5 -> 11.4 ms (four Q: 4.0 -> 2.0 ms).
+// products of the trailing update (slices of V and of U's columns, W = V^T U, W' = S W, U -= V W'), with eight digits:
+// Q then is as near to the exact one as by FP64 FMAs, and G errs by the QR's and the T update's 49 bits only (T by FMAs,
+// error of G against extended precision: 18x18, L = 30 1.41e-13 with FMAs or eight digits, 1.71e-13 with
+// seven; 18x10, L = 37 2.07 / 2.07 / 2.15e-13; 12x12, L = 40 1.38 / 1.38 / 1.44e-13). On the FP64 pipe
+// (k_formq_b) the 4/3 N^3 flops were 30-45 % of an FP64 evaluation: 12x12, L = 120, 256 fields with G take 62 ms that
+// way, 53.0 with eight digits and 51.7 with seven; 18x10, L = 37, 50 fields 13.3, 11.3 and 11.2 ms.
 template <int BP>
 cudaError_t launch_form_q(slmc_ctx* c, int nf, cudaStream_t s) {
     const QrtArgs a = qrt_args(c);
     const int N = a.N;
-    const size_t sm1 = gemm1_smem(BP), sm2 = gemm2_smem(), smV = sizeof(double) * (size_t)N * (BP + 1);
-    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_gemm2<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_slice_V<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smV);
+    const size_t sm1 = gemm1_smem<8>(BP), sm2 = gemm2_smem<8>(), smV = sizeof(double) * (size_t)N * (BP + 1);
+    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP, true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_gemm2<BP, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_slice_V<BP, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smV);
     if (e != cudaSuccess) return e;
     const CUtensorMap& mapV1 = BP == 32 ? c->qt_mapV1_32 : c->qt_mapV1_16;
     const CUtensorMap& mapC = BP == 32 ? c->qt_mapC96 : c->qt_mapC112;
     k_qrt_identity<<<dim3(std::min(64, (N * N + 1023) / 1024), nf), 256, 0, s>>>(c->U, N);
     for (int p = (N - 1) / BP * BP; p >= 0; p -= BP) {
         const int n_t = N - p;
-        k_qrt_slice_V<BP><<<nf, 256, sizeof(double) * (size_t)n_t * (BP + 1), s>>>(
+        k_qrt_slice_V<BP, 8><<<nf, 256, sizeof(double) * (size_t)n_t * (BP + 1), s>>>(
             c->QR, a.V1, c->qt_eV1, a.V2, c->qt_eV2, N, p, a.kpad, a.mpad, a.plane1, a.plane2, c->fbase);
-        k_qrt_slice_C<<<dim3((n_t + 7) / 8, nf), 256, 0, s>>>(c->U, nullptr, a.Cs, c->qt_eC, N, p, p, a.kpad, a.jpad, a.planeC,
+        k_qrt_slice_C<8><<<dim3((n_t + 7) / 8, nf), 256, 0, s>>>(c->U, nullptr, a.Cs, c->qt_eC, N, p, p, a.kpad, a.jpad, a.planeC,
                                                               c->fbase);
-        k_qrt_gemm1<BP, true><<<dim3((n_t + 127 - BP) / (128 - BP), nf), kQT, sm1, s>>>(
+        k_qrt_gemm1<BP, true, 8><<<dim3((n_t + 127 - BP) / (128 - BP), nf), kQT, sm1, s>>>(
             mapC, mapV1, c->qt_eC, c->qt_eV1, c->tau, c->Sws, a.Ws, c->qt_eW, N, p, n_t, a.kpad, a.jpad, a.wpad, a.planeW,
             c->fbase, c->err);
-        k_qrt_gemm2<BP><<<dim3((n_t + kNC - 1) / kNC, a.mpad / 128 - p / 128, nf), kQT, sm2, s>>>(
+        k_qrt_gemm2<BP, 8><<<dim3((n_t + kNC - 1) / kNC, a.mpad / 128 - p / 128, nf), kQT, sm2, s>>>(
             c->qt_mapV2, c->qt_mapW, c->qt_eV2, c->qt_eW, nullptr, c->U, N, p, p, n_t, a.mpad, a.wpad, c->fbase, c->err);
     }
     return cudaGetLastError();
@@ -835,7 +862,7 @@ bool qrt_supported(int N) { return N >= 2 && N <= kMaxN; }
 // Sizes of the slice buffers (BF16 elements) and exponent arrays of a context with F fields.
 void qrt_sizes(int N, int F, size_t* bf16_elems, size_t* int_elems) {
     const size_t kpad = (N + 63) / 64 * 64, mpad = (N + 127) / 128 * 128, wpad = kpad;
-    *bf16_elems = (size_t)kS * F * (mpad * kpad + kVRows * kpad + mpad * 64 + wpad * 64);
+    *bf16_elems = (size_t)kDMax * F * (mpad * kpad + kVRows * kpad + mpad * 64 + wpad * 64);
     *int_elems = (size_t)F * (mpad + kVRows + mpad + wpad + 1);
 }
 
@@ -850,13 +877,13 @@ cudaError_t qrt_init(slmc_ctx* c, void* bf16_base, int* int_base) {
     const size_t kpad = c->qt_kpad, mpad = c->qt_mpad, wpad = c->qt_wpad;
     __nv_bfloat16* b = reinterpret_cast<__nv_bfloat16*>(bf16_base);
     c->qt_C = b;
-    b += (size_t)kS * F * mpad * kpad;
+    b += (size_t)kDMax * F * mpad * kpad;
     c->qt_V1 = b;
-    b += (size_t)kS * F * kVRows * kpad;
+    b += (size_t)kDMax * F * kVRows * kpad;
     c->qt_V2 = b;
-    b += (size_t)kS * F * mpad * 64;
+    b += (size_t)kDMax * F * mpad * 64;
     c->qt_W = b;
-    b += (size_t)kS * F * wpad * 64;
+    b += (size_t)kDMax * F * wpad * 64;
     c->qt_eC = int_base;
     c->qt_eV1 = c->qt_eC + F * mpad;
     c->qt_eV2 = c->qt_eV1 + F * kVRows;
@@ -867,12 +894,12 @@ cudaError_t qrt_init(slmc_ctx* c, void* bf16_base, int* int_base) {
     cudaError_t e = cudaMemset(bf16_base, 0, nb16 * sizeof(__nv_bfloat16));
     if (e == cudaSuccess) e = cudaMemset(int_base, 0, nint * sizeof(int));
     if (e != cudaSuccess) return e;
-    if (!make_map_sw128(&c->qt_mapC96, c->qt_C, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kpad, F * mpad, kS, 96) ||
-        !make_map_sw128(&c->qt_mapC112, c->qt_C, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kpad, F * mpad, kS, 112) ||
-        !make_map_sw128(&c->qt_mapV1_32, c->qt_V1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kpad, F * kVRows, kS, 32) ||
-        !make_map_sw128(&c->qt_mapV1_16, c->qt_V1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kpad, F * kVRows, kS, 16) ||
-        !make_map_sw128(&c->qt_mapV2, c->qt_V2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 64, F * mpad, kS, 128) ||
-        !make_map_sw128(&c->qt_mapW, c->qt_W, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 64, F * wpad, kS, kNC))
+    if (!make_map_sw128(&c->qt_mapC96, c->qt_C, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kpad, F * mpad, kDMax, 96) ||
+        !make_map_sw128(&c->qt_mapC112, c->qt_C, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kpad, F * mpad, kDMax, 112) ||
+        !make_map_sw128(&c->qt_mapV1_32, c->qt_V1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kpad, F * kVRows, kDMax, 32) ||
+        !make_map_sw128(&c->qt_mapV1_16, c->qt_V1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kpad, F * kVRows, kDMax, 16) ||
+        !make_map_sw128(&c->qt_mapV2, c->qt_V2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 64, F * mpad, kDMax, 128) ||
+        !make_map_sw128(&c->qt_mapW, c->qt_W, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 64, F * wpad, kDMax, kNC))
         return cudaErrorInvalidValue;
     return cudaSuccess;
 }

@@ -296,7 +296,7 @@ SLMC_API int slmc_set_dense_slices(slmc_ctx* ctx, int dense);
  *            below 2^-48 of their row and column scales.
  *   path = 1: FP64 FMAs (tiled triangular GEMM).
  *   path = 2: the tensor-core kernel with every tile on its FP64 fallback (for tests).
- * The DQMC updates use the same path for N > 64 and path 1 up to there. Errors: SLMC_ERR_ARG for other values. */
+ * The DQMC updates always use path 1. Errors: SLMC_ERR_ARG for other values. */
 SLMC_API int slmc_set_tupdate_path(slmc_ctx* ctx, int path);
 
 /* How the pre-pivoted blocked QR (qr_mode SLMC_QR_PREPIVOT) applies each panel's block of BP
@@ -314,8 +314,8 @@ SLMC_API int slmc_set_tupdate_path(slmc_ctx* ctx, int path);
  *            per panel on the caller's stream. For N > 64 Q is formed in FP64 through such products with
  *            eight digits (56 bits, as near to the exact Q as by FP64 FMAs; 4 more launches per panel).
  *   path = 1: the one-kernel FP64 QR (trailing updates with FP64 FMAs), Q formed with FP64 FMAs.
- * The DQMC updates follow it for N > 64 (the one-kernel QR up to there); qr_mode SLMC_QR_PIVOTED is
- * unaffected. Errors: SLMC_ERR_ARG for other
+ * The DQMC updates follow it for N > 64, on path 0 with eight digits in the trailing updates too (the one-kernel QR up
+ * to there), so that G is as accurate on either path; qr_mode SLMC_QR_PIVOTED is unaffected. Errors: SLMC_ERR_ARG for other
  * values, SLMC_ERR_UNSUPPORTED for path 0 when N > 896. */
 SLMC_API int slmc_set_qr_path(slmc_ctx* ctx, int path);
 

@@ -668,29 +668,29 @@ int slmc_cumulative_update(slmc_ctx* c, double* x, int n, const double* J, int n
 }
 
 namespace {
-// One FP64 step of the stabilised chain on the product already in Y: pivoted QR, Q, T, on the same paths as the
-// determinant's. At N <= 64 the one-kernel QR and the FP64 T update have fewer launches than the work is worth.
+// One FP64 step of the stabilised chain on the product already in Y: pivoted QR, Q, T. QR and Q through the tensor
+// products of the determinant's QR with eight digits, T by FP64 FMAs: the Green's functions that these chains
+// form decide every local move, and 49 bits in QR and T left them up to 100 times further off (error of G against
+// extended precision, QR and Q by FMAs / eight digits: 9x8, L = 40 4.4e-15 / 4.5e-15, 16x16, L = 160 3.2e-14 / 3.2e-14; all
+// with seven 5.5e-13, 3.9e-12). A sweep of 152 chains of 12x12, L = 120: 181 ms, 201 with QR and Q by FMAs, 161
+// with seven digits throughout. At N <= 64 the one-kernel QR has fewer launches than the work is worth.
 int chain_step64(slmc_ctx* c, int nf, cudaStream_t s) {
     c->cur_units = nf;
-    const bool tc = slmc::qrt_form_q_active(c);
     if (c->p.qr_mode == SLMC_QR_PIVOTED) {
         SLMC_LAUNCH(SLMC_PROF_QR, 1, s, slmc::qr_pivoted(c, nf, s));
         SLMC_LAUNCH(SLMC_PROF_FORMQ, 1, s, slmc::form_q(c, nf, s));
-    } else if (tc) {
+    } else if (slmc::qrt_form_q_active(c)) {
         const int np = slmc::qrt_panels(c);
         for (int t = 0; t < np; ++t) {
-            SLMC_LAUNCH(SLMC_PROF_QR, 1, s, slmc::qrt_panel(c, nf, t, s));
-            if (t + 1 < np) SLMC_LAUNCH(SLMC_PROF_QRTC, 3, s, slmc::qrt_trailing(c, nf, t, s));
+            SLMC_LAUNCH(SLMC_PROF_QR, 1, s, slmc::qrt_panel(c, nf, t, s, true));
+            if (t + 1 < np) SLMC_LAUNCH(SLMC_PROF_QRTC, 3, s, slmc::qrt_trailing(c, nf, t, s, true));
         }
         SLMC_LAUNCH(SLMC_PROF_FORMQ, slmc::qrt_form_q_launches(c), s, slmc::qrt_form_q(c, nf, s));
     } else {
         SLMC_LAUNCH(SLMC_PROF_QR, 1, s, slmc::qr_blocked(c, nf, s));
         SLMC_LAUNCH(SLMC_PROF_FORMQ, 1, s, slmc::form_q_blocked(c, nf, false, s));
     }
-    if (tc)
-        SLMC_LAUNCH(SLMC_PROF_TUPDATE, slmc::t_update_launches(c), s, slmc::t_update(c, nf, s));
-    else
-        SLMC_LAUNCH(SLMC_PROF_TUPDATE, 1, s, slmc::t_update_tiled(c, nf, s));
+    SLMC_LAUNCH(SLMC_PROF_TUPDATE, 1, s, slmc::t_update_tiled(c, nf, s));
     return SLMC_OK;
 }
 

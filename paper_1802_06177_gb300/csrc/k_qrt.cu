@@ -57,8 +57,8 @@ constexpr int kVRows = 32;                   // rows of the V1 slice buffer per 
 constexpr int kRing = 3;
 constexpr int kDMax = 8;
 
-// What depends on the number of digits D per operand: seven (49 bits, the trailing updates) or eight (56 bits, the
-// formation of Q in FP64; oz_line.cuh's digits). Products a + b <= D - 1 in D levels.
+// What depends on the number of digits D per operand: seven (49 bits, the trailing updates) or eight (56 bits, Q in
+// FP64 and the trailing updates of the DQMC chains; oz_line.cuh's digits). Products a + b <= D - 1 in D levels.
 template <int D>
 struct Dig {
     // K chunks (64 rows) per accumulator set of W^T = C^T V: a level's sum of absolute terms is at most 36864 per K
@@ -219,7 +219,7 @@ __device__ __forceinline__ void slice_V(const double* Vp, __nv_bfloat16* __restr
     }
 }
 
-template <int BP, int kPT>
+template <int BP, int kPT, int D>
 __global__ void __launch_bounds__(kPT, kPT == 256 ? 3 : 1)
     k_qrt_panel(double* __restrict__ Yall, double* __restrict__ lnD_all, double* __restrict__ QRall,
                 double* __restrict__ tau_all, int* __restrict__ perm_all, int* __restrict__ sgnU,
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kPT, kPT == 256 ? 3 : 1)
         if (bad) atomicOr(err, SLMC_EBIT_NONFINITE);
         return;
     }
-    slice_V<BP, kPT, 7>(Vp, V1, eV1, V2, eV2, N, p, gf, kpad, mpad, plane1, plane2);
+    slice_V<BP, kPT, D>(Vp, V1, eV1, V2, eV2, N, p, gf, kpad, mpad, plane1, plane2);
 }
 
 // ---- slices of the trailing columns ---------------------------------------------------------
@@ -779,37 +779,37 @@ QrtArgs qrt_args(const slmc_ctx* c) {
     return a;
 }
 
-template <int BP, int kPT>
+template <int BP, int kPT, int D>
 cudaError_t launch_panel(slmc_ctx* c, int nf, int t, cudaStream_t s) {
     const QrtArgs a = qrt_args(c);
     const int p = t * BP;
     const size_t smP = PanelSmem<BP>::bytes(a.N, p, p + BP >= a.N);
-    cudaError_t e = cudaFuncSetAttribute(k_qrt_panel<BP, kPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_qrt_panel<BP, kPT, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)std::max(PanelSmem<BP>::bytes(a.N, 0, a.N <= BP), smP));
     if (e != cudaSuccess) return e;
-    k_qrt_panel<BP, kPT><<<nf, kPT, smP, s>>>(c->Y, c->lnD, c->QR, c->tau, c->perm, c->sgnU, c->Sws, c->err, a.N, t,
+    k_qrt_panel<BP, kPT, D><<<nf, kPT, smP, s>>>(c->Y, c->lnD, c->QR, c->tau, c->perm, c->sgnU, c->Sws, c->err, a.N, t,
                                               c->qt_lnDn, c->qt_ntriv, a.V1, c->qt_eV1, a.V2, c->qt_eV2, a.kpad,
                                               a.mpad, a.plane1, a.plane2, c->fbase);
     return cudaGetLastError();
 }
 
 // Trailing update of panel t (t < last panel): slices of C, W'^T = (C^T V) S, C -= V W'.
-template <int BP>
+template <int BP, int D>
 cudaError_t launch_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s) {
     const QrtArgs a = qrt_args(c);
-    const size_t sm1 = gemm1_smem<7>(BP), sm2 = gemm2_smem<7>();
-    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP, false, 7>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_gemm2<BP, 7>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+    const size_t sm1 = gemm1_smem<D>(BP), sm2 = gemm2_smem<D>();
+    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP, false, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_gemm2<BP, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
     if (e != cudaSuccess) return e;
     const CUtensorMap& mapV1 = BP == 32 ? c->qt_mapV1_32 : c->qt_mapV1_16;
     const int N = a.N, p = t * BP, j0 = p + BP, n_t = N - j0;
-    k_qrt_slice_C<7><<<dim3((n_t + 7) / 8, nf), 256, 0, s>>>(c->Y, c->perm, a.Cs, c->qt_eC, N, p, j0, a.kpad, a.jpad,
+    k_qrt_slice_C<D><<<dim3((n_t + 7) / 8, nf), 256, 0, s>>>(c->Y, c->perm, a.Cs, c->qt_eC, N, p, j0, a.kpad, a.jpad,
                                                           a.planeC, c->fbase);
     const CUtensorMap& mapC = BP == 32 ? c->qt_mapC96 : c->qt_mapC112;
-    k_qrt_gemm1<BP, false, 7><<<dim3((n_t + 127 - BP) / (128 - BP), nf), kQT, sm1, s>>>(
+    k_qrt_gemm1<BP, false, D><<<dim3((n_t + 127 - BP) / (128 - BP), nf), kQT, sm1, s>>>(
         mapC, mapV1, c->qt_eC, c->qt_eV1, c->tau, c->Sws, a.Ws, c->qt_eW, N, p, n_t, a.kpad, a.jpad, a.wpad, a.planeW,
         c->fbase, c->err);
-    k_qrt_gemm2<BP, 7><<<dim3((n_t + kNC - 1) / kNC, a.mpad / 128 - p / 128, nf), kQT, sm2, s>>>(
+    k_qrt_gemm2<BP, D><<<dim3((n_t + kNC - 1) / kNC, a.mpad / 128 - p / 128, nf), kQT, sm2, s>>>(
         c->qt_mapV2, c->qt_mapW, c->qt_eV2, c->qt_eW, c->perm, c->Y, N, p, j0, n_t, a.mpad, a.wpad, c->fbase, c->err);
     return cudaGetLastError();
 }
@@ -921,14 +921,25 @@ int qrt_panels(const slmc_ctx* c) {
     return (c->N + BP - 1) / BP;
 }
 
-cudaError_t qrt_panel(slmc_ctx* c, int nf, int t, cudaStream_t s) {
+namespace {
+template <int D>
+cudaError_t panel(slmc_ctx* c, int nf, int t, cudaStream_t s) {
     if (nf <= c->num_sms)
-        return qr_panel_width(c) == 32 ? launch_panel<32, 512>(c, nf, t, s) : launch_panel<16, 512>(c, nf, t, s);
-    return qr_panel_width(c) == 32 ? launch_panel<32, 256>(c, nf, t, s) : launch_panel<16, 256>(c, nf, t, s);
+        return qr_panel_width(c) == 32 ? launch_panel<32, 512, D>(c, nf, t, s) : launch_panel<16, 512, D>(c, nf, t, s);
+    return qr_panel_width(c) == 32 ? launch_panel<32, 256, D>(c, nf, t, s) : launch_panel<16, 256, D>(c, nf, t, s);
+}
+template <int D>
+cudaError_t trailing(slmc_ctx* c, int nf, int t, cudaStream_t s) {
+    return qr_panel_width(c) == 32 ? launch_trailing<32, D>(c, nf, t, s) : launch_trailing<16, D>(c, nf, t, s);
+}
+}  // namespace
+
+cudaError_t qrt_panel(slmc_ctx* c, int nf, int t, cudaStream_t s, bool eight) {
+    return eight ? panel<8>(c, nf, t, s) : panel<7>(c, nf, t, s);
 }
 
-cudaError_t qrt_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s) {
-    return qr_panel_width(c) == 32 ? launch_trailing<32>(c, nf, t, s) : launch_trailing<16>(c, nf, t, s);
+cudaError_t qrt_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s, bool eight) {
+    return eight ? trailing<8>(c, nf, t, s) : trailing<7>(c, nf, t, s);
 }
 
 }  // namespace slmc

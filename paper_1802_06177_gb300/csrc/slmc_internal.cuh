@@ -211,8 +211,9 @@ void qrt_sizes(int N, int F, size_t* bf16_elems, size_t* int_elems);
 cudaError_t qrt_init(slmc_ctx* c, void* bf16_base, int* int_base);
 bool qrt_active(const slmc_ctx* c);
 int qrt_panels(const slmc_ctx* c);
-cudaError_t qrt_panel(slmc_ctx* c, int nf, int t, cudaStream_t s);     // factor panel t (1 launch)
-cudaError_t qrt_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s);  // its trailing update (3 launches)
+// factor panel t (1 launch) and its trailing update (3 launches), with seven or eight digits per operand
+cudaError_t qrt_panel(slmc_ctx* c, int nf, int t, cudaStream_t s, bool eight = false);
+cudaError_t qrt_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s, bool eight = false);
 bool qrt_form_q_active(const slmc_ctx* c);
 int qrt_form_q_launches(const slmc_ctx* c);
 cudaError_t qrt_form_q(slmc_ctx* c, int nf, cudaStream_t s);  // Q (FP64) of the last QR into U

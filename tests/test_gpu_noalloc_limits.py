@@ -23,3 +23,20 @@ def test_largest_fp32_field_of_529_sites():
     with pytest.raises(SlmcError) as e:
         logdet_noalloc(x, Lx, Lx, L + 1, n_s=n_s, precision="fp32")
     assert e.value.status == 5
+
+
+@pytest.mark.parametrize("Lx,Ly,L,n_s,qr_mode,general", [(4, 4, 40, 10, "prepivot", False), (8, 8, 20, 6, "prepivot", False),
+                                                         (9, 8, 40, 10, "prepivot", True), (4, 4, 40, 10, "pivoted", True)])
+def test_fp64_arithmetic_is_the_documented_one(Lx, Ly, L, n_s, qr_mode, general):
+    """The one-launch determinant up to 64 sites, the general kernels with FP64 FMAs above and in the pivoted mode."""
+    from paper_1802_06177_gb300.slmc import logdet_noalloc
+    x = cuda(inputs.mixed_fields(5, Lx, Ly, L, seed=12))
+    got, sg = logdet_noalloc(x, Lx, Ly, L, n_s=n_s, qr_mode=qr_mode)
+    ctx = make_ctx(Lx, L, n_s, Ly=Ly, max_fields=5, qr_mode=qr_mode)
+    if general:
+        ctx.set_tupdate_path(1)
+        ctx.set_qr_path(1)
+    n0 = ctx.launch_count()
+    want, sw = ctx.logdet(x)
+    assert (ctx.launch_count() - n0 > 1) == general
+    assert torch.equal(got, want) and torch.equal(sg, sw)

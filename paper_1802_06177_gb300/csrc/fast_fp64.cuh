@@ -9,7 +9,8 @@ namespace slmc {
 // Square root and quotient of normal numbers of moderate exponent (others take the library's) by Newton steps from an
 // FP32 estimate of the significand: Goldschmidt's coupled iteration for the root with a final residual correction,
 // Newton's for the reciprocal and Markstein's correction of the quotient. Six and five FP64 instructions; results
-// are within one unit in the last place of the correctly rounded ones (10^8 random arguments).
+// are within one unit in the last place of the correctly rounded ones, for any FP32 estimate within the documented two
+// units of rsqrtf (tests/test_fast_fp64.py).
 __device__ __forceinline__ double fast_sqrt(double a) {
     const int hi = __double2hiint(a), ex = (hi >> 20) - 1023;
     if (ex < -900 || ex > 900) return sqrt(a);

@@ -17,9 +17,9 @@
 //    along y commute); the mu factors of B_l and B_l^-1 cancel, and the wrap becomes four
 //    in-place circulant transforms along the lines of G, folded by the factor's symmetry
 //    (circ.cuh): about N^2 (Lx + Ly) FP64 operations instead of the 4 N^3 of two dense products;
-//  * G stays in shared memory when it fits (N <= 160), else in global memory (L2-resident). For N > 64 the
-//    accepted moves of a slice are delayed in batches (Ad, Bd in shared memory, with the running diagonal of G for
-//    the decisions): each new move needs only the current column and row of G, and the batch is added to G in one
+//  * G stays in shared memory when it and the vectors beside it fit in 227 KB (up to N = 165), else in global memory
+//    (L2-resident). For N > 64 the accepted moves of a slice are delayed in batches (Ad, Bd in shared memory, with the
+//    running diagonal of G for the decisions) where there is room for them (up to N = 147): each new move needs only the current column and row of G, and the batch is added to G in one
 //    pass. With G in shared memory a batch is 16 moves, one K step of the tensor-instruction update of oz_line.cuh
 //    (each entry's sum of 16 products rounded once, 56-bit digits): the N^2 FMAs per move were most of the kernel
 //    (40 slices, 128 chains, immediate / batched: 12x12 34.2 / 23.8 ms, 10x10 16.7 / 12.8, 9x8 8.6 / 7.9, 8x8 5.6 /
@@ -527,7 +527,7 @@ cudaError_t launch_slices(slmc_ctx* c, double* x, double* G, int nf, int chain0,
     const bool in_smem = dqmc_smem_bytes(c->N, nc, true) <= (size_t)optin;
     // Batches of up to kd accepted moves (delayed updates). G in shared memory: 16 moves are one K step of the
     // tensor-instruction update, where there is room for them and N is large enough for the update to outweigh the
-    // batch's bookkeeping (N = 72 gains 8%, N = 64 loses 6%, above); else, and for N > 150, which leaves no room for
+    // batch's bookkeeping (N = 72 gains 8%, N = 64 loses 6%, above); else, and from N = 150 on, where no room is left for
     // the batch, moves are applied at once (batches flushed by FP64 FMAs measured slower than that:
     // the same FMAs and the columns on top). G in global memory: batches of 32 by FMAs, one pass over G each.
     int kd = 0;

@@ -4,7 +4,7 @@
 //   ln|det(I + B_L ... B_1)| = sum ln D_b + ln|det M|,  sign = det(U) sign(det M),
 //   G = (I + B_L ... B_1)^-1 = M^-1 D_b^-1 U^T.
 // M is factored by a blocked right-looking LU with partial pivoting (one CTA per field; the
-// unblocked kernel covers N > 842, whose panel does not fit in shared memory); G is
+// unblocked kernel covers N > 880, whose panel does not fit in shared memory); G is
 // solved by blocked triangular solves, 32 right-hand sides per CTA (for N > 842, whose
 // right-hand sides do not fit in shared memory, one warp per column).
 #include <cfloat>
@@ -16,6 +16,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
+constexpr int MAXR = 32;  // rows per lane of the unblocked kernels (N <= 1024)
 
 // M (column-major, written over Y) from U (column-major), T (row-major) and lnD.
 __global__ void __launch_bounds__(kThreads) k_assemble_M(const double* __restrict__ Uall, const double* __restrict__ Tall,
@@ -41,7 +42,6 @@ __global__ void __launch_bounds__(kThreads) k_assemble_M(const double* __restric
     }
 }
 
-template <int MAXR>
 __global__ void __launch_bounds__(kThreads) k_lu(double* __restrict__ Mall, int* __restrict__ piv_all,
                                                  const double* __restrict__ lnD_all, const int* __restrict__ sgnU,
                                                  double* __restrict__ lndet, int* __restrict__ sign,
@@ -152,7 +152,6 @@ __global__ void __launch_bounds__(kThreads) k_lu(double* __restrict__ Mall, int*
 
 // G[:, j] = M^-1 (D_b^-1 U^T)[:, j] with the LU factors of M; one warp per column, the
 // right-hand side kept in shared memory. Output row-major G[f][i][j].
-template <int MAXR>
 __global__ void __launch_bounds__(256) k_greens(const double* __restrict__ LUall, const int* __restrict__ piv_all,
                                                 const double* __restrict__ Uall, const double* __restrict__ lnD_all,
                                                 double* __restrict__ Gout, int N) {
@@ -489,29 +488,27 @@ __global__ void __launch_bounds__(256) k_greens_blk(const double* __restrict__ L
     }
 }
 
-template <int MAXR>
 cudaError_t launch_final(slmc_ctx* c, int nf, double* lndet, int* sign, cudaStream_t s, bool assemble) {
     const int N = c->N;
     if (assemble) k_assemble_M<<<nf, kThreads, 2 * N * sizeof(double), s>>>(c->U, c->Ta, c->lnD, c->Y, N);
     const size_t smem = (size_t)N * kLS * sizeof(double);
-    if (smem <= 227 * 1024) {  // blocked LU (the panel fits in shared memory)
+    if (smem <= 227 * 1024) {  // blocked LU: the panel fits in shared memory up to N = 880
         cudaError_t e = cudaFuncSetAttribute(k_lu_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         k_lu_blk<<<nf, 256, smem, s>>>(c->Y, c->piv, c->lnD, c->sgnU, lndet, sign, c->err, N);
         return cudaGetLastError();
     }
-    k_lu<MAXR><<<nf, kThreads, N * sizeof(double), s>>>(c->Y, c->piv, c->lnD, c->sgnU, lndet, sign, c->err, N);
+    k_lu<<<nf, kThreads, N * sizeof(double), s>>>(c->Y, c->piv, c->lnD, c->sgnU, lndet, sign, c->err, N);
     return cudaGetLastError();
 }
 
-template <int MAXR>
 cudaError_t launch_greens(slmc_ctx* c, int nf, double* G, cudaStream_t s) {
     const int N = c->N;
     const size_t smem = (size_t)8 * N * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_greens<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_greens, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((N + 7) / 8, nf);
-    k_greens<MAXR><<<grid, 256, smem, s>>>(c->Y, c->piv, c->U, c->lnD, G, N);
+    k_greens<<<grid, 256, smem, s>>>(c->Y, c->piv, c->U, c->lnD, G, N);
     return cudaGetLastError();
 }
 
@@ -522,16 +519,7 @@ namespace slmc {
 namespace {
 cudaError_t final_dispatch(slmc_ctx* c, int nf, double* lndet, int* sign, cudaStream_t s, bool assemble) {
     if (c->N <= kSmallN) return small_final_lu(c, nf, lndet, sign, s, assemble);
-    switch (rows_per_lane_class(c->N)) {
-        case 1: return launch_final<1>(c, nf, lndet, sign, s, assemble);
-        case 2: return launch_final<2>(c, nf, lndet, sign, s, assemble);
-        case 4: return launch_final<4>(c, nf, lndet, sign, s, assemble);
-        case 5: return launch_final<5>(c, nf, lndet, sign, s, assemble);
-        case 8: return launch_final<8>(c, nf, lndet, sign, s, assemble);
-        case 12: return launch_final<12>(c, nf, lndet, sign, s, assemble);
-        case 18: return launch_final<18>(c, nf, lndet, sign, s, assemble);
-        default: return launch_final<32>(c, nf, lndet, sign, s, assemble);
-    }
+    return launch_final(c, nf, lndet, sign, s, assemble);
 }
 }  // namespace
 
@@ -549,23 +537,14 @@ cudaError_t final_greens(slmc_ctx* c, int nf, double* G, cudaStream_t s) {
     const int N = c->N;
     if (N <= kSmallN) return small_final_greens(c, nf, G, s);
     const size_t smem = (size_t)N * kGS * sizeof(double) + (size_t)N * (sizeof(double) + sizeof(int));
-    if (smem <= 227 * 1024) {  // blocked solve (the column-per-warp kernel below covers larger N)
+    if (smem <= 227 * 1024) {  // blocked solve up to N = 842, a column per warp above
         cudaError_t e = cudaFuncSetAttribute(k_greens_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         dim3 grid((N + kGB - 1) / kGB, nf);
         k_greens_blk<<<grid, 256, smem, s>>>(c->Y, c->piv, c->U, c->lnD, G, N);
         return cudaGetLastError();
     }
-    switch (rows_per_lane_class(c->N)) {
-        case 1: return launch_greens<1>(c, nf, G, s);
-        case 2: return launch_greens<2>(c, nf, G, s);
-        case 4: return launch_greens<4>(c, nf, G, s);
-        case 5: return launch_greens<5>(c, nf, G, s);
-        case 8: return launch_greens<8>(c, nf, G, s);
-        case 12: return launch_greens<12>(c, nf, G, s);
-        case 18: return launch_greens<18>(c, nf, G, s);
-        default: return launch_greens<32>(c, nf, G, s);
-    }
+    return launch_greens(c, nf, G, s);
 }
 
 }  // namespace slmc

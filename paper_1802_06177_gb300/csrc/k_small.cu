@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(Dim<NMAX>::threads, NMAX == 16 ? 4 : (NMAX == 
     __syncthreads();
     bool bad = false;
     for (int l0 = 0; l0 < L; l0 += n_s) {
-        slices<NMAX, LMAX, false>(B, v, xf, N, Lx, Ly, L, l0, min(L, l0 + n_s), dtlam, emu);
+        slices<NMAX, LMAX>(B, v, xf, N, Lx, Ly, L, l0, min(L, l0 + n_s), dtlam, emu);
         qr<NMAX>(B, A, v, N);
         t_update<NMAX>(A, T, v, N);
         form_q<NMAX>(A, B, v, N);

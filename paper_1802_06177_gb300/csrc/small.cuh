@@ -43,7 +43,6 @@ struct Vecs {
     double sc[kScMax][NMAX];       // slice scales of a group
     double cx[kSmallCoef], cy[kSmallCoef];  // folded coefficients of E_x, E_y
     double lbuf[2][NMAX];          // multipliers of the current / next LU step
-    double logabs;
     int perm[NMAX];
     int src[NMAX];                 // row interchanges as a permutation
     int piv[2];
@@ -82,16 +81,13 @@ __device__ __forceinline__ void half_line(double* g, int stride, const double* _
 }
 
 template <int NMAX>
-__device__ __forceinline__ void short_pass(double* P, const double* __restrict__ t, const double* in_sc, const double* out_sc,
-                                           int N, int n, int lines, int step_l, int stride) {
+__device__ __forceinline__ void short_pass(double* P, const double* __restrict__ t, const double* out_sc, int N,
+                                           int n, int lines, int step_l, int stride) {
     constexpr int ld = Dim<NMAX>::ld, NT = Dim<NMAX>::threads;
     for (int q0 = 0; q0 < 2 * N * lines; q0 += NT) {  // uniform trip count: the halves meet at a warp barrier
         const int q = q0 + threadIdx.x, li = (q >> 1) / N, jj = (q >> 1) - li * N, o = li * step_l;
         const bool on = q < 2 * N * lines;
         double* g = P + (on ? jj * ld + o : 0);
-        if (in_sc && on && (q & 1) == 0)
-            for (int m = 0; m < n; ++m) g[m * stride] *= in_sc[o + m * stride];
-        __syncwarp();
 #define SLMC_SHORT(k) \
     case k: half_line<k>(g, stride, t, q & 1, out_sc ? out_sc + (on ? o : 0) : nullptr, on); break;  // off lanes: no store
         switch (n) {
@@ -101,10 +97,10 @@ __device__ __forceinline__ void short_pass(double* P, const double* __restrict__
     }
 }
 
-// P <- B_{c1} ... B_{c0} P (plain) for the field columns c0 .. c1 - 1 in order, or with trans the transposed
-// slices E diag(s) from c1 - 1 down to c0: circulant transforms along the x and the y lines of every column.
+// P <- B_{c1} ... B_{c0} P for the field columns c0 .. c1 - 1 in order: circulant transforms along the x and the y lines
+// of every column, then the slice's scales.
 // v.cx, v.cy: folded coefficients, or the factors less the identity for NMAX = 16 (short_pass).
-template <int NMAX, int LMAX, bool kTrans>
+template <int NMAX, int LMAX>
 __device__ __forceinline__ void slices(double* P, Vecs<NMAX>& v, const double* __restrict__ xf, int N, int Lx, int Ly,
                                        int L, int c0, int c1, double dtlam, double emu) {
     constexpr int ld = Dim<NMAX>::ld, NT = Dim<NMAX>::threads;
@@ -113,22 +109,20 @@ __device__ __forceinline__ void slices(double* P, Vecs<NMAX>& v, const double* _
         const int nb = min(kScMax, c1 - b0);  // field columns of this batch, in the order of the slices
         for (int idx = tid; idx < nb * N; idx += NT) {
             const int i = idx / nb, k = idx - i * nb;
-            const int c = kTrans ? c1 - 1 - (b0 - c0) - k : b0 + k;
-            v.sc[k][i] = exp(-dtlam * xf[(size_t)i * L + c]) * emu;
+            v.sc[k][i] = exp(-dtlam * xf[(size_t)i * L + b0 + k]) * emu;
         }
         __syncthreads();
         for (int k = 0; k < nb; ++k)
             for (int pass = 0; pass < 2; ++pass) {
                 const int lines = pass ? Lx : Ly, step_l = pass ? 1 : Lx, stride = pass ? Lx : 1, n = pass ? Ly : Lx;
-                const double* in_sc = kTrans && pass == 0 ? v.sc[k] : nullptr;
-                const double* out_sc = !kTrans && pass == 1 ? v.sc[k] : nullptr;
+                const double* out_sc = pass ? v.sc[k] : nullptr;
                 if constexpr (NMAX == 16) {
-                    short_pass<NMAX>(P, pass ? v.cy : v.cx, in_sc, out_sc, N, n, lines, step_l, stride);
+                    short_pass<NMAX>(P, pass ? v.cy : v.cx, out_sc, N, n, lines, step_l, stride);
                 } else {
                     for (int q = tid; q < N * lines; q += NT) {
                         const int li = q / N, jj = q - li * N, o = li * step_l;
-                        circ::apply_any<LMAX>(n, P + jj * ld + o, stride, pass ? v.cy : v.cx, in_sc ? in_sc + o : nullptr,
-                                              stride, out_sc ? out_sc + o : nullptr, stride);
+                        circ::apply_any<LMAX>(n, P + jj * ld + o, stride, pass ? v.cy : v.cx, nullptr, 0,
+                                              out_sc ? out_sc + o : nullptr, stride);
                     }
                 }
                 __syncthreads();

@@ -238,9 +238,33 @@ def qr_trailing_issued(N):
     return t
 
 
-def class_work(cls, wl, nsl_mean, precision="fp32", qrt=False):
+def folded_line(n):
+    """(FMAs, additions) of one folded transform of a line of n sites (csrc/circ.cuh)."""
+    h, hm = n // 2, (n - 1) // 2
+    if n < 4 or n % 2:
+        return (h + 1) ** 2 + hm ** 2, 4 * hm
+    even, odd = (h + 1) // 2, (h - 1) // 2  # halves of the second fold, with the middle site where h is even
+    mid = 1 if h % 2 == 0 else 0
+    return (even + mid) ** 2 + even ** 2 + (odd + mid) ** 2 + odd ** 2, 4 * hm + 4 * even + 4 * odd
+
+
+def slice_pipe_flops(wl, dense=False):
+    """FP64-pipe flops of one FP64 slice of one field: the dense product; direct sums over the lines of up to 4 x 4
+    sites; none for sides 9 to 16, whose transforms run on the tensor instruction; else folded transforms."""
+    N, n = float(wl.N), wl.Lx
+    if dense:
+        return 2.0 * N ** 3
+    if 9 <= n <= 16:
+        return 0.0
+    if N <= 16:
+        return 2.0 * N * N * (2 * n)
+    fma, add = folded_line(n)
+    return N * 2 * n * (2.0 * fma + add)
+
+
+def class_work(cls, wl, nsl_mean, precision="fp32", qrt=False, dense=False):
     N, L = wl.N, wl.L
-    if cls == "slice" and precision == "fp64":  # separable exp(-dtau K): N^2 (Lx + Ly) FMAs per slice
+    if cls == "slice" and precision == "fp64" and not dense:  # separable exp(-dtau K): N^2 (Lx + Ly) FMAs of the method
         return 2.0 * N ** 2 * (2 * wl.Lx) * nsl_mean, "flop"
     if cls == "slice":
         return 2.0 * N ** 3 * nsl_mean, "flop"
@@ -596,7 +620,8 @@ def run_gpu(args):
     npan = len(qrt_panel_sizes(wl.N))
     per_qr = {"qr": npan, "qrtc": max(1, npan - 1)}.get(dom, 1) if qrt else 1
     dom_calls, dom_units = dom_calls / per_qr, dom_units / per_qr
-    work, kind = class_work(dom, wl, nsl_mean, args.precision, qrt)
+    q_tc = qrt and wl.N > 64  # FP64 Q through the products of the QR's trailing updates
+    work, kind = class_work(dom, wl, nsl_mean, args.precision, qrt, args.dense_slices)
     roof = None
     if work:
         fields_per_call = dom_units / max(dom_calls, 1)
@@ -621,6 +646,10 @@ def run_gpu(args):
             roof = dict(common, bound="alu", pipe="fp64" if fp64_cls else "fp32", achieved=achieved, peak=peak,
                         unit="TFLOP/s", frac=achieved / peak, peak_probed=pk, frac_of_probed=achieved / pk,
                         traffic=traffic, peak_source=src)
+            if args.precision == "fp64" and ((dom == "slice" and not args.dense_slices) or (dom == "formq" and q_tc)):
+                roof.update(unit="TFLOP/s (FP64 equivalent)", frac=None, frac_of_probed=None,
+                            note="achieved counts the method's FMAs; folded sums or the tensor instruction leave half of "
+                                 "them or none to the FP64 pipe, so it is no fraction of that pipe's peak")
         elif kind == "flop" and dom == "qrtc":
             t = tensor_use(wl, nf, ngroups, args.precision, prof, peaks).get("qrtc:" + args.precision)
             if t:
@@ -674,20 +703,20 @@ def run_gpu(args):
 
     # FP64-pipe work of one evaluation of the step (QR per group, Q of the final group (FP64 in
     # every mode; the other groups' Q is FP64 only in FP64 mode; through the tensor cores with the
-    # QR's trailing updates for N > 64), final LU, G, and FP64 slices in FP64 mode; the T update
-    # runs on the tensor cores) against the step time
+    # QR's trailing updates for N > 64), final LU, G, and what FP64 slices leave to that pipe in FP64
+    # mode; the T update runs on the tensor cores) against the step time
     N3 = float(wl.N) ** 3
     w_qr = qr_panel_flops(wl.N) if qrt else (4.0 / 3.0) * N3  # the panels alone when the trailing updates are TC
-    q_tc = qrt and wl.N > 64
     w64 = ngroups * w_qr + (0.0 if q_tc else (4.0 / 3.0) * N3 * (ngroups if args.precision == "fp64" else 1)) \
         + (2.0 / 3.0 + (2.0 if args.mode == "step" else 0.0)) * N3
-    if args.precision == "fp64":  # slices through the separable exp(-dtau K): N^2 (Lx + Ly) FMAs each
-        w64 += 2.0 * float(wl.N) ** 2 * (2 * wl.Lx) * wl.L
+    slice64 = slice_pipe_flops(wl, args.dense_slices) if args.precision == "fp64" else 0.0
+    w64 += slice64 * wl.L
     ach64 = w64 * nf * world / (ms_step / 1e3) / 1e12 / world
     fp64_step = {"flop_per_eval": w64, "achieved_per_gpu": ach64, "unit": "TFLOP/s",
                  "frac_of_nominal": ach64 / NOMINAL["fp64_tflops"], "frac_of_probed": ach64 / probed["fp64_tflops"],
                  "excludes": "T update (tensor cores)" + (", QR trailing updates (tensor cores)" if qrt else "")
-                 + (", FP64 Q (tensor cores)" if q_tc else "")}
+                 + (", FP64 Q (tensor cores)" if q_tc else "")
+                 + (", FP64 slices (tensor instruction)" if args.precision == "fp64" and not slice64 else "")}
     dtype = {"fp64": "f64", "fp32": "f32 slices + f64 stabilisation",
              "tf32x3": "tf32x3 slices (tensor cores) + f64 stabilisation",
              "bf16x9": "bf16x9 exact-sliced slices (tensor cores) + f64 stabilisation"}[args.precision] + \

@@ -55,49 +55,81 @@ __global__ void __launch_bounds__(kThreads) k_bose(const double* __restrict__ x,
     if (threadIdx.x == 0) lnw[f] = (lndet ? 2.0 * lndet[f] : 0.0) + acc[0];
 }
 
-// Feature sums of one field per CTA; a warp walks rows (sites), its lanes the slices. Eleven FP64 operations per
-// value bound it: 2000 fields of 12x12,
-// L = 120 take 1.36 ms (0.6 ms of FP64 issue, 41 us of memory traffic). With nine more FP64 operations and three
-// integer divisions per value, and the regression below as it was, a fit of them took 5.5 ms against 1.45 ms.
-__global__ void __launch_bounds__(kThreads) k_features(const double* __restrict__ x, int Lx, int Ly, int L, double a2,
-                                                       double dtau, const double* __restrict__ J,
+// n / d for the divisors of a lattice (half the slices, Lx) by one multiply-high: exact while n d < 2^32
+// (q = floor(n ceil(2^32 / d) / 2^32)); magic 0 selects the division.
+__device__ __forceinline__ int fast_div(int n, int d, uint32_t magic) {
+    return magic ? (int)__umulhi((uint32_t)n, magic) : n / d;
+}
+
+// Feature sums of one field per CTA, eleven FP64 operations per value, the bound from a few thousand values on: a
+// field of 12x12, L = 120 has 46 us of FP64 issue. Threads take values 256 apart, whatever rows they lie in (the site and
+// slice advance by additions, the neighbours' rows come from a table), and load four values' operands before they use
+// them; 152 / 1000 fields of 12x12, L = 120 take 61 / 364 us, of 4x4, L = 40 12 / 23 us, of 16x16, L = 160 132 / 846 us.
+// With a row per warp and its lanes on the slices they took 104 / 686, 16 / 54 and 130 / 870 us: only row lengths of
+// a multiple of 128 filled the unrolled loop.
+__global__ void __launch_bounds__(kThreads) k_features(const double* __restrict__ x, int Lx, int Ly, int L, uint32_t ml,
+                                                       uint32_t mlx, int di, double a2, double dtau, const double* __restrict__ J,
                                                        double* __restrict__ F, int ldF, double* __restrict__ lnw_eff) {
-    __shared__ double red[5][kThreads / 32];
+    constexpr int U = 4;  // values in flight
+    __shared__ double red[5][kThreads], feat[5];
+    __shared__ int nbx[SLMC_MAX_N], nby[SLMC_MAX_N];  // first element of the rows of a site's neighbours
     const int f = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int N = Lx * Ly;
-    const double* xf = x + (size_t)f * N * L;
+    const int N = Lx * Ly, NL = N * L;
+    const double* xf = x + (size_t)f * NL;
+    for (int i = threadIdx.x; i < N; i += kThreads) {
+        const int iy = fast_div(i, Lx, mlx), ix = i - iy * Lx;
+        nbx[i] = (i + (ix + 1 == Lx ? 1 - Lx : 1)) * L;
+        nby[i] = (iy + 1 == Ly ? ix : i + Lx) * L;
+    }
+    __syncthreads();
     double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     const double h2 = -0.5 * a2, h4 = -0.25 * a2;
-    for (int i = warp; i < N; i += kThreads / 32) {
-        const int iy = i / Lx, ix = i - iy * Lx;
-        const double* xi = xf + (size_t)i * L;
-        const double* xx = xf + (size_t)((ix + 1 == Lx ? 0 : ix + 1) + Lx * iy) * L;
-        const double* xy = xf + (size_t)(ix + Lx * (iy + 1 == Ly ? 0 : iy + 1)) * L;
-#pragma unroll 4
-        for (int l = lane; l < L; l += 32) {
-            const double v = xi[l], vt = xi[l + 1 == L ? 0 : l + 1];
-            const double nb = xx[l] + xy[l];
-            const double v2 = v * v, v4 = v2 * v2, d = vt - v;
+    const int dl = kThreads - di * L;  // di = kThreads / L
+    int i = fast_div(threadIdx.x, L, ml), l = threadIdx.x - i * L;
+    for (unsigned w0 = threadIdx.x & ~31u; w0 < (unsigned)NL; w0 += U * kThreads) {  // first value of the warp
+        double v[U], vt[U], vx[U], vy[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            v[u] = vt[u] = vx[u] = vy[u] = 0.0;  // adds nothing
+            if (i < N) {
+                const double* xi = xf + i * L;
+                v[u] = xi[l];
+                vt[u] = xi[l + 1 == L ? 0 : l + 1];
+                vx[u] = xf[nbx[i] + l];
+                vy[u] = xf[nby[i] + l];
+            }
+            i += di;
+            l += dl;
+            if (l >= L) {
+                l -= L;
+                ++i;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (w0 + u * kThreads >= (unsigned)NL) break;
+            const double nb = vx[u] + vy[u];
+            const double v2 = v[u] * v[u], v4 = v2 * v2, d = vt[u] - v[u];
             acc[0] = fma(d, d, acc[0]);
             acc[1] = fma(v2, fma(0.25, v2, h2), acc[1]);
             acc[2] = fma(v4, fma(1.0 / 6.0, v2, h4), acc[2]);
-            acc[3] = fma(v, nb, acc[3]);
-            acc[4] = fma(v, vt, acc[4]);
+            acc[3] = fma(v[u], nb, acc[3]);
+            acc[4] = fma(v[u], vt[u], acc[4]);
         }
     }
+    // one warp per sum: over the warps first, then over the lanes (13 additions of five warps)
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-        const double t = slmc::warp_allsum(acc[q]);
-        if (lane == 0) red[q][warp] = t;
+    for (int q = 0; q < 5; ++q) red[q][threadIdx.x] = acc[q];
+    __syncthreads();
+    if (warp < 5) {
+        double t = red[warp][lane];
+#pragma unroll
+        for (int w = 1; w < kThreads / 32; ++w) t += red[warp][lane + 32 * w];
+        t = slmc::warp_allsum(t);
+        if (lane == 0) feat[warp] = t;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double feat[5];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            feat[q] = red[q][0];
-            for (int w = 1; w < kThreads / 32; ++w) feat[q] += red[q][w];
-        }
         if (F)
             for (int q = 0; q < 5; ++q) F[(size_t)f * ldF + q] = feat[q];
         if (lnw_eff) {
@@ -134,12 +166,6 @@ __device__ __forceinline__ float trunc_f32(double v) {
     if (t < 0x00100000) m = 0u;
     if (t >= 0x0ff00000) m = 0x7f800000u;
     return __uint_as_float((m & 0x7fffffffu) | ((uint32_t)hi & 0x80000000u));
-}
-
-// n / d for the divisors of a lattice (half the slices, Lx) by one multiply-high: exact while n d < 2^32
-// (q = floor(n ceil(2^32 / d) / 2^32)); magic 0 selects the division.
-__device__ __forceinline__ int fast_div(int n, int d, uint32_t magic) {
-    return magic ? (int)__umulhi((uint32_t)n, magic) : n / d;
 }
 
 // Couplings and constants of one chain's sweeps, FP64 for the exact rule and FP32 for the fast test, kept in
@@ -759,7 +785,8 @@ cudaError_t bose_log_weight(slmc_ctx* c, const double* x, int nf, const double* 
 cudaError_t eff_features(slmc_ctx* c, const double* x, int nf, const double* J, double* F, int ldF, double* lnw_eff,
                          cudaStream_t s) {
     const double a = c->p.lambda / (c->p.omega0 * c->p.omega0);
-    k_features<<<nf, kThreads, 0, s>>>(x, c->p.Lx, c->p.Ly, c->L, a * a, c->p.dtau, J, F, ldF, lnw_eff);
+    k_features<<<nf, kThreads, 0, s>>>(x, c->p.Lx, c->p.Ly, c->L, div_magic(kThreads, c->L), div_magic(c->N, c->p.Lx),
+                                       kThreads / c->L, a * a, c->p.dtau, J, F, ldF, lnw_eff);
     return cudaGetLastError();
 }
 

@@ -620,7 +620,7 @@ def run_gpu(args):
     npan = len(qrt_panel_sizes(wl.N))
     per_qr = {"qr": npan, "qrtc": max(1, npan - 1)}.get(dom, 1) if qrt else 1
     dom_calls, dom_units = dom_calls / per_qr, dom_units / per_qr
-    q_tc = qrt and wl.N > 64  # FP64 Q through the products of the QR's trailing updates
+    q_tc = qrt and wl.N > 80  # FP64 Q through the products of the QR's trailing updates
     work, kind = class_work(dom, wl, nsl_mean, args.precision, qrt, args.dense_slices)
     roof = None
     if work:
@@ -703,7 +703,7 @@ def run_gpu(args):
 
     # FP64-pipe work of one evaluation of the step (QR per group, Q of the final group (FP64 in
     # every mode; the other groups' Q is FP64 only in FP64 mode; through the tensor cores with the
-    # QR's trailing updates for N > 64), final LU, G, and what FP64 slices leave to that pipe in FP64
+    # QR's trailing updates for N > 80), final LU, G, and what FP64 slices leave to that pipe in FP64
     # mode; the T update runs on the tensor cores) against the step time
     N3 = float(wl.N) ** 3
     w_qr = qr_panel_flops(wl.N) if qrt else (4.0 / 3.0) * N3  # the panels alone when the trailing updates are TC

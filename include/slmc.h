@@ -311,7 +311,7 @@ SLMC_API int slmc_set_tupdate_path(slmc_ctx* ctx, int path);
  *            accumulator), and each entry is rounded once to FP64. Each product entry then differs
  *            from the exact product of the operands by below 2^-44 K max|a_row| max|b_column| (K
  *            the inner dimension): normwise the size of the FP64 loop's own rounding. 4 launches
- *            per panel on the caller's stream. For N > 64 Q is formed in FP64 through such products with
+ *            per panel on the caller's stream. From N = 81 on Q is formed in FP64 through such products with
  *            eight digits (56 bits, as near to the exact Q as by FP64 FMAs; 4 more launches per panel).
  *   path = 1: the one-kernel FP64 QR (trailing updates with FP64 FMAs), Q formed with FP64 FMAs.
  * The DQMC updates follow it for N > 64, on path 0 with eight digits in the trailing updates too (the one-kernel QR up

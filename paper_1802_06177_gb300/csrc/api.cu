@@ -679,13 +679,16 @@ int chain_step64(slmc_ctx* c, int nf, cudaStream_t s) {
     if (c->p.qr_mode == SLMC_QR_PIVOTED) {
         SLMC_LAUNCH(SLMC_PROF_QR, 1, s, slmc::qr_pivoted(c, nf, s));
         SLMC_LAUNCH(SLMC_PROF_FORMQ, 1, s, slmc::form_q(c, nf, s));
-    } else if (slmc::qrt_form_q_active(c)) {
+    } else if (slmc::qrt_active(c) && c->N > slmc::kSmallN) {
         const int np = slmc::qrt_panels(c);
         for (int t = 0; t < np; ++t) {
             SLMC_LAUNCH(SLMC_PROF_QR, 1, s, slmc::qrt_panel(c, nf, t, s, true));
             if (t + 1 < np) SLMC_LAUNCH(SLMC_PROF_QRTC, 3, s, slmc::qrt_trailing(c, nf, t, s, true));
         }
-        SLMC_LAUNCH(SLMC_PROF_FORMQ, slmc::qrt_form_q_launches(c), s, slmc::qrt_form_q(c, nf, s));
+        if (slmc::qrt_form_q_active(c))
+            SLMC_LAUNCH(SLMC_PROF_FORMQ, slmc::qrt_form_q_launches(c), s, slmc::qrt_form_q(c, nf, s));
+        else
+            SLMC_LAUNCH(SLMC_PROF_FORMQ, 1, s, slmc::form_q_blocked(c, nf, false, s));
     } else {
         SLMC_LAUNCH(SLMC_PROF_QR, 1, s, slmc::qr_blocked(c, nf, s));
         SLMC_LAUNCH(SLMC_PROF_FORMQ, 1, s, slmc::form_q_blocked(c, nf, false, s));

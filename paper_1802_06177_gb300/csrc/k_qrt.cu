@@ -904,8 +904,13 @@ cudaError_t qrt_init(slmc_ctx* c, void* bf16_base, int* int_base) {
     return cudaSuccess;
 }
 
-// Below, a panel's four launches outweigh the FP64 kernel (one or two panels in all).
-constexpr int kFormQMinN = 65;
+// From three panels on, four launches a panel against one in all: with few fields FP64 FMAs are faster up to about 100
+// sites, with many the products from 66 on. The path may not depend on the number of fields (the split into batches
+// leaves results as they are), so the line lies where what either side loses is even. FP64 evaluations with G, L = 40, FMAs
+// / products, 1, 64, 152, 512 fields: N = 72 3.56 / 3.86, 4.01 / 4.39, 5.23 / 5.42, 11.6 / 11.2 ms; N = 81 4.16 / 4.44,
+// 4.68 / 4.98, 6.13 / 6.27, 14.2 / 13.4; N = 100 5.88 / 6.12, 6.82 / 6.91, 9.15 / 8.76, 21.1 / 19.2; N = 132 7.59 / 7.71,
+// 9.75 / 9.45, 14.2 / 13.2, 37.2 / 32.9.
+constexpr int kFormQMinN = 81;
 
 bool qrt_active(const slmc_ctx* c) { return c->qt_C && c->qr_path == 0 && qrt_supported(c->N); }
 

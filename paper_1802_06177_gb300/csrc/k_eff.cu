@@ -620,21 +620,19 @@ __device__ __forceinline__ void givens_absorb(double (&Rrow)[7], double a, int l
     }
 }
 
-// Absorbs nconf rows into the triangle, kFitRows per pass, by Householder reflections of [R; rows] in one CTA:
-// the rows stay in registers (four per thread), and the reflector of column k touches row k of R and the rows
+// Absorbs nconf rows into the triangle, up to 2048 per pass, by Householder reflections of [R; rows] in one CTA:
+// the rows stay in registers (up to four per thread), and the reflector of column k touches row k of R and the rows
 // only. The products of column k with itself and with the columns right of it are reduced together (one block
 // reduction per column); scaling by the reflector's normalisation comes after. Row k of R takes the sign that
-// makes its diagonal non-negative, as the Givens merge below leaves it. A chain of Givens rotations per warp
-// (63 rows, seven hypots and divisions each) and a tree of triangle merges stood here before; 2000 rows take 95 us with
-// the kernels around it. Couplings against quad precision over 24 fits: 1.2e-13 (2.4e-13 before).
-constexpr int kFitThreads = 512, kFitPer = 4, kFitRows = kFitThreads * kFitPer;
+// makes its diagonal non-negative, as the Givens merge below leaves it. A fit of 4x4, L = 40 takes
+// 60 us with 6 to 100 rows, 103 with 500, 128 with 2000 (512 threads whatever the rows: 100 with 6, 192 with 2000). Couplings against quad precision over 24 fits: 1.2e-13.
+constexpr int kFitThreads = 512, kFitMinThreads = 224 /* a warp per column */, kFitPer = 4;
 
 __global__ void __launch_bounds__(kFitThreads) k_fit_accumulate(double* __restrict__ R, const double* __restrict__ feat,
                                                                 int ldF, const double* __restrict__ lnw, int nconf,
                                                                 double sc) {
-    constexpr int NW = kFitThreads / 32;
-    __shared__ double sR[49], ref[6], part[7][NW], dot[7], par[2];  // par: tau, scal
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ double sR[49], ref[6], part[7][kFitThreads / 32], dot[7], par[2];  // par: tau, scal
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x, NW = T / 32;
     if (tid == 0 && R[55] == 0.0) {
         for (int q = 0; q < 5; ++q) R[49 + q] = feat[q];
         R[54] = lnw[0];
@@ -645,11 +643,12 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_accumulate(double* __restri
     if (tid >= 64 && tid < 70) ref[tid - 64] = R[49 + tid - 64];
     __syncthreads();
     const double inv = 1.0 / sc;
-    for (int c0 = 0; c0 < nconf; c0 += kFitRows) {
+    for (int c0 = 0; c0 < nconf; c0 += kFitPer * T) {
         double a[kFitPer][7];
+        const int left = nconf - c0 - 32 * warp, nr = left <= 0 ? 0 : min(kFitPer, (left + T - 1) / T);  // the warp's rows
 #pragma unroll
         for (int r = 0; r < kFitPer; ++r) {
-            const int c = c0 + r * kFitThreads + tid;
+            const int c = c0 + r * T + tid;
             const bool on = c < nconf;
             a[r][0] = on ? 1.0 : 0.0;
 #pragma unroll
@@ -661,9 +660,12 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_accumulate(double* __restri
 #pragma unroll
             for (int m = k; m < 7; ++m) {
                 double t = 0.0;
+                if (nr > 0) {
 #pragma unroll
-                for (int r = 0; r < kFitPer; ++r) t = fma(a[r][k], a[r][m], t);
-                t = slmc::warp_allsum(t);
+                    for (int r = 0; r < kFitPer; ++r)
+                        if (r < nr) t = fma(a[r][k], a[r][m], t);
+                    t = slmc::warp_allsum(t);
+                }
                 if (lane == 0) part[m][warp] = t;
             }
             __syncthreads();
@@ -700,7 +702,8 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_accumulate(double* __restri
             for (int m = k + 1; m < 7; ++m) {
                 const double d = dot[m] * scal;
 #pragma unroll
-                for (int r = 0; r < kFitPer; ++r) a[r][m] = fma(-d, a[r][k], a[r][m]);
+                for (int r = 0; r < kFitPer; ++r)
+                    if (r < nr) a[r][m] = fma(-d, a[r][k], a[r][m]);
             }
             __syncthreads();  // part and dot are rewritten by the next column
         }
@@ -902,7 +905,9 @@ cudaError_t fit_begin(slmc_ctx* c, double* R, cudaStream_t s) {
 }
 
 cudaError_t fit_accumulate(slmc_ctx* c, double* R, const double* feat, const double* lnw, int nconf, cudaStream_t s) {
-    k_fit_accumulate<<<1, kFitThreads, 0, s>>>(R, feat, 8, lnw, nconf, (double)c->N * c->L);
+    // a row per thread while they fit: warps without rows would only lengthen the FP64 queue
+    const int threads = std::min(kFitThreads, std::max(kFitMinThreads, (nconf + 31) / 32 * 32));
+    k_fit_accumulate<<<1, threads, 0, s>>>(R, feat, 8, lnw, nconf, (double)c->N * c->L);
     return cudaGetLastError();
 }
 

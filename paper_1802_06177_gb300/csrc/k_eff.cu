@@ -625,7 +625,8 @@ __device__ __forceinline__ void givens_absorb(double (&Rrow)[7], double a, int l
 // only. The products of column k with itself and with the columns right of it are reduced together (one block
 // reduction per column); scaling by the reflector's normalisation comes after. Row k of R takes the sign that
 // makes its diagonal non-negative, as the Givens merge below leaves it. A fit of 4x4, L = 40 takes
-// 60 us with 6 to 100 rows, 103 with 500, 128 with 2000 (512 threads whatever the rows: 100 with 6, 192 with 2000). Couplings against quad precision over 24 fits: 1.2e-13.
+// 60 us with 6 to 100 rows, 103 with 500, 128 with 2000 (512 threads whatever the rows: 100 with 6, 192 with 2000).
+// Couplings against quad precision, geometric mean of 120 fits: 1.6e-13.
 constexpr int kFitThreads = 512, kFitMinThreads = 224 /* a warp per column */, kFitPer = 4;
 
 __global__ void __launch_bounds__(kFitThreads) k_fit_accumulate(double* __restrict__ R, const double* __restrict__ feat,
@@ -858,7 +859,9 @@ cudaError_t eff_chain_sweeps(slmc_ctx* c, double* x, int nf, int chain0, const d
     const int sites = c->N * (c->L / 2), iters = (sites + 1023) / 1024;
     const int threads = std::max(64, ((sites + iters - 1) / iters + 31) / 32 * 32);
     const size_t smem = (size_t)c->N * (c->L + 1) * sizeof(double) + 3 * (size_t)c->N;
-    cudaError_t e = cudaFuncSetAttribute(k_chain_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the largest chain's, whatever this one's: contexts of other sizes on other threads set it too
+    constexpr int kMost = (kChainSites + SLMC_MAX_N) * (int)sizeof(double) + 3 * SLMC_MAX_N;
+    cudaError_t e = cudaFuncSetAttribute(k_chain_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
     if (e != cudaSuccess) return e;
     k_chain_sweeps<<<nf, threads, smem, s>>>(
         x, c->p.Lx, c->p.Ly, c->L, div_magic(sites, c->L / 2), div_magic(c->N, c->p.Lx), J, c->p.dtau, a * a,

@@ -4,7 +4,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <mutex>
 #include <new>
+#include <unordered_map>
 
 #include "slmc_internal.cuh"
 
@@ -320,6 +322,17 @@ void free_ctx(slmc_ctx* c) {
 }  // namespace
 
 namespace slmc {
+cudaError_t raise_smem_limit(const void* kernel, size_t bytes) {
+    static std::mutex mutex;
+    static auto* most = new std::unordered_map<const void*, size_t>;  // (never destroyed: used until the last call)
+    std::lock_guard<std::mutex> lock(mutex);
+    size_t& m = (*most)[kernel];
+    const size_t want = std::max(m, bytes);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want);
+    if (e == cudaSuccess) m = want;
+    return e;
+}
+
 // Shared with the allocation-free entry point (k_noalloc.cu): parameter validation and the
 // stabilised UDT chain + LU of slmc_logdet for one batch of fields.
 int validate_params(const slmc_params* p) { return validate(p); }

@@ -539,7 +539,7 @@ cudaError_t launch_slices(slmc_ctx* c, double* x, double* G, int nf, int chain0,
         if (dqmc_smem_bytes(c->N, nc, false, kd) > (size_t)optin) kd = 0;
     }
     const size_t bytes = dqmc_smem_bytes(c->N, nc, in_smem, kd);
-    e = cudaFuncSetAttribute(k_dqmc_slices<LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    e = slmc::allow_smem(k_dqmc_slices<LMAX>, bytes);
     if (e != cudaSuccess) return e;
     k_dqmc_slices<LMAX><<<nf, kThreads, bytes, s>>>(
         x, G, c->p.Lx, c->p.Ly, c->L, l0, nsl, c->p.dtau, c->kron, c->p.lambda, c->p.omega0 * c->p.omega0,

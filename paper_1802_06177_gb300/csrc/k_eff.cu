@@ -859,9 +859,7 @@ cudaError_t eff_chain_sweeps(slmc_ctx* c, double* x, int nf, int chain0, const d
     const int sites = c->N * (c->L / 2), iters = (sites + 1023) / 1024;
     const int threads = std::max(64, ((sites + iters - 1) / iters + 31) / 32 * 32);
     const size_t smem = (size_t)c->N * (c->L + 1) * sizeof(double) + 3 * (size_t)c->N;
-    // the largest chain's, whatever this one's: contexts of other sizes on other threads set it too
-    constexpr int kMost = (kChainSites + SLMC_MAX_N) * (int)sizeof(double) + 3 * SLMC_MAX_N;
-    cudaError_t e = cudaFuncSetAttribute(k_chain_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+    cudaError_t e = slmc::allow_smem(k_chain_sweeps, smem);
     if (e != cudaSuccess) return e;
     k_chain_sweeps<<<nf, threads, smem, s>>>(
         x, c->p.Lx, c->p.Ly, c->L, div_magic(sites, c->L / 2), div_magic(c->N, c->p.Lx), J, c->p.dtau, a * a,

@@ -493,7 +493,7 @@ cudaError_t launch_final(slmc_ctx* c, int nf, double* lndet, int* sign, cudaStre
     if (assemble) k_assemble_M<<<nf, kThreads, 2 * N * sizeof(double), s>>>(c->U, c->Ta, c->lnD, c->Y, N);
     const size_t smem = (size_t)N * kLS * sizeof(double);
     if (smem <= 227 * 1024) {  // blocked LU: the panel fits in shared memory up to N = 880
-        cudaError_t e = cudaFuncSetAttribute(k_lu_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = slmc::allow_smem(k_lu_blk, smem);
         if (e != cudaSuccess) return e;
         k_lu_blk<<<nf, 256, smem, s>>>(c->Y, c->piv, c->lnD, c->sgnU, lndet, sign, c->err, N);
         return cudaGetLastError();
@@ -505,7 +505,7 @@ cudaError_t launch_final(slmc_ctx* c, int nf, double* lndet, int* sign, cudaStre
 cudaError_t launch_greens(slmc_ctx* c, int nf, double* G, cudaStream_t s) {
     const int N = c->N;
     const size_t smem = (size_t)8 * N * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_greens, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_greens, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((N + 7) / 8, nf);
     k_greens<<<grid, 256, smem, s>>>(c->Y, c->piv, c->U, c->lnD, G, N);
@@ -538,7 +538,7 @@ cudaError_t final_greens(slmc_ctx* c, int nf, double* G, cudaStream_t s) {
     if (N <= kSmallN) return small_final_greens(c, nf, G, s);
     const size_t smem = (size_t)N * kGS * sizeof(double) + (size_t)N * (sizeof(double) + sizeof(int));
     if (smem <= 227 * 1024) {  // blocked solve up to N = 842, a column per warp above
-        cudaError_t e = cudaFuncSetAttribute(k_greens_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = slmc::allow_smem(k_greens_blk, smem);
         if (e != cudaSuccess) return e;
         dim3 grid((N + kGB - 1) / kGB, nf);
         k_greens_blk<<<grid, 256, smem, s>>>(c->Y, c->piv, c->U, c->lnD, G, N);

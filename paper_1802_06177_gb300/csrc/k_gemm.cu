@@ -106,7 +106,7 @@ cudaError_t launch_panel(const T* A, size_t a_stride, const double* B, const int
     constexpr int NB = kWarps * CPT;
     const size_t smem = (size_t)(2 * NB * N + N) * sizeof(T);
     auto kern = k_panel<T, MAXR, CPT, TRI>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((N + NB - 1) / NB, nf);
     kern<<<grid, 256, smem, s>>>(A, a_stride, B, perm, out, x, N, L, l0, nsl, dtlam, add_identity);
@@ -313,8 +313,7 @@ cudaError_t launch_slice_f32_kb(const slmc_ctx* c, int nf, int l0, int nsl, cuda
     const int N = c->N;
     constexpr int NBP = NCG * NBT + 4;
     const size_t smem = ((size_t)2 * N * NBP + (size_t)2 * KB * N) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k_slice_f32<RPT, NBT, KB, NCG, TRC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_slice_f32<RPT, NBT, KB, NCG, TRC>, smem);
     if (e != cudaSuccess) return e;
     constexpr int NB = NCG * NBT;
     dim3 grid((N + NB - 1) / NB, nf);

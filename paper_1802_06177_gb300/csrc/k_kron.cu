@@ -89,7 +89,7 @@ cudaError_t launch_oz(slmc_ctx* c, const double* x, int nf, int l0, int nsl, cud
     for (int w = 48; w <= 64; w += 16)
         if ((N + w - 1) / w * w <= (N + NB - 1) / NB * NB && fixed + (size_t)w * (N | 1) * sizeof(double) <= 112 * 1024) NB = w;
     const size_t smem = fixed + (size_t)NB * (N | 1) * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_slice_oz<kTrans>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_slice_oz<kTrans>, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((N + NB - 1) / NB, nf);
     k_slice_oz<kTrans><<<grid, kThreads, smem, s>>>(c->U, c->Y, x, c->kron, c->p.Lx, c->p.Ly, c->L, l0, nsl,
@@ -147,8 +147,7 @@ cudaError_t launch_kron(slmc_ctx* c, const double* x, int nf, int l0, int nsl, c
     const size_t fixed = (size_t)N + slmc::circ::ncoef(c->p.Lx) + slmc::circ::ncoef(c->p.Ly);
     const int NB = (fixed + (size_t)kNBF * (N | 1)) * sizeof(double) <= 227 * 1024 ? kNBF : kNBFLarge;
     const size_t smem = (fixed + (size_t)NB * (N | 1)) * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_slice_kron<LMAX, kTrans>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = slmc::allow_smem(k_slice_kron<LMAX, kTrans>, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((N + NB - 1) / NB, nf);
     k_slice_kron<LMAX, kTrans><<<grid, kThreads, smem, s>>>(c->U, c->Y, x, c->kron, c->p.Lx, c->p.Ly, c->L, l0, nsl,

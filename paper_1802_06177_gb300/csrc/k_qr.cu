@@ -317,7 +317,7 @@ template <int MAXR>
 cudaError_t launch_qr(slmc_ctx* c, int nf, cudaStream_t s) {
     const int N = c->N;
     const size_t smem = (size_t)N * (8 * sizeof(double) + 2 * sizeof(int));
-    cudaError_t e = cudaFuncSetAttribute(k_qrp<MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_qrp<MAXR>, smem);
     if (e != cudaSuccess) return e;
     k_qrp<MAXR><<<nf, kThreads, smem, s>>>(c->Y, c->lnD, c->QR, c->tau, c->perm, c->sgnU, c->err, N);
     return cudaGetLastError();

@@ -386,7 +386,7 @@ int qr_cluster_size(const slmc_ctx* c, int nf) {
 template <int BP>
 cudaError_t launch_qrb(slmc_ctx* c, int nf, cudaStream_t s) {
     const size_t smem = QrSmem<BP>::bytes(c->N);
-    cudaError_t e = cudaFuncSetAttribute(k_qrb<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_qrb<BP>, smem);
     if (e != cudaSuccess) return e;
     const int C = qr_cluster_size(c, nf);
     if (C == 1) {
@@ -411,7 +411,7 @@ cudaError_t launch_qrb(slmc_ctx* c, int nf, cudaStream_t s) {
 template <int BP>
 cudaError_t launch_formq_b(slmc_ctx* c, int nf, cudaStream_t s) {
     const size_t smem = sizeof(double) * ((size_t)c->N * (BP + 1) + BP * BP + kWarps * BP * kCT);
-    cudaError_t e = cudaFuncSetAttribute(k_formq_b<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_formq_b<BP>, smem);
     if (e != cudaSuccess) return e;
     // column blocks per field: at least the QR's cluster size, and enough for about two CTAs per SM
     int cb = qr_cluster_size(c, nf);
@@ -432,7 +432,7 @@ cudaError_t launch_formq32(slmc_ctx* c, int nf, cudaStream_t s) {
         if (nw < 1) return cudaErrorInvalidValue;
     }
     const size_t smem = fixed + nw * per_warp;
-    cudaError_t e = cudaFuncSetAttribute(k_formq32<BP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_formq32<BP>, smem);
     if (e != cudaSuccess) return e;
     const int groups = (N + 7) / 8;
     k_formq32<BP><<<dim3(nf, (groups + nw - 1) / nw), nw * 32, smem, s>>>(c->QR, c->Sws, c->U32, N, ld);

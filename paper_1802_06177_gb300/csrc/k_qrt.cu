@@ -784,8 +784,7 @@ cudaError_t launch_panel(slmc_ctx* c, int nf, int t, cudaStream_t s) {
     const QrtArgs a = qrt_args(c);
     const int p = t * BP;
     const size_t smP = PanelSmem<BP>::bytes(a.N, p, p + BP >= a.N);
-    cudaError_t e = cudaFuncSetAttribute(k_qrt_panel<BP, kPT, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)std::max(PanelSmem<BP>::bytes(a.N, 0, a.N <= BP), smP));
+    cudaError_t e = slmc::allow_smem(k_qrt_panel<BP, kPT, D>, smP);
     if (e != cudaSuccess) return e;
     k_qrt_panel<BP, kPT, D><<<nf, kPT, smP, s>>>(c->Y, c->lnD, c->QR, c->tau, c->perm, c->sgnU, c->Sws, c->err, a.N, t,
                                               c->qt_lnDn, c->qt_ntriv, a.V1, c->qt_eV1, a.V2, c->qt_eV2, a.kpad,
@@ -798,8 +797,8 @@ template <int BP, int D>
 cudaError_t launch_trailing(slmc_ctx* c, int nf, int t, cudaStream_t s) {
     const QrtArgs a = qrt_args(c);
     const size_t sm1 = gemm1_smem<D>(BP), sm2 = gemm2_smem<D>();
-    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP, false, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_gemm2<BP, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+    cudaError_t e = slmc::allow_smem(k_qrt_gemm1<BP, false, D>, sm1);
+    if (e == cudaSuccess) e = slmc::allow_smem(k_qrt_gemm2<BP, D>, sm2);
     if (e != cudaSuccess) return e;
     const CUtensorMap& mapV1 = BP == 32 ? c->qt_mapV1_32 : c->qt_mapV1_16;
     const int N = a.N, p = t * BP, j0 = p + BP, n_t = N - j0;
@@ -831,9 +830,9 @@ cudaError_t launch_form_q(slmc_ctx* c, int nf, cudaStream_t s) {
     const QrtArgs a = qrt_args(c);
     const int N = a.N;
     const size_t sm1 = gemm1_smem<8>(BP), sm2 = gemm2_smem<8>(), smV = sizeof(double) * (size_t)N * (BP + 1);
-    cudaError_t e = cudaFuncSetAttribute(k_qrt_gemm1<BP, true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_gemm2<BP, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_qrt_slice_V<BP, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smV);
+    cudaError_t e = slmc::allow_smem(k_qrt_gemm1<BP, true, 8>, sm1);
+    if (e == cudaSuccess) e = slmc::allow_smem(k_qrt_gemm2<BP, 8>, sm2);
+    if (e == cudaSuccess) e = slmc::allow_smem(k_qrt_slice_V<BP, 8>, smV);
     if (e != cudaSuccess) return e;
     const CUtensorMap& mapV1 = BP == 32 ? c->qt_mapV1_32 : c->qt_mapV1_16;
     const CUtensorMap& mapC = BP == 32 ? c->qt_mapC96 : c->qt_mapC112;

@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(Dim<NMAX>::threads) k_small_greens(const doubl
 template <int NMAX>
 cudaError_t launch_small_lu(slmc_ctx* c, int nf, double* lndet, int* sign, cudaStream_t s, bool assemble) {
     const size_t smem = (size_t)Dim<NMAX>::mat * sizeof(double) + sizeof(Vecs<NMAX>);
-    cudaError_t e = cudaFuncSetAttribute(k_small_lu<NMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_small_lu<NMAX>, smem);
     if (e != cudaSuccess) return e;
     k_small_lu<NMAX><<<nf, Dim<NMAX>::threads, smem, s>>>(c->U, c->Ta, c->lnD, c->Y, c->piv, c->sgnU, lndet, sign, c->err,
                                                          c->N, assemble ? 1 : 0);
@@ -174,7 +174,7 @@ cudaError_t launch_small_lu(slmc_ctx* c, int nf, double* lndet, int* sign, cudaS
 template <int NMAX>
 cudaError_t launch_small_greens(slmc_ctx* c, int nf, double* G, cudaStream_t s) {
     const size_t smem = ((size_t)Dim<NMAX>::mat + 2 * NMAX) * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_small_greens<NMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_small_greens<NMAX>, smem);
     if (e != cudaSuccess) return e;
     k_small_greens<NMAX><<<nf, Dim<NMAX>::threads, smem, s>>>(c->Y, c->piv, c->U, c->lnD, G, c->N);
     return cudaGetLastError();
@@ -183,7 +183,7 @@ cudaError_t launch_small_greens(slmc_ctx* c, int nf, double* G, cudaStream_t s) 
 template <int NMAX, int LMAX>
 cudaError_t launch_small(slmc_ctx* c, const double* x, int nf, double* lndet, int* sign, double* G, cudaStream_t s) {
     const size_t smem = 3 * (size_t)Dim<NMAX>::mat * sizeof(double) + sizeof(Vecs<NMAX>);
-    cudaError_t e = cudaFuncSetAttribute(k_small_logdet<NMAX, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_small_logdet<NMAX, LMAX>, smem);
     if (e != cudaSuccess) return e;
     k_small_logdet<NMAX, LMAX><<<nf, Dim<NMAX>::threads, smem, s>>>(x, c->kron, lndet, sign, G, c->err, c->N, c->p.Lx, c->p.Ly, c->L,
                                                          c->p.n_s, c->p.dtau * c->p.lambda, exp(c->p.dtau * c->p.mu));

@@ -226,7 +226,7 @@ cudaError_t tc_slice_group(slmc_ctx* c, const double* x, int nf, int l0, int nsl
     uint32_t* p0 = reinterpret_cast<uint32_t*>(c->tc_p[0]);
     k_tc_split_in<<<1024, 256, 0, s>>>(c->U32, c->tc_y32[0], p0, N, Npad, c->max_fields, total);
     const size_t smem = 1024 + (size_t)kStages * kNP * (128 * kAtom + (size_t)NT * kAtom);
-    cudaError_t e = cudaFuncSetAttribute(k_tc_slice, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = slmc::allow_smem(k_tc_slice, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((N + 127) / 128, (N + NT - 1) / NT, nf);
     for (int q = 0; q < nsl; ++q) {

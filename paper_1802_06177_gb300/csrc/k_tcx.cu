@@ -379,7 +379,7 @@ cudaError_t launch_group(const slmc_ctx* c, int nf, int l0, int nsl, cudaStream_
     if (fa.sharedSizeBytes + fixed + 2 * kStageBytes > limit) return cudaErrorInvalidConfiguration;
     const int stages = (int)std::min<size_t>(kMaxStages, (limit - fa.sharedSizeBytes - fixed) / kStageBytes);
     const size_t smem = fixed + (size_t)stages * kStageBytes;
-    e = cudaFuncSetAttribute(k_tcx_group<MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = slmc::allow_smem(k_tcx_group<MT, NT>, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((c->N + NT - 1) / NT, nf);
     k_tcx_group<MT, NT><<<grid, kThreads, smem, s>>>(c->tcx_mapF, c->tcx_eF, c->U32, c->Y, c->sc32, c->N, Npad,

@@ -367,15 +367,15 @@ cudaError_t t_update(slmc_ctx* c, int nf, cudaStream_t s) {
     const int CB = rows_per_block(N), RB = rows_per_block(N);
     const size_t smB = (size_t)N * (CB + 1) * sizeof(double) + (size_t)N * sizeof(int);
     const size_t smA = (size_t)RB * (N + 1) * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_tt_slice_B, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smB);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tt_slice_A, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smA);
+    cudaError_t e = slmc::allow_smem(k_tt_slice_B, smB);
+    if (e == cudaSuccess) e = slmc::allow_smem(k_tt_slice_A, smA);
     if (e != cudaSuccess) return e;
     k_tt_slice_B<<<dim3((N + CB - 1) / CB, nf), 256, smB, s>>>(c->Ta, c->perm, B, c->tt_eB, c->tt_flag, N, npad, MT,
                                                                c->fbase, pb, CB);
     k_tt_slice_A<<<dim3((N + RB - 1) / RB, nf), 256, smA, s>>>(c->QR, A, c->tt_eA, c->tt_flag, N, npad, mpad, MT,
                                                                c->fbase, pa, RB);
     const size_t smem = 1024 + 2 * (size_t)kBChunk + (size_t)kRingA * kATile;
-    e = cudaFuncSetAttribute(k_tt_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = slmc::allow_smem(k_tt_gemm, smem);
     if (e != cudaSuccess) return e;
     k_tt_gemm<<<dim3(npad / kNT, MT, nf), kThreads, smem, s>>>(c->tt_mapA, c->tt_mapB, c->tt_eA, c->tt_eB, c->tt_flag,
                                                                c->QR, c->Ta, c->perm, c->Tb, N, npad, mpad, MT,

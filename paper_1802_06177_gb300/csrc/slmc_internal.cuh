@@ -146,6 +146,15 @@ namespace slmc {
 // Stencil size of the FP32 rounding residual of F in the FP32 slice products.
 constexpr int kLoStencil = 32;
 
+// Lets a kernel be launched with that many bytes of dynamic shared memory. The limit belongs to the kernel, not to the
+// launch, and contexts of several sizes share it between host threads: it only ever grows, so no call lowers what
+// another has set before its launch.
+cudaError_t raise_smem_limit(const void* kernel, size_t bytes);
+template <typename K>
+cudaError_t allow_smem(K* kernel, size_t bytes) {
+    return raise_smem_limit(reinterpret_cast<const void*>(kernel), bytes);
+}
+
 inline int rows_per_lane_class(int N) {
     const int r = (N + 31) / 32;
     if (r <= 1) return 1;

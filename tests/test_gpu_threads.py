@@ -1,5 +1,5 @@
-"""Contexts of different sizes used by several host threads at once: the one-launch sweeps ask for shared memory by
-the chain's size, and a launch must not meet the limit that another thread's smaller chain has set meanwhile."""
+"""Contexts of different sizes used by several host threads at once: kernels ask for shared memory by the lattice's
+size, and a launch must not meet the limit that another thread's smaller lattice has set meanwhile."""
 import threading
 
 import numpy as np
@@ -13,16 +13,21 @@ pytestmark = pytest.mark.gpu
 J = np.array([0.0, 45.0, 0.6, 0.01, 0.1, 0.2])
 
 
-def test_updates_of_two_sizes_on_two_threads():
-    # 8x8, L = 100 needs 52 KB, more than a kernel has without asking; the updates loop inside the library
-    sizes, errors, out = ((8, 100, 2, 400), (4, 8, 4, 8000)), [], {}
+# Sides, slices, chains and updates of either thread, the updates looping inside the library. One-launch sweeps of 8x8,
+# L = 100 need 52 KB, more than a kernel has without asking; of 16x16 and 8x10 every kernel of a determinant differs.
+@pytest.mark.parametrize("sizes,precision", [(((8, 8, 100, 2, 400), (4, 4, 8, 4, 8000)), "fp64"),
+                                             (((16, 16, 8, 2, 400), (8, 10, 8, 2, 800)), "fp64"),
+                                             (((16, 16, 8, 2, 400), (8, 10, 8, 2, 800)), "fp32"),
+                                             (((16, 16, 8, 2, 400), (8, 10, 8, 2, 800)), "bf16x9")])
+def test_updates_of_two_sizes_on_two_threads(sizes, precision):
+    errors, out = [], {}
 
-    def work(k, Lx, L, n, updates):
+    def work(k, Lx, Ly, L, n, updates):
         try:
             with torch.cuda.stream(torch.cuda.Stream()):
-                ctx = make_ctx(Lx, L, 10, max_fields=n, sweep_delta=0.4, seed=k)
+                ctx = make_ctx(Lx, L, 10, Ly=Ly, precision=precision, max_fields=n, sweep_delta=0.4, seed=k)
                 ctx.set_wolff(1)
-                x, Jt = cuda(inputs.gaussian_fields(n, Lx, Lx, L, seed=k)), cuda(J)
+                x, Jt = cuda(inputs.gaussian_fields(n, Lx, Ly, L, seed=k)), cuda(J)
                 lnw, _ = ctx.chain_init(x, want_cdw=False)
                 ctx.cumulative_update(x, Jt, 1, updates, 0, lnw)
                 ctx.get_error()

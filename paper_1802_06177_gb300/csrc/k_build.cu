@@ -32,8 +32,8 @@ __global__ void k_hopping_exp(double* __restrict__ E, int Lx, int Ly, double dta
 // e[d] = (1/Ld) sum_n cos(2 pi n d / Ld) exp(+-2 dtau t cos(2 pi n / Ld)); the sums over
 // x and y separate because the hopping along x and along y commute. Block q of tab holds
 // [E_x | E_x^-1 | E_y | E_y^-1][q], and kKronMaxLine behind it the same less the identity. The sums go over the
-// exponentials less one: every slice multiplies by the same entries, so their rounding adds up over N L factors in ln det, and this way
-// it is that of a number ten times smaller than the diagonal.
+// exponentials less one: every slice multiplies by the same entries, so their rounding adds up over N L factors in
+// ln det, and this way it is that of a number ten times smaller than the diagonal.
 __global__ void k_kron_tables(double* __restrict__ tab, int Lx, int Ly, double dtau_t2) {
     const int q = blockIdx.x, d = threadIdx.x;
     const int Ld = q < 2 ? Lx : Ly;

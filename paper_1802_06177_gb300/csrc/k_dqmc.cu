@@ -19,8 +19,8 @@
 //    (circ.cuh): about N^2 (Lx + Ly) FP64 operations instead of the 4 N^3 of two dense products;
 //  * G stays in shared memory when it and the vectors beside it fit in 227 KB (up to N = 165), else in global memory
 //    (L2-resident). For N > 64 the accepted moves of a slice are delayed in batches (Ad, Bd in shared memory, with the
-//    running diagonal of G for the decisions) where there is room for them (up to N = 147): each new move needs only the current column and row of G, and the batch is added to G in one
-//    pass. With G in shared memory a batch is 16 moves, one K step of the tensor-instruction update of oz_line.cuh
+//    running diagonal of G for the decisions) where there is room for them (up to N = 147): each new move needs only
+//    the current column and row of G, and the batch is added to G in one pass. With G in shared memory a batch is 16 moves, one K step of the tensor-instruction update of oz_line.cuh
 //    (each entry's sum of 16 products rounded once, 56-bit digits): the N^2 FMAs per move were most of the kernel
 //    (40 slices, 128 chains, immediate / batched: 12x12 34.2 / 23.8 ms, 10x10 16.7 / 12.8, 9x8 8.6 / 7.9, 8x8 5.6 /
 //    6.0, where moves stay immediate). With G in global memory it is up to 32 moves, added by FMAs in the order of

@@ -204,11 +204,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_formq_b(const double* __restric
 // Q in FP32 (mixed modes), same arithmetic per entry as k_formq_b<BP, float> (each sum one FMA chain in the same
 // order, so the same bits) with the operands in shared memory: a warp keeps 8 columns of Q there from the first
 // panel to the last, and each phase is a register tile. W = V^T Q: a lane's four reflectors are BP / 4
-// apart, its columns 128 / BP apart, four rows per 16-byte load; W' = S W: a reflector per lane; Q -= V W': four rows per lane and
-// the warp's 8 columns. The row stride is 4 mod 32 floats, so 16-byte accesses a column apart meet no bank
-// conflicts. Reading Q's columns from global memory one broadcast word at a time, a 24x24 evaluation of
-// 32 fields (30 groups) spent 99 ms here and now 36; a 16x16 evaluation of 512 fields took 235 ms and now 218. Groups of 8 columns go round the CTAs of a field, which evens out the triangular work
-// (columns left of a panel are still unit vectors and are skipped).
+// apart, its columns 128 / BP apart, four rows per 16-byte load; W' = S W: a reflector per lane; Q -= V W': four rows
+// per lane and the warp's 8 columns. The row stride is 4 mod 32 floats, so 16-byte accesses a column apart meet no bank
+// conflicts. Groups of 8 columns go round the CTAs of a field, which evens out the triangular work (columns left of a
+// panel are still unit vectors and are skipped). A 24x24 evaluation of 32 fields (30 groups) spends 36 ms here, 99 with
+// Q's columns read from global memory one broadcast word at a time.
 template <int BP>
 __global__ void __launch_bounds__(256, 2) k_formq32(const double* __restrict__ QRall, const double* __restrict__ Sall,
                                                     float* __restrict__ Uall, int N, int ld) {

@@ -26,6 +26,8 @@
 //                    W'^T = W^T S and its slices, one exponent per trailing column;
 //   k_qrt_gemm2<BP>  C -= V W' on the tensor cores (M = rows, N = 32 trailing columns, K = BP), the
 //                    FP64 read-modify-write of C in the epilogue.
+// The same kernels form Q in FP64 and, in the chains of DQMC, the trailing updates with eight digits (56 bits) per
+// operand and levels 0..7, which leaves the error of FP64 FMAs (Dig, launch_form_q).
 // Outputs are those of k_qrb (packed QR, tau, perm, new ln D, sgnU, the panels' S). All waits are
 // clock-bounded and set SLMC_EBIT_TIMEOUT; a CTA that gives up drains its copies and frees its
 // tensor memory.
@@ -166,8 +168,9 @@ __device__ __forceinline__ void wy_triangle_blocked(const double* G, int ldg, co
 // The panel is a chain of column steps (dot products, warp reductions, square root and divisions, one block
 // barrier each), so what counts is how many panels an SM works on at once, beside the trailing updates of the
 // other sub-batches: 8 warps per field, and shared memory for rows p.. only (PanelSmem; 77 KB for the first
-// panel of N = 256, 42 KB for the fifth, against 102 KB and 16 warps before). With at most one field per SM nothing
-// shares it, and 16 warps shorten the chain (24x24, 32 fields: 656 against 665 ms per evaluation).
+// panel of N = 256, 42 KB for the fifth; with 16 warps and 102 KB whatever the panel a 16x16 evaluation of 512 fields took
+// 294 ms, with these 283). With at most one field per SM nothing shares it, and 16 warps shorten the chain (24x24, 32
+// fields: 656 against 665 ms per evaluation).
 
 // Shared memory of panel t: V (rows p.. of the panel), the last panel's S and Gram matrix, the scales, the first
 // panel's ordering keys, tau, beta, the permutation.

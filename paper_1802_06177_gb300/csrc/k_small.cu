@@ -1,6 +1,6 @@
 // FP64 determinant and Green's function of small lattices (N <= 64) in one launch, one CTA per field
-// (small.cuh holds the steps and what bounds them). The per-group kernels it replaces were launch latency at
-// these sizes: a 4x4, L = 40 determinant took about 28 launches.
+// (small.cuh holds the steps and what bounds them): the general kernels are launch latency at these sizes, about 28
+// launches for a determinant of 4x4, L = 40.
 #include <algorithm>
 
 #include "small.cuh"

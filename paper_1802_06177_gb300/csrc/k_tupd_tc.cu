@@ -23,9 +23,9 @@
 // seven A slices of each 64-wide K chunk through a 3-tile ring and the seven B slices double-buffered,
 // one thread issues the MMAs, eight warps drain the accumulators, stage the tile in shared memory
 // and write T_new row-major with coalesced stores; 32 columns per CTA keep the accumulators at
-// 7 x 32 tensor-memory columns and the shared memory near 105 KB, so two CTAs share an SM). Row-tile mt starts its K loop at row 128 mt
-// (Rt is zero to the left of its diagonal). All waits are clock-bounded as in the other
-// tensor-core kernels.
+// 7 x 32 tensor-memory columns and the shared memory near 105 KB, so two CTAs share an SM). Row-tile mt starts
+// its K loop at row 128 mt (Rt is zero to the left of its diagonal). All waits are clock-bounded as in the
+// other tensor-core kernels.
 #include <cuda_bf16.h>
 
 #include "slice7.cuh"

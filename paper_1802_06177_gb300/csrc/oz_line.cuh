@@ -7,10 +7,10 @@
 // registers. Lines of up to 16 values: 16 of them (the same line of 16 columns) are the rows of A, cut per row into
 // eight 7-bit digits against the row's power of two (as slice7.cuh with one digit more: 56 bits, so the slicing
 // error is 2^-56 of the row's largest value, below the FP64 sum's own rounding); the factor's digits, less the
-// identity (build), are B, laid out in fragment order once per CTA. The 36 products a + b <= 7 of a tile are summed per level in FP32, exactly (at most
-// 41 thousand per index of K <= 16), combined in two 64-bit integers and rounded once with integer operations: about
-// 50 integer and FP32 instructions per value and pass, no FP64. tcgen05 would need the digits in shared memory and
-// the sums back from tensor memory for 36 instructions of K = 16.
+// identity (build), are B, laid out in fragment order once per CTA. The 36 products a + b <= 7 of a tile are summed per
+// level in FP32, exactly (at most 41 thousand per index of K <= 16), combined in two 64-bit integers and rounded once
+// with integer operations: about 50 integer and FP32 instructions per value and pass, no FP64. tcgen05 would need the
+// digits in shared memory and the sums back from tensor memory for 36 instructions of K = 16.
 #pragma once
 
 #include <cuda_bf16.h>

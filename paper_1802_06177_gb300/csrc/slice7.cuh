@@ -65,7 +65,7 @@ __device__ __forceinline__ uint32_t bf16x2_of(float q0, float q1) {
 }
 
 // (hi 2^28 + lo) 2^k rounded once to FP64 (to nearest, ties to even), assembled with integer operations: the two
-// conversions, the FMA and the scaling it replaces took 64 issue cycles of the FP64 pipe per warp, the bound of
+// conversions, the FMA and the scaling of an FP64 combination take 64 issue cycles of the FP64 pipe per warp, the bound of
 // the epilogues that combine level sums. |hi| < 2^50, |lo| < 2^60.
 __device__ __forceinline__ double combine(long long hi, long long lo, int k) {
     unsigned long long l = (unsigned long long)hi << 28;

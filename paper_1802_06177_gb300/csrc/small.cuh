@@ -5,12 +5,13 @@
 //
 // What bounds it: for N <= 36 the chain of column steps; for N = 64 the FP64 pipe (an SM issues one FP64 warp
 // instruction per 16 to 19 cycles). One warp issues one per 64 cycles, however many lanes are active and however
-// independent they are, so the chain is as long as the number of FP64 instructions one warp runs in sequence. Columns are held in registers by groups of G lanes:
-// thread G j + g owns rows g, g + G, ... of column j, so a dot product is a run of FMAs per thread and log2 G
-// additions across the group (a column per warp would spend five of every nine on the reduction); square root and divisions are short Newton forms, the two divisions of a
-// reflector in neighbouring lanes of one instruction stream; and a group's slice scales are exponentiated
-// together before its slices. 64 fields of 4x4, L = 40 with G: 784 us by per-step kernels, 401 us by the first
-// version of this kernel, 326 us with folded transforms, 241 us now.
+// independent they are, so the chain is as long as the number of FP64 instructions one warp runs in sequence. Columns
+// are held in registers by groups of G lanes: thread G j + g owns rows g, g + G, ... of column j, so a dot product is a
+// run of FMAs per thread and log2 G additions across the group (a column per warp would spend five of every nine on the
+// reduction); square root and divisions are short Newton forms, the two divisions of a reflector in neighbouring lanes
+// of one instruction stream; and a group's slice scales are exponentiated together before its slices. With G, L = 40,
+// 64 fields of 4x4 take 242 us (general kernels, a launch per step: 784), 16 of 2x32 2.3 ms (5.0), although the instance
+// for lines of 17 to 32 sites spills (2.7 KB of registers per thread).
 //
 // Matrices in shared memory: element (r, c) of a column-major one at c * ld + r, of a row-major one at
 // r * ld + c, ld = NMAX + 1; rows and columns beyond N are zero.
@@ -57,8 +58,8 @@ __device__ __forceinline__ double group_sum(double v) {
 }
 
 // One pass of a transform over short lines (n <= 8, the 4x4 class): two lanes per line, each half of the outputs by
-// direct sums (t: the factor less the identity). At this size the folded transform's chain (18 FP64 instructions for a line of 4 on two warps) is
-// longer than eight direct ones on four.
+// direct sums (t: the factor less the identity). At this size the folded transform's chain (18 FP64 instructions for a
+// line of 4 on two warps) is longer than eight direct ones on four.
 template <int n>
 __device__ __forceinline__ void half_line(double* g, int stride, const double* __restrict__ t, int half,
                                           const double* out_sc, bool on) {

@@ -947,7 +947,7 @@ def run_dqmc(args):
             "config": {"workload": wl.name, "model": "holstein_2d", "N": N, "Lx": Lx, "L": L, "n_s": wl.n_s,
                        "chains_per_gpu": nf, "block_updates_per_sweep": args.dqmc_block, "sweep_delta": 0.5,
                        "parallelism": "replicas x%d" % world,
-                       "l2": "per-chain G in shared memory (N <= 160) or L2; fields %.0f MB" % (h2d / 1e6)},
+                       "l2": "per-chain G in shared memory (N <= 165) or L2; fields %.0f MB" % (h2d / 1e6)},
             "e2e": {"value": nf * world / (e2e_ms / 1e3), "unit": DQMC_UNIT, "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": h2d + 8 * nf},
             "gpu_launches": launches, "roofline": roof, "cpu_baseline": cpu, "clocks": clk,

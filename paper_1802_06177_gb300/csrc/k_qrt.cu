@@ -64,7 +64,8 @@ constexpr int kDMax = 8;
 template <int D>
 struct Dig {
     // K chunks (64 rows) per accumulator set of W^T = C^T V: a level's sum of absolute terms is at most 36864 per K
-    // index with seven digits, 40960 with eight, and stays below 2^24
+    // index with seven digits, 40960 with eight, and stays below 2^24. Tensor memory holds two sets of eight levels of 32
+    // reflectors (panels of 32 end at N = 667, eleven chunks) or four of 16 (three needed at N = 896)
     static constexpr int kSegChunks = D == 7 ? 7 : 6;
     // the digits' units 2^(e - 6) per operand and the level weights 2^(-7 level)
     static constexpr int kUnitShift = 2 * 6 + 7 * (D - 1);
